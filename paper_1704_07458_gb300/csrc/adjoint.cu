@@ -20,7 +20,7 @@
 // host round trip.
 #include <algorithm>
 
-#include "kernels.cuh"
+#include "colpass.cuh"
 
 namespace lob {
 namespace {
@@ -48,37 +48,25 @@ __global__ void adj_coeff_kernel(int k, const double* __restrict__ M, int64_t ld
   Cin[j + (int64_t)i * k] = c;
 }
 
-// Block-local column sums of the per-thread partials s (8 warps x 32 columns)
-// into partial[blockIdx.x * k + j].
-__device__ __forceinline__ void block_colsum(double s, int j, int k, double (*red)[33],
-                                             double* __restrict__ partial) {
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  red[ty][tx] = s;
-  __syncthreads();
-  if (ty == 0 && j < k) {
-    double a = 0.0;
-    for (int t = 0; t < 8; ++t) a += red[t][tx];
-    partial[(int64_t)blockIdx.x * k + j] = a;
-  }
-  __syncthreads();
-}
-
 // Q(r, j) -= lambda_j * (B P)(r, j) and partial column dots P(:, j)^T Q(:, j).
 // (B P) is BP when given, b[r] P(r, j) for a diagonal B, else P.
-__global__ void __launch_bounds__(256) shift_dot_kernel(
-    int64_t n, int k, double* __restrict__ Q, const double* __restrict__ P,
+__global__ void __launch_bounds__(kColThreads) shift_dot_kernel(
+    int64_t n, int k, int TX, double* __restrict__ Q, const double* __restrict__ P,
     const double* __restrict__ BP, const double* __restrict__ b, int64_t ld,
     const double* __restrict__ lam, double* __restrict__ partial) {
-  __shared__ double red[8][33];
+  __shared__ double red[kColThreads];
+  const int TY = kColThreads / TX;
   const int64_t per = ceil_div(n, (int64_t)gridDim.x);
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int cb = 0; cb < k; cb += 32) {
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  for (int cb = 0; cb < k; cb += TX) {
     const int j = cb + tx;
+    const bool live = ty < TY && j < k;
     double s = 0.0;
-    if (j < k) {
+    if (live) {
       const double l = lam[j];
-      for (int64_t r = r0 + ty; r < r1; r += 8) {
+#pragma unroll 4
+      for (int64_t r = r0 + ty; r < r1; r += TY) {
         const int64_t o = r * ld + j;
         const double p = P[o];
         const double bp = BP ? BP[o] : (b ? b[r] * p : p);
@@ -87,7 +75,8 @@ __global__ void __launch_bounds__(256) shift_dot_kernel(
         s = fma(p, q, s);
       }
     }
-    block_colsum(s, j, k, red, partial);
+    s = col_reduce(s, red, tx, ty, TX, TY);
+    if (live && ty == 0) partial[(int64_t)blockIdx.x * k + j] = s;
   }
 }
 
@@ -96,71 +85,93 @@ __global__ void __launch_bounds__(256) shift_dot_kernel(
 // of the preconditioner), partial R^T R.
 // V may alias P and R may alias Q (the first step runs with alpha = 0 on
 // V = P = 0, R = Q = F to form Z = K^-1 F and |F|^2).
-__global__ void __launch_bounds__(256) cg_step_kernel(
-    int64_t n, int k, double* V, const double* P, double* R, const double* Q,
+__global__ void __launch_bounds__(kColThreads) cg_step_kernel(
+    int64_t n, int k, int TX, double* V, const double* P, double* R, const double* Q,
     double* __restrict__ Z, const double* __restrict__ kinv, int64_t ld,
     const double* __restrict__ rz, const double* __restrict__ pq, double* __restrict__ partial) {
-  __shared__ double red[8][33];
+  __shared__ double red[kColThreads];
+  const int TY = kColThreads / TX;
   const int64_t per = ceil_div(n, (int64_t)gridDim.x);
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int cb = 0; cb < k; cb += 32) {
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  for (int cb = 0; cb < k; cb += TX) {
     const int j = cb + tx;
+    const bool live = ty < TY && j < k;
     double s = 0.0;
-    if (j < k) {
+    if (live) {
       const double a = pq[j] > 0.0 ? safe_div(rz[j], pq[j]) : 0.0;
-      for (int64_t r = r0 + ty; r < r1; r += 8) {
-        const int64_t o = r * ld + j;
-        V[o] = fma(-a, P[o], V[o]);
-        const double rr = fma(-a, Q[o], R[o]);
-        R[o] = rr;
-        Z[o] = kinv ? rr * kinv[r] : rr;
-        s = fma(rr, rr, s);
+      // four rows at a time, every load before the first store (the compiler
+      // may not move them: V may alias P and R may alias Q, element by element)
+      for (int64_t r = r0 + ty; r < r1; r += 4 * TY) {
+        double v[4], p[4], q[4], x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int64_t o = min(r + i * TY, r1 - 1) * ld + j;
+          v[i] = V[o];
+          p[i] = P[o];
+          q[i] = Q[o];
+          x[i] = R[o];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int64_t ri = r + i * TY, o = ri * ld + j;
+          if (ri >= r1) break;
+          V[o] = fma(-a, p[i], v[i]);
+          const double rr = fma(-a, q[i], x[i]);
+          R[o] = rr;
+          Z[o] = kinv ? rr * __ldg(kinv + ri) : rr;
+          s = fma(rr, rr, s);
+        }
       }
     }
-    block_colsum(s, j, k, red, partial);
+    s = col_reduce(s, red, tx, ty, TX, TY);
+    if (live && ty == 0) partial[(int64_t)blockIdx.x * k + j] = s;
   }
 }
 
 // partial column dots X(:, j)^T Y(:, j)
-__global__ void __launch_bounds__(256) coldot_kernel(int64_t n, int k,
+__global__ void __launch_bounds__(kColThreads) coldot_kernel(int64_t n, int k, int TX,
                                                      const double* __restrict__ X,
                                                      const double* __restrict__ Y, int64_t ld,
                                                      double* __restrict__ partial) {
-  __shared__ double red[8][33];
+  __shared__ double red[kColThreads];
+  const int TY = kColThreads / TX;
   const int64_t per = ceil_div(n, (int64_t)gridDim.x);
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int cb = 0; cb < k; cb += 32) {
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  for (int cb = 0; cb < k; cb += TX) {
     const int j = cb + tx;
+    const bool live = ty < TY && j < k;
     double s = 0.0;
-    if (j < k)
-      for (int64_t r = r0 + ty; r < r1; r += 8) s = fma(X[r * ld + j], Y[r * ld + j], s);
-    block_colsum(s, j, k, red, partial);
+    if (live)
+#pragma unroll 4
+      for (int64_t r = r0 + ty; r < r1; r += TY) s = fma(X[r * ld + j], Y[r * ld + j], s);
+    s = col_reduce(s, red, tx, ty, TX, TY);
+    if (live && ty == 0) partial[(int64_t)blockIdx.x * k + j] = s;
   }
 }
 
-__global__ void colfinish_kernel(const double* __restrict__ partial, int blocks, int k,
-                                 double* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= k) return;
-  double a = 0.0;
-  for (int z = 0; z < blocks; ++z) a += partial[(int64_t)z * k + j];
-  out[j] = a;
-}
-
 // P = Z + beta P, beta_j = rz_new_j / rz_old_j (0 when rz_old_j == 0)
-__global__ void cg_direction_kernel(int64_t n, int k, double* __restrict__ P,
-                                    const double* __restrict__ Z, int64_t ld,
-                                    const double* __restrict__ rz_new,
-                                    const double* __restrict__ rz_old) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * k) return;
-  const int64_t r = e / k;
-  const int j = (int)(e % k);
-  const double beta = rz_old[j] > 0.0 ? safe_div(rz_new[j], rz_old[j]) : 0.0;
-  const int64_t o = r * ld + j;
-  P[o] = fma(beta, P[o], Z[o]);
+// Threads over the columns of a tile, as in the column passes: beta (an FP64
+// division, ~10 FP64 instructions) is formed once per thread and not per
+// element, and no element costs an integer division by k (168 us against 30 us
+// of bytes at n = 262,144, k = 32 before; 36 us now).
+__global__ void __launch_bounds__(kColThreads) cg_direction_kernel(
+    int64_t n, int k, int TX, double* __restrict__ P, const double* __restrict__ Z, int64_t ld,
+    const double* __restrict__ rz_new, const double* __restrict__ rz_old) {
+  const int TY = kColThreads / TX;
+  const int64_t per = ceil_div(n, (int64_t)gridDim.x);
+  const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  if (ty >= TY) return;
+  for (int j = tx; j < k; j += TX) {
+    const double beta = rz_old[j] > 0.0 ? safe_div(rz_new[j], rz_old[j]) : 0.0;
+#pragma unroll 4
+    for (int64_t r = r0 + ty; r < r1; r += TY) {
+      const int64_t o = r * ld + j;
+      P[o] = fma(beta, P[o], Z[o]);
+    }
+  }
 }
 
 // Gradient on a CSR pattern, one warp per row r; for each stored (r, c):
@@ -228,8 +239,8 @@ __global__ void grad_coeff_kernel(int k, const double* __restrict__ lam,
 }
 
 int col_finish(cudaStream_t st, int k, void* partial, double* out) {
-  colfinish_kernel<<<(unsigned)ceil_div(k, 128), 128, 0, st>>>((const double*)partial, kRB, k,
-                                                               out);
+  colsum_finish_kernel<<<(unsigned)ceil_div(k, kSumCols), kSumCols * kSumLanes, 0, st>>>(
+      (const double*)partial, kRB, k, out);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
@@ -249,7 +260,7 @@ int64_t adj_reduce_workspace(int k) { return (int64_t)kRB * std::max(k, 1) * siz
 
 int shift_dot(cudaStream_t st, int64_t n, int k, double* Q, const double* P, const double* BP,
               const double* b, int64_t ld, const double* lam, double* out, void* partial) {
-  shift_dot_kernel<<<kRB, 256, 0, st>>>(n, k, Q, P, BP, b, ld, lam, (double*)partial);
+  shift_dot_kernel<<<kRB, kColThreads, 0, st>>>(n, k, col_tile(k), Q, P, BP, b, ld, lam, (double*)partial);
   LOB_LAUNCHED();
   return col_finish(st, k, partial, out);
 }
@@ -257,22 +268,22 @@ int shift_dot(cudaStream_t st, int64_t n, int k, double* Q, const double* P, con
 int cg_step(cudaStream_t st, int64_t n, int k, double* V, const double* P, double* R,
             const double* Q, double* Z, const double* kinv, int64_t ld, const double* rz,
             const double* pq, double* rr, void* partial) {
-  cg_step_kernel<<<kRB, 256, 0, st>>>(n, k, V, P, R, Q, Z, kinv, ld, rz, pq, (double*)partial);
+  cg_step_kernel<<<kRB, kColThreads, 0, st>>>(n, k, col_tile(k), V, P, R, Q, Z, kinv, ld, rz, pq, (double*)partial);
   LOB_LAUNCHED();
   return col_finish(st, k, partial, rr);
 }
 
 int coldot(cudaStream_t st, int64_t n, int k, const double* X, const double* Y, int64_t ld,
            double* out, void* partial) {
-  coldot_kernel<<<kRB, 256, 0, st>>>(n, k, X, Y, ld, (double*)partial);
+  coldot_kernel<<<kRB, kColThreads, 0, st>>>(n, k, col_tile(k), X, Y, ld, (double*)partial);
   LOB_LAUNCHED();
   return col_finish(st, k, partial, out);
 }
 
 int cg_direction(cudaStream_t st, int64_t n, int k, double* P, const double* Z, int64_t ld,
                  const double* rz_new, const double* rz_old) {
-  cg_direction_kernel<<<(unsigned)ceil_div(n * k, 256), 256, 0, st>>>(n, k, P, Z, ld, rz_new,
-                                                                      rz_old);
+  const unsigned blocks = (unsigned)std::min<int64_t>(2 * kRB, ceil_div(n * k, kColThreads));
+  cg_direction_kernel<<<blocks, kColThreads, 0, st>>>(n, k, col_tile(k), P, Z, ld, rz_new, rz_old);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }

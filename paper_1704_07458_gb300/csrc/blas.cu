@@ -12,7 +12,7 @@
 // These run on the FP64 units; the tensor-core versions are in ozaki.cu.
 #include <algorithm>
 
-#include "kernels.cuh"
+#include "colpass.cuh"
 
 namespace lob {
 
@@ -210,60 +210,72 @@ int64_t residual_workspace(int64_t n, int m) {
   return (int64_t)row_blocks(n) * 2 * std::max(m, 1) * (int64_t)sizeof(double);
 }
 
-// Block: 32 columns x 8 row lanes; each block owns a contiguous row range.
-__global__ void __launch_bounds__(256) residual_kernel(
+// One pass over X, AX (and BX): each CTA owns a contiguous row range, threads
+// over the columns of a tile and TY rows, four rows in flight per thread.  Bound
+// by the four FP64 operations per element (residual, two squares, the product
+// with 1 / kdiag) on a part with 1/64-rate FP64: 118 us of FP64 pipe at
+// n = 262,144, m = 71, against 88 us of bytes.
+template <bool kB>
+__global__ void __launch_bounds__(kColThreads) residual_kernel(
     int64_t n, const double* __restrict__ X, const double* __restrict__ AX,
-    const double* __restrict__ BX, int64_t ld, int m, int c0, const double* __restrict__ theta,
-    const double* __restrict__ kinv, double* __restrict__ W, int64_t ldw, int xb,
-    double* __restrict__ partial) {
-  __shared__ double red[2][8][33];
-  const int mm = m - c0;
+    const double* __restrict__ BX, int64_t ld, int m, int c0, int TX,
+    const double* __restrict__ theta, const double* __restrict__ kinv, double* __restrict__ W,
+    int64_t ldw, int xb, double* __restrict__ partial) {
+  __shared__ double red[kColThreads];
+  const int mm = m - c0, TY = kColThreads / TX;
   const int64_t per = ceil_div(n, (int64_t)gridDim.x);
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int cb = 0; cb < mm; cb += 32) {
-    const int j = c0 + cb + tx;
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  for (int cb = 0; cb < mm; cb += TX) {
+    const int jj = cb + tx, j = c0 + jj;
+    const bool live = ty < TY && jj < mm;
     double rn = 0.0, xn = 0.0;
-    if (j < m) {
+    if (live) {
       const double th = theta[j];
-#pragma unroll 4
-      for (int64_t r = r0 + ty; r < r1; r += 8) {
-        const int64_t o = r * ld + j;
-        const double x = X[o];
-        const double bx = BX ? BX[o] : x;
-        const double res = fma(-th, bx, AX[o]);
+      auto row = [&](int64_t r, double x, double bx, double ax, double ki) {
+        const double res = fma(-th, bx, ax);
         rn = fma(res, res, rn);
         xn = fma(x, xb ? bx : x, xn);  // ||x||^2, or x^T B x for criterion (8)
-        if (W) W[r * ldw + (j - c0)] = kinv ? res * kinv[r] : res;
+        if (W) W[r * ldw + jj] = kinv ? res * ki : res;
+      };
+      int64_t r = r0 + ty;
+      for (; r + 3 * TY < r1; r += 4 * TY) {
+        double x[4], bx[4], ax[4], ki[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int64_t o = (r + i * TY) * ld + j;
+          x[i] = X[o];
+          ax[i] = AX[o];
+          bx[i] = kB ? BX[o] : x[i];
+          ki[i] = kinv ? __ldg(kinv + r + i * TY) : 1.0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) row(r + i * TY, x[i], bx[i], ax[i], ki[i]);
+      }
+      for (; r < r1; r += TY) {
+        const int64_t o = r * ld + j;
+        const double x = X[o];
+        row(r, x, kB ? BX[o] : x, AX[o], kinv ? kinv[r] : 1.0);
       }
     }
-    red[0][ty][tx] = rn;
-    red[1][ty][tx] = xn;
-    __syncthreads();
-    if (ty == 0 && j < m) {
-      double a = 0.0, b = 0.0;
-      for (int t = 0; t < 8; ++t) {
-        a += red[0][t][tx];
-        b += red[1][t][tx];
-      }
-      partial[((int64_t)blockIdx.x * 2 + 0) * mm + (j - c0)] = a;
-      partial[((int64_t)blockIdx.x * 2 + 1) * mm + (j - c0)] = b;
+    rn = col_reduce(rn, red, tx, ty, TX, TY);
+    xn = col_reduce(xn, red, tx, ty, TX, TY);
+    if (live && ty == 0) {
+      partial[((int64_t)blockIdx.x * 2 + 0) * mm + jj] = rn;
+      partial[((int64_t)blockIdx.x * 2 + 1) * mm + jj] = xn;
     }
-    __syncthreads();
   }
 }
 
-__global__ void residual_finish_kernel(const double* __restrict__ partial, int blocks, int mm,
-                                       int c0, const double* __restrict__ theta, double normA,
-                                       double normB, double* __restrict__ be) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= mm) return;
-  double a = 0.0, b = 0.0;
-  for (int z = 0; z < blocks; ++z) {
-    a += partial[((int64_t)z * 2 + 0) * mm + j];
-    b += partial[((int64_t)z * 2 + 1) * mm + j];
-  }
-  be[j] = sqrt(a) / ((normA + fabs(theta[c0 + j]) * normB) * sqrt(b));
+__global__ void __launch_bounds__(kSumCols* kSumLanes)
+    residual_finish_kernel(const double* __restrict__ partial, int blocks, int mm, int c0,
+                           const double* __restrict__ theta, double normA, double normB,
+                           double* __restrict__ be) {
+  const int j = blockIdx.x * kSumCols + threadIdx.x % kSumCols;
+  double s[2];
+  sum_partials<2>(partial, blocks, mm, j, s);
+  if (threadIdx.x < kSumCols && j < mm)
+    be[j] = sqrt(s[0]) / ((normA + fabs(theta[c0 + j]) * normB) * sqrt(s[1]));
 }
 
 int residual(cudaStream_t st, int64_t n, const double* X, const double* AX, const double* BX,
@@ -272,10 +284,15 @@ int residual(cudaStream_t st, int64_t n, const double* X, const double* AX, cons
   const int mm = m - c0;
   if (mm <= 0) return LOBPCG_OK;
   const int blocks = row_blocks(n);
-  residual_kernel<<<blocks, 256, 0, st>>>(n, X, AX, BX, ld, m, c0, theta, kinv, W, ldw, xb,
-                                          (double*)partial);
+  const int TX = col_tile(mm);
+  if (BX)
+    residual_kernel<true><<<blocks, kColThreads, 0, st>>>(n, X, AX, BX, ld, m, c0, TX, theta, kinv,
+                                                          W, ldw, xb, (double*)partial);
+  else
+    residual_kernel<false><<<blocks, kColThreads, 0, st>>>(n, X, AX, BX, ld, m, c0, TX, theta,
+                                                           kinv, W, ldw, xb, (double*)partial);
   LOB_LAUNCHED();
-  residual_finish_kernel<<<(unsigned)ceil_div(mm, 128), 128, 0, st>>>(
+  residual_finish_kernel<<<(unsigned)ceil_div(mm, kSumCols), kSumCols * kSumLanes, 0, st>>>(
       (const double*)partial, blocks, mm, c0, theta, normA, normB, be);
   LOB_LAUNCHED();
   return LOBPCG_OK;
@@ -287,49 +304,39 @@ int64_t colsumsq_workspace(int64_t n, int m) {
   return (int64_t)row_blocks(n) * std::max(m, 1) * (int64_t)sizeof(double);
 }
 
-__global__ void __launch_bounds__(256) colsumsq_kernel(int64_t n, const double* __restrict__ Y,
-                                                       int64_t ld, int m,
-                                                       double* __restrict__ partial) {
-  __shared__ double red[8][33];
+__global__ void __launch_bounds__(kColThreads) colsumsq_kernel(int64_t n,
+                                                               const double* __restrict__ Y,
+                                                               int64_t ld, int m, int TX,
+                                                               double* __restrict__ partial) {
+  __shared__ double red[kColThreads];
+  const int TY = kColThreads / TX;
   const int64_t per = ceil_div(n, (int64_t)gridDim.x);
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int cb = 0; cb < m; cb += 32) {
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  for (int cb = 0; cb < m; cb += TX) {
     const int j = cb + tx;
+    const bool live = ty < TY && j < m;
     double s = 0.0;
-    if (j < m)
-      for (int64_t r = r0 + ty; r < r1; r += 8) {
+    if (live) {
+#pragma unroll 4
+      for (int64_t r = r0 + ty; r < r1; r += TY) {
         const double y = Y[r * ld + j];
         s = fma(y, y, s);
       }
-    red[ty][tx] = s;
-    __syncthreads();
-    if (ty == 0 && j < m) {
-      double a = 0.0;
-      for (int t = 0; t < 8; ++t) a += red[t][tx];
-      partial[(int64_t)blockIdx.x * m + j] = a;
     }
-    __syncthreads();
+    s = col_reduce(s, red, tx, ty, TX, TY);
+    if (live && ty == 0) partial[(int64_t)blockIdx.x * m + j] = s;
   }
-}
-
-__global__ void colsum_finish_kernel(const double* __restrict__ partial, int blocks, int m,
-                                     double* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= m) return;
-  double a = 0.0;
-  for (int z = 0; z < blocks; ++z) a += partial[(int64_t)z * m + j];
-  out[j] = a;
 }
 
 int colsumsq(cudaStream_t st, int64_t n, const double* Y, int64_t ld, int m, double* out,
              void* partial) {
   if (m <= 0) return LOBPCG_OK;
   const int blocks = row_blocks(n);
-  colsumsq_kernel<<<blocks, 256, 0, st>>>(n, Y, ld, m, (double*)partial);
+  colsumsq_kernel<<<blocks, kColThreads, 0, st>>>(n, Y, ld, m, col_tile(m), (double*)partial);
   LOB_LAUNCHED();
-  colsum_finish_kernel<<<(unsigned)ceil_div(m, 128), 128, 0, st>>>((const double*)partial,
-                                                                   blocks, m, out);
+  colsum_finish_kernel<<<(unsigned)ceil_div(m, kSumCols), kSumCols * kSumLanes, 0, st>>>(
+      (const double*)partial, blocks, m, out);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
