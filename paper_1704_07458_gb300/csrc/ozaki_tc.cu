@@ -11,7 +11,7 @@
 //
 // GB300 mapping:
 //  * one CTA per SM owns a 128 x NT output tile (Gram: 256 threads; update:
-//    512 compute threads and one issuer warp),
+//    512 compute threads and a helper warpgroup),
 //    NT <= 96 a multiple of 16: tcgen05.mma kind::f16, M = 128, N = NT, K = 16;
 //  * the contraction runs in chunks of 16 (rows of U and V for the Gram,
 //    columns of S for the update), grouped in blocks of 256 that share one
@@ -21,12 +21,11 @@
 //    2^-24 resp. 2^-32 of level 0) share one inexact accumulator.  4 or 5
 //    accumulators x NT columns fit the 512 TMEM columns, and TMEM is read once
 //    per block instead of once per chunk;
-//  * the raw FP64 operands stream into three shared-memory stages by cp.async,
-//    two chunks ahead of use, so that no thread waits on a global load; the
-//    tensor core multiplies chunk c while the compute threads cut chunk c + 1
-//    (two digit-plane stages in the Gram, three in the update); the digits of
-//    the small matrix C of the update are cut once per call and arrive by
-//    cp.async.bulk two chunks ahead;
+//  * Gram: the raw FP64 operands stream into three shared-memory stages by
+//    cp.async, two chunks ahead of use; the tensor core multiplies chunk c while
+//    the compute threads cut chunk c + 1 (two digit-plane stages).  Update: see
+//    its kernel; the digits of the small matrix C are cut once per call and
+//    arrive by cp.async.bulk four chunks ahead;
 //  * the shared exponents come from a streaming pre-pass at full occupancy
 //    (per 256-row block and column for the Gram, per row for the update), so
 //    the tensor-core kernels never wait on a global load of their own;
@@ -34,6 +33,7 @@
 //    (and, for the update, sets a status bit that the solver reads with its
 //    per-iteration scalars) and the CTA returns instead of hanging.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.cuh"
 #include "ozaki_common.cuh"
@@ -106,6 +106,96 @@ __device__ __forceinline__ void digits(double x, int E, float (&d)[S]) {
   d[0] = (float)(int)(G >> (8 * (S - 1)));
 }
 
+// The same digits with about half the instructions, for exponent bounds away
+// from the ends of the range: every step is a 32-bit operation.  ke is
+// (digit_ke<S>() + E) << 20 modulo 2^32.  With M = the 53-bit mantissa at the
+// top of 64 bits, F' = M >> q keeps 8 bits below the last digit; one's
+// complement for a negative x and 0x80 added to every byte then round half up
+// in magnitude (the byte below the last digit) and balance the digits at once,
+// so byte b of the sum is digit + 128.  S = 7 has no room for those 8 bits:
+// one rounding bit, and the low byte is the last digit.  Needs 64 <= q for a
+// zero or subnormal x (its implicit bit is set here), so E > kFastEMin, and
+// E < kFastEMax for q < 4096.
+constexpr int kFastEMin = -900, kFastEMax = 1500;
+constexpr int kEZeroFast = 1100;  // stands for kEZero: every shift clears the value
+
+template <int S>
+__host__ __device__ constexpr int digit_ke() { return 1079 - 8 * S + (S >= 7 ? 7 : 0); }
+
+template <int S>
+__device__ __forceinline__ uint2 biased_bytes(double x, uint32_t ke) {
+  const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
+  const uint32_t q = (ke - (xh & 0x7FF00000u)) >> 20;
+  const uint32_t mh = (xh & 0x000FFFFFu) | 0x00100000u;
+  const uint32_t Mh = __funnelshift_l(xl, mh, 11), Ml = xl << 11;
+  // 64-bit right shift by any q: the shifts clamp at 32 instead of wrapping
+  uint32_t Fl, Fh;
+  asm("shr.u32 %0, %1, %2;\n" : "=r"(Fh) : "r"(Mh), "r"(q));
+  asm("shr.u32 %0, %1, %2;\n"
+      : "=r"(Fl)
+      : "r"(__funnelshift_rc(Ml, Mh, q)), "r"((uint32_t)max((int)q - 32, 0)));
+  const uint32_t sg = (uint32_t)((int)xh >> 31);
+  constexpr unsigned long long bias =
+      S >= 7 ? 0x0080808080808080ULL : (0x8080808080808080ULL >> (8 * (7 - S)));
+  uint2 g;
+  if (S >= 7) {  // round half up, then two's complement
+    asm("add.cc.u32 %0, %0, 1;\n\taddc.u32 %1, %1, 0;\n" : "+r"(Fl), "+r"(Fh));
+    Fl = __funnelshift_r(Fl, Fh, 1);
+    Fh >>= 1;
+    Fl ^= sg;
+    Fh ^= sg;
+    asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %2;\n" : "+r"(Fl), "+r"(Fh) : "r"(sg));
+  } else {
+    Fl ^= sg;
+    Fh ^= sg;
+  }
+  asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %4, %5;\n"
+      : "=r"(g.x), "=r"(g.y)
+      : "r"(Fl), "r"((uint32_t)bias), "r"(Fh), "r"((uint32_t)(bias >> 32)));
+  return g;
+}
+
+// pre-weighted digit s of a biased fixed-point value, as a float exact in BF16
+template <int S, int s>
+__device__ __forceinline__ float byte_digit(uint2 g) {
+  constexpr int b = S - 1 - s + (S >= 7 ? 0 : 1);
+  uint32_t t;
+  if (s == 0) {  // nine bits: the leading digit reaches +128
+    t = b == 3 ? __byte_perm(__byte_perm(g.x, g.y, 0x4343), 0x4B000000u, 0x7410)
+               : __byte_perm(b < 4 ? g.x : g.y, 0x4B000000u, 0x7400u | ((b & 3) + 1) << 4 | (b & 3));
+  } else {
+    t = __byte_perm(b < 4 ? g.x : g.y, 0x4B000000u, 0x7540u | (uint32_t)(b & 3));
+  }
+  // 0x4B000000 + u is 2^23 + u as a float; minus (2^23 + 128), scaled by 2^-8s (exact)
+  const float sc = __uint_as_float((uint32_t)(127 - 8 * s) << 23);
+  return fmaf(__uint_as_float(t), sc, -8388736.0f * sc);
+}
+
+// plane s of 8 consecutive K values: four packed BF16 pairs
+template <int S, int s>
+__device__ __forceinline__ void plane8(const uint2 (&g)[8], uint32_t (&w)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    w[i] = __byte_perm(__float_as_uint(byte_digit<S, s>(g[2 * i])),
+                       __float_as_uint(byte_digit<S, s>(g[2 * i + 1])), 0x7632);
+}
+
+// the biased fixed-point value of the general split: any exponent bound
+template <int S>
+__device__ __noinline__ uint2 biased_bytes_any(double x, int E) {
+  const long long bits = __double_as_longlong(x);
+  const int be = (int)((bits >> 52) & 0x7FF);
+  const long long mant = (bits & 0x000FFFFFFFFFFFFFLL) | ((long long)(be != 0) << 52);
+  const int t = min(max(2 - (max(be, 1) - 1076 + 8 * S - E), 0), 63);
+  const long long F = (((mant << 3) >> t) + 1) >> 1;
+  long long G = bits < 0 ? -F : F;
+  constexpr unsigned long long bias =
+      S >= 7 ? 0x0080808080808080ULL : (0x8080808080808080ULL >> (8 * (7 - S)));
+  if (S < 7) G *= 256;
+  const unsigned long long B = (unsigned long long)G + bias;
+  return make_uint2((uint32_t)B, (uint32_t)(B >> 32));
+}
+
 // 8 consecutive K values of one M/N index -> S planes, one 16-byte shared
 // store per plane (K-major core-matrix row: 8 BF16 along K).
 template <int S>
@@ -162,6 +252,26 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
       : "r"(taddr));
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float v[4]) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// One lane of the (converged) warp.  An elected lane, unlike a test of the
+// thread index, is known to be the only one, so MMA operands stay in uniform
+// registers instead of being moved there lane by lane.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.b32 %0, 1, 0, P;\n\t}\n"
+      : "=r"(p));
+  return p != 0;
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
@@ -249,19 +359,55 @@ __device__ __forceinline__ long long shr_sat(long long v, int k) {
   return k <= 0 ? v : (k > 62 ? 0 : (v >> k));
 }
 
-// v * 2^e + y0 rounded to FP64 (error below 1 ulp), integer operations only.
-__device__ __forceinline__ double assemble_i64(long long v, int e, double y0) {
-  if ((__double_as_longlong(y0) << 1) == 0) return int_to_double_fast(v, e);  // y0 = +-0, no FP64 op
-  long long my;
-  int ey;
-  double_parts(y0, my, ey);
-  if (v == 0) return y0;
-  const int top = max(e + bitlen(v), ey + bitlen(my));
-  const int base = top - 61;
-  const int kv = e - base, ky = ey - base;
-  const long long a = kv >= 0 ? (v << kv) : shr_sat(v, -kv);
-  const long long b = ky >= 0 ? (my << ky) : shr_sat(my, -ky);
-  return int_to_double(a + b, base);
+// v * 2^e in FP64 for the usual case |v| < 2^51 and a normal result: the
+// integer is added to the bits of 1.5 * 2^52, one FP64 subtraction (exact)
+// normalises it, and the exponent field takes e.  One FP64 instruction per
+// output is pipe time that nothing else uses and replaces a 64-bit leading
+// zero count, two variable shifts and a rounding.
+__device__ __forceinline__ double i64_scaled(long long v, int e) {
+  const int hi = (int)(v >> 32);
+  if ((unsigned)(hi + 0x00080000) < 0x00100000u) {
+    const double d = __hiloint2double(hi + 0x43380000, (int)v) - 6755399441055744.0;
+    const int dh = __double2hiint(d);
+    if ((unsigned)(((dh >> 20) & 0x7FF) + e - 1) < 2046u && v != 0)
+      return __hiloint2double(dh + (int)((unsigned)e << 20), __double2loint(d));
+  }
+  return int_to_double(v, e);
+}
+
+// float -> int without the conversion unit (which takes 16 values per clock
+// and SM): f + kMagic for |f| <= 2^22 holds the integer nearest f in its low
+// mantissa bits, as_int(f + kMagic) - kMagicInt.
+constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+constexpr int kMagicInt = 0x4B400000;
+
+// The accumulators of one output as in acc_to_i64, summed by wide
+// multiply-adds.  Four conversions per output would bound the drain of TMEM
+// (32 cycles per warp and output on the conversion unit), during which the
+// tensor core waits, so levels 0 and 1 go through the FP32 adder: level 0 is an
+// integer of at most 2^22, level 1 of at most 2^23 in units of 2^-8, split into
+// 2 h + l.  The integer offsets of the magic constant leave by one constant.
+template <int S>
+__device__ __forceinline__ long long acc_sum(const float (&v)[5]) {
+  constexpr int NA = nacc<S>();
+  static_assert(NA >= 3, "levels 0 and 1 have accumulators of their own");
+  const float hm = fmaf(v[1], 128.0f, kMagic), h = hm - kMagic;
+  const float lm = fmaf(v[1], 256.0f, -2.0f * h) + kMagic;
+  const int i0 = __float_as_int(v[0] + kMagic);
+  const int i1 = 2 * __float_as_int(hm) + __float_as_int(lm);  // modulo 2^32, offset below
+  long long T = 0;
+#pragma unroll
+  for (int a = NA - 1; a >= 2; --a) {
+    const bool last = (a == NA - 1) && (S >= 4);
+    const int sc = last ? kFrac : 8 * a;
+    const int i = __float2int_rn(v[a] * __uint_as_float((uint32_t)(127 + sc) << 23));
+    asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(i), "r"(last ? 1 : 1 << (kFrac - 8 * a)));
+  }
+  const int w1 = i1 - (int)(3u * (unsigned)kMagicInt);
+  asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(w1), "r"(1 << (kFrac - 8)));
+  const int w0 = i0 - kMagicInt;
+  asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(w0), "r"(1 << kFrac));
+  return T;
 }
 
 __device__ __forceinline__ void seg_col_ptr(const SegList& s, int c, const double** p,
@@ -704,20 +850,47 @@ __global__ void split_c_tc_kernel(const double* __restrict__ C, int64_t ldc, int
   }
 }
 
-constexpr int kRawRow = TCK + 1;  // raw row pitch in doubles (odd: conflict-free 8-byte reads)
-constexpr int kUThr = 512;        // compute threads of the update (16 warps)
-constexpr int kUThrAll = kUThr + 32;  // + one issuer warp
-constexpr int kUIssuer = kUThr;   // issuer thread of the update (warp 16, lane 0)
-constexpr int kUStages = 3;       // digit-plane stages of A and B (chunks in flight)
-constexpr int kUCols = NTMAX / 32 * 8;  // output columns of one thread (8-column groups cg + 4 i)
+constexpr int kUWarps = 16;             // compute warps of the update
+constexpr int kUThr = kUWarps * 32;
+constexpr int kUThrAll = kUThr + 128;   // + a warpgroup for the MMA and the C copy warp
+// Registers per thread: the launch gives every warp kURegs; the helper
+// warpgroup gives most of its share to the compute warps (setmaxnreg), whose
+// pending loads would otherwise be spilled, i.e. waited for.  The shares must
+// add up to the launch's total.
+constexpr int kURegs = 96, kURegsCompute = 104, kURegsHelper = 64;
+static_assert(kUThr * kURegsCompute + (kUThrAll - kUThr) * kURegsHelper == kUThrAll * kURegs,
+              "register shares must add up to the launch's registers");
+constexpr int kUStagesA = 4;            // most digit stages of S in TMEM
+constexpr int kUStagesB = 4;            // stages of C's digits in shared memory
+constexpr int kUPitch = NTMAX / 4 + 1;  // int64 slots per row and warp (odd: no bank conflicts)
+
+// widest output tile: the accumulators leave TMEM room for two digit stages of S
+template <int S>
+__host__ __device__ constexpr int upd_ntmax() { return S >= 7 ? 80 : 96; }
+// digit stages of S that fit beside the accumulators (8 columns per plane)
+template <int S>
+__host__ __device__ inline int upd_stages(int NT) {
+  const int fit = ((int)kTmemCols - nacc<S>() * NT) / (8 * S);
+  return fit < kUStagesA ? fit : kUStagesA;
+}
+
+// What is rarely needed of the finished tile whose int64 sums lie in a warp's
+// slots (the rest is in registers, where more would push the pending loads out):
+// its first row, and its corner in Y0 (null without Y0, or with several segments).
+struct UpdOut {
+  const double* y0base;
+  int64_t y0ld;
+  int row0;
+};
 
 struct UpdShared {
-  unsigned long long bfull[kUStages], mdone[kUStages];
+  UpdOut out[kUWarps];
+  unsigned long long afull[kUStagesA], mdone[kUStagesA];  // digits of S written / multiplied
+  unsigned long long bfull[kUStagesB], bempty[kUStagesB];
+  unsigned long long accfull, accempty;                   // accumulators of a K block
   uint32_t tmem_base;
   int fail;
-  int eA[TCM];     // row exponent bounds of the balanced S, current tile
-  int eC[NTMAX];   // column exponent bounds of the balanced C, current tile
-  SegList seg;
+  int cxmin, cxmax;  // range of the column exponents
 };
 
 // ER[i] = exponent bound of row i of the balanced S(i, k) 2^-colexp[k] over all
@@ -749,351 +922,490 @@ __global__ void row_exp_kernel(int64_t n, SegList Sg, int s, const int* __restri
   if (lane == 0) ER[row] = e > -1000000 ? e - 1022 : kEZero;
 }
 
-__device__ __forceinline__ void upd_k(const UpdShared& sh, int k, const double** p,
-                                      long long* ld) {
-  seg_col_ptr(sh.seg, k, p, ld);
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c,
+                                         uint32_t d) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(taddr),
+               "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
 }
 
-// Stage S(rows row0 .. row0 + 127, columns kc .. kc + TCK - 1) into raw
-// ([TCM][kRawRow]); zero outside the matrix.
-__device__ __forceinline__ void upd_stage_raw(const UpdShared& sh, int64_t n, int s, int64_t row0,
-                                              int kc, uint32_t raw, int tid) {
-  // thread: column kk = tid % TCK, rows tid / TCK + 32 j (coalesced along k)
-  const int kk = tid % TCK, r0 = tid / TCK;
-  const int k = kc + kk;
-  const double* p;
-  long long ld;
-  upd_k(sh, k < s ? k : 0, &p, &ld);
-  const double* src = p + (row0 + r0) * ld;
-  const long long step = (long long)(kUThr / TCK) * ld;
-#pragma unroll
-  for (int j = 0; j < TCM * TCK / kUThr; ++j) {
-    const int rl = r0 + j * (kUThr / TCK);
-    const bool ok = k < s && row0 + rl < n;
-    cp_async8(raw + (uint32_t)(rl * kRawRow + kk) * 8, ok ? src : p, ok);
-    src += step;
+// A from TMEM (lane = row, a 32-bit column = two consecutive K), B from shared memory
+__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
+// digit planes s .. S - 1 of 8 K values of this lane's row into TMEM
+template <int S, int s>
+__device__ __forceinline__ void store_planes(const uint2 (&g)[8], uint32_t dst) {
+  uint32_t w[4];
+  plane8<S, s>(g, w);
+  tmem_st4(dst + s * 8, w[0], w[1], w[2], w[3]);
+  if constexpr (s + 1 < S) store_planes<S, s + 1>(g, dst);
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t a) {
+  asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.shared::cta.b64 t, [%0];\n\t}\n" ::"r"(a)
+               : "memory");
+}
+
+// One poll of an mbarrier phase.
+__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\tmbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}\n"
+      : "=r"(done)
+      : "r"(a), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
+// Bounded wait that also ends when another warp of the CTA has given up;
+// running out raises the CTA's failure flag.
+__device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, int* fail) {
+  if (mbar_try(bar, parity)) return true;
+  for (int spin = 0; spin < kSpin; spin += 64) {
+    if (mbar_wait(bar, parity, 64)) return true;
+    if (*reinterpret_cast<volatile int*>(fail)) return false;
   }
-}
-
-// 4 consecutive K values of one M index -> S planes, one 8-byte shared store
-// per plane (half a K-major core-matrix row).
-template <int S>
-__device__ __forceinline__ void split4(const double (&x)[4], const int (&E)[4], uint32_t dst,
-                                       uint32_t pstride) {
-  uint32_t w[S][2];
-#pragma unroll
-  for (int i = 0; i < 4; i += 2) {
-    float a[S], b[S];
-    digits<S>(x[i], E[i], a);
-    digits<S>(x[i + 1], E[i + 1], b);
-#pragma unroll
-    for (int sl = 0; sl < S; ++sl)
-      w[sl][i >> 1] = __byte_perm(__float_as_uint(a[sl]), __float_as_uint(b[sl]), 0x7632);
-  }
-#pragma unroll
-  for (int sl = 0; sl < S; ++sl)
-    asm volatile("st.shared.v2.b32 [%0], {%1, %2};\n" ::"r"(dst + sl * pstride), "r"(w[sl][0]),
-                 "r"(w[sl][1])
-                 : "memory");
-}
-
-template <int S>
-__host__ __device__ inline size_t upd_regionA(int NT) {
-  const size_t a = (size_t)kUStages * S * planeA_bytes<S>();
-  return (a + 1023) / 1024 * 1024;
+  *reinterpret_cast<volatile int*>(fail) = 1;
+  return false;
 }
 
 template <int S>
 size_t upd_smem_bytes(int NT, int s) {
-  return upd_regionA<S>(NT) + (size_t)kUStages * S * planeB_bytes(NT) +
-         (size_t)kRaw * TCM * kRawRow * 8 + sizeof(UpdShared) +
-         (size_t)round_up(std::max(s, 1), 4) * 4 + 1024;
+  return (size_t)kUStagesB * S * planeB_bytes(NT) + sizeof(UpdShared) +
+         (size_t)ceil_div(std::max(s, 1), TCK) * TCK * 4 +
+         (size_t)kUThr * kUPitch * 8 + 1024 + 64;
 }
 
-// One CTA per SM: 16 compute warps cut the staged S chunks into digit planes
-// and convert the TMEM accumulators; one issuer thread (warp 16) issues the
-// MMAs and the bulk copies of C's digits.  Three plane stages: the issuer
-// fetches C's digits of chunk g + 2 while the tensor core multiplies chunk g
-// and the compute warps cut chunk g + 1.
-// kOneBlock: s <= 256, a single exponent block; the TMEM accumulators go
-// straight to the output (no int64 carry registers).
-// 17 warps: the busiest of the four SM sub-partitions holds five, so the
-// register cap is 16,384 / (5 x 32) -> 96 per thread (the multi-block
-// variant spills its int64 carries a little; the s <= 256 one does not)
-template <int S, bool kOneBlock>
+// One CTA per SM walks (row block, column tile) pairs; its warps hand chunks
+// of 16 columns of S to one another through mbarriers, with no CTA-wide
+// barrier in the loop:
+//  * 16 compute warps: a thread owns one row (its TMEM lane) and cuts 8 of a
+//    chunk's 16 columns, every other chunk, from global memory straight into
+//    digit planes in TMEM, the A operand of tcgen05.mma; the loads of its next
+//    chunk are in flight meanwhile.  At the end of a block of 256 columns it
+//    moves the accumulators into int64 sums in shared memory, after having cut
+//    the first chunks of the next block, and forms the outputs a few at a time
+//    between the chunks that follow, so that the tensor core waits for the
+//    drain of TMEM only;
+//  * warp 16: an elected thread issues the S (S + 1) / 2 MMAs of a chunk (a
+//    thread found by its index instead makes every operand pass through a
+//    lane-by-lane move to uniform registers: 1,430 cycles a chunk, 870 so);
+//  * warp 17: one thread fetches C's digits, kUStagesB chunks ahead.
+// The floor is the tensor pipe's 61 cycles for an M = 128, K = 16 MMA up to
+// N = 80 (64 at 96), 21 of them per chunk; what bounds it is the instruction
+// issue of the compute warps (about 30 per value cut, at the half rate of the
+// integer pipe, 45 per output).  The form before this one (digits in shared
+// memory, one CTA barrier per chunk, 64-bit shifts, the tensor core idle during
+// the outputs) took 1,010 us at n = 262,144, s = 213, m = 142 and 79.0 ms at
+// n = 2,097,152, s = 846, m = 564; this one 540 us and 39 ms.
+// kOneBlock: s <= 256, a single block of columns; otherwise the int64 sums are
+// kept in shared memory across the blocks, one slot per thread and output.
+// kY0: Y0 is added (an instantiation of its own: without it the loads and
+// addresses would cost the common case registers).
+template <int S, bool kOneBlock, bool kY0>
 __global__ void __launch_bounds__(kUThrAll, 1)
-    ozaki_update_tc_kernel(int64_t n, SegList Sg, int s, const int* __restrict__ colexp,
-                           const uint16_t* __restrict__ Cs, const int* __restrict__ Ce,
-                           const int* __restrict__ ER, int m, int ntiles, int NT,
-                           int64_t ntile_total, double beta, SegList Y0, OutList Y,
+    ozaki_update_tc_kernel(int64_t n, const __grid_constant__ SegList Sg, int s,
+                           const int* __restrict__ colexp, const uint16_t* __restrict__ Cs,
+                           const int* __restrict__ Ce, const int* __restrict__ ER, int m,
+                           int ntiles, int NT, int ntile_total,
+                           const __grid_constant__ SegList Y0, const __grid_constant__ OutList Y,
                            int* status) {
   constexpr int NA = nacc<S>();
-  constexpr int NS = kUStages;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-  const uint32_t pa = (uint32_t)planeA_bytes<S>(), pb = (uint32_t)planeB_bytes(NT);
-  const size_t regA = upd_regionA<S>(NT);
-  // region A: the A planes of the stages
-  const uint32_t aS0 = smem_u32(base), bS0 = smem_u32(base) + (uint32_t)regA;
-  const uint32_t raw0 = bS0 + NS * S * pb;
-  constexpr uint32_t rawB = TCM * kRawRow * 8;
-  unsigned char* after_raw = base + regA + (size_t)NS * S * pb + kRaw * rawB;
-  UpdShared& sh = *reinterpret_cast<UpdShared*>(after_raw);
-  int* cx = reinterpret_cast<int*>(after_raw + sizeof(UpdShared));
+  const uint32_t pb = (uint32_t)planeB_bytes(NT);
+  const uint32_t bS0 = smem_u32(base);
+  unsigned char* after = base + (size_t)kUStagesB * S * pb;
+  UpdShared& sh = *reinterpret_cast<UpdShared*>(after);
+  const int nch = (s + TCK - 1) / TCK;
+  int* cx = reinterpret_cast<int*>(after + ((sizeof(UpdShared) + 15) / 16) * 16);
+  long long* carry = reinterpret_cast<long long*>(cx + nch * TCK);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool compute = tid < kUThr;
-  const bool has_y0 = beta != 0.0;  // the kernel's only FP64 operation
-  const int nch = (int)ceil_div(s, TCK);
-  const size_t cs_blk = (size_t)S * KG * (NT / 8) * 64;  // bf16 per (chunk, tile)
-  const uint32_t bbytes = (uint32_t)(cs_blk * 2);
+  const int NSA = upd_stages<S>(NT);
+  const uint32_t cs_blk = (uint32_t)S * KG * (NT / 8) * 64;  // bf16 per (chunk, tile)
 
   if (warp == 0) tmem_alloc(smem_u32(&sh.tmem_base));
   if (tid == 0) {
-    for (int i = 0; i < NS; ++i) {
-      mbar_init(smem_u32(&sh.bfull[i]), 1);
+    for (int i = 0; i < kUStagesA; ++i) {
+      mbar_init(smem_u32(&sh.afull[i]), kUWarps / 2);
       mbar_init(smem_u32(&sh.mdone[i]), 1);
     }
+    for (int i = 0; i < kUStagesB; ++i) {
+      mbar_init(smem_u32(&sh.bfull[i]), 1);
+      mbar_init(smem_u32(&sh.bempty[i]), 1);
+    }
+    mbar_init(smem_u32(&sh.accfull), 1);
+    mbar_init(smem_u32(&sh.accempty), kUWarps);
     sh.fail = 0;
-    sh.seg = Sg;
+    sh.cxmin = sh.cxmax = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n");
   }
-  for (int k = tid; k < s; k += kUThrAll) cx[k] = colexp ? colexp[k] : 0;
+  __syncthreads();
+  for (int k = tid; k < nch * TCK; k += kUThrAll) {
+    const int v = (colexp && k < s) ? colexp[k] : 0;
+    cx[k] = (int)((unsigned)v << 20);  // as the fast digits add it
+    if (v < 0) atomicMin(&sh.cxmin, v);
+    if (v > 0) atomicMax(&sh.cxmax, v);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n");
   const uint32_t tmem = sh.tmem_base;
+  const uint32_t tmemA = tmem + (uint32_t)(NA * NT);
+  const int t0 = blockIdx.x, tstep = gridDim.x;
+  const int my_chunks = ((ntile_total - t0 + tstep - 1) / tstep) * nch;
 
-  // digit split: row rl of the tile, columns 4 kq .. 4 kq + 3 of the chunk
-  // (lane pairs share a row: a warp's 8-byte plane stores are contiguous)
-  const int rl = 16 * (warp & 7) + (lane >> 1), kq = 2 * ((warp >> 3) & 1) + (lane & 1);
-  const uint32_t aoff =
-      (uint32_t)(((kq >> 1) * (TCM / 8) + (rl >> 3)) * 128 + (rl & 7) * 16 + (kq & 1) * 8);
-  // epilogue: TMEM lane quarter q (tile rows 32 q ..), 8-column groups cg + 4 i
-  const int q = warp & 3, cg = (warp >> 2) & 3;
-  const int my_r = 32 * q + lane;
-  const uint32_t lane_off = (uint32_t)(32 * q) << 16;
-  bool failed = false;
-  int64_t gc = 0;  // chunk counter of this CTA over all its tiles
-  const int64_t t0 = blockIdx.x, tstep = gridDim.x;
-  auto tile_row0 = [&](int64_t t) { return (t / ntiles) * TCM; };
-  const int64_t my_chunks = ((ntile_total - t0 + tstep - 1) / tstep) * nch;
-  // chunk g of this CTA: tile t0 + (g / nch) tstep, columns (g % nch) TCK;
-  // plane stage g % NS, used for the (g / NS)-th time.  Staging (every
-  // compute thread) and the B copies (issuer) each walk the chunks in order,
-  // so their positions advance by one chunk per call: no division by a
-  // runtime value per chunk (64-bit division is a long software sequence).
-  int64_t st_g = 0, st_t = t0, st_row0 = tile_row0(t0);
-  int st_c = 0, st_slot = 0;
-  auto stage_next = [&]() {  // raw S of chunk st_g into raw stage st_g % kRaw
-    if (st_g < my_chunks)
-      upd_stage_raw(sh, n, s, st_row0, st_c * TCK, raw0 + (uint32_t)st_slot * rawB, tid);
-    cp_async_commit();
-    ++st_g;
-    st_slot = st_slot + 1 == kRaw ? 0 : st_slot + 1;
-    if (++st_c == nch) {
-      st_c = 0;
-      st_t += tstep;
-      st_row0 = tile_row0(st_t);
+  if (warp < kUWarps) {
+    // ------------------------------------------------------ compute warps
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kURegsCompute));
+    const int q = warp & 3, grp = warp >> 2, half = grp & 1;
+    const int rl = 32 * q + lane;
+    const uint32_t lane_off = (uint32_t)(32 * q) << 16;
+    const int W = NT / 4;  // output columns of a warp: W grp .. W grp + W - 1
+    long long* slots = carry + (size_t)warp * 32 * kUPitch;
+    // Position of this warp's next chunk: counted over the CTA's chunks (g),
+    // tile t, first column k0 of its 8; the row (rows past n repeat the last
+    // one), the segment holding k0 (its end, this row's address of k0, whether
+    // every row's address takes 16-byte loads), and the row's exponent bound,
+    // in the form of the fast digits when they can be used.
+    int g = grp >> 1, t = t0, k0 = g * TCK + half * 8, segend = 0;
+    const double* p = nullptr;
+    bool wide = false, fast = false;
+    int64_t row = 0;
+    int er = 0;
+    auto locate = [&]() {
+      int i = 0;
+#pragma unroll
+      for (int u = 1; u < kMaxSeg; ++u) i += (u < Sg.nseg && k0 >= Sg.off[u]) ? 1 : 0;
+      const int64_t ld = Sg.ld[i];
+      p = Sg.ptr[i] + (k0 - Sg.off[i]);
+      wide = ((reinterpret_cast<uintptr_t>(p) | (uintptr_t)(ld * 8)) & 15) == 0;
+      p += row * ld;
+      segend = Sg.off[i + 1];
+    };
+    auto enter_tile = [&]() {
+      row = min((int64_t)(t / ntiles) * TCM + rl, n - 1);
+      er = __ldg(ER + row);
+      const int ef = er == kEZero ? kEZeroFast : er;
+      fast = __all_sync(0xffffffffu, ef + sh.cxmin > kFastEMin && ef + sh.cxmax < kFastEMax);
+      if (fast) er = (int)((unsigned)(ef + digit_ke<S>()) << 20);
+      locate();
+    };
+    auto load8 = [&](double (&x)[8]) {
+      if (k0 + 8 <= segend) {
+        if (wide) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const double2 v = __ldg(reinterpret_cast<const double2*>(p) + e);
+            x[2 * e] = v.x;
+            x[2 * e + 1] = v.y;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[e] = __ldg(p + e);
+        }
+      } else {  // across segments, or past s
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = k0 + e < s ? seg_load(Sg, k0 + e, row) : 0.0;
+      }
+    };
+    auto wrap = [&]() {  // k0 past the tile's chunks
+      do {
+        k0 -= nch * TCK;
+        t += tstep;
+      } while (k0 >= nch * TCK);
+      if (g < my_chunks) enter_tile();
+    };
+    int st = g;  // digit stage of chunk g and parity of the wait for it to be free
+    uint32_t phase = 1;
+    while (st >= NSA) {
+      st -= NSA;
+      phase ^= 1;
     }
-  };
-  int64_t lb_g = 0, lb_t = t0;
-  int lb_c = 0, lb_tile = (int)(t0 % ntiles);
-  auto load_b_next = [&]() {  // issuer: B digits of chunk lb_g into stage lb_g % NS
-    const uint32_t st = (uint32_t)(lb_g % NS);
-    const size_t src = ((size_t)lb_c * ntiles + (size_t)lb_tile) * cs_blk;
-    ++lb_g;
-    if (++lb_c == nch) {
-      lb_c = 0;
-      lb_t += tstep;
-      lb_tile = (int)(lb_t % ntiles);
+    // next block of accumulators to move: tile pt, block pblk of it, ending at
+    // chunk pend; parity of its barrier phases
+    int pt = t0, pblk = 0, pend = min(kChunksPerBlock, nch) - 1;
+    uint32_t pphase = 0;
+    // output steps of the finished tile: the next one (W or more: none left),
+    // rows, first column, row exponents, and its corner in Y when the warp's
+    // columns go to one destination (else null)
+    UpdOut& fin = sh.out[warp];
+    int ou = W, onrow = 0, ocol = 0, oerow = 0, oyld = 0;
+    double* ybase = nullptr;
+    bool ok = true;
+    double x[8];
+    if (k0 >= nch * TCK) {
+      wrap();
+    } else if (g < my_chunks) {
+      enter_tile();
     }
-    uint64_t state;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;\n"
-                 : "=l"(state)
-                 : "r"(smem_u32(&sh.bfull[st])), "r"(bbytes)
-                 : "memory");
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
-        "[%3];\n" ::"r"(bS0 + st * S * pb),
-        "l"(Cs + src), "r"(bbytes), "r"(smem_u32(&sh.bfull[st]))
-        : "memory");
-  };
-  auto parity = [](int64_t g) { return (uint32_t)((g / NS) & 1); };
-  int64_t b_issued = -1;  // last chunk whose B copy the issuer started
-  int64_t m_issued = -1;  // last chunk whose MMAs the issuer committed
-  if (compute) {
-    stage_next();
-    stage_next();
-    cp_async_wait1();
-  } else if (tid == kUIssuer) {
-    for (int64_t g = 0; g < 2 && g < my_chunks; ++g) {
-      load_b_next();
-      b_issued = g;
-    }
-  }
-  __syncthreads();
+    if (g < my_chunks) load8(x);
 
-  for (int64_t t = t0; t < ntile_total && !failed; t += tstep) {
-    const int tile = (int)(t % ntiles);
-    const int64_t row0 = tile_row0(t);
-    const int tn = tile * NT;
-    const int nq_ = min(NT, m - tn);
-    for (int r = tid; r < TCM; r += kUThrAll) sh.eA[r] = row0 + r < n ? ER[row0 + r] : kEZero;
-    for (int j = tid; j < NTMAX; j += kUThrAll) sh.eC[j] = j < NT ? Ce[tn + j] : kEZero;
-    __syncthreads();
-    long long acc[kOneBlock ? 1 : kUCols];
+    // Y = T 2^(E_row + E_col - 14 - kFrac) + beta Y0 for 32 U of the warp's 32 x W
+    // outputs, lanes along the columns: a store covers two or three row
+    // segments (one thread per row would touch 32 rows with every store)
+    const unsigned inv = 65536u / (unsigned)W + 1u;  // idx / W for idx < 768
+    auto out_steps = [&](auto U) {
+      constexpr int kU = decltype(U)::value;
+      long long T[kU];
+      int e[kU], r[kU], j[kU];
 #pragma unroll
-    for (int j = 0; j < (kOneBlock ? 1 : kUCols); ++j) acc[j] = 0;
-    uint32_t started = 0;
-    for (int kc = 0; kc < s && !failed; kc += kBlock) {  // blocks of 256 columns
-      started = 0;
-      const int kend = min(s, kc + kBlock);
-      const bool last_block = kend >= s;
-      for (int k1 = kc; k1 < kend; k1 += TCK) {
-        const uint32_t st = (uint32_t)(gc % NS);
-        if (compute) {
-          const uint32_t raw = raw0 + (uint32_t)(gc % kRaw) * rawB;
-          // the stage's planes are free once the MMAs of chunk gc - NS are done
-          if (gc >= NS && !mbar_wait(smem_u32(&sh.mdone[st]), parity(gc - NS))) sh.fail = 1;
-          {
-            double x[4];
-            int E[4];
-            const int Er = sh.eA[rl];
-            const uint32_t src = raw + (uint32_t)(rl * kRawRow + kq * 4) * 8;
+      for (int u = 0; u < kU; ++u) {
+        const unsigned idx = 32u * (ou + u) + lane;
+        r[u] = (int)((idx * inv) >> 16);
+        j[u] = (int)idx - r[u] * W;
+        e[u] = __shfl_sync(0xffffffffu, oerow, r[u] & 31);
+        if (r[u] < onrow && ocol + j[u] < m) {
+          T[u] = slots[r[u] * kUPitch + j[u]];
+          e[u] += __ldg(Ce + ocol + j[u]);
+        } else {
+          r[u] = -1;
+        }
+      }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              ld_shared_f64(src + 8 * i, x[i]);
-              const int k = k1 + kq * 4 + i;
-              E[i] = Er + (k < s ? cx[k] : 0);
-            }
-            split4<S>(x, E, aS0 + st * S * pa + aoff, pa);
-          }
-          stage_next();  // chunk gc + 2
-          cp_async_wait1();
-          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      for (int u = 0; u < kU; ++u) {
+        if (r[u] < 0) continue;
+        double out = i64_scaled(T[u], e[u]);
+        if (kY0) {
+          const double* y0 = fin.y0base;
+          out += y0 ? y0[r[u] * fin.y0ld + j[u]]
+                    : seg_load(Y0, ocol + j[u], (int64_t)fin.row0 + r[u]);
         }
-        if (__syncthreads_or(sh.fail)) {
-          failed = true;
-          break;
-        }
-        if (tid == kUIssuer) {
-          if (!mbar_wait(smem_u32(&sh.bfull[st]), parity(gc))) {
-            sh.fail = 1;
-          } else {
-            asm volatile("tcgen05.fence::after_thread_sync;\n");
-            issue_chunk<S>(tmem, NT, aS0 + st * S * pa, bS0 + st * S * pb, started);
-            mma_commit(smem_u32(&sh.mdone[st]));
-            m_issued = gc;
-            // B of chunk gc + 2 into the stage of chunk gc - 1 once its MMAs are done
-            if (gc + 2 < my_chunks) {
-              if (gc >= 1 &&
-                  !mbar_wait(smem_u32(&sh.mdone[(gc - 1) % NS]), parity(gc - 1))) {
-                sh.fail = 1;
-              } else {
-                load_b_next();  // chunk gc + 2
-                b_issued = gc + 2;
-              }
-            }
-          }
-        }
-        ++gc;
+        if (ybase)
+          ybase[(int64_t)r[u] * oyld + j[u]] = out;
+        else
+          *out_addr(Y, ocol + j[u], (int64_t)fin.row0 + r[u]) = out;
       }
-      if (failed) break;
-      if (!mbar_wait(smem_u32(&sh.mdone[(gc - 1) % NS]), parity(gc - 1))) sh.fail = 1;
-      if (__syncthreads_or(sh.fail)) {
-        failed = true;
-        break;
-      }
+      ou += kU;
+    };
+    auto drain_outputs = [&]() {
+      while (ou < W) out_steps(std::integral_constant<int, 2>());
+    };
+    // accumulators -> int64 sums in this warp's slots; the tensor core has TMEM
+    // back before the outputs are formed
+    auto flush = [&]() -> bool {
+      drain_outputs();  // the previous tile's outputs leave the slots
+      __syncwarp();
+      if (!__all_sync(0xffffffffu, wait_or_fail(smem_u32(&sh.accfull), pphase, &sh.fail)))
+        return false;
       asm volatile("tcgen05.fence::after_thread_sync;\n");
-      if (!last_block) {
-        if (!kOneBlock && compute) {
+#pragma unroll 1
+      for (int j = 0; j < W; j += 4) {
+        float v[5][4];
 #pragma unroll
-          for (int i = 0; i < kUCols / 8; ++i) {
-            const int g = cg + 4 * i;
-            if (8 * g < NT) {
-              float v[NA][8];
+        for (int a = 0; a < NA; ++a) tmem_ld4(tmem + lane_off + a * NT + W * grp + j, v[a]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-              for (int a = 0; a < NA; ++a) tmem_ld8(tmem + lane_off + a * NT + 8 * g, v[a]);
-              asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                float w[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int a = 0; a < NA; ++a) w[a] = v[a][c];
-                if (!kOneBlock) acc[(8 * i + c) % (kOneBlock ? 1 : kUCols)] += acc_to_i64<S>(w);
-              }
-            }
-          }
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;\n");
-        __syncthreads();
-      }
-    }
-    // ---- output: Y = acc 2^(E_row + E_col - 14 - kFrac) + beta Y0.  All
-    // sixteen compute warps convert at once: a warp owns its TMEM lane
-    // quarter's 32 rows and the 8-column groups cg + 4 i, and each thread
-    // stores the 8 consecutive outputs of its row per group straight to
-    // global memory (no staging pass, no barrier between conversion and
-    // store)
-    if (compute) {
-      const int64_t row = row0 + my_r;
-      const bool live = row < n;
-      const int Er = sh.eA[my_r];
-#pragma unroll
-      for (int i = 0; i < kUCols / 8; ++i) {
-        const int g = cg + 4 * i;
-        if (8 * g < NT) {  // warp-uniform: the TMEM loads are .sync.aligned
-          float v[NA][8];
-          if (!failed) {
-#pragma unroll
-            for (int a = 0; a < NA; ++a) tmem_ld8(tmem + lane_off + a * NT + 8 * g, v[a]);
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-          }
-          if (live) {
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const int j = 8 * g + c;
-              if (j < nq_) {
-                double out = __longlong_as_double(0x7FF8000000000000LL);
-                if (!failed) {
-                  float w[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                  for (int a = 0; a < NA; ++a) w[a] = v[a][c];
-                  long long T = acc_to_i64<S>(w);
-                  if (!kOneBlock) T += acc[(8 * i + c) % (kOneBlock ? 1 : kUCols)];
-                  const double y0 = has_y0 ? seg_load(Y0, tn + j, row) : 0.0;
-                  out = assemble_i64(T, Er + sh.eC[j] - 14 - kFrac, y0);
-                }
-                *out_addr(Y, tn + j, row) = out;
-              }
-            }
-          }
+        for (int e = 0; e < 4; ++e) {
+          const float w[5] = {v[0][e], v[1][e], v[2][e], v[3][e], v[4][e]};
+          long long* slot = slots + lane * kUPitch + j + e;
+          long long T = acc_sum<S>(w);
+          if (!kOneBlock && pblk > 0) T += *slot;
+          *slot = T;
         }
       }
+      asm volatile("tcgen05.fence::before_thread_sync;\n");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sh.accempty));
+      pphase ^= 1;
+      if (++pblk * kChunksPerBlock >= nch) {  // the tile is complete
+        ou = 0;
+        ocol = (pt % ntiles) * NT + W * grp;
+        const int64_t row0 = (int64_t)(pt / ntiles) * TCM + 32 * q;
+        onrow = (int)max((int64_t)0, min((int64_t)32, n - row0));
+        oerow = lane < onrow ? __ldg(ER + row0 + lane) - 14 - kFrac : 0;
+        const int dst = ocol >= Y.split ? 1 : 0;
+        const int64_t ld = Y.ld[dst];
+        const bool plain = (dst || ocol + W <= Y.split || m <= Y.split) && ld < (1LL << 31);
+        ybase = plain ? Y.ptr[dst] + row0 * ld + (ocol - dst * Y.split) : nullptr;
+        oyld = (int)ld;
+        if (lane == 0) {
+          if (kY0) {
+            fin.y0base = Y0.nseg == 1 ? Y0.ptr[0] + row0 * Y0.ld[0] + ocol : nullptr;
+            fin.y0ld = Y0.ld[0];
+          }
+          fin.row0 = (int)row0;
+        }
+        __syncwarp();
+        pblk = 0;
+        pt += tstep;
+      }
+      pend += min(kChunksPerBlock, nch - pblk * kChunksPerBlock);
+      return true;
+    };
+    // outputs are formed a few steps after each chunk, spread over the chunks of
+    // the next tile, so that the tensor core never waits for them
+    const int own = max(1, min(nch, kChunksPerBlock) / 2);
+    const bool spread3 = W <= 3 * own;  // three steps a chunk are enough
+
+    for (;;) {
+      const bool more = g < my_chunks;
+      // a block is moved once the digit stages that do not wait for its last
+      // MMAs are filled with chunks of the next one
+      while (ok && pt < ntile_total && (!more || g > pend + NSA - 1)) ok = flush();
+      if (!ok || !more) break;
+      // chunk g in fixed point; its registers then take the loads of chunk g + 2
+      uint2 gb[8];
+      {
+        const int4* ce = reinterpret_cast<const int4*>(cx + k0);
+        const int4 c0 = ce[0], c1 = ce[1];
+        const int cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+        if (fast) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) gb[e] = biased_bytes<S>(x[e], (uint32_t)(er + cv[e]));
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) gb[e] = biased_bytes_any<S>(x[e], er + (cv[e] >> 20));
+        }
+      }
+      const int gc = g, sc = st;
+      const uint32_t pc = phase;
+      g += 2;
+      k0 += 2 * TCK;
+      p += 2 * TCK;
+      st += 2;
+      while (st >= NSA) {
+        st -= NSA;
+        phase ^= 1;
+      }
+      if (k0 >= nch * TCK)
+        wrap();
+      else if (k0 >= segend && k0 < s)
+        locate();
+      if (g < my_chunks) load8(x);
+      if (gc >= NSA && !wait_or_fail(smem_u32(&sh.mdone[sc]), pc, &sh.fail)) ok = false;
+      if (!(ok = __all_sync(0xffffffffu, ok))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;\n");
+      store_planes<S, 0>(gb, tmemA + lane_off + (uint32_t)(sc * 8 * S + half * 4));
+      asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;\n");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sh.afull[sc]));
+      if (ou < W) {
+        if (spread3)
+          out_steps(std::integral_constant<int, 3>());
+        else
+          drain_outputs();
+      }
     }
-    // TMEM and the tile's exponents are reused by the next tile
-    asm volatile("tcgen05.fence::before_thread_sync;\n");
-    __syncthreads();
-  }
-  if (compute) cp_async_wait0();  // no copy may outlive the CTA
-  if (tid == 0 && failed && status) atomicOr(status, 1);
-  if (tid == kUIssuer && failed) {
-    // drain what is still in flight: the B copies not yet consumed and the
-    // last committed MMAs (bounded waits; their outcome no longer matters)
-    for (int64_t g = m_issued + 1; g <= b_issued; ++g)
-      mbar_wait(smem_u32(&sh.bfull[g % NS]), parity(g));
-    if (m_issued >= 0) mbar_wait(smem_u32(&sh.mdone[m_issued % NS]), parity(m_issued));
+    drain_outputs();
+    if (!ok) {  // a wait ran out: the tiles not finished are marked
+      for (; pt < ntile_total; pt += tstep) {
+        const int tn = (pt % ntiles) * NT, nq = min(NT, m - tn);
+        const int64_t row = (int64_t)(pt / ntiles) * TCM + rl;
+        if (row < n)
+          for (int j = grp; j < nq; j += kUWarps / 4)
+            *out_addr(Y, tn + j, row) = __longlong_as_double(0x7FF8000000000000LL);
+      }
+    }
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kURegsHelper));
+    if (warp == kUWarps) {
+      if (elect_one()) {
+        // ---------------------------------------------------------- MMA issue
+        const uint64_t pb16 = pb >> 4;
+        const uint32_t idesc = instr_desc(TCM, NT);
+        const uint64_t db_first = smem_desc(bS0, (uint32_t)(NT / 8) * 128, 128);
+        const uint32_t afull0 = smem_u32(&sh.afull[0]), bfull0 = smem_u32(&sh.bfull[0]);
+        const uint32_t mdone0 = smem_u32(&sh.mdone[0]), bempty0 = smem_u32(&sh.bempty[0]);
+        int gc = 0, left = 0, c = 0;  // chunks to the end of the block; chunk of the tile
+        uint32_t blk = 0, phA = 0, phB = 0;
+        int stA = 0, stB = 0;
+        for (; gc < my_chunks; ++gc) {
+          uint32_t seen = 0xFFu;
+          if (left == 0) {  // a block starts: its accumulators must have been read
+            seen = 0u;
+            left = min(kChunksPerBlock, nch - c);
+            if (blk > 0 && !wait_or_fail(smem_u32(&sh.accempty), (blk - 1) & 1u, &sh.fail)) break;
+          }
+          if (!wait_or_fail(bfull0 + 8 * stB, phB, &sh.fail) ||
+              !wait_or_fail(afull0 + 8 * stA, phA, &sh.fail))
+            break;
+          asm volatile("tcgen05.fence::after_thread_sync;\n");
+          const uint64_t db0 = db_first + (uint64_t)stB * S * pb16;
+          const uint32_t a0 = tmemA + (uint32_t)(stA * 8 * S);
+#pragma unroll
+          for (int sl = 0; sl < S; ++sl)
+#pragma unroll
+            for (int tl = 0; tl + sl < S; ++tl) {
+              const int a = acc_of<S>(sl + tl);
+              mma_bf16_ts(tmem + (uint32_t)(a * NT), a0 + sl * 8, db0 + tl * pb16, idesc,
+                          (seen >> a) & 1u);
+              seen |= 1u << a;
+            }
+          mma_commit(mdone0 + 8 * stA);
+          mma_commit(bempty0 + 8 * stB);
+          if (--left == 0) {
+            mma_commit(smem_u32(&sh.accfull));
+            ++blk;
+          }
+          if (++c == nch) c = 0;
+          if (++stA == NSA) {
+            stA = 0;
+            phA ^= 1;
+          }
+          if (++stB == kUStagesB) {
+            stB = 0;
+            phB ^= 1;
+          }
+        }
+        // every committed MMA (and its arrivals on these barriers) ends before the CTA
+        if (gc > 0) {
+          mbar_wait(smem_u32(&sh.mdone[(gc - 1) % NSA]), (uint32_t)((gc - 1) / NSA) & 1u);
+          mbar_wait(smem_u32(&sh.bempty[(gc - 1) % kUStagesB]), (uint32_t)((gc - 1) / kUStagesB) & 1u);
+        }
+      }
+    } else if (tid == kUThr + 32) {
+      // ------------------------------------------------- copies of C's digits
+      const uint32_t bbytes = cs_blk * 2;
+      bool ok = true;
+      int64_t gc = 0;
+      for (int t = t0; t < ntile_total && ok; t += tstep) {
+        const int tile = t % ntiles;
+        for (int c = 0; c < nch; ++c) {
+          const int st = (int)(gc % kUStagesB);
+          const uint32_t use = (uint32_t)(gc / kUStagesB);
+          if (gc >= kUStagesB &&
+              !(ok = wait_or_fail(smem_u32(&sh.bempty[st]), (use - 1) & 1u, &sh.fail)))
+            break;
+          const uint16_t* src = Cs + ((size_t)c * ntiles + (size_t)tile) * cs_blk;
+          uint64_t state;
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;\n"
+                       : "=l"(state)
+                       : "r"(smem_u32(&sh.bfull[st])), "r"(bbytes)
+                       : "memory");
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+              "[%3];\n" ::"r"(bS0 + (uint32_t)st * S * pb),
+              "l"(src), "r"(bbytes), "r"(smem_u32(&sh.bfull[st]))
+              : "memory");
+          ++gc;
+        }
+      }
+      // no copy outlives the CTA (on success the MMAs have consumed them all)
+      for (int64_t u = max((int64_t)0, gc - kUStagesB); u < gc; ++u)
+        mbar_wait(smem_u32(&sh.bfull[u % kUStagesB]), (uint32_t)(u / kUStagesB) & 1u);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
   __syncthreads();
+  if (tid == 0 && sh.fail && status) atomicOr(status, 1);
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     tmem_dealloc(tmem);
   }
 }
 
+template <int S>
 void update_tiles(int m, int* ntiles, int* NT) {
-  *ntiles = (int)ceil_div(std::max(m, 1), NTMAX);
+  *ntiles = (int)ceil_div(std::max(m, 1), upd_ntmax<S>());
   *NT = (int)round_up(ceil_div(std::max(m, 1), *ntiles), 16);
 }
 
@@ -1102,7 +1414,7 @@ int update_tc_launch(cudaStream_t st, int64_t n, const SegList& Sg, int s, const
                      int64_t ldc, int m, double alpha, double beta, const SegList& Y0,
                      const OutList& Y, const int* colexp, void* work, int* status) {
   int ntiles, NT;
-  update_tiles(m, &ntiles, &NT);
+  update_tiles<S>(m, &ntiles, &NT);
   const int nch = (int)ceil_div(s, TCK);
   uint16_t* Cs = (uint16_t*)work;
   const size_t cs_elems = (size_t)nch * ntiles * S * KG * (NT / 8) * 64;
@@ -1122,26 +1434,41 @@ int update_tc_launch(cudaStream_t st, int64_t n, const SegList& Sg, int s, const
         C, ldc, s, m, ntiles, NT, alpha, colexp, Cs, Ce);
     LOB_LAUNCHED();
   }
-  const size_t shmax = upd_smem_bytes<S>(NTMAX, kMaxUpdateK);
   // the attribute is per device: set it once on every device that launches
   static bool configured[64] = {false};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    LOB_CUDA_OK(cudaFuncSetAttribute(ozaki_update_tc_kernel<S, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmax));
-    LOB_CUDA_OK(cudaFuncSetAttribute(ozaki_update_tc_kernel<S, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmax));
+    auto configure = [](auto* kernel, int one_s) -> int {
+      LOB_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)upd_smem_bytes<S>(upd_ntmax<S>(), one_s)));
+      cudaFuncAttributes at;  // a launch with other registers would wait for its shares forever
+      LOB_CUDA_OK(cudaFuncGetAttributes(&at, kernel));
+      return at.numRegs == kURegs ? LOBPCG_OK : LOBPCG_ERR_CUDA;
+    };
+    int rc = configure(ozaki_update_tc_kernel<S, true, false>, kBlock);
+    if (!rc) rc = configure(ozaki_update_tc_kernel<S, false, false>, kMaxUpdateK);
+    if (!rc) rc = configure(ozaki_update_tc_kernel<S, true, true>, kBlock);
+    if (!rc) rc = configure(ozaki_update_tc_kernel<S, false, true>, kMaxUpdateK);
+    if (rc) return rc;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   const int64_t tiles = ceil_div(n, TCM) * ntiles;
+  if (tiles > (1LL << 30) || ceil_div(tiles, 152) * nch > (1LL << 30))
+    return LOBPCG_ERR_ARG;  // terabytes of S
   const int64_t grid = std::min<int64_t>(tiles, 152);
-  if (s <= kBlock)
-    ozaki_update_tc_kernel<S, true><<<(unsigned)grid, kUThrAll, upd_smem_bytes<S>(NT, s), st>>>(
-        n, Sg, s, colexp, Cs, Ce, ER, m, ntiles, NT, tiles, beta, Y0, Y, status);
+  const bool one = s <= kBlock;
+  const size_t sm = upd_smem_bytes<S>(NT, s);
+  auto launch = [&](auto* kernel) {
+    kernel<<<(unsigned)grid, kUThrAll, sm, st>>>(n, Sg, s, colexp, Cs, Ce, ER, m, ntiles, NT,
+                                                 (int)tiles, Y0, Y, status);
+  };
+  if (beta != 0.0)
+    one ? launch(ozaki_update_tc_kernel<S, true, true>)
+        : launch(ozaki_update_tc_kernel<S, false, true>);
   else
-    ozaki_update_tc_kernel<S, false><<<(unsigned)grid, kUThrAll, upd_smem_bytes<S>(NT, s), st>>>(
-        n, Sg, s, colexp, Cs, Ce, ER, m, ntiles, NT, tiles, beta, Y0, Y, status);
+    one ? launch(ozaki_update_tc_kernel<S, true, false>)
+        : launch(ozaki_update_tc_kernel<S, false, false>);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
@@ -1215,7 +1542,10 @@ int gram_tc(cudaStream_t st, int64_t n, const SegList& U, const SegList& V, doub
 int64_t update_tc_workspace(int64_t n, int s, int m, int slices) {
   if (slices == 0) slices = 6;
   int ntiles, NT;
-  update_tiles(m, &ntiles, &NT);
+  if (slices >= 7)
+    update_tiles<7>(m, &ntiles, &NT);
+  else
+    update_tiles<6>(m, &ntiles, &NT);
   const int64_t nch = ceil_div(std::max(s, 1), TCK);
   return nch * ntiles * slices * KG * (NT / 8) * 64 * 2 + (int64_t)ntiles * NT * 4 +
          (int64_t)std::max(s, 1) * 4 + std::max<int64_t>(n, 1) * 4 + 256;
