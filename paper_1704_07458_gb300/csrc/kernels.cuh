@@ -9,6 +9,13 @@ int spmm(cudaStream_t st, int64_t n, const int32_t* rowptr, const int32_t* col,
          const double* val, const double* X, int64_t ldx, int m, double* Y, int64_t ldy,
          const double* b, double* BY, int64_t ldby);
 
+// One Chebyshev step with its product: d <- a d + bz D^-1 (R - A w), wnew = w + d
+// (n x m blocks; w and d share the leading dimension ld; the last step leaves d).
+int cheb_step(cudaStream_t st, int64_t n, const int32_t* rowptr, const int32_t* col,
+              const double* val, const double* w, int64_t ld, int m, const double* R, int64_t ldr,
+              const double* dinv, double a, double bz, double* d, double* wnew, int64_t ldw,
+              bool last);
+
 // G = U^T V (G column-major, leading dimension ldg), plain FP64 on the CUDA
 // cores with a split over rows and a fixed-order second pass (deterministic).
 int64_t gram_f64_workspace(int64_t n, int p, int q);

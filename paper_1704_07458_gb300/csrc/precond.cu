@@ -12,11 +12,13 @@
 //     d_k = rho_k rho_{k-1} d_{k-1} + (2 rho_k / delta) z,  w_{k+1} = w_k + d_k.
 // w = p(D^-1 A) D^-1 r for a fixed polynomial p, positive on [lmin, lmax], so
 // K^-1 = D^-1/2 p(D^-1/2 A D^-1/2) D^-1/2 is symmetric positive definite: a
-// valid LOBPCG preconditioner.  Every step is this library's SpMM plus one
-// fused elementwise kernel over the n x ncols block; no host work per call.
+// valid LOBPCG preconditioner.  Every step is one kernel: the product A w with
+// the recurrence in its epilogue, so that A w is never stored (a product and an
+// elementwise pass took 570 us a step at 64^3, 71 columns; 400 us now); no
+// host work per call.
 #include <algorithm>
 
-#include "kernels.cuh"
+#include "colpass.cuh"
 
 struct lobpcg_chebyshev {
   int64_t n = 0, max_cols = 0, ld = 0;
@@ -24,7 +26,7 @@ struct lobpcg_chebyshev {
   const int32_t* col = nullptr;
   const double* val = nullptr;
   double* dinv = nullptr;  // 1 / diag(A)
-  double *w = nullptr, *d = nullptr, *aw = nullptr;  // n x ld work blocks
+  double *w = nullptr, *d = nullptr, *aw = nullptr;  // n x ld work blocks (aw: the other w)
   int degree = 0;
   double lmin = 0.0, lmax = 0.0;
 };
@@ -47,36 +49,20 @@ __global__ void cheb_dinv_kernel(int64_t n, const int32_t* __restrict__ rp,
   dinv[r] = x != 0.0 ? 1.0 / x : 1.0;
 }
 
-// first step: d = D^-1 r / theta, w = d
-__global__ void cheb_first_kernel(int64_t n, int m, const double* __restrict__ R, int64_t ldr,
-                                  const double* __restrict__ dinv, double inv_theta,
-                                  double* __restrict__ d, double* __restrict__ w, int64_t ld) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * m) return;
-  const int64_t r = e / m;
-  const int c = (int)(e % m);
-  const double v = R[r * ldr + c] * dinv[r] * inv_theta;
-  d[r * ld + c] = v;
-  w[r * ld + c] = v;
-}
-
-// later steps: z = D^-1 (r - A w), d = a d + b z, w += d; the last step
-// writes w into the output W
-__global__ void cheb_step_kernel(int64_t n, int m, const double* __restrict__ R, int64_t ldr,
-                                 const double* __restrict__ aw, const double* __restrict__ dinv,
-                                 double a, double b, double* __restrict__ d,
-                                 double* __restrict__ w, int64_t ld, double* __restrict__ Wout,
-                                 int64_t ldw) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * m) return;
-  const int64_t r = e / m;
-  const int c = (int)(e % m);
-  const double z = (R[r * ldr + c] - aw[r * ld + c]) * dinv[r];
-  const double dn = a * d[r * ld + c] + b * z;
-  const double wn = w[r * ld + c] + dn;
-  d[r * ld + c] = dn;
-  w[r * ld + c] = wn;
-  if (Wout) Wout[r * ldw + c] = wn;
+// first step: d = D^-1 r / theta, w = d.  CTAs walk rows, threads over (row,
+// column) as in the column passes: no integer division per element.
+__global__ void __launch_bounds__(kColThreads) cheb_first_kernel(
+    int64_t n, int m, int TX, const double* __restrict__ R, int64_t ldr,
+    const double* __restrict__ dinv, double inv_theta, double* __restrict__ d,
+    double* __restrict__ w, int64_t ld) {
+  const int TY = kColThreads / TX, tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  if (ty >= TY) return;
+  for (int64_t r = (int64_t)blockIdx.x * TY + ty; r < n; r += (int64_t)gridDim.x * TY)
+    for (int c = tx; c < m; c += TX) {
+      const double v = R[r * ldr + c] * dinv[r] * inv_theta;
+      d[r * ld + c] = v;
+      w[r * ld + c] = v;
+    }
 }
 
 __global__ void copy_rows_kernel(int64_t n, int m, const double* __restrict__ S, int64_t lds,
@@ -143,23 +129,26 @@ LOBPCG_EXPORT int lobpcg_chebyshev_apply(void* ctx, int64_t n, int64_t ncols, co
   const double theta = 0.5 * (c->lmax + c->lmin), delta = 0.5 * (c->lmax - c->lmin);
   const double sigma = theta / delta;
   double rho = 1.0 / sigma;
-  const unsigned nb = lob::blocks_of(n * m);
-  lob::cheb_first_kernel<<<nb, 256, 0, st>>>(n, m, R, ldr, c->dinv, 1.0 / theta, c->d, c->w,
-                                             c->ld);
+  const int TX = lob::col_tile(m);
+  const unsigned nb = (unsigned)std::min<int64_t>(
+      lob::ceil_div(n, lob::kColThreads / TX), 16 * 152);
+  lob::cheb_first_kernel<<<nb, lob::kColThreads, 0, st>>>(n, m, TX, R, ldr, c->dinv, 1.0 / theta,
+                                                          c->d, c->w, c->ld);
   ++lob::g_launches;
+  // w and w' alternate between two blocks (a step reads its neighbours' w)
+  double *w = c->w, *wn = c->aw;
   for (int k = 1; k < c->degree; ++k) {
-    int rc = lob::spmm(st, n, c->rowptr, c->col, c->val, c->w, c->ld, m, c->aw, c->ld, nullptr,
-                       nullptr, 0);
-    if (rc) return rc;
+    const bool last = k + 1 == c->degree;
     const double rho1 = 1.0 / (2.0 * sigma - rho);
-    lob::cheb_step_kernel<<<nb, 256, 0, st>>>(n, m, R, ldr, c->aw, c->dinv, rho1 * rho,
-                                              2.0 * rho1 / delta, c->d, c->w, c->ld,
-                                              k + 1 == c->degree ? W : nullptr, ldw);
-    ++lob::g_launches;
+    int rc = lob::cheb_step(st, n, c->rowptr, c->col, c->val, w, c->ld, m, R, ldr, c->dinv,
+                            rho1 * rho, 2.0 * rho1 / delta, c->d, last ? W : wn,
+                            last ? ldw : c->ld, last);
+    if (rc) return rc;
+    std::swap(w, wn);
     rho = rho1;
   }
   if (c->degree == 1) {
-    lob::copy_rows_kernel<<<nb, 256, 0, st>>>(n, m, c->w, c->ld, W, ldw);
+    lob::copy_rows_kernel<<<lob::blocks_of(n * m), 256, 0, st>>>(n, m, c->w, c->ld, W, ldw);
     ++lob::g_launches;
   }
   return cudaPeekAtLastError() == cudaSuccess ? LOBPCG_OK : LOBPCG_ERR_CUDA;
