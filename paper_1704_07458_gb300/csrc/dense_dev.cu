@@ -198,39 +198,26 @@ __global__ void __launch_bounds__(256) trinv64_kernel(int n, const double* R, in
 }
 
 // ------------------------------------------- FP32 tridiagonalisation
-// Householder reduction of the symmetric A (FP64, both triangles averaged)
-// to tridiagonal T = Q^T A Q in FP32 (the reduction of LAPACK's sytd2, lower
-// variant): one CTA, the lower triangle packed in shared memory.  Outputs d
-// (n), e (n - 1), the reflectors v_k (column k of V, rows k + 1 .. n - 1,
-// v_k[k + 1] = 1), tau (n) and scal[0] = ||A||_F.
+// Householder reduction of the symmetric A (FP64) to tridiagonal T = Q^T A Q
+// in FP32 (the reduction of LAPACK's sytd2, lower variant): one CTA, the lower
+// triangle packed in shared memory.  Outputs d (n), e (n - 1), the reflectors
+// v_k (column k of V, rows k + 1 .. n - 1, v_k[k + 1] = 1) and tau (n).  For
+// orders above kTridRegMax, whose matrix does not fit the registers.
 __device__ __forceinline__ int pk(int n, int i, int j) {  // (i >= j) packed lower, column-major
   return j * n - (j * (j - 1)) / 2 + (i - j);
 }
 
 __global__ void __launch_bounds__(1024, 1) tridiag32_kernel(int n, const double* A, int lda,
                                                             float* d, float* e, float* V, int ldv,
-                                                            float* tau, double* scal) {
+                                                            float* tau) {
   extern __shared__ float P[];  // n (n + 1) / 2
   __shared__ float v[256], p[256];
   __shared__ float wpart[32];
   __shared__ float s_tau;
-  __shared__ double fro[32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  double f = 0.0;
   for (int j = warp; j < n; j += 32)
-    for (int i = j + lane; i < n; i += 32) {
-      const double a = 0.5 * (A[i + (int64_t)j * lda] + A[j + (int64_t)i * lda]);
-      P[pk(n, i, j)] = (float)a;
-      f += (i == j ? 1.0 : 2.0) * a * a;
-    }
-  for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-  if (lane == 0) fro[warp] = f;
+    for (int i = j + lane; i < n; i += 32) P[pk(n, i, j)] = (float)A[i + (int64_t)j * lda];
   __syncthreads();
-  if (t == 0) {
-    double s = 0.0;
-    for (int w = 0; w < 32; ++w) s += fro[w];
-    scal[0] = sqrt(s);
-  }
   for (int k = 0; k + 2 < n; ++k) {
     const int m = n - k - 1;  // length of the reflected column x = A(k+1 .. n-1, k)
     if (warp == 0) {
@@ -306,131 +293,146 @@ __global__ void __launch_bounds__(1024, 1) tridiag32_kernel(int n, const double*
   }
 }
 
-// The same reduction with the lower triangle kept in a full n x ld array
-// (ld = n rounded up to odd, n <= kTridFull) in shared memory: the product
-// p = tau A22 v runs one thread per row (row i reads A(i, j), j <= i, along
-// its row and A(j, i), j > i, down its column; with an odd ld both patterns
-// are free of bank conflicts across a warp), four accumulators per thread;
-// the rank-2 update touches the lower triangle only.
-constexpr int kTridFull = 223;
+// The same reduction with the whole symmetric matrix in registers (n <= 224):
+// thread (ty, tx) of 16 warps x 32 lanes holds A(ty + 16 r, tx + 32 c), so a
+// warp owns complete rows, the products A v and the rank-2 update run without
+// touching memory, and a step costs two barriers: one for the column that the
+// owners of its elements publish, one for p = tau A v.  Every warp forms the
+// reflector and p^T v for itself (a few shuffles) instead of waiting for one
+// that does.  Tiles left of or above the trailing block are skipped.  Bound by
+// the chain of a step (two reductions of five shuffles, a square root, two
+// divisions, two barriers); with the matrix in shared memory each element cost
+// two loads and a store per step (811 us at n = 213; 394 us now).
+constexpr int kTridRegMax = 224;
 
-__global__ void __launch_bounds__(1024, 1) tridiag32_full_kernel(int n, const double* A, int lda,
-                                                                 float* d, float* e, float* V,
-                                                                 int ldv, float* tau,
-                                                                 double* scal) {
-  extern __shared__ float F[];  // n x ld, F[i * ld + j] = A(i, j) for j <= i
-  __shared__ float v[256], p[256];
-  __shared__ float wpart[32];
-  __shared__ float s_tau;
-  __shared__ double fro[32];
-  const int ld = n | 1;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  double f = 0.0;
-  for (int i = warp; i < n; i += 32)
-    for (int j = lane; j <= i; j += 32) {
-      const double a = 0.5 * (A[i + (int64_t)j * lda] + A[j + (int64_t)i * lda]);
-      F[i * ld + j] = (float)a;
-      f += (i == j ? 1.0 : 2.0) * a * a;
+template <int NB>
+struct TridiagShared {
+  float xs[2][32 * NB], ps[32 * NB];
+};
+
+// The steps k whose next column k + 1 lies in column tile C0: tiles left of it
+// and row tiles above 2 C0 are finished, and every register index is static.
+template <int NB, int C0>
+__device__ __forceinline__ void tridiag_phase(int n, float (&a)[2 * NB][NB], TridiagShared<NB>& sh,
+                                              float* d, float* e, float* V, int ldv, float* tau) {
+  constexpr int NR = 2 * NB, R0 = 2 * C0;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int kend = min(n - 2, 32 * C0 + 31);
+#pragma unroll 1
+  for (int k = C0 > 0 ? 32 * C0 - 1 : 0; k < kend; ++k) {
+    const float* x = sh.xs[k & 1];
+    __syncthreads();  // column k is complete; p of the step before has been read
+    // reflector of x(k + 1 : n): v_{k+1} = 1, v_j = x_j scale
+    float vj[NB], ss = 0.f;
+#pragma unroll
+    for (int c = C0; c < NB; ++c) {
+      const int j = tx + 32 * c;
+      vj[c] = j > k ? x[j] : 0.f;  // rows past n are zero
+      ss = fmaf(j == k + 1 ? 0.f : vj[c], vj[c], ss);
     }
-  for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-  if (lane == 0) fro[warp] = f;
-  __syncthreads();
-  if (t == 0) {
-    double sacc = 0.0;
-    for (int w = 0; w < 32; ++w) sacc += fro[w];
-    scal[0] = sqrt(sacc);
-  }
-  for (int k = 0; k + 2 < n; ++k) {
-    const int m = n - k - 1;
-    const int o = k + 1;  // first row / column of the trailing block
-    if (warp == 0) {
-      // x = A(k+1 .. n-1, k): column k below the diagonal (stride ld)
-      float ss = 0.f;
-      for (int i = 1 + lane; i < m; i += 32) {
-        const float x = F[(o + i) * ld + k];
-        ss = fmaf(x, x, ss);
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, q);
+    const float alpha = x[k + 1];
+    float tk = 0.f, beta = alpha, scale = 0.f;
+    if (ss > 0.f) {
+      beta = -copysignf(sqrtf(alpha * alpha + ss), alpha);
+      tk = (beta - alpha) / beta;
+      scale = 1.f / (alpha - beta);
+    }
+#pragma unroll
+    for (int c = C0; c < NB; ++c) vj[c] = tx + 32 * c == k + 1 ? 1.f : vj[c] * scale;
+    if (ty == 0) {
+#pragma unroll
+      for (int c = C0; c < NB; ++c) {
+        const int j = tx + 32 * c;
+        if (j > k && j < n) V[j + (int64_t)k * ldv] = vj[c];
       }
-      for (int q = 16; q > 0; q >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, q);
-      const float alpha = F[o * ld + k];
-      float tk = 0.f, beta = alpha, scale = 0.f;
-      if (ss > 0.f) {
-        beta = -copysignf(sqrtf(alpha * alpha + ss), alpha);
-        tk = (beta - alpha) / beta;
-        scale = 1.f / (alpha - beta);
-      }
-      for (int i = lane; i < m; i += 32) {
-        const float vi = i == 0 ? 1.f : (tk != 0.f ? F[(o + i) * ld + k] * scale : 0.f);
-        v[i] = vi;
-        V[(o + i) + (int64_t)k * ldv] = vi;
-      }
-      if (lane == 0) {
-        s_tau = tk;
-        d[k] = F[k * ld + k];
+      if (tx == 0) {
+        d[k] = x[k];
         e[k] = beta;
         tau[k] = tk;
       }
     }
-    __syncthreads();
-    const float tk = s_tau;
-    if (tk == 0.f) continue;
-    // p_i = tau sum_j A22(i, j) v_j: four consecutive lanes per row, lane
-    // sub of a row takes the j = sub (mod 4) terms of the stored lower
-    // triangle (row part j <= i, column part j > i), a shuffle sums them
-    float pv = 0.f;
-    {
-      const int r = t >> 2, sub = t & 3;
-      float a0 = 0.f, a1 = 0.f;
-      if (r < m) {
-        const int gi = o + r;
-        const float* row = F + gi * ld + o;  // A(gi, o + j), j <= r
-        int j = sub;
-        for (; j + 4 <= r; j += 8) {
-          a0 = fmaf(row[j], v[j], a0);
-          a1 = fmaf(row[j + 4], v[j + 4], a1);
-        }
-        for (; j <= r; j += 4) a0 = fmaf(row[j], v[j], a0);
-        // j > r: A(o + j, gi) = F[(o + j) * ld + gi]; first j = r + 1 + ((sub - r - 1) mod 4)
-        j = r + 1 + ((sub - r - 1) & 3);
-        for (; j + 4 < m; j += 8) {
-          a0 = fmaf(F[(o + j) * ld + gi], v[j], a0);
-          a1 = fmaf(F[(o + j + 4) * ld + gi], v[j + 4], a1);
-        }
-        for (; j < m; j += 4) a0 = fmaf(F[(o + j) * ld + gi], v[j], a0);
-      }
-      float sacc = a0 + a1;
-      sacc += __shfl_xor_sync(0xffffffffu, sacc, 1);
-      sacc += __shfl_xor_sync(0xffffffffu, sacc, 2);
-      if (r < m && sub == 0) {
-        sacc *= tk;
-        p[r] = sacc;
-        pv = sacc * v[r];
+    // p_i = tau sum_j A(i, j) v_j of this warp's rows: lane sums, reduced by
+    // halving (each exchange halves the values a lane carries)
+    float s[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) s[r] = 0.f;
+#pragma unroll
+    for (int c = C0; c < NB; ++c)
+#pragma unroll
+      for (int r = R0; r < NR; ++r) s[r] = fmaf(a[r][c], vj[c], s[r]);
+#pragma unroll
+    for (int h = 8; h > 0; h >>= 1) {  // lane bit 2h keeps the upper h of 2h values
+      const bool up = (tx & (2 * h)) != 0;
+#pragma unroll
+      for (int r = 0; r < h; ++r) {
+        const float send = up ? s[r] : s[r + h], keep = up ? s[r + h] : s[r];
+        s[r] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
       }
     }
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+    if ((tx & 1) == 0 && (tx >> 1) < NR) sh.ps[ty + 16 * (tx >> 1)] = tk * s[0];
+    __syncthreads();
+    // K = tau p^T v / 2, w = p - K v, A -= v w^T + w v^T
+    float wj[NB], pv = 0.f;
+#pragma unroll
+    for (int c = C0; c < NB; ++c) {
+      wj[c] = sh.ps[tx + 32 * c];
+      pv = fmaf(wj[c], vj[c], pv);
+    }
+#pragma unroll
     for (int q = 16; q > 0; q >>= 1) pv += __shfl_xor_sync(0xffffffffu, pv, q);
-    if (lane == 0) wpart[warp] = pv;
-    __syncthreads();
-    float ptv = 0.f;
-    for (int w = 0; w < 32; ++w) ptv += wpart[w];
-    const float K = 0.5f * tk * ptv;
-    // rank-2 update of the lower triangle: A22(i, j) -= v_i w_j + w_i v_j
-    for (int i = warp; i < m; i += 32) {
-      float* row = F + (o + i) * ld + o;
-      const float vi = v[i], wi = p[i] - K * v[i];
-      for (int j = lane; j <= i; j += 32) row[j] = row[j] - (vi * (p[j] - K * v[j]) + wi * v[j]);
+    const float K = 0.5f * tk * pv;
+#pragma unroll
+    for (int c = C0; c < NB; ++c) wj[c] = fmaf(-K, vj[c], wj[c]);
+    const bool own = tx == ((k + 1) & 31);  // column k + 1, published for the next step
+    float* xn = sh.xs[(k + 1) & 1];
+#pragma unroll
+    for (int r = R0; r < NR; ++r) {
+      const int i = ty + 16 * r;
+      const float vi = i == k + 1 ? 1.f : (i > k ? x[i] * scale : 0.f);
+      const float wi = fmaf(-K, vi, sh.ps[i]);
+#pragma unroll
+      for (int c = C0; c < NB; ++c) a[r][c] -= fmaf(vi, wj[c], wi * vj[c]);
+      if (own) xn[i] = a[r][C0];
     }
-    __syncthreads();
   }
-  if (t == 0) {
-    if (n >= 2) {
-      d[n - 2] = F[(n - 2) * ld + (n - 2)];
-      d[n - 1] = F[(n - 1) * ld + (n - 1)];
-      e[n - 2] = F[(n - 1) * ld + (n - 2)];
-      tau[n - 2] = 0.f;
-    } else {
-      d[0] = F[0];
+  if constexpr (C0 + 1 < NB) {
+    // the last step above published column 32 C0 + 31; the rows of finished
+    // tiles that the next phase's x no longer reads stay as they are
+    tridiag_phase<NB, C0 + 1>(n, a, sh, d, e, V, ldv, tau);
+  }
+}
+
+template <int NB>
+__global__ void __launch_bounds__(512, 1) tridiag32_reg_kernel(int n, const double* __restrict__ A,
+                                                               int lda, float* d, float* e,
+                                                               float* V, int ldv, float* tau) {
+  constexpr int NR = 2 * NB;
+  __shared__ TridiagShared<NB> sh;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  float a[NR][NB];
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int c = 0; c < NB; ++c) {
+      const int i = ty + 16 * r, j = tx + 32 * c;
+      a[r][c] = (i < n && j < n) ? (float)A[j + (int64_t)i * lda] : 0.f;
     }
-    tau[n - 1] = 0.f;
-  }
+  if (tx == 0)
+#pragma unroll
+    for (int r = 0; r < NR; ++r) sh.xs[0][ty + 16 * r] = a[r][0];
+  tridiag_phase<NB, 0>(n, a, sh, d, e, V, ldv, tau);
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int c = 0; c < NB; ++c) {
+      const int i = ty + 16 * r, j = tx + 32 * c;
+      if (i == j && i < n && i + 2 >= n) d[i] = a[r][c];
+      if (i == n - 1 && j == n - 2) e[n - 2] = a[r][c];
+    }
+  if (threadIdx.x < 2 && n >= 2) tau[n - 2 + threadIdx.x] = 0.f;
 }
 
 // --------------------------- tridiagonal eigenvalues and eigenvectors
@@ -453,65 +455,78 @@ __device__ __forceinline__ float hash_unit(uint32_t a, uint32_t b) {
 }
 
 // lam[j], j = 0 .. n-1: the eigenvalues of T by multisection on the Sturm
-// count (count(x) = number of eigenvalues below x, LAPACK's pivmin guard),
-// four lanes per eigenvalue evaluating four interior points of the interval
-// at once (each round narrows it five-fold), to FP32 resolution.
+// count (count(x) = number of eigenvalues below x, LAPACK's pivmin guard), a
+// warp per eigenvalue evaluating 32 interior points of the interval at once
+// (each round narrows it 33-fold: five rounds to FP32 resolution), with the
+// approximate division (two ulps; the values only start an iteration that FP64
+// refines).  A round is a chain of n quotients, so its count is what to save:
+// four points per eigenvalue and IEEE division took 204 us at n = 213; 51 us
+// now.  bounds[0], bounds[1]: ||T|| bound and pivot guard for the eigenvectors.
 __global__ void __launch_bounds__(256) bisect_kernel(int n, const float* __restrict__ dg,
                                                      const float* __restrict__ eg,
-                                                     float* __restrict__ lam) {
-  __shared__ float d[256], e2[256];
-  __shared__ float s_gl, s_gu, s_piv;
-  const int t = threadIdx.x;
-  for (int i = t; i < n; i += blockDim.x) {
-    d[i] = dg[i];
-    const float ei = i + 1 < n ? eg[i] : 0.f;
-    e2[i] = ei * ei;
+                                                     float* __restrict__ lam,
+                                                     float* __restrict__ bounds) {
+  __shared__ float d[256], e2[257];
+  __shared__ float s_gl[8], s_gu[8], s_em[8];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  float gl = FLT_MAX, gu = -FLT_MAX, emax2 = 0.f;
+  if (t == 0) e2[0] = 0.f;  // e2[i]: square of the entry above d[i]
+  if (t < n) {
+    const float di = dg[t], el = t > 0 ? eg[t - 1] : 0.f, er = t + 1 < n ? eg[t] : 0.f;
+    d[t] = di;
+    e2[t + 1] = er * er;
+    const float r = fabsf(el) + fabsf(er);
+    gl = di - r;
+    gu = di + r;
+    emax2 = er * er;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    gl = fminf(gl, __shfl_xor_sync(0xffffffffu, gl, o));
+    gu = fmaxf(gu, __shfl_xor_sync(0xffffffffu, gu, o));
+    emax2 = fmaxf(emax2, __shfl_xor_sync(0xffffffffu, emax2, o));
+  }
+  if (lane == 0) {
+    s_gl[warp] = gl;
+    s_gu[warp] = gu;
+    s_em[warp] = emax2;
   }
   __syncthreads();
-  if (t == 0) {
-    float gl = FLT_MAX, gu = -FLT_MAX, emax2 = 0.f;
-    for (int i = 0; i < n; ++i) {
-      const float r = (i > 0 ? sqrtf(e2[i - 1]) : 0.f) + (i + 1 < n ? sqrtf(e2[i]) : 0.f);
-      gl = fminf(gl, d[i] - r);
-      gu = fmaxf(gu, d[i] + r);
-      emax2 = fmaxf(emax2, e2[i]);
-    }
-    const float tnorm = fmaxf(fabsf(gl), fabsf(gu));
-    const float pivmin = FLT_MIN * fmaxf(1.f, emax2);
-    s_gl = gl - 2.f * FLT_EPSILON * tnorm * n - pivmin;
-    s_gu = gu + 2.f * FLT_EPSILON * tnorm * n + pivmin;
-    s_piv = pivmin;
+  for (int w = 0; w < 8; ++w) {
+    gl = fminf(gl, s_gl[w]);
+    gu = fmaxf(gu, s_gu[w]);
+    emax2 = fmaxf(emax2, s_em[w]);
   }
-  __syncthreads();
-  const int g = (blockIdx.x * blockDim.x + t) >> 2, q = t & 3;
-  const bool active = g < n;
-  const float pivmin = s_piv;
-  float lo = s_gl, hi = s_gu;
-  for (int round = 0; round < 24; ++round) {
+  const float tnorm = fmaxf(fabsf(gl), fabsf(gu));
+  const float pivmin = FLT_MIN * fmaxf(1.f, emax2);
+  if (blockIdx.x == 0 && t == 0) {
+    bounds[0] = tnorm;
+    bounds[1] = pivmin;
+  }
+  const int g = blockIdx.x * 8 + warp;
+  if (g >= n) return;
+  float lo = gl - 2.f * FLT_EPSILON * tnorm * n - pivmin;
+  float hi = gu + 2.f * FLT_EPSILON * tnorm * n + pivmin;
+  for (int round = 0; round < 12; ++round) {
     const float wdt = hi - lo;
-    const bool conv = !(wdt > 2.f * FLT_EPSILON * fmaxf(fabsf(lo), fabsf(hi)) + pivmin);
-    // the four lanes of a group share lo, hi: they stop together
-    const float x = lo + (float)(q + 1) * 0.2f * wdt;
+    if (!(wdt > 2.f * FLT_EPSILON * fmaxf(fabsf(lo), fabsf(hi)) + pivmin)) break;
+    const float step = wdt * (1.f / 33.f);
+    const float x = lo + (float)(lane + 1) * step;
     int c = 0;
-    if (active && !conv) {
-      float qq = 1.f;
-      for (int i = 0; i < n; ++i) {
-        qq = d[i] - x - (i > 0 ? e2[i - 1] / qq : 0.f);
-        if (fabsf(qq) < pivmin) qq = -pivmin;
-        c += qq < 0.f;
-      }
+    float q = 1.f;
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+      q = d[i] - x - __fdividef(e2[i], q);
+      if (fabsf(q) < pivmin) q = -pivmin;
+      c += q < 0.f;
     }
-    // first of the four points with count > g: the eigenvalue lies below it
-    const unsigned above = __ballot_sync(0xffffffffu, active && !conv && c > g);
-    const unsigned grp = (above >> ((t & 31) & ~3)) & 0xFu;
-    const int first = grp ? __ffs(grp) - 1 : 4;
-    const float x0 = lo + (float)first * 0.2f * wdt, x1 = lo + (float)(first + 1) * 0.2f * wdt;
-    if (!conv) {
-      lo = first == 0 ? lo : x0;
-      hi = first == 4 ? hi : x1;
-    }
+    // first of the points with count > g: the eigenvalue lies below it
+    const unsigned above = __ballot_sync(0xffffffffu, c > g);
+    const int first = above ? __ffs(above) - 1 : 32;
+    const float x0 = lo + (float)first * step, x1 = lo + (float)(first + 1) * step;
+    lo = first == 0 ? lo : x0;
+    hi = first == 32 ? hi : x1;
   }
-  if (active && q == 0) lam[g] = 0.5f * (lo + hi);
+  if (lane == 0) lam[g] = 0.5f * (lo + hi);
 }
 
 // Inverse iteration (two steps) for eigenvalue lam[j] of T, one thread per j
@@ -520,16 +535,17 @@ __global__ void __launch_bounds__(256) bisect_kernel(int n, const float* __restr
 // from j so that members of a tight cluster start in different directions.
 // Per-thread work arrays live in shared memory interleaved by lane.  Y(:, j)
 // (FP32, n x n column-major) receives the unit eigenvector of T.
+// The pivots are stored as reciprocals, so the substitutions hold no division.
 __global__ void __launch_bounds__(32) tridiag_eig_kernel(int n, const float* __restrict__ dg,
                                                          const float* __restrict__ eg,
                                                          const float* __restrict__ lam,
+                                                         const float* __restrict__ bounds,
                                                          float* __restrict__ Y, int ldy) {
-  extern __shared__ float ws[];  // d, e, e^2 (3 n) then 6 arrays of n x 32
+  extern __shared__ float ws[];  // d, e (2 n) then 6 arrays of n x 32
   float* d = ws;
   float* e = ws + n;
-  float* e2 = ws + 2 * n;
-  float* u0 = ws + 3 * n;
-  float* u1 = u0 + 32 * n;
+  float* iu = ws + 2 * n;
+  float* u1 = iu + 32 * n;
   float* u2 = u1 + 32 * n;
   float* lm = u2 + 32 * n;
   float* y = lm + 32 * n;
@@ -537,84 +553,68 @@ __global__ void __launch_bounds__(32) tridiag_eig_kernel(int n, const float* __r
   const int lane = threadIdx.x;
   for (int i = lane; i < n; i += 32) {
     d[i] = dg[i];
-    const float ei = i + 1 < n ? eg[i] : 0.f;
-    e[i] = ei;
-    e2[i] = ei * ei;
+    e[i] = i + 1 < n ? eg[i] : 0.f;
   }
   __syncwarp();
-  float gl = FLT_MAX, gu = -FLT_MAX, emax2 = 0.f;
-  for (int i = 0; i < n; ++i) {
-    const float r = (i > 0 ? fabsf(e[i - 1]) : 0.f) + (i + 1 < n ? fabsf(e[i]) : 0.f);
-    gl = fminf(gl, d[i] - r);
-    gu = fmaxf(gu, d[i] + r);
-    emax2 = fmaxf(emax2, e2[i]);
-  }
-  const float tnorm = fmaxf(fabsf(gl), fabsf(gu));
-  const float pivmin = FLT_MIN * fmaxf(1.f, emax2);
   const int j = blockIdx.x * 32 + lane;
   if (j >= n) return;
   const float L = lam[j];
   // ---- LU with partial pivoting of T - L I (rows i, i + 1 may swap):
-  // U has diagonal u0, superdiagonals u1, u2; multipliers in lm, swaps in sw
-  const float pert = FLT_EPSILON * tnorm + pivmin;
+  // U has diagonal 1 / iu, superdiagonals u1, u2; multipliers in lm, swaps in sw
+  const float pert = FLT_EPSILON * bounds[0] + bounds[1];
 #define AT(arr, i) arr[(i) * 32 + lane]
+  auto recip = [&](float u) {
+    if (fabsf(u) < pert) u = u < 0.f ? -pert : pert;
+    return __fdividef(1.f, u);
+  };
   float diag = d[0] - L, sup = n > 1 ? e[0] : 0.f;
   for (int i = 0; i + 1 < n; ++i) {
     const float sub = e[i], nd = d[i + 1] - L, ns = i + 2 < n ? e[i + 1] : 0.f;
-    if (fabsf(diag) >= fabsf(sub)) {
-      if (diag == 0.f) diag = pert;
-      const float mlt = sub / diag;
-      AT(lm, i) = mlt;
-      AT(sw, i) = 0.f;
-      AT(u0, i) = diag;
-      AT(u1, i) = sup;
-      AT(u2, i) = 0.f;
-      diag = nd - mlt * sup;
-      sup = ns;
-    } else {
-      const float mlt = diag / sub;
-      AT(lm, i) = mlt;
-      AT(sw, i) = 1.f;
-      AT(u0, i) = sub;
-      AT(u1, i) = nd;
-      AT(u2, i) = ns;
-      diag = sup - mlt * nd;
-      sup = -mlt * ns;
-    }
+    const bool keep = fabsf(diag) >= fabsf(sub);
+    if (keep && diag == 0.f) diag = pert;
+    const float mlt = __fdividef(keep ? sub : diag, keep ? diag : sub);
+    AT(lm, i) = mlt;
+    AT(sw, i) = keep ? 0.f : 1.f;
+    AT(iu, i) = recip(keep ? diag : sub);
+    AT(u1, i) = keep ? sup : nd;
+    AT(u2, i) = keep ? 0.f : ns;
+    diag = keep ? nd - mlt * sup : sup - mlt * nd;
+    sup = keep ? ns : -mlt * ns;
   }
-  if (fabsf(diag) < pert) diag = diag < 0.f ? -pert : pert;
-  AT(u0, n - 1) = diag;
-  for (int i = 0; i < n; ++i) AT(y, i) = hash_unit((uint32_t)j, (uint32_t)i);
+  AT(iu, n - 1) = recip(diag);
+  float sc = 1.f;
   for (int step = 0; step < 2; ++step) {
-    // forward: apply the row operations
+    // forward: apply the row operations (to the start vector, then to the
+    // scaled solution of the first step)
+    float yi = step == 0 ? hash_unit((uint32_t)j, 0u) : AT(y, 0) * sc;
+#pragma unroll 4
     for (int i = 0; i + 1 < n; ++i) {
-      const float c = AT(lm, i);
-      if (AT(sw, i) == 0.f) {
-        AT(y, i + 1) -= c * AT(y, i);
-      } else {
-        const float yi = AT(y, i), yi1 = AT(y, i + 1);
-        AT(y, i) = yi1;
-        AT(y, i + 1) = yi - c * yi1;
-      }
+      const float yn = step == 0 ? hash_unit((uint32_t)j, (uint32_t)(i + 1)) : AT(y, i + 1) * sc;
+      const bool swp = AT(sw, i) != 0.f;
+      const float c = AT(lm, i), top = swp ? yn : yi, bot = swp ? yi : yn;
+      AT(y, i) = top;
+      yi = bot - c * top;
     }
     // back substitution with U
-    float nrm = 0.f;
+    float y1 = 0.f, y2 = 0.f, nrm = 0.f, s = yi;
+#pragma unroll 4
     for (int i = n - 1; i >= 0; --i) {
-      float s = AT(y, i);
-      if (i + 1 < n) s -= AT(u1, i) * AT(y, i + 1);
-      if (i + 2 < n) s -= AT(u2, i) * AT(y, i + 2);
-      float u = AT(u0, i);
-      if (fabsf(u) < pert) u = u < 0.f ? -pert : pert;
-      const float xi = s / u;
-      AT(y, i) = xi;
-      nrm = fmaxf(nrm, fabsf(xi));
+      if (i + 1 < n) s = AT(y, i) - AT(u1, i) * y1;
+      if (i + 2 < n) s -= AT(u2, i) * y2;
+      y2 = y1;
+      y1 = s * AT(iu, i);
+      AT(y, i) = y1;
+      nrm = fmaxf(nrm, fabsf(y1));
     }
-    const float sc = nrm > 0.f ? 1.f / nrm : 1.f;
-    for (int i = 0; i < n; ++i) AT(y, i) *= sc;
+    sc = nrm > 0.f ? 1.f / nrm : 1.f;
   }
   float s2 = 0.f;
-  for (int i = 0; i < n; ++i) s2 = fmaf(AT(y, i), AT(y, i), s2);
-  const float inv = s2 > 0.f ? rsqrtf(s2) : 0.f;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) {
+    const float v = AT(y, i) * sc;
+    s2 = fmaf(v, v, s2);
+  }
+  const float inv = s2 > 0.f ? sc * rsqrtf(s2) : 0.f;
   for (int i = 0; i < n; ++i) Y[i + (int64_t)j * ldy] = AT(y, i) * inv;
 #undef AT
 }
@@ -627,16 +627,24 @@ __global__ void __launch_bounds__(32) tridiag_eig_kernel(int n, const float* __r
 __global__ void __launch_bounds__(1024, 1) cluster_orth_kernel(int n, const float* __restrict__ lam,
                                                                float* __restrict__ Y, int ldy) {
   __shared__ int runs[2 * 128];
-  __shared__ int nruns;
+  __shared__ int nruns, near;
+  __shared__ float ls[256];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // the eigenvalues are ascending: the largest magnitude is at an end
+  const float thr = 1e-5f * fmaxf(fabsf(lam[0]), fabsf(lam[n - 1]));
+  if (t == 0) nruns = near = 0;
+  __syncthreads();
+  if (t < n) {
+    ls[t] = lam[t];
+    if (t > 0 && lam[t] - lam[t - 1] <= thr) near = 1;
+  }
+  __syncthreads();
+  if (!near) return;  // no cluster: the usual case ends without the serial scan
   if (t == 0) {
-    float tn = 0.f;
-    for (int i = 0; i < n; ++i) tn = fmaxf(tn, fabsf(lam[i]));
-    const float thr = 1e-5f * tn;
     int nr = 0;
     for (int a = 0; a < n;) {
       int b = a + 1;
-      while (b < n && lam[b] - lam[b - 1] <= thr) ++b;
+      while (b < n && ls[b] - ls[b - 1] <= thr) ++b;
       if (b - a >= 2 && nr < 128) {
         runs[2 * nr] = a;
         runs[2 * nr + 1] = b - a;
@@ -671,50 +679,60 @@ __global__ void __launch_bounds__(1024, 1) cluster_orth_kernel(int n, const floa
 }
 
 // Z = Q Y with Q = H_0 H_1 ... H_{n-3}, H_k = I - tau_k v_k v_k^T: reflectors
-// applied from the last to the first, each column of Y independently (one
-// half-warp per column, 16 columns per CTA).  The reflectors are staged in
-// shared memory (packed, strictly lower part) so that the n sequential
-// reflector steps read no global memory.  Z is written in FP64.
+// applied from the last to the first, each column of Y independently: a warp
+// per column, the column in registers, the reflectors staged in shared memory
+// (packed, strictly lower part).  Bound by the chain of a reflector (a dot
+// product's five shuffles): with half a warp per column and the column in
+// shared memory a reflector took a microsecond (203 us at n = 213; 53 us
+// now).  Z is written in FP64.
 __device__ __forceinline__ int vpk(int n, int k) {  // start of reflector k (rows k+1 .. n-1)
   return k * (n - 1) - (k * (k - 1)) / 2;
 }
 
+template <int NB>
 __global__ void __launch_bounds__(256) backtransform_kernel(int n, const float* __restrict__ V,
                                                             int ldv, const float* __restrict__ tau,
                                                             const float* __restrict__ Y, int ldy,
                                                             double* __restrict__ Z, int ldz) {
-  extern __shared__ float bs[];
-  float* vp = bs;                          // n (n - 1) / 2
-  float* ys = bs + (n * (n - 1)) / 2;      // 16 x n
+  extern __shared__ float vp[];  // n (n - 1) / 2
   __shared__ float ts[256];
-  const int t = threadIdx.x, c = t >> 4, r = t & 15;
-  for (int k = 0; k + 1 < n; ++k) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int k = warp; k + 1 < n; k += 8) {
     const int base = vpk(n, k), len = n - 1 - k;
-    for (int i = t; i < len; i += blockDim.x) vp[base + i] = V[(k + 1 + i) + (int64_t)k * ldv];
+    for (int i = lane; i < len; i += 32) vp[base + i] = V[(k + 1 + i) + (int64_t)k * ldv];
   }
   for (int k = t; k < n; k += blockDim.x) ts[k] = tau[k];
-  const int col = blockIdx.x * 16 + c;
-  const bool active = col < n;
-  float* y = ys + c * n;
-  if (active)
-    for (int i = r; i < n; i += 16) y[i] = Y[i + (int64_t)col * ldy];
+  const int col = blockIdx.x * 8 + warp;
+  float y[NB];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) {
+    const int i = lane + 32 * c;
+    y[c] = (i < n && col < n) ? Y[i + (int64_t)col * ldy] : 0.f;
+  }
   __syncthreads();
-  const unsigned mask = 0xFFFFu << (16 * ((t >> 4) & 1));
+  if (col >= n) return;
   for (int k = n - 3; k >= 0; --k) {
     const float tk = ts[k];
     if (tk == 0.f) continue;
     const float* v = vp + vpk(n, k) - (k + 1);  // v[i] for i = k+1 .. n-1
-    float sacc = 0.f;
-    if (active)
-      for (int i = k + 1 + r; i < n; i += 16) sacc = fmaf(v[i], y[i], sacc);
-    for (int o = 8; o > 0; o >>= 1) sacc += __shfl_xor_sync(mask, sacc, o);
-    sacc *= tk;
-    if (active)
-      for (int i = k + 1 + r; i < n; i += 16) y[i] = fmaf(-sacc, v[i], y[i]);
-    __syncwarp(mask);
+    float vr[NB], s = 0.f;
+#pragma unroll
+    for (int c = 0; c < NB; ++c) {
+      const int i = lane + 32 * c;
+      vr[c] = (i > k && i < n) ? v[i] : 0.f;
+      s = fmaf(vr[c], y[c], s);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    s *= tk;
+#pragma unroll
+    for (int c = 0; c < NB; ++c) y[c] = fmaf(-s, vr[c], y[c]);
   }
-  if (active)
-    for (int i = r; i < n; i += 16) Z[i + (int64_t)col * ldz] = (double)y[i];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) {
+    const int i = lane + 32 * c;
+    if (i < n) Z[i + (int64_t)col * ldz] = (double)y[c];
+  }
 }
 
 // -------------------------------------------- FP64 refinement steps
@@ -837,73 +855,108 @@ __global__ void oa_next_kernel(const int* cur, const unsigned long long* emax, i
     next[0] = (cur[0] || __longlong_as_double((long long)emax[0]) <= 1e-10) ? 1 : 0;
 }
 
-// Final pass on S = X^T A X, G = X^T X of the refined X (one CTA): order by
-// d_i = s_ii, and group the sorted positions into runs: positions k < j join
-// one run (with everything between them) when |s_ij| > 8 eps ||A||_F, i.e.
-// pairs the first-order steps did not decouple (clusters, and pairs whose
-// correction the steps' guard refused).  Outside the runs every coupling is
-// then below 8 eps ||A||_F (row norms below 8 sqrt(n) eps ||A||_F), so the
-// run blocks' FP64 Jacobi finishes the decomposition.  Checks ||I - G||_F at
-// rounding level, finite values and runs no wider than kMaxRunDev; writes the
-// permutation, the runs, the eigenvalues w (ascending) and status[0] = 0 on
-// success, else a bit mask (1 orthogonality, 2 wide run, 8 non-finite) and
-// the caller falls back.
-__global__ void __launch_bounds__(1024, 1) eig_finalize_kernel(int n, const double* __restrict__ GS,
-                                                               const double* __restrict__ scal,
-                                                               int* __restrict__ perm,
-                                                               int* __restrict__ runs,
-                                                               int* __restrict__ nruns_out,
-                                                               double* __restrict__ w,
-                                                               int* status) {
-  __shared__ double dv[256];
-  __shared__ int pm[256], pos[256], reach[256];
-  __shared__ double red[32];
-  __shared__ int s_bad;
+// Final pass on S = X^T A X, G = X^T X of the refined X: order by d_i = s_ii,
+// and group the sorted positions into runs: positions k < j join one run (with
+// everything between them) when |s_ij| > 8 eps ||A||_F, i.e. pairs the
+// first-order steps did not decouple (clusters, and pairs whose correction the
+// steps' guard refused).  Outside the runs every coupling is then below
+// 8 eps ||A||_F (row norms below 8 sqrt(n) eps ||A||_F), so the run blocks' FP64
+// Jacobi finishes the decomposition.  Checks ||I - G||_F at rounding level,
+// finite values and runs no wider than kMaxRunDev; writes the permutation, the
+// runs, the eigenvalues w (ascending) and status[0] = 0 on success, else a bit
+// mask (1 orthogonality, 2 wide run, 8 non-finite) and the caller falls back.
+//
+// The n^2 work (norm and couplings) runs over the whole GPU, a warp per column,
+// with comparisons on the bit patterns: on one CTA its FP64 instructions alone
+// took 80 us at n = 213 (108 us in all; 9 us now).
+__device__ __forceinline__ long long order_key(double x) {  // sorts as x does (NaN at an end)
+  const long long b = __double_as_longlong(x);
+  return b < 0 ? (long long)(0x8000000000000000ULL - (unsigned long long)b) : b;
+}
+
+// reach[pos(i)]: furthest sorted position coupled to column i; part[i]: column
+// i's share of ||I - G||_F^2; perm and w; nonfin[0] = 1 for a non-finite d_i.
+__global__ void __launch_bounds__(256) eig_scan_kernel(int n, const double* __restrict__ GS,
+                                                       const double* __restrict__ scal,
+                                                       int* __restrict__ perm,
+                                                       int* __restrict__ reach,
+                                                       double* __restrict__ part,
+                                                       double* __restrict__ w, int* nonfin) {
+  __shared__ long long key[256];
+  __shared__ int pos[256];
   const double* G = GS;
   const double* S = GS + (int64_t)n * n;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  if (t < n) dv[t] = S[t + (int64_t)t * n];
-  if (t == 0) s_bad = 0;
+  const int t = threadIdx.x, lane = t & 31;
+  double dt = 0.0;
+  if (t < n) {
+    dt = S[t + (int64_t)t * n];
+    key[t] = order_key(dt);
+  }
   __syncthreads();
   if (t < n) {  // rank of d_t (ties by index)
     int r = 0;
-    const double x = dv[t];
-    for (int j = 0; j < n; ++j) r += (dv[j] < x || (dv[j] == x && j < t)) ? 1 : 0;
-    pm[r] = t;
+    const long long kt = key[t];
+    for (int j = 0; j < n; ++j) r += (key[j] < kt || (key[j] == kt && j < t)) ? 1 : 0;
     pos[t] = r;
-    if (!isfinite(x)) atomicOr(&s_bad, 8);
+    if (blockIdx.x == 0) {
+      perm[r] = t;
+      w[r] = dt;
+      if ((__double_as_longlong(dt) & 0x7FF0000000000000LL) == 0x7FF0000000000000LL) nonfin[0] = 1;
+    }
   }
+  __syncthreads();
+  const int i = blockIdx.x * 8 + (t >> 5);
+  if (i >= n) return;
+  const long long thr = __double_as_longlong(8.0 * kEps64 * scal[0]);  // >= 0: ordered as bits
+  int rmax = pos[i];
   double b = 0.0;
-  for (int e = t; e < n * n; e += blockDim.x) {
-    const int i = e % n, j = e / n;
-    const double r = (i == j ? 1.0 : 0.0) - G[e];
+  for (int j = lane; j < n; j += 32) {
+    const long long m = __double_as_longlong(S[j + (int64_t)i * n]) & 0x7FFFFFFFFFFFFFFFLL;
+    if (j != i && m > thr) rmax = max(rmax, pos[j]);
+    const double r = (i == j ? 1.0 : 0.0) - G[j + (int64_t)i * n];
     b = fma(r, r, b);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    rmax = max(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  if (lane == 0) {
+    reach[pos[i]] = rmax;
+    part[i] = b;
+  }
+}
+
+__global__ void __launch_bounds__(256) eig_finalize_kernel(int n, const int* __restrict__ reach_g,
+                                                           const double* __restrict__ part,
+                                                           int* __restrict__ runs,
+                                                           int* __restrict__ nruns_out,
+                                                           int* nonfin, int* status) {
+  __shared__ int reach[256];
+  __shared__ double red[8];
+  __shared__ int coupled;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t == 0) coupled = 0;
+  __syncthreads();
+  double b = t < n ? part[t] : 0.0;
+  if (t < n) {
+    reach[t] = reach_g[t];
+    if (reach[t] != t) coupled = 1;
   }
   for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
   if (lane == 0) red[warp] = b;
   __syncthreads();
-  const double thr = 8.0 * kEps64 * scal[0];
-  // furthest sorted position coupled to each position (a warp per column of
-  // S, contiguous reads; S is symmetric to rounding)
-  for (int tt = warp; tt < n; tt += 32) {
-    const int i = pm[tt];
-    int rmax = tt;
-    for (int j = lane; j < n; j += 32)
-      if (j != i && !(fabs(S[j + (int64_t)i * n]) <= thr)) rmax = max(rmax, pos[j]);
-    for (int o = 16; o > 0; o >>= 1) rmax = max(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-    if (lane == 0) reach[tt] = rmax;
-  }
-  __syncthreads();
-  if (t == 0) {
-    double sb = 0.0;
-    for (int q = 0; q < 32; ++q) sb += red[q];
-    if (!(sqrt(sb) <= 64.0 * n * kEps64)) s_bad |= 1;
-    int nr = 0;
+  if (t != 0) return;
+  double sb = 0.0;
+  for (int q = 0; q < 8; ++q) sb += red[q];
+  int bad = nonfin[0] ? 8 : 0, nr = 0;
+  nonfin[0] = 0;
+  if (!(sqrt(sb) <= 64.0 * n * kEps64)) bad |= 1;
+  if (coupled)
     for (int k = 0; k < n;) {
       int e2 = reach[k];
       for (int j = k; j <= e2; ++j) e2 = max(e2, reach[j]);
       const int m = e2 - k + 1;
-      if (m > kMaxRunDev) s_bad |= 2;
+      if (m > kMaxRunDev) bad |= 2;
       if (m >= 2) {
         runs[2 * nr] = k;
         runs[2 * nr + 1] = m;
@@ -911,14 +964,8 @@ __global__ void __launch_bounds__(1024, 1) eig_finalize_kernel(int n, const doub
       }
       k = e2 + 1;
     }
-    nruns_out[0] = nr;
-  }
-  __syncthreads();
-  if (t < n) {
-    perm[t] = pm[t];
-    w[t] = dv[pm[t]];
-  }
-  if (t == 0) status[0] = s_bad;
+  nruns_out[0] = nr;
+  status[0] = bad;
 }
 
 // Zo(:, k) = X(:, perm[k]) (column permutation into the output).
@@ -1119,13 +1166,42 @@ __global__ void eig1_kernel(const double* A, double* Z, double* w, int* status) 
   status[0] = 0;
 }
 
-// S = (A + A^T) / 2 (n x n)
-__global__ void symmetrize_copy_kernel(int n, const double* __restrict__ A, int lda,
-                                       double* __restrict__ S, int lds) {
+// S = (A + A^T) / 2 (n x n), with each CTA's share of ||S||_F^2
+__global__ void __launch_bounds__(256) symmetrize_copy_kernel(int n, const double* __restrict__ A,
+                                                              int lda, double* __restrict__ S,
+                                                              int lds, double* __restrict__ part) {
+  __shared__ double red[8];
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)n * n) return;
-  const int i = (int)(e % n), j = (int)(e / n);
-  S[i + (int64_t)j * lds] = 0.5 * (A[i + (int64_t)j * lda] + A[j + (int64_t)i * lda]);
+  double v = 0.0;
+  if (e < (int64_t)n * n) {
+    const int i = (int)(e % n), j = (int)(e / n);
+    v = 0.5 * (A[i + (int64_t)j * lda] + A[j + (int64_t)i * lda]);
+    S[i + (int64_t)j * lds] = v;
+  }
+  v *= v;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int q = 0; q < 8; ++q) s += red[q];
+    part[blockIdx.x] = s;
+  }
+}
+
+// out[0] = sqrt of the sum of m partials (m <= 256, fixed order)
+__global__ void __launch_bounds__(256) norm_finish_kernel(int m, const double* __restrict__ part,
+                                                          double* out) {
+  __shared__ double red[8];
+  double v = threadIdx.x < m ? part[threadIdx.x] : 0.0;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int q = 0; q < 8; ++q) s += red[q];
+    out[0] = sqrt(s);
+  }
 }
 
 __global__ void copy_block_cm_kernel(int rows, int cols, const double* __restrict__ S, int lds,
@@ -1437,13 +1513,13 @@ int DevDense::init(int64_t nmax_) {
   ok = ok && g((void**)&f32v, 4 * (size_t)nmax * sizeof(float));
   ok = ok && g((void**)&vec, (8 * (size_t)nmax + 256) * sizeof(double));
   ok = ok && g((void**)&scal, 16 * sizeof(double));
-  ok = ok && g((void**)&ints, (4 * (size_t)nmax + 64) * sizeof(int));
+  ok = ok && g((void**)&ints, (5 * (size_t)nmax + 64) * sizeof(int));
   ok = ok && g((void**)&part, (size_t)tiles * kMaxKs * 256 * sizeof(double));
   ok = ok && g((void**)&cnt, (size_t)tiles * sizeof(unsigned));
   if (!ok) return LOBPCG_ERR_OOM;
   cnt_tiles = tiles;
   if (cudaMemset(cnt, 0, (size_t)tiles * sizeof(unsigned)) != cudaSuccess) return LOBPCG_ERR_CUDA;
-  if (cudaMemset(ints, 0, (4 * (size_t)nmax + 64) * sizeof(int)) != cudaSuccess)
+  if (cudaMemset(ints, 0, (5 * (size_t)nmax + 64) * sizeof(int)) != cudaSuccess)
     return LOBPCG_ERR_CUDA;
   if (cudaDeviceSynchronize() != cudaSuccess) return LOBPCG_ERR_CUDA;
   return LOBPCG_OK;
@@ -1517,15 +1593,16 @@ int dev_syev(DenseLayer& L, int n, const double* A, int lda, double* Z, int ldz,
   if (dev < 0 || dev >= 64 || !configured[dev]) {
     LOB_CUDA_OK(cudaFuncSetAttribute(tridiag32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kDevDenseMax * (kDevDenseMax + 1) / 2 * 4));
-    LOB_CUDA_OK(cudaFuncSetAttribute(tridiag32_full_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kTridFull * (kTridFull | 1) * 4));
     LOB_CUDA_OK(cudaFuncSetAttribute(tridiag_eig_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (3 * kDevDenseMax + 6 * 32 * kDevDenseMax) * 4));
-    LOB_CUDA_OK(cudaFuncSetAttribute(backtransform_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (kDevDenseMax * (kDevDenseMax - 1) / 2 + 16 * kDevDenseMax) * 4));
+                                     (2 * kDevDenseMax + 6 * 32 * kDevDenseMax) * 4));
+    constexpr int vbytes = kDevDenseMax * (kDevDenseMax - 1) / 2 * 4;
+    const void* bt[8] = {(const void*)backtransform_kernel<1>, (const void*)backtransform_kernel<2>,
+                         (const void*)backtransform_kernel<3>, (const void*)backtransform_kernel<4>,
+                         (const void*)backtransform_kernel<5>, (const void*)backtransform_kernel<6>,
+                         (const void*)backtransform_kernel<7>, (const void*)backtransform_kernel<8>};
+    for (const void* f : bt)
+      LOB_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, vbytes));
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   if (n == 1) {
@@ -1540,29 +1617,52 @@ int dev_syev(DenseLayer& L, int n, const double* A, int lda, double* Z, int ldz,
   double* normA = D.scal;  // scal[0] = ||A||_F
   // the refinement multiplies by the symmetric part of A (a projected
   // matrix formed by products is symmetric only to rounding)
-  symmetrize_copy_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, A, lda, D.Zt, n);
+  // (its norm partials lie where the refinement's vectors will)
+  symmetrize_copy_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, A, lda, D.Zt, n, D.vec);
+  DLAUNCH(L);
+  norm_finish_kernel<<<1, 256, 0, L.st>>>((int)nblk((int64_t)n * n), D.vec, normA);
   DLAUNCH(L);
   A = D.Zt;
   lda = n;
-  if (n <= kTridFull)
-    tridiag32_full_kernel<<<1, 1024, (size_t)n * (n | 1) * 4, L.st>>>(n, A, lda, d32, e32, D.V32,
-                                                                      n, tau32, normA);
-  else
+  const int nb = (int)ceil_div(n, 32);
+  float* bounds = reinterpret_cast<float*>(D.scal + 8);
+  auto tridiag = [&](auto* kernel) {
+    kernel<<<1, 512, 0, L.st>>>(n, A, lda, d32, e32, D.V32, n, tau32);
+  };
+  if (n > kTridRegMax)
     tridiag32_kernel<<<1, 1024, (size_t)n * (n + 1) / 2 * 4, L.st>>>(n, A, lda, d32, e32, D.V32,
-                                                                     n, tau32, normA);
+                                                                     n, tau32);
+  else if (nb == 1) tridiag(tridiag32_reg_kernel<1>);
+  else if (nb == 2) tridiag(tridiag32_reg_kernel<2>);
+  else if (nb == 3) tridiag(tridiag32_reg_kernel<3>);
+  else if (nb == 4) tridiag(tridiag32_reg_kernel<4>);
+  else if (nb == 5) tridiag(tridiag32_reg_kernel<5>);
+  else if (nb == 6) tridiag(tridiag32_reg_kernel<6>);
+  else tridiag(tridiag32_reg_kernel<7>);
   DLAUNCH(L);
-  bisect_kernel<<<(unsigned)ceil_div(4 * n, 256), 256, 0, L.st>>>(n, d32, e32, lam32);
+  bisect_kernel<<<(unsigned)ceil_div(n, 8), 256, 0, L.st>>>(n, d32, e32, lam32, bounds);
   DLAUNCH(L);
-  tridiag_eig_kernel<<<(unsigned)ceil_div(n, 32), 32, (size_t)(3 * n + 6 * 32 * n) * 4, L.st>>>(
-      n, d32, e32, lam32, D.Y32, n);
+  tridiag_eig_kernel<<<(unsigned)ceil_div(n, 32), 32, (size_t)(2 * n + 6 * 32 * n) * 4, L.st>>>(
+      n, d32, e32, lam32, bounds, D.Y32, n);
   DLAUNCH(L);
   cluster_orth_kernel<<<1, 1024, 0, L.st>>>(n, lam32, D.Y32, n);
   DLAUNCH(L);
   // X (first n columns of XA) = Q Y
   double* X = D.XA;
-  backtransform_kernel<<<(unsigned)ceil_div(n, 16), 256,
-                         (size_t)((n * (n - 1)) / 2 + 16 * n) * 4, L.st>>>(
-      n, D.V32, n, tau32, D.Y32, n, X, n);
+  auto back = [&](auto* kernel) {
+    kernel<<<(unsigned)ceil_div(n, 8), 256, (size_t)(n * (n - 1)) / 2 * 4, L.st>>>(
+        n, D.V32, n, tau32, D.Y32, n, X, n);
+  };
+  switch (nb) {
+    case 1: back(backtransform_kernel<1>); break;
+    case 2: back(backtransform_kernel<2>); break;
+    case 3: back(backtransform_kernel<3>); break;
+    case 4: back(backtransform_kernel<4>); break;
+    case 5: back(backtransform_kernel<5>); break;
+    case 6: back(backtransform_kernel<6>); break;
+    case 7: back(backtransform_kernel<7>); break;
+    default: back(backtransform_kernel<8>); break;
+  }
   DLAUNCH(L);
   return dev_syev_refine(L, n, Z, ldz, w, status, kRefSteps);
 }
@@ -1632,7 +1732,12 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
   if ((rc = dev_gemm(L, true, false, n, 2 * n, n, 1.0, X, n, D.XA, n, 0.0, nullptr, 0, G, n,
                      nullptr)))
     return rc;
-  eig_finalize_kernel<<<1, 1024, 0, L.st>>>(n, D.GS, normA, perm, runs, nruns, w, status);
+  int* nonfin = D.ints + 4 * D.nmax + 60;
+  int* reach = D.ints + 4 * D.nmax + 64;
+  eig_scan_kernel<<<(unsigned)ceil_div(n, 8), 256, 0, L.st>>>(n, D.GS, normA, perm, reach, D.vec, w,
+                                                              nonfin);
+  DLAUNCH(L);
+  eig_finalize_kernel<<<1, 256, 0, L.st>>>(n, reach, D.vec, runs, nruns, nonfin, status);
   DLAUNCH(L);
   permute_cols_dev_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, X, n, perm, Z, ldz);
   DLAUNCH(L);
