@@ -528,8 +528,7 @@ LOBPCG_EXPORT int lobpcg_gram(int64_t n, const double* U, int64_t ldu, int64_t p
   const int64_t need = lobpcg_gram_workspace(n, p, q, mode, slices);
   void* own = nullptr;
   if (!work) {
-    if (cudaMallocAsync(&own, (size_t)std::max<int64_t>(need, 16), st) != cudaSuccess)
-      return LOBPCG_ERR_OOM;
+    if (lob::scratch_alloc(&own, (size_t)need, st)) return LOBPCG_ERR_OOM;
     work = own;
     work_bytes = need;
   }
@@ -539,7 +538,7 @@ LOBPCG_EXPORT int lobpcg_gram(int64_t n, const double* U, int64_t ldu, int64_t p
                : mode == LOBPCG_GEMM_OZAKI
                      ? lob::gram_ozaki(st, n, Us, Vs, G, ldg, slices, work, work_bytes)
                      : lob::gram_f64(st, n, Us, Vs, G, ldg, work, work_bytes);
-  if (own) cudaFreeAsync(own, st);
+  lob::scratch_free(own, st);
   return rc;
 }
 
@@ -577,12 +576,12 @@ LOBPCG_EXPORT int lobpcg_update(int64_t n, const double* S, int64_t lds, int64_t
     const int64_t need = tc ? lob::update_tc_workspace(n, (int)s, (int)m, slices)
                             : lob::update_ozaki_workspace(n, (int)s, (int)m, slices);
     void* own = nullptr;
-    if (need > 0 && cudaMallocAsync(&own, (size_t)need, st) != cudaSuccess) return LOBPCG_ERR_OOM;
+    if (need > 0 && lob::scratch_alloc(&own, (size_t)need, st)) return LOBPCG_ERR_OOM;
     int rc = tc ? lob::update_tc(st, n, Ss, C, ldc, (int)m, alpha, beta, Y0s, out, slices, own,
                                  need)
                 : lob::update_ozaki(st, n, Ss, C, ldc, (int)m, alpha, beta, Y0s, out, slices,
                                     own, need);
-    if (own) cudaFreeAsync(own, st);
+    lob::scratch_free(own, st);
     return rc;
   }
   return lob::update_f64(st, n, Ss, C, ldc, (int)m, alpha, beta, Y0s, out);
@@ -599,14 +598,14 @@ LOBPCG_EXPORT int lobpcg_residual(int64_t n, const double* X, const double* AX,
   cudaStream_t st = (cudaStream_t)stream;
   void* part = nullptr;
   const size_t pb = (size_t)lob::residual_workspace(n, (int)(m - c0));
-  if (cudaMallocAsync(&part, pb + (kdiag ? (size_t)n * sizeof(double) : 0), st) != cudaSuccess)
+  if (lob::scratch_alloc(&part, pb + (kdiag ? (size_t)n * sizeof(double) : 0), st))
     return LOBPCG_ERR_OOM;
   double* kinv = kdiag ? (double*)((char*)part + pb) : nullptr;
   int rc = kdiag ? lob::reciprocal(st, n, kdiag, kinv) : LOBPCG_OK;
   if (!rc)
     rc = lob::residual(st, n, X, AX, BX, ld, (int)m, (int)c0, theta, kinv, W, ldw, normA, normB,
                        be, part);
-  cudaFreeAsync(part, st);
+  lob::scratch_free(part, st);
   return rc;
 }
 

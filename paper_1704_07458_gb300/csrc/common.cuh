@@ -64,6 +64,11 @@ __device__ __forceinline__ double* out_addr(const OutList& o, int c, int64_t row
   return c < o.split ? o.ptr[0] + row * o.ld[0] + c : o.ptr[1] + row * o.ld[1] + (c - o.split);
 }
 
+// Device scratch in stream order from this library's pool (scratch.cu).
+int scratch_alloc(void** p, size_t bytes, cudaStream_t st);
+void scratch_free(void* p, cudaStream_t st);
+void scratch_trim();  // the current device's kept memory goes back
+
 // Kernel launch counter (host side, per process) used for the stats.
 extern int64_t g_launches;
 

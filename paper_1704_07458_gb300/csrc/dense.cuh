@@ -33,6 +33,10 @@ struct DevDense {
   int cnt_tiles = 0;
   int init(int64_t n_max);
   void release();
+  // Layout of the buffers in one block for orders up to n_max: bytes needed;
+  // with a base, the pointers are set (the first clear_bytes of the block must
+  // be zero before the first use).
+  size_t carve(int64_t n_max, char* base, size_t* clear_bytes);
 };
 
 struct DenseLayer {

@@ -1492,35 +1492,52 @@ unsigned nblk(int64_t total) { return (unsigned)std::max<int64_t>(1, ceil_div(to
 
 // ==================================================================== host
 
-int DevDense::init(int64_t nmax_) {
-  nmax = (int)std::min<int64_t>(nmax_, kDevDenseMax);
-  const size_t nn = (size_t)nmax * nmax;
-  const int tiles = (int)(ceil_div(nmax, kGT) * ceil_div(2 * nmax, kGT));
-  auto g = [&](void** p, size_t bytes) {
-    if (cudaMalloc(p, std::max<size_t>(bytes, 16)) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    bufs.push_back(*p);
-    return true;
+size_t DevDense::carve(int64_t nmax_, char* base, size_t* clear_bytes) {
+  const int nm = (int)std::min<int64_t>(nmax_, kDevDenseMax);
+  const size_t nn = (size_t)nm * nm;
+  const int tiles = (int)(ceil_div(nm, kGT) * ceil_div(2 * nm, kGT));
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    char* p = base ? base + at : nullptr;
+    at += (bytes + 255) / 256 * 256;
+    return (void*)p;
   };
-  bool ok = true;
-  for (double** b : {&X, &X1, &E, &Zt, &T1, &T2, &T3, &T4}) ok = ok && g((void**)b, nn * sizeof(double));
-  ok = ok && g((void**)&XA, 2 * nn * sizeof(double));   // [X | A X]
-  ok = ok && g((void**)&GS, 2 * nn * sizeof(double));   // [G | S]
-  ok = ok && g((void**)&V32, nn * sizeof(float));
-  ok = ok && g((void**)&Y32, nn * sizeof(float));
-  ok = ok && g((void**)&f32v, 4 * (size_t)nmax * sizeof(float));
-  ok = ok && g((void**)&vec, (8 * (size_t)nmax + 256) * sizeof(double));
-  ok = ok && g((void**)&scal, 16 * sizeof(double));
-  ok = ok && g((void**)&ints, (5 * (size_t)nmax + 64) * sizeof(int));
-  ok = ok && g((void**)&part, (size_t)tiles * kMaxKs * 256 * sizeof(double));
-  ok = ok && g((void**)&cnt, (size_t)tiles * sizeof(unsigned));
-  if (!ok) return LOBPCG_ERR_OOM;
-  cnt_tiles = tiles;
-  if (cudaMemset(cnt, 0, (size_t)tiles * sizeof(unsigned)) != cudaSuccess) return LOBPCG_ERR_CUDA;
-  if (cudaMemset(ints, 0, (5 * (size_t)nmax + 64) * sizeof(int)) != cudaSuccess)
-    return LOBPCG_ERR_CUDA;
+  unsigned* c = (unsigned*)take((size_t)tiles * sizeof(unsigned));
+  int* in = (int*)take((5 * (size_t)nm + 64) * sizeof(int));
+  if (clear_bytes) *clear_bytes = at;
+  double* m[8];
+  for (double*& p : m) p = (double*)take(nn * sizeof(double));
+  double* xa = (double*)take(2 * nn * sizeof(double));  // [X | A X]
+  double* gs = (double*)take(2 * nn * sizeof(double));  // [G | S]
+  float* v32 = (float*)take(nn * sizeof(float));
+  float* y32 = (float*)take(nn * sizeof(float));
+  float* fv = (float*)take(4 * (size_t)nm * sizeof(float));
+  double* ve = (double*)take((8 * (size_t)nm + 256) * sizeof(double));
+  double* sc = (double*)take(16 * sizeof(double));
+  double* pt = (double*)take((size_t)tiles * kMaxKs * 256 * sizeof(double));
+  if (base) {
+    nmax = nm;
+    cnt_tiles = tiles;
+    cnt = c;
+    ints = in;
+    X = m[0]; X1 = m[1]; E = m[2]; Zt = m[3];
+    T1 = m[4]; T2 = m[5]; T3 = m[6]; T4 = m[7];
+    XA = xa; GS = gs; V32 = v32; Y32 = y32; f32v = fv; vec = ve; scal = sc; part = pt;
+  }
+  return at;
+}
+
+int DevDense::init(int64_t nmax_) {
+  size_t clear = 0;
+  const size_t bytes = carve(nmax_, nullptr, &clear);
+  void* p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return LOBPCG_ERR_OOM;
+  }
+  bufs.push_back(p);
+  carve(nmax_, (char*)p, nullptr);
+  if (cudaMemset(p, 0, clear) != cudaSuccess) return LOBPCG_ERR_CUDA;
   if (cudaDeviceSynchronize() != cudaSuccess) return LOBPCG_ERR_CUDA;
   return LOBPCG_OK;
 }

@@ -1134,6 +1134,7 @@ LOBPCG_EXPORT void lobpcg_destroy(lobpcg_t h) {
   if (!h) return;
   cudaStreamSynchronize(h->st);
   delete h;
+  scratch_trim();
 }
 
 LOBPCG_EXPORT const char* lobpcg_last_error(lobpcg_t h) { return h ? h->err.c_str() : "null handle"; }
