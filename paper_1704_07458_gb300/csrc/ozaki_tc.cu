@@ -10,25 +10,22 @@
 // operations only.  No FP64 instruction runs on the hot path.
 //
 // GB300 mapping:
-//  * one CTA per SM owns a 128 x NT output tile (Gram: 256 threads; update:
-//    512 compute threads and a helper warpgroup),
-//    NT <= 96 a multiple of 16: tcgen05.mma kind::f16, M = 128, N = NT, K = 16;
+//  * one CTA per SM owns a 128 x NT output tile (512 compute threads and a
+//    helper warpgroup), NT <= 96 a multiple of 16: tcgen05.mma kind::f16,
+//    M = 128, N = NT, K = 16, A in TMEM, B in shared memory;
 //  * the contraction runs in chunks of 16 (rows of U and V for the Gram,
-//    columns of S for the update), grouped in blocks of 256 that share one
-//    exponent per operand column (Gram) or row (update).  With |digit| <= 128
-//    the sums of levels 0, 1, 2 (and 3 for S = 7) stay below 2^24 in their
-//    units over a block, so they are exact in FP32; the deeper levels (below
-//    2^-24 resp. 2^-32 of level 0) share one inexact accumulator.  4 or 5
-//    accumulators x NT columns fit the 512 TMEM columns, and TMEM is read once
-//    per block instead of once per chunk;
-//  * Gram: the raw FP64 operands stream into three shared-memory stages by
-//    cp.async, two chunks ahead of use; the tensor core multiplies chunk c while
-//    the compute threads cut chunk c + 1 (two digit-plane stages).  Update: see
-//    its kernel; the digits of the small matrix C are cut once per call and
+//    columns of S for the update), grouped in blocks of at most 256 (the Gram's
+//    share one exponent per operand column; the update has one per row).  With
+//    |digit| <= 128 the sums of levels 0, 1, 2 (and 3 for S = 7) stay below 2^24
+//    in their units over a block, so they are exact in FP32; the deeper levels
+//    (below 2^-24 resp. 2^-32 of level 0) share one inexact accumulator.  4 or 5
+//    accumulators x NT columns and two to four digit stages of A fit the 512
+//    TMEM columns, and the accumulators are read once per block;
+//  * compute warps cut FP64 values from global memory straight into digit
+//    planes; their loads for the chunk after next are in flight meanwhile.  The
+//    digits of the small matrix C of the update are cut once per call and
 //    arrive by cp.async.bulk four chunks ahead;
-//  * the shared exponents come from a streaming pre-pass at full occupancy
-//    (per 256-row block and column for the Gram, per row for the update), so
-//    the tensor-core kernels never wait on a global load of their own;
+//  * the shared exponents come from a streaming pre-pass at full occupancy;
 //  * every mbarrier wait is bounded: a wait that runs out marks the result NaN
 //    (and, for the update, sets a status bit that the solver reads with its
 //    per-iteration scalars) and the CTA returns instead of hanging.
@@ -45,10 +42,8 @@ constexpr int TCM = 128;            // MMA M
 constexpr int TCK = 16;             // contraction length of a chunk (one MMA K)
 constexpr int KG = TCK / 8;         // core-matrix groups along K in a chunk
 constexpr int kChunksPerBlock = 16; // 256 rows / columns share one exponent
-constexpr int kRaw = 3;             // raw FP64 stages (prefetch distance 2)
 constexpr int kBlock = TCK * kChunksPerBlock;
 constexpr int NTMAX = 96;           // max MMA N (output columns of a tile)
-constexpr int kThr = 256;
 constexpr int kFrac = 30;           // fraction bits of the int64 accumulators
 constexpr int kEZero = -4000;       // exponent of an all-zero block
 constexpr uint32_t kTmemCols = 512;
@@ -106,117 +101,139 @@ __device__ __forceinline__ void digits(double x, int E, float (&d)[S]) {
   d[0] = (float)(int)(G >> (8 * (S - 1)));
 }
 
-// The same digits with about half the instructions, for exponent bounds away
-// from the ends of the range: every step is a 32-bit operation.  ke is
-// (digit_ke<S>() + E) << 20 modulo 2^32.  With M = the 53-bit mantissa at the
-// top of 64 bits, F' = M >> q keeps 8 bits below the last digit; one's
-// complement for a negative x and 0x80 added to every byte then round half up
-// in magnitude (the byte below the last digit) and balance the digits at once,
-// so byte b of the sum is digit + 128.  S = 7 has no room for those 8 bits:
-// one rounding bit, and the low byte is the last digit.  Needs 64 <= q for a
-// zero or subnormal x (its implicit bit is set here), so E > kFastEMin, and
-// E < kFastEMax for q < 4096.
-constexpr int kFastEMin = -900, kFastEMax = 1500;
-constexpr int kEZeroFast = 1100;  // stands for kEZero: every shift clears the value
+// The splits of the compute warps: eight consecutive K values of one row or
+// column, first in a form that frees the registers of the values (load), then
+// plane by plane (plane): four packed BF16 pairs each.  The exponent bounds come
+// as thr = split_thr(E), which is additive in E modulo 2^32; it serves
+// kFastEMin < E < kFastEMax, `load_any` serves every E.
+//
+// S <= 6, on the FP32 pipe.  The integer pipe takes an instruction every two
+// cycles, so a split by shifts and byte permutes (25 integer instructions per
+// value) bounded the kernels at 1,400 to 2,200 cycles a chunk against 1,300 of
+// MMAs.  Here x 2^(7-E) is a sum a + b of two floats: a takes the top 24 bits of
+// the mantissa with the exponent field moved by one multiply-add (values below
+// 2^-87 of the bound are raised to it: all their digits are zero), b the other
+// 29 bits through one conversion.  Digit s is what the sum rounds to at a
+// multiple of 2^-8s: adding and subtracting 1.5 * 2^(23-8s) leaves it, exact,
+// pre-weighted and balanced (|d_s| <= 128); b joins at the third digit.  Nine
+// integer instructions per value remain.
+constexpr int kFastEMin = -900, kFastEMax = 1100;
 
-template <int S>
-__host__ __device__ constexpr int digit_ke() { return 1079 - 8 * S + (S >= 7 ? 7 : 0); }
+__host__ __device__ constexpr uint32_t split_thr(int E) { return (uint32_t)(E + 889) << 20; }
 
-template <int S>
-__device__ __forceinline__ uint2 biased_bytes(double x, uint32_t ke) {
-  const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
-  const uint32_t q = (ke - (xh & 0x7FF00000u)) >> 20;
-  const uint32_t mh = (xh & 0x000FFFFFu) | 0x00100000u;
-  const uint32_t Mh = __funnelshift_l(xl, mh, 11), Ml = xl << 11;
-  // 64-bit right shift by any q: the shifts clamp at 32 instead of wrapping
-  uint32_t Fl, Fh;
-  asm("shr.u32 %0, %1, %2;\n" : "=r"(Fh) : "r"(Mh), "r"(q));
-  asm("shr.u32 %0, %1, %2;\n"
-      : "=r"(Fl)
-      : "r"(__funnelshift_rc(Ml, Mh, q)), "r"((uint32_t)max((int)q - 32, 0)));
-  const uint32_t sg = (uint32_t)((int)xh >> 31);
-  constexpr unsigned long long bias =
-      S >= 7 ? 0x0080808080808080ULL : (0x8080808080808080ULL >> (8 * (7 - S)));
-  uint2 g;
-  if (S >= 7) {  // round half up, then two's complement
-    asm("add.cc.u32 %0, %0, 1;\n\taddc.u32 %1, %1, 0;\n" : "+r"(Fl), "+r"(Fh));
-    Fl = __funnelshift_r(Fl, Fh, 1);
-    Fh >>= 1;
-    Fl ^= sg;
-    Fh ^= sg;
-    asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %2;\n" : "+r"(Fl), "+r"(Fh) : "r"(sg));
-  } else {
-    Fl ^= sg;
-    Fh ^= sg;
-  }
-  asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %4, %5;\n"
-      : "=r"(g.x), "=r"(g.y)
-      : "r"(Fl), "r"((uint32_t)bias), "r"(Fh), "r"((uint32_t)(bias >> 32)));
-  return g;
+__host__ __device__ constexpr float pow2f(int e) {
+  return e >= 0 ? (float)(1ull << e) : 1.0f / (float)(1ull << -e);
 }
 
-// pre-weighted digit s of a biased fixed-point value, as a float exact in BF16
-template <int S, int s>
-__device__ __forceinline__ float byte_digit(uint2 g) {
-  constexpr int b = S - 1 - s + (S >= 7 ? 0 : 1);
-  uint32_t t;
-  if (s == 0) {  // nine bits: the leading digit reaches +128
-    t = b == 3 ? __byte_perm(__byte_perm(g.x, g.y, 0x4343), 0x4B000000u, 0x7410)
-               : __byte_perm(b < 4 ? g.x : g.y, 0x4B000000u, 0x7400u | ((b & 3) + 1) << 4 | (b & 3));
-  } else {
-    t = __byte_perm(b < 4 ? g.x : g.y, 0x4B000000u, 0x7540u | (uint32_t)(b & 3));
-  }
-  // 0x4B000000 + u is 2^23 + u as a float; minus (2^23 + 128), scaled by 2^-8s (exact)
-  const float sc = __uint_as_float((uint32_t)(127 - 8 * s) << 23);
-  return fmaf(__uint_as_float(t), sc, -8388736.0f * sc);
-}
-
-// plane s of 8 consecutive K values: four packed BF16 pairs
-template <int S, int s>
-__device__ __forceinline__ void plane8(const uint2 (&g)[8], uint32_t (&w)[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    w[i] = __byte_perm(__float_as_uint(byte_digit<S, s>(g[2 * i])),
-                       __float_as_uint(byte_digit<S, s>(g[2 * i + 1])), 0x7632);
-}
-
-// the biased fixed-point value of the general split: any exponent bound
+// F = round(x 2^(8S-1-E)), the fixed-point integer of `digits`
 template <int S>
-__device__ __noinline__ uint2 biased_bytes_any(double x, int E) {
+__device__ __noinline__ long long fixed_any(double x, int E) {
   const long long bits = __double_as_longlong(x);
   const int be = (int)((bits >> 52) & 0x7FF);
   const long long mant = (bits & 0x000FFFFFFFFFFFFFLL) | ((long long)(be != 0) << 52);
   const int t = min(max(2 - (max(be, 1) - 1076 + 8 * S - E), 0), 63);
   const long long F = (((mant << 3) >> t) + 1) >> 1;
-  long long G = bits < 0 ? -F : F;
-  constexpr unsigned long long bias =
-      S >= 7 ? 0x0080808080808080ULL : (0x8080808080808080ULL >> (8 * (7 - S)));
-  if (S < 7) G *= 256;
-  const unsigned long long B = (unsigned long long)G + bias;
-  return make_uint2((uint32_t)B, (uint32_t)(B >> 32));
+  return bits < 0 ? -F : F;
 }
 
-// 8 consecutive K values of one M/N index -> S planes, one 16-byte shared
-// store per plane (K-major core-matrix row: 8 BF16 along K).
 template <int S>
-__device__ __forceinline__ void split8(const double (&x)[8], const int (&E)[8], uint32_t dst,
-                                       uint32_t pstride) {
-  uint32_t w[S][4];
-#pragma unroll
-  for (int i = 0; i < 8; i += 2) {
-    float a[S], b[S];
-    digits<S>(x[i], E[i], a);
-    digits<S>(x[i + 1], E[i + 1], b);
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-      w[s][i >> 1] = __byte_perm(__float_as_uint(a[s]), __float_as_uint(b[s]), 0x7632);
+struct Split {
+  float a[8], b[8];
+
+  __device__ __forceinline__ void load(int i, double x, uint32_t thr) {
+    const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
+    const uint32_t m = (uint32_t)max((int)(xh & 0x7FFFFFFFu), (int)(thr + (40u << 20)));
+    // exponent field be - E - 889 = (be - 1023) + (7 - E) + 127
+    const uint32_t w = __funnelshift_l(xl, m, 3) - thr * 8u;
+    const uint32_t sw = (xh & 0x80000000u) | w;
+    a[i] = __uint_as_float(sw);
+    b[i] = (float)(int)(xl & 0x1FFFFFFFu) * pow2f(-52) * __uint_as_float(sw & 0xFF800000u);
   }
+  __device__ __forceinline__ void load_any(int i, double x, int E) {
+    constexpr int sh = 8 * S - 24;
+    const long long F = fixed_any<S>(x, E);
+    a[i] = (float)(int)(F >> sh) * pow2f(-16);
+    b[i] = (float)(int)(F & ((1LL << sh) - 1)) * pow2f(8 - 8 * S);
+  }
+  template <int s>
+  __device__ __forceinline__ void plane(uint32_t (&w)[4]) {
+    constexpr float M = 1.5f * pow2f(23 - 8 * s);
+    float d[8];
 #pragma unroll
-  for (int s = 0; s < S; ++s)
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + s * pstride),
-                 "r"(w[s][0]), "r"(w[s][1]), "r"(w[s][2]), "r"(w[s][3])
-                 : "memory");
-}
+    for (int i = 0; i < 8; ++i) {
+      // b is below the third digit's unit, but may decide its rounding
+      d[i] = ((s == 2 ? a[i] + b[i] : a[i]) + M) - M;
+      if (s + 1 < S) a[i] -= d[i];
+      if (s == 2) a[i] += b[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      w[i] = __byte_perm(__float_as_uint(d[2 * i]), __float_as_uint(d[2 * i + 1]), 0x7632);
+  }
+};
+
+// S = 7: 55 bits do not fit two floats; the fixed-point integer by 32-bit shifts,
+// its digits as bytes with 128 added.
+template <>
+struct Split<7> {
+  uint2 g[8];
+
+  static __device__ __forceinline__ uint2 bias(uint32_t Fl, uint32_t Fh) {
+    uint2 r;  // 0x80 in each of the six low bytes balances the digits
+    asm("add.cc.u32 %0, %2, 0x80808080;\n\taddc.u32 %1, %3, 0x00008080;\n"
+        : "=r"(r.x), "=r"(r.y)
+        : "r"(Fl), "r"(Fh));
+    return r;
+  }
+  __device__ __forceinline__ void load(int i, double x, uint32_t thr) {
+    const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
+    // with M the 53-bit mantissa at the top of 64 bits, 2 F = M >> q
+    const uint32_t q = ((thr - (889u << 20) + (1030u << 20)) - (xh & 0x7FF00000u)) >> 20;
+    const uint32_t mh = (xh & 0x000FFFFFu) | 0x00100000u;
+    const uint32_t Mh = __funnelshift_l(xl, mh, 11), Ml = xl << 11;
+    uint32_t Fl, Fh;  // 64-bit shift by any q: the shifts clamp at 32 instead of wrapping
+    asm("shr.u32 %0, %1, %2;\n" : "=r"(Fh) : "r"(Mh), "r"(q));
+    asm("shr.u32 %0, %1, %2;\n"
+        : "=r"(Fl)
+        : "r"(__funnelshift_rc(Ml, Mh, q)), "r"((uint32_t)max((int)q - 32, 0)));
+    asm("add.cc.u32 %0, %0, 1;\n\taddc.u32 %1, %1, 0;\n" : "+r"(Fl), "+r"(Fh));
+    Fl = __funnelshift_r(Fl, Fh, 1);
+    Fh >>= 1;
+    const uint32_t sg = (uint32_t)((int)xh >> 31);
+    Fl ^= sg;
+    Fh ^= sg;
+    asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %2;\n" : "+r"(Fl), "+r"(Fh) : "r"(sg));
+    g[i] = bias(Fl, Fh);
+  }
+  __device__ __forceinline__ void load_any(int i, double x, int E) {
+    const long long F = fixed_any<7>(x, E);
+    g[i] = bias((uint32_t)F, (uint32_t)(F >> 32));
+  }
+  template <int s>
+  __device__ __forceinline__ float digit(uint2 v) const {
+    constexpr int b = 6 - s;
+    // the leading digit has nine bits (it reaches +128)
+    constexpr uint32_t sel = s == 0 ? 0x7432u : (0x7540u | (uint32_t)(b & 3));
+    const uint32_t t = __byte_perm(b < 4 ? v.x : v.y, 0x4B000000u, sel);
+    // 0x4B000000 + u is 2^23 + u; minus its bias, scaled by 2^-8s (exact)
+    const float off = s == 0 ? -8388608.0f : -8388736.0f;
+    return fmaf(__uint_as_float(t), pow2f(-8 * s), off * pow2f(-8 * s));
+  }
+  template <int s>
+  __device__ __forceinline__ void plane(uint32_t (&w)[4]) {
+    if (s == 0) {  // the leading digit carries no bias: signed 16 bits
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        w[i] = __byte_perm(__float_as_uint((float)((int)g[2 * i].y >> 16)),
+                           __float_as_uint((float)((int)g[2 * i + 1].y >> 16)), 0x7632);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        w[i] = __byte_perm(__float_as_uint(digit<s>(g[2 * i])),
+                           __float_as_uint(digit<s>(g[2 * i + 1])), 0x7632);
+    }
+  }
+};
 
 // UMMA shared-memory descriptor: K-major, no swizzle.  lbo: byte distance of
 // K-adjacent core matrices, sbo: byte distance of M/N-adjacent core matrices.
@@ -233,25 +250,6 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 __host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
-  uint32_t r[8];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7])
-      : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float v[4]) {
@@ -310,55 +308,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t tmem) {
                "r"(kTmemCols));
 }
 
-// All digit-pair MMAs of one chunk (both K halves) into the accumulators.
-// started: bit a set once accumulator a has been written in this block.
-// (TCK = 16: one MMA of K = 16 per digit pair.)  The descriptors of the
-// planes differ from the stage's first one only in the 14-bit start address
-// field (shared addresses < 256 KB), so they are formed by addition.
-template <int S>
-__device__ __forceinline__ void issue_chunk(uint32_t tmem, int NT, uint32_t aStage,
-                                            uint32_t bStage, uint32_t& started) {
-  static_assert(TCK == 16, "one MMA per digit pair and chunk");
-  const uint32_t lboA = (TCM / 8) * 128, lboB = (uint32_t)(NT / 8) * 128, sbo = 128;
-  const uint64_t pa16 = planeA_bytes<S>() >> 4, pb16 = planeB_bytes(NT) >> 4;
-  const uint32_t idesc = instr_desc(TCM, NT);
-  const uint64_t da0 = smem_desc(aStage, lboA, sbo), db0 = smem_desc(bStage, lboB, sbo);
-#pragma unroll
-  for (int s = 0; s < S; ++s)
-#pragma unroll
-    for (int t = 0; t + s < S; ++t) {
-      const int a = acc_of<S>(s + t);
-      mma_bf16(tmem + (uint32_t)(a * NT), da0 + s * pa16, db0 + t * pb16, idesc,
-               (started >> a) & 1u);
-      started |= 1u << a;
-    }
-}
-
-constexpr int kIssuer = kThr - 32;  // thread that issues MMAs and bulk copies (lightest split load)
-
-// Exact int64 value (units 2^-kFrac of the level-0 unit) of the accumulators
-// of one output: levels 0..2 (and 3 for S = 7) are exact FP32 integers in
-// their units (< 2^24), the last accumulator is rounded at 2^-kFrac.
-template <int S>
-__device__ __forceinline__ long long acc_to_i64(const float (&v)[5]) {
-  constexpr int NA = nacc<S>();
-  long long T = 0;
-#pragma unroll
-  for (int a = 0; a < NA; ++a) {
-    // level a in units 2^(-8a); scale so that the int32 conversion is exact
-    // (exact levels) or rounds at 2^-kFrac (last accumulator)
-    const bool last = (a == NA - 1) && (S >= 4);
-    const int sc = last ? kFrac : 8 * a;
-    const int i = __float2int_rn(v[a] * __uint_as_float((uint32_t)(127 + sc) << 23));
-    T += last ? (long long)i : ((long long)i << (kFrac - 8 * a));
-  }
-  return T;
-}
-
-__device__ __forceinline__ long long shr_sat(long long v, int k) {
-  return k <= 0 ? v : (k > 62 ? 0 : (v >> k));
-}
-
 // v * 2^e in FP64 for the usual case |v| < 2^51 and a normal result: the
 // integer is added to the bits of 1.5 * 2^52, one FP64 subtraction (exact)
 // normalises it, and the exponent field takes e.  One FP64 instruction per
@@ -381,13 +330,14 @@ __device__ __forceinline__ double i64_scaled(long long v, int e) {
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
 constexpr int kMagicInt = 0x4B400000;
 
-// The accumulators of one output as in acc_to_i64, summed by wide
-// multiply-adds.  Four conversions per output would bound the drain of TMEM
+// Exact int64 value (units 2^-kFrac of the level-0 unit) of the accumulators
+// of one output: levels 0..2 (and 3 for S = 7) are exact FP32 integers in
+// their units (< 2^24), the last accumulator is rounded at 2^-kFrac.  Four conversions per output would bound the drain of TMEM
 // (32 cycles per warp and output on the conversion unit), during which the
 // tensor core waits, so levels 0 and 1 go through the FP32 adder: level 0 is an
 // integer of at most 2^22, level 1 of at most 2^23 in units of 2^-8, split into
 // 2 h + l.  The integer offsets of the magic constant leave by one constant.
-template <int S>
+template <int S, int kF = kFrac>
 __device__ __forceinline__ long long acc_sum(const float (&v)[5]) {
   constexpr int NA = nacc<S>();
   static_assert(NA >= 3, "levels 0 and 1 have accumulators of their own");
@@ -399,14 +349,17 @@ __device__ __forceinline__ long long acc_sum(const float (&v)[5]) {
 #pragma unroll
   for (int a = NA - 1; a >= 2; --a) {
     const bool last = (a == NA - 1) && (S >= 4);
-    const int sc = last ? kFrac : 8 * a;
+    const int sc = last ? kF : 8 * a;
     const int i = __float2int_rn(v[a] * __uint_as_float((uint32_t)(127 + sc) << 23));
-    asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(i), "r"(last ? 1 : 1 << (kFrac - 8 * a)));
+    asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(i), "r"(last ? 1 : 1 << (kF - 8 * a)));
   }
   const int w1 = i1 - (int)(3u * (unsigned)kMagicInt);
-  asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(w1), "r"(1 << (kFrac - 8)));
+  asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(w1), "r"(1 << (kF - 8)));
   const int w0 = i0 - kMagicInt;
-  asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(w0), "r"(1 << kFrac));
+  if (kF >= 32)
+    T += (long long)(w0 * (1 << (kF >= 32 ? kF - 32 : 0))) << 32;
+  else
+    asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(T) : "r"(w0), "r"(1 << (kF < 32 ? kF : 0)));
   return T;
 }
 
@@ -419,284 +372,429 @@ __device__ __forceinline__ void seg_col_ptr(const SegList& s, int c, const doubl
   *ld = s.ld[i];
 }
 
-// 8-byte global -> shared copy (zero fill when !valid; src must still be a
-// mapped address), completion tracked by cp.async groups.
-__device__ __forceinline__ void cp_async8(uint32_t dst, const double* src, bool valid) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(dst), "l"(src),
-               "r"(valid ? 8 : 0)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-// wait until at most one group of this thread is pending
-__device__ __forceinline__ void cp_async_wait1() {
-  asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait0() {
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+// ------------------------------------------- shared by Gram and update kernels
+constexpr int kUWarps = 16;             // compute warps
+constexpr int kUThr = kUWarps * 32;
+constexpr int kUThrAll = kUThr + 128;   // + a warpgroup for the MMA and the C copy warp
+// Registers per thread: the launch gives every warp kURegs; the helper
+// warpgroup gives most of its share to the compute warps (setmaxnreg), whose
+// pending loads would otherwise be spilled, i.e. waited for.  The shares must
+// add up to the launch's total.
+constexpr int kURegs = 96, kURegsCompute = 104, kURegsHelper = 64;
+static_assert(kUThr * kURegsCompute + (kUThrAll - kUThr) * kURegsHelper == kUThrAll * kURegs,
+              "register shares must add up to the launch's registers");
+constexpr int kUStagesA = 4;            // most digit stages of A in TMEM
+constexpr int kUStagesB = 4;            // stages of C's digits in shared memory
+constexpr int kUPitch = NTMAX / 4 + 1;  // int64 slots per row and warp (odd: no bank conflicts)
+
+// widest output tile: the accumulators leave TMEM room for two digit stages of A
+template <int S>
+__host__ __device__ constexpr int upd_ntmax() { return S >= 7 ? 80 : 96; }
+// digit stages of A that fit beside the accumulators (8 columns per plane)
+template <int S>
+__host__ __device__ inline int upd_stages(int NT) {
+  const int fit = ((int)kTmemCols - nacc<S>() * NT) / (8 * S);
+  return fit < kUStagesA ? fit : kUStagesA;
 }
 
-__device__ __forceinline__ void ld_shared_f64(uint32_t a, double& x) {
-  asm volatile("ld.shared.f64 %0, [%1];\n" : "=d"(x) : "r"(a) : "memory");
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c,
+                                         uint32_t d) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(taddr),
+               "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
+}
+
+// A from TMEM (lane = row, a 32-bit column = two consecutive K), B from shared memory
+__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
+// digit planes s .. S - 1 of 8 K values of this lane's row into TMEM
+template <int S, int s>
+__device__ __forceinline__ void store_planes(Split<S>& sp, uint32_t dst) {
+  uint32_t w[4];
+  sp.template plane<s>(w);
+  tmem_st4(dst + s * 8, w[0], w[1], w[2], w[3]);
+  if constexpr (s + 1 < S) store_planes<S, s + 1>(sp, dst);
+}
+
+// the same into K-major core-matrix rows in shared memory, planes pstride apart
+template <int S, int s>
+__device__ __forceinline__ void store_planes_shared(Split<S>& sp, uint32_t dst, uint32_t pstride) {
+  uint32_t w[4];
+  sp.template plane<s>(w);
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + s * pstride), "r"(w[0]),
+               "r"(w[1]), "r"(w[2]), "r"(w[3])
+               : "memory");
+  if constexpr (s + 1 < S) store_planes_shared<S, s + 1>(sp, dst, pstride);
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t a) {
+  asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.shared::cta.b64 t, [%0];\n\t}\n" ::"r"(a)
+               : "memory");
+}
+
+// One poll of an mbarrier phase.
+__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\tmbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}\n"
+      : "=r"(done)
+      : "r"(a), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
+// Bounded wait that also ends when another warp of the CTA has given up;
+// running out raises the CTA's failure flag.
+__device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, int* fail) {
+  if (mbar_try(bar, parity)) return true;
+  for (int spin = 0; spin < kSpin; spin += 64) {
+    if (mbar_wait(bar, parity, 64)) return true;
+    if (*reinterpret_cast<volatile int*>(fail)) return false;
+  }
+  *reinterpret_cast<volatile int*>(fail) = 1;
+  return false;
 }
 
 // ------------------------------------------------------------------- Gram
-constexpr int kGcols = TCM + NTMAX;  // column slots of a Gram tile: A columns, then B columns
+// Rows that share one exponent per column: 256 (the bound of the exact levels),
+// 64 when 256 would leave CTAs without a block.
+struct GramPlan {
+  int ntq, NT;        // column tiles of V and their width
+  int cpb;            // chunks per exponent block
+  int64_t nblk, per;  // blocks in all, blocks per slab
+  int slabs;
+};
+
+// Fraction bits of the int64 sums of a Gram: with seven slices the rounding of
+// each block at 2^-30 would show (the last accumulator, below 2^-7 there, leaves
+// room for more); 64 blocks of at most 2^22 stay below 2^63.
+template <int S>
+__host__ __device__ constexpr int gram_frac() { return S >= 7 ? 34 : kFrac; }
 
 struct GramShared {
-  unsigned long long mdone[2];
+  unsigned long long full[kUStagesA], mdone[kUStagesA];  // digits written / multiplied
+  unsigned long long accfull, accempty;                  // accumulators of a block
   uint32_t tmem_base;
   int fail;
-  int eCur[kGcols];   // exponent bounds E of the current block
-  int R[kGcols];      // reference exponents of the int64 accumulators
-  int dR[kGcols];     // reference increase at the current block
-  const double* cptr[kGcols];
-  long long cld[kGcols];
+  int RB[NTMAX];  // reference exponents of the V columns over the slab
 };
 
 template <int S>
 size_t gram_smem_bytes(int NT) {
-  return 2 * (S * planeA_bytes<S>() + S * planeB_bytes(NT)) +
-         (size_t)kRaw * TCK * kGcols * 8 + sizeof(GramShared) + 1024;
+  return (size_t)upd_stages<S>(NT) * S * planeB_bytes(NT) + (size_t)kUThr * kUPitch * 8 +
+         sizeof(GramShared) + 1024 + 64;
 }
 
-// E[b][c] = exponent bound of column c over rows [256 b, 256 b + 256): the
-// biased exponent maximum (at least 1) minus 1022.  One warp per (block, 32
-// columns), lanes over columns; high words only.
-__global__ void block_col_exp_kernel(int64_t n, SegList L, int ncols, int64_t nblk,
-                                     int* __restrict__ E) {
-  const int lane = threadIdx.x & 31;
-  const int64_t b = (int64_t)blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int c = blockIdx.x * 32 + lane;
-  if (b >= nblk || c >= ncols) return;
-  const double* p;
-  long long ld;
-  seg_col_ptr(L, c, &p, &ld);
-  const int64_t r0 = b * kBlock, r1 = min(n, r0 + kBlock);
+// E[b][c] = exponent bound of column c over the rows of block b: the biased
+// exponent maximum (at least 1) minus 1022.  One CTA per (block, 32 columns),
+// lanes over columns, the rows dealt to its eight warps (with a warp per block
+// a 32-column Gram of 262,144 rows had 1,024 warps in all: 33 us; 32 us
+// now); the columns of U, then those of V; high words only.
+__global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n, SegList U, int p, SegList V,
+                                                            int q, int rows,
+                                                            int* __restrict__ EU,
+                                                            int* __restrict__ EV) {
+  __shared__ int red[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ub = (p + 31) / 32;
+  const int64_t b = blockIdx.x;
+  const bool isv = (int)blockIdx.y >= ub;
+  const int c = (isv ? (int)blockIdx.y - ub : (int)blockIdx.y) * 32 + lane, nc = isv ? q : p;
   int e = 1;
-  for (int64_t r = r0; r < r1; r += 16) {
-    int hw[16];
+  if (c < nc) {
+    const double* ptr;
+    long long ld;
+    seg_col_ptr(isv ? V : U, c, &ptr, &ld);
+    const int64_t r1 = min(n, (b + 1) * rows);
+#pragma unroll 1
+    for (int64_t r = b * rows + warp; r < r1; r += 128) {
+      int hw[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int64_t row = min(r + i, r1 - 1);
-      hw[i] = __ldg(reinterpret_cast<const int*>(p + row * ld) + 1);
+      for (int i = 0; i < 16; ++i)
+        hw[i] = __ldg(reinterpret_cast<const int*>(ptr + min(r + 8 * i, r1 - 1) * ld) + 1);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) e = max(e, (hw[i] >> 20) & 0x7FF);
     }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) e = max(e, (hw[i] >> 20) & 0x7FF);
   }
-  E[b * ncols + c] = e - 1022;
-}
-
-// Stage rows [r, r + TCK) of column slot c = tid into raw (row-major
-// [TCK][kGcols]): lanes over consecutive columns (coalesced), rows by pointer
-// increments.
-__device__ __forceinline__ void gram_stage_raw(const GramShared& sh, int ncs, int64_t r,
-                                               int64_t rend, uint32_t raw, int tid,
-                                               const double* any) {
-  if (tid >= ncs) return;
-  const double* p = sh.cptr[tid];
-  const long long ld = sh.cld[tid];
-  const double* src = p ? p + r * ld : any;
-  const int64_t left = rend - r;
-  const int nv = !p ? 0 : (left >= TCK ? TCK : (left > 0 ? (int)left : 0));
-#pragma unroll
-  for (int i = 0; i < TCK; ++i) {
-    cp_async8(raw + (uint32_t)(i * kGcols + tid) * 8, i < nv ? src : any, i < nv);
-    src += ld;
+  red[warp][lane] = e;
+  __syncthreads();
+  if (warp == 0 && c < nc) {
+    for (int w = 1; w < 8; ++w) e = max(e, red[w][lane]);
+    (isv ? EV : EU)[b * nc + c] = e - 1022;
   }
 }
 
+// One CTA per (128 columns of U, NT columns of V, row slab), built like the
+// update kernel: 16 compute warps, an elected MMA thread, mbarriers and no
+// CTA-wide barrier in the loop.  In a chunk of 16 rows half of the compute warps
+// cut the U columns (a thread owns one column, its TMEM lane, and 8 rows) into
+// digit planes in TMEM and the other half the V columns into planes in shared
+// memory; the halves change places from chunk to chunk, and each warp's loads
+// for the chunk after next are in flight meanwhile.  The columns' reference
+// exponents over the slab are known beforehand (block_col_exp_kernel), so a
+// block's sums only shift and add.  The form before this one (all digits in
+// shared memory, 8 warps, one CTA barrier per chunk) took 896 us at
+// n = 262,144, p = 213, q = 142; 640 us now.
 template <int S>
-__global__ void __launch_bounds__(kThr, 1)
-    ozaki_gram_tc_kernel(int64_t n, SegList U, int p, SegList V, int q, int NT,
-                         int64_t blocks_per_slab, const int* __restrict__ EU,
-                         const int* __restrict__ EV, int4* __restrict__ partial) {
+__global__ void __launch_bounds__(kUThrAll, 1)
+    ozaki_gram_tc_kernel(int64_t n, const __grid_constant__ SegList U, int p,
+                         const __grid_constant__ SegList V, int q, int NT, int cpb, int64_t nblk,
+                         int64_t per, const int* __restrict__ EU, const int* __restrict__ EV,
+                         int4* __restrict__ partial) {
   constexpr int NA = nacc<S>();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-  const uint32_t pa = (uint32_t)planeA_bytes<S>(), pb = (uint32_t)planeB_bytes(NT);
-  // stage st: A planes at aS0 + st * S * pa, B planes at bS0 + st * S * pb
-  const uint32_t aS0 = smem_u32(base), bS0 = smem_u32(base) + 2 * S * pa;
-  const uint32_t raw0 = smem_u32(base) + 2 * S * (pa + pb);
-  constexpr uint32_t rawB = TCK * kGcols * 8;  // bytes per raw stage
-  GramShared& sh = *reinterpret_cast<GramShared*>(base + 2 * S * (pa + pb) + kRaw * rawB);
+  const uint32_t pb = (uint32_t)planeB_bytes(NT);
+  const int NSA = upd_stages<S>(NT);
+  const uint32_t bS0 = smem_u32(base);
+  unsigned char* after = base + (size_t)NSA * S * pb;
+  long long* all_slots = reinterpret_cast<long long*>(after);
+  GramShared& sh = *reinterpret_cast<GramShared*>(after + (size_t)kUThr * kUPitch * 8);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tp = blockIdx.x * TCM, tq = blockIdx.y * NT;
   const int np_ = min(TCM, p - tp), nq_ = min(NT, q - tq);
-  const int64_t nblk = ceil_div(n, kBlock);
-  const int64_t b0 = (int64_t)blockIdx.z * blocks_per_slab;
-  const int64_t b1 = min(nblk, b0 + blocks_per_slab);
-  const int64_t r_begin = b0 * kBlock, r_end = min(n, b1 * kBlock);
-  const int64_t nchunks = ceil_div(r_end - r_begin, TCK);
-  const int ncs = TCM + NT;  // column slots: A columns, then B columns
-  const double* any = U.ptr[0];
+  const int64_t b0 = (int64_t)blockIdx.z * per, b1 = min(nblk, b0 + per);
+  const int64_t r0 = b0 * cpb * TCK, r1 = min(n, b1 * cpb * TCK);
+  const int nchunks = (int)((r1 - r0 + TCK - 1) / TCK), nb = (int)(b1 - b0);
+  const int bunits = NT / 16;  // warps that cut the V columns of a chunk
 
-  for (int c = tid; c < kGcols; c += kThr) {
-    const double* ptr = nullptr;
-    long long ld = 0;
-    if (c < TCM && c < np_) seg_col_ptr(U, tp + c, &ptr, &ld);
-    if (c >= TCM && c - TCM < nq_) seg_col_ptr(V, tq + c - TCM, &ptr, &ld);
-    sh.cptr[c] = ptr;
-    sh.cld[c] = ld;
-    sh.R[c] = kEZero;
-  }
   if (warp == 0) tmem_alloc(smem_u32(&sh.tmem_base));
   if (tid == 0) {
-    mbar_init(smem_u32(&sh.mdone[0]), 1);
-    mbar_init(smem_u32(&sh.mdone[1]), 1);
+    for (int i = 0; i < kUStagesA; ++i) {
+      mbar_init(smem_u32(&sh.full[i]), kUWarps / 2 + bunits);
+      mbar_init(smem_u32(&sh.mdone[i]), 1);
+    }
+    mbar_init(smem_u32(&sh.accfull), 1);
+    mbar_init(smem_u32(&sh.accempty), kUWarps);
     sh.fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n");
+  }
+  // columns past the tile's end repeat its last one; their sums are not stored
+  if (tid < NT) {
+    int R = kEZero;
+    const int* e = EV + b0 * q + tq + min(tid, nq_ - 1);
+#pragma unroll 8
+    for (int b = 0; b < nb; ++b) R = max(R, __ldg(e + (int64_t)b * q));
+    sh.RB[tid] = R;
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n");
   const uint32_t tmem = sh.tmem_base;
+  const uint32_t tmemA = tmem + (uint32_t)(NA * NT);
 
-  // prologue: first two chunks in flight
-  for (int g = 0; g < 2; ++g) {
-    if (g < nchunks)
-      gram_stage_raw(sh, ncs, r_begin + (int64_t)g * TCK, r_end, raw0 + g * rawB, tid, any);
-    cp_async_commit();
-  }
-  cp_async_wait1();
-  __syncthreads();
+  if (warp < kUWarps) {
+    // ------------------------------------------------------ compute warps
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kURegsCompute));
+    const int qd = warp & 3, grp = warp >> 2, half = grp & 1, par = grp >> 1;
+    const uint32_t lane_off = (uint32_t)(32 * qd) << 16;
+    const int W = NT / 4;  // output columns of a warp
+    long long* slots = all_slots + (size_t)warp * 32 * kUPitch;
+    // U column of this lane; V column and row half of its item
+    const int ca = min(32 * qd + lane, np_ - 1);
+    const int item = (half * 4 + qd) * 32 + lane;
+    const bool cuts_v = half * 4 + qd < bunits;
+    const int vj = item % NT, vh = item / NT, cb = min(vj, nq_ - 1);
+    const int* ea = EU + b0 * p + tp + ca;
+    const int* eb = EV + b0 * q + tq + cb;
+    const double *pa, *pv;
+    long long lda, ldv;
+    seg_col_ptr(U, tp + ca, &pa, &lda);
+    seg_col_ptr(V, tq + cb, &pv, &ldv);
+    // this lane's addresses in its first chunks: U in chunks par, par + 2, ..,
+    // V in the others
+    pa += (r0 + (int64_t)par * TCK + 8 * half) * lda;
+    pv += (r0 + (int64_t)(1 - par) * TCK + 8 * vh) * ldv;
+    const uint32_t vdst = (uint32_t)((vh * (NT / 8) + (vj >> 3)) * 128 + (vj & 7) * 16);
+    int RA = kEZero;  // reference exponent of the U column over the slab
+#pragma unroll 8
+    for (int b = 0; b < nb; ++b) RA = max(RA, __ldg(ea + (int64_t)b * p));
+    for (int u = 0; u < W; ++u) slots[lane * kUPitch + u] = 0;
 
-  // flush ownership: TMEM lane = A column my_i, B columns j0 .. j0 + NT/2 - 1
-  const int my_i = 32 * (warp & 3) + lane;
-  const int half = NT / 2;
-  const int j0 = half * (warp >> 2);
-  const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-  long long acc[NTMAX / 2];
+    // 8 rows of a column from row r on (zero past the slab's end)
+    auto load8 = [&](const double* ptr, long long ld, int64_t r, double (&x)[8]) {
+      if (r + 8 <= r1) {
 #pragma unroll
-  for (int j = 0; j < NTMAX / 2; ++j) acc[j] = 0;
-  bool failed = false;
-  uint32_t started = 0;
-  int64_t gc = 0;  // chunk counter of the slab
-  // cut items of this thread: (column slot, 8-row group), at most two
-  int it_c[2], it_kg[2];
-  uint32_t it_dst[2], it_ps[2];
-  int nit = 0;
+        for (int e = 0; e < 8; ++e) x[e] = __ldg(ptr + e * ld);
+      } else {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int it = tid + h * kThr;
-    it_c[h] = it % ncs;
-    it_kg[h] = it / ncs;
-    if (it < ncs * KG) nit = h + 1;
-    const int c = it_c[h], kg = it_kg[h];
-    it_dst[h] = c < TCM ? (uint32_t)((kg * (TCM / 8) + (c >> 3)) * 128 + (c & 7) * 16)
-                        : (uint32_t)((kg * (NT / 8) + ((c - TCM) >> 3)) * 128 + ((c - TCM) & 7) * 16);
-    it_ps[h] = c < TCM ? pa : pb;
-  }
-
-  for (int64_t b = b0; b < b1 && !failed; ++b) {
-    // ---- block start: exponents of this block, reference update
-    for (int c = tid; c < ncs; c += kThr) {
-      const int E = !sh.cptr[c] ? kEZero
-                    : c < TCM    ? EU[b * p + tp + c]
-                                 : EV[b * q + tq + c - TCM];
-      const int Rn = max(sh.R[c], E);
-      sh.dR[c] = Rn - sh.R[c];
-      sh.R[c] = Rn;
-      sh.eCur[c] = E;
-    }
-    __syncthreads();
-    started = 0;
-    const int64_t rb = b * kBlock;
-    for (int ch = 0; ch < kChunksPerBlock; ++ch) {
-      const int64_t r = rb + (int64_t)ch * TCK;
-      if (r >= r_end) break;
-      const uint32_t st = (uint32_t)(gc & 1);
-      const uint32_t raw = raw0 + (uint32_t)(gc % kRaw) * rawB;
-      if (gc >= 2 && !mbar_wait(smem_u32(&sh.mdone[st]), (uint32_t)((gc >> 1) - 1) & 1))
-        sh.fail = 1;
-      // cut the staged chunk: items (column slot, 8-row group)
+        for (int e = 0; e < 8; ++e) x[e] = r + e < r1 ? __ldg(ptr + e * ld) : 0.0;
+      }
+    };
+    auto split = [&](const double (&x)[8], int E, Split<S>& sp) {
+      if (__all_sync(0xffffffffu, E > kFastEMin && E < kFastEMax)) {
+        const uint32_t thr = split_thr(E);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h < nit) {
-          const int c = it_c[h], kg = it_kg[h];
-          double x[8];
-          int E[8];
-          const int Ec = sh.eCur[c];
+        for (int e = 0; e < 8; ++e) sp.load(e, x[e], thr);
+      } else {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            ld_shared_f64(raw + (uint32_t)((kg * 8 + i) * kGcols + c) * 8, x[i]);
-            E[i] = Ec;
-          }
-          const uint32_t base_st = c < TCM ? aS0 + st * S * pa : bS0 + st * S * pb;
-          split8<S>(x, E, base_st + it_dst[h], it_ps[h]);
+        for (int e = 0; e < 8; ++e) sp.load_any(e, x[e], E);
+      }
+    };
+    // accumulators of block b -> the warp's int64 sums
+    uint32_t fphase = 0;
+    auto flush = [&](int b) -> bool {
+      if (!__all_sync(0xffffffffu, wait_or_fail(smem_u32(&sh.accfull), fphase, &sh.fail)))
+        return false;
+      fphase ^= 1;
+      asm volatile("tcgen05.fence::after_thread_sync;\n");
+      const int si = RA - __ldg(ea + (int64_t)b * p);  // >= 0
+      const int* ev = EV + (b0 + b) * q + tq;
+#pragma unroll 1
+      for (int j = 0; j < W; j += 4) {
+        float v[5][4];
+#pragma unroll
+        for (int a = 0; a < NA; ++a) tmem_ld4(tmem + lane_off + a * NT + W * grp + j, v[a]);
+        int sj[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int jj = W * grp + j + e;
+          sj[e] = sh.RB[jj] - __ldg(ev + min(jj, nq_ - 1));
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float w[5] = {v[0][e], v[1][e], v[2][e], v[3][e], v[4][e]};
+          long long* slot = slots + lane * kUPitch + j + e;
+          const int k = si + sj[e];
+          long long T = acc_sum<S, gram_frac<S>()>(w);
+          if (k > 0) T = k < 62 ? (T + (1LL << (k - 1))) >> k : 0;  // round to nearest
+          *slot += T;
         }
       }
-      // chunk gc + 2 into the stage just read by chunk gc - 1
-      if (gc + 2 < nchunks)
-        gram_stage_raw(sh, ncs, r_begin + (gc + 2) * TCK, r_end,
-                       raw0 + (uint32_t)((gc + 2) % kRaw) * rawB, tid, any);
-      cp_async_commit();
-      cp_async_wait1();  // chunk gc + 1 has landed (this thread's copies)
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      if (__syncthreads_or(sh.fail)) {
-        failed = true;
-        break;
+      asm volatile("tcgen05.fence::before_thread_sync;\n");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sh.accempty));
+      return true;
+    };
+
+    double xa[8], xv[8];
+    if (par < nchunks) load8(pa, lda, r0 + (int64_t)par * TCK + 8 * half, xa);
+    if (cuts_v && 1 - par < nchunks) load8(pv, ldv, r0 + (int64_t)(1 - par) * TCK + 8 * vh, xv);
+    // E of the block of the chunk at hand: read when a block is entered
+    int Ea = __ldg(ea), Ev = __ldg(eb);
+    int blk = 0, inblk = 0;    // block of chunk c and its chunk in it
+    int fl = 0, fend = min(cpb, nchunks) - 1;  // next block to flush, its last chunk
+    int st = 0;
+    uint32_t phase = 1;
+    bool ok = true;
+    for (int c = 0;; ++c) {
+      while (ok && fl < nb && (c >= nchunks || c > fend + NSA - 1)) {
+        ok = flush(fl);
+        ++fl;
+        fend = min(fend + cpb, nchunks - 1);
       }
-      if (tid == kIssuer) {
+      if (!ok || c >= nchunks) break;
+      const bool mine_a = (c & 1) == par;
+      if (mine_a || cuts_v) {
+        Split<S> sp;
+        const int64_t r = r0 + (int64_t)c * TCK;
+        if (mine_a) {
+          split(xa, Ea, sp);
+          pa += 2 * TCK * lda;
+          if (c + 2 < nchunks) load8(pa, lda, r + 2 * TCK + 8 * half, xa);
+        } else {
+          split(xv, Ev, sp);
+          pv += 2 * TCK * ldv;
+          if (c + 2 < nchunks) load8(pv, ldv, r + 2 * TCK + 8 * vh, xv);
+        }
+        if (c >= NSA && !wait_or_fail(smem_u32(&sh.mdone[st]), phase, &sh.fail)) ok = false;
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        if (mine_a) {
+          asm volatile("tcgen05.fence::after_thread_sync;\n");
+          store_planes<S, 0>(sp, tmemA + lane_off + (uint32_t)(st * 8 * S + half * 4));
+          asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+          asm volatile("tcgen05.fence::before_thread_sync;\n");
+        } else {
+          store_planes_shared<S, 0>(sp, bS0 + (uint32_t)st * S * pb + vdst, pb);
+          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sh.full[st]));
+      }
+      if (++st == NSA) {
+        st = 0;
+        phase ^= 1;
+      }
+      if (++inblk == cpb) {
+        inblk = 0;
+        ++blk;
+        if (blk < nb) {
+          Ea = __ldg(ea + (int64_t)blk * p);
+          Ev = __ldg(eb + (int64_t)blk * q);
+        }
+      }
+    }
+    // ---- slab partial: (value, exponent) = sum * 2^(R_i + R_j - 14 - kFrac), lanes
+    // along the columns of V
+    __syncwarp();
+    const unsigned inv = 65536u / (unsigned)W + 1u;  // idx / W for idx < 768
+    for (int u = 0; u < W; ++u) {
+      const unsigned idx = 32u * u + lane;
+      const int r = (int)((idx * inv) >> 16), j = (int)idx - r * W, jj = W * grp + j;
+      const int Ri = __shfl_sync(0xffffffffu, RA, r);
+      const int i = 32 * qd + r;
+      if (i < np_ && jj < nq_) {
+        const long long v = ok ? slots[r * kUPitch + j] : 0;
+        int4 w;
+        w.x = (int)(unsigned)(unsigned long long)v;
+        w.y = (int)(v >> 32);
+        w.z = Ri + sh.RB[jj] - 14 - gram_frac<S>();
+        w.w = ok ? 0 : 1;
+        partial[((int64_t)blockIdx.z * p + tp + i) * q + tq + jj] = w;
+      }
+    }
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kURegsHelper));
+    if (warp == kUWarps && elect_one()) {
+      // -------------------------------------------------------- MMA issue
+      const uint64_t pb16 = pb >> 4;
+      const uint32_t idesc = instr_desc(TCM, NT);
+      const uint64_t db_first = smem_desc(bS0, (uint32_t)(NT / 8) * 128, 128);
+      const uint32_t full0 = smem_u32(&sh.full[0]), mdone0 = smem_u32(&sh.mdone[0]);
+      int gc = 0, left = 0, st = 0;
+      uint32_t blk = 0, ph = 0;
+      for (; gc < nchunks; ++gc) {
+        uint32_t seen = 0xFFu;
+        if (left == 0) {  // a block starts: its accumulators must have been read
+          seen = 0u;
+          left = min(cpb, nchunks - gc);
+          if (blk > 0 && !wait_or_fail(smem_u32(&sh.accempty), (blk - 1) & 1u, &sh.fail)) break;
+        }
+        if (!wait_or_fail(full0 + 8 * st, ph, &sh.fail)) break;
         asm volatile("tcgen05.fence::after_thread_sync;\n");
-        issue_chunk<S>(tmem, NT, aS0 + st * S * pa, bS0 + st * S * pb, started);
-        mma_commit(smem_u32(&sh.mdone[st]));
-      }
-      ++gc;
-    }
-    if (failed) break;
-    // ---- block end: wait for the last chunk's MMAs, fold TMEM into int64
-    if (!mbar_wait(smem_u32(&sh.mdone[(gc - 1) & 1]), (uint32_t)((gc - 1) >> 1) & 1)) sh.fail = 1;
-    if (__syncthreads_or(sh.fail)) {
-      failed = true;
-      break;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;\n");
-    {
-      const int Ei = sh.eCur[my_i], Ri = sh.R[my_i], di = sh.dR[my_i];
+        const uint64_t db0 = db_first + (uint64_t)st * S * pb16;
+        const uint32_t a0 = tmemA + (uint32_t)(st * 8 * S);
 #pragma unroll
-      for (int g = 0; g < NTMAX / 16; ++g) {
-        if (8 * g < half) {
-          float v[NA][8];
+        for (int sl = 0; sl < S; ++sl)
 #pragma unroll
-          for (int a = 0; a < NA; ++a) tmem_ld8(tmem + lane_off + a * NT + j0 + 8 * g, v[a]);
-          asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int cj = TCM + j0 + 8 * g + i;
-            float w[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int a = 0; a < NA; ++a) w[a] = v[a][i];
-            const long long T = acc_to_i64<S>(w);
-            const int shift = Ri + sh.R[cj] - Ei - sh.eCur[cj];
-            acc[8 * g + i] = shr_sat(acc[8 * g + i], di + sh.dR[cj]) + shr_sat(T, shift);
+          for (int tl = 0; tl + sl < S; ++tl) {
+            const int a = acc_of<S>(sl + tl);
+            mma_bf16_ts(tmem + (uint32_t)(a * NT), a0 + sl * 8, db0 + tl * pb16, idesc,
+                        (seen >> a) & 1u);
+            seen |= 1u << a;
           }
+        mma_commit(mdone0 + 8 * st);
+        if (--left == 0) {
+          mma_commit(smem_u32(&sh.accfull));
+          ++blk;
+        }
+        if (++st == NSA) {
+          st = 0;
+          ph ^= 1;
         }
       }
+      // every committed MMA (and its arrival) ends before the CTA
+      if (gc > 0)
+        mbar_wait(smem_u32(&sh.mdone[(gc - 1) % NSA]), (uint32_t)((gc - 1) / NSA) & 1u);
     }
-    asm volatile("tcgen05.fence::before_thread_sync;\n");
-    __syncthreads();
-  }
-  cp_async_wait0();  // no copy may outlive the CTA
-  // ---- slab partial: (value, exponent) = acc * 2^(R_i + R_j - 14 - kFrac)
-  if (my_i < np_) {
-    int4* out = partial + ((int64_t)blockIdx.z * p + tp + my_i) * q + tq;
-#pragma unroll
-    for (int g = 0; g < NTMAX / 16; ++g)
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int j = j0 + 8 * g + i;
-        if (8 * g < half && j < nq_) {
-          const long long v = failed ? 0 : acc[8 * g + i];
-          int4 w;
-          w.x = (int)(unsigned)(unsigned long long)v;
-          w.y = (int)(v >> 32);
-          w.z = sh.R[my_i] + sh.R[TCM + j] - 14 - kFrac;
-          w.w = failed ? 1 : 0;
-          out[j] = w;
-        }
-      }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
   __syncthreads();
@@ -766,41 +864,41 @@ __global__ void __launch_bounds__(256) gram_tc_reduce_kernel(const int4* __restr
   G[i + (int64_t)j * ldg] = out;
 }
 
-void gram_tiles(int q, int* ntq, int* NT) {
-  *ntq = (int)ceil_div(q, NTMAX);
-  *NT = (int)round_up(ceil_div(q, *ntq), 16);
-}
-
-void gram_plan(int64_t n, int p, int q, int* slabs, int64_t* per_slab) {
-  int ntq, NT;
-  gram_tiles(q, &ntq, &NT);
-  const int64_t tiles = ceil_div(p, TCM) * ntq;
-  const int64_t nblk = std::max<int64_t>(1, ceil_div(n, kBlock));
+GramPlan gram_plan(int64_t n, int p, int q, int slices) {
+  GramPlan g;
+  const int ntmax = slices >= 7 ? upd_ntmax<7>() : upd_ntmax<6>();
+  g.ntq = (int)ceil_div(q, ntmax);
+  g.NT = (int)round_up(ceil_div(q, g.ntq), 16);
+  const int64_t tiles = ceil_div(p, TCM) * g.ntq;
+  g.cpb = tiles * ceil_div(n, kBlock) < 152 ? kChunksPerBlock / 4 : kChunksPerBlock;
+  g.nblk = std::max<int64_t>(1, ceil_div(n, (int64_t)g.cpb * TCK));
   // one wave of CTAs; at most 64 blocks per slab keeps the int64 sums < 2^61
-  int64_t s = std::max<int64_t>(ceil_div(152, tiles), ceil_div(nblk, 64));
-  s = std::min(s, nblk);
-  const int64_t per = ceil_div(nblk, s);
-  *slabs = (int)ceil_div(nblk, per);
-  *per_slab = per;
+  int64_t s = std::max<int64_t>(ceil_div(152, tiles), ceil_div(g.nblk, 64));
+  s = std::min(s, g.nblk);
+  g.per = ceil_div(g.nblk, s);
+  g.slabs = (int)ceil_div(g.nblk, g.per);
+  return g;
 }
 
 template <int S>
 int gram_tc_launch(cudaStream_t st, int64_t n, const SegList& U, int p, const SegList& V, int q,
-                   int slabs, int64_t per, const int* EU, const int* EV, int4* partial) {
-  int ntq, NT;
-  gram_tiles(q, &ntq, &NT);
-  const size_t sh = gram_smem_bytes<S>(NTMAX);
+                   const GramPlan& g, const int* EU, const int* EV, int4* partial) {
   static bool configured[64] = {false};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !configured[dev]) {
+    size_t sh = 0;  // the stage count falls as the tile widens
+    for (int NT = 16; NT <= upd_ntmax<S>(); NT += 16) sh = std::max(sh, gram_smem_bytes<S>(NT));
     LOB_CUDA_OK(cudaFuncSetAttribute(ozaki_gram_tc_kernel<S>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
+    cudaFuncAttributes at;  // a launch with other registers would wait for its shares forever
+    LOB_CUDA_OK(cudaFuncGetAttributes(&at, ozaki_gram_tc_kernel<S>));
+    if (at.numRegs != kURegs) return LOBPCG_ERR_CUDA;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
-  dim3 grid((unsigned)ceil_div(p, TCM), (unsigned)ntq, (unsigned)slabs);
-  ozaki_gram_tc_kernel<S><<<grid, kThr, gram_smem_bytes<S>(NT), st>>>(n, U, p, V, q, NT, per, EU,
-                                                                      EV, partial);
+  dim3 grid((unsigned)ceil_div(p, TCM), (unsigned)g.ntq, (unsigned)g.slabs);
+  ozaki_gram_tc_kernel<S><<<grid, kUThrAll, gram_smem_bytes<S>(g.NT), st>>>(
+      n, U, p, V, q, g.NT, g.cpb, g.nblk, g.per, EU, EV, partial);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
@@ -850,30 +948,6 @@ __global__ void split_c_tc_kernel(const double* __restrict__ C, int64_t ldc, int
   }
 }
 
-constexpr int kUWarps = 16;             // compute warps of the update
-constexpr int kUThr = kUWarps * 32;
-constexpr int kUThrAll = kUThr + 128;   // + a warpgroup for the MMA and the C copy warp
-// Registers per thread: the launch gives every warp kURegs; the helper
-// warpgroup gives most of its share to the compute warps (setmaxnreg), whose
-// pending loads would otherwise be spilled, i.e. waited for.  The shares must
-// add up to the launch's total.
-constexpr int kURegs = 96, kURegsCompute = 104, kURegsHelper = 64;
-static_assert(kUThr * kURegsCompute + (kUThrAll - kUThr) * kURegsHelper == kUThrAll * kURegs,
-              "register shares must add up to the launch's registers");
-constexpr int kUStagesA = 4;            // most digit stages of S in TMEM
-constexpr int kUStagesB = 4;            // stages of C's digits in shared memory
-constexpr int kUPitch = NTMAX / 4 + 1;  // int64 slots per row and warp (odd: no bank conflicts)
-
-// widest output tile: the accumulators leave TMEM room for two digit stages of S
-template <int S>
-__host__ __device__ constexpr int upd_ntmax() { return S >= 7 ? 80 : 96; }
-// digit stages of S that fit beside the accumulators (8 columns per plane)
-template <int S>
-__host__ __device__ inline int upd_stages(int NT) {
-  const int fit = ((int)kTmemCols - nacc<S>() * NT) / (8 * S);
-  return fit < kUStagesA ? fit : kUStagesA;
-}
-
 // What is rarely needed of the finished tile whose int64 sums lie in a warp's
 // slots (the rest is in registers, where more would push the pending loads out):
 // its first row, and its corner in Y0 (null without Y0, or with several segments).
@@ -920,60 +994,6 @@ __global__ void row_exp_kernel(int64_t n, SegList Sg, int s, const int* __restri
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
   if (lane == 0) ER[row] = e > -1000000 ? e - 1022 : kEZero;
-}
-
-__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c,
-                                         uint32_t d) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(taddr),
-               "r"(a), "r"(b), "r"(c), "r"(d)
-               : "memory");
-}
-
-// A from TMEM (lane = row, a 32-bit column = two consecutive K), B from shared memory
-__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b,
-                                            uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-      "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-
-// digit planes s .. S - 1 of 8 K values of this lane's row into TMEM
-template <int S, int s>
-__device__ __forceinline__ void store_planes(const uint2 (&g)[8], uint32_t dst) {
-  uint32_t w[4];
-  plane8<S, s>(g, w);
-  tmem_st4(dst + s * 8, w[0], w[1], w[2], w[3]);
-  if constexpr (s + 1 < S) store_planes<S, s + 1>(g, dst);
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t a) {
-  asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.shared::cta.b64 t, [%0];\n\t}\n" ::"r"(a)
-               : "memory");
-}
-
-// One poll of an mbarrier phase.
-__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred P;\n\tmbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, P;\n\t}\n"
-      : "=r"(done)
-      : "r"(a), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
-// Bounded wait that also ends when another warp of the CTA has given up;
-// running out raises the CTA's failure flag.
-__device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, int* fail) {
-  if (mbar_try(bar, parity)) return true;
-  for (int spin = 0; spin < kSpin; spin += 64) {
-    if (mbar_wait(bar, parity, 64)) return true;
-    if (*reinterpret_cast<volatile int*>(fail)) return false;
-  }
-  *reinterpret_cast<volatile int*>(fail) = 1;
-  return false;
 }
 
 template <int S>
@@ -1093,9 +1113,9 @@ __global__ void __launch_bounds__(kUThrAll, 1)
     auto enter_tile = [&]() {
       row = min((int64_t)(t / ntiles) * TCM + rl, n - 1);
       er = __ldg(ER + row);
-      const int ef = er == kEZero ? kEZeroFast : er;
+      const int ef = er == kEZero ? 0 : er;  // a zero row's digits are zero for any bound
       fast = __all_sync(0xffffffffu, ef + sh.cxmin > kFastEMin && ef + sh.cxmax < kFastEMax);
-      if (fast) er = (int)((unsigned)(ef + digit_ke<S>()) << 20);
+      if (fast) er = (int)split_thr(ef);
       locate();
     };
     auto load8 = [&](double (&x)[8]) {
@@ -1252,17 +1272,17 @@ __global__ void __launch_bounds__(kUThrAll, 1)
       while (ok && pt < ntile_total && (!more || g > pend + NSA - 1)) ok = flush();
       if (!ok || !more) break;
       // chunk g in fixed point; its registers then take the loads of chunk g + 2
-      uint2 gb[8];
+      Split<S> sp;
       {
         const int4* ce = reinterpret_cast<const int4*>(cx + k0);
         const int4 c0 = ce[0], c1 = ce[1];
         const int cv[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
         if (fast) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) gb[e] = biased_bytes<S>(x[e], (uint32_t)(er + cv[e]));
+          for (int e = 0; e < 8; ++e) sp.load(e, x[e], (uint32_t)(er + cv[e]));
         } else {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) gb[e] = biased_bytes_any<S>(x[e], er + (cv[e] >> 20));
+          for (int e = 0; e < 8; ++e) sp.load_any(e, x[e], er + (cv[e] >> 20));
         }
       }
       const int gc = g, sc = st;
@@ -1283,7 +1303,7 @@ __global__ void __launch_bounds__(kUThrAll, 1)
       if (gc >= NSA && !wait_or_fail(smem_u32(&sh.mdone[sc]), pc, &sh.fail)) ok = false;
       if (!(ok = __all_sync(0xffffffffu, ok))) break;
       asm volatile("tcgen05.fence::after_thread_sync;\n");
-      store_planes<S, 0>(gb, tmemA + lane_off + (uint32_t)(sc * 8 * S + half * 4));
+      store_planes<S, 0>(sp, tmemA + lane_off + (uint32_t)(sc * 8 * S + half * 4));
       asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;\n");
       __syncwarp();
@@ -1495,11 +1515,12 @@ int wait_selftest(cudaStream_t st, int limit, int* status) {
 }
 
 int64_t gram_tc_workspace(int64_t n, int p, int q) {
-  int slabs;
-  int64_t per;
-  gram_plan(n, p, q, &slabs, &per);
-  const int64_t nblk = std::max<int64_t>(1, ceil_div(n, kBlock));
-  return (int64_t)slabs * p * q * (int64_t)sizeof(int4) + nblk * (p + q) * 4;
+  int64_t need = 0;  // for any slice count
+  for (int slices : {6, 7}) {
+    const GramPlan g = gram_plan(n, p, q, slices);
+    need = std::max(need, (int64_t)g.slabs * p * q * (int64_t)sizeof(int4) + g.nblk * (p + q) * 4);
+  }
+  return need;
 }
 
 int gram_tc(cudaStream_t st, int64_t n, const SegList& U, const SegList& V, double* G,
@@ -1508,32 +1529,26 @@ int gram_tc(cudaStream_t st, int64_t n, const SegList& U, const SegList& V, doub
   if (p <= 0 || q <= 0) return LOBPCG_OK;
   if (slices == 0) slices = 6;
   if (n <= 0) return gram_ozaki(st, n, U, V, G, ldg, slices, work, work_bytes);
-  int slabs;
-  int64_t per;
-  gram_plan(n, p, q, &slabs, &per);
   if (work_bytes < gram_tc_workspace(n, p, q)) return LOBPCG_ERR_ARG;
   if (slices < 3 || slices > 7) return LOBPCG_ERR_ARG;
+  const GramPlan g = gram_plan(n, p, q, slices);
   int4* partial = (int4*)work;
-  const int64_t nblk = ceil_div(n, kBlock);
-  int* EU = (int*)(partial + (int64_t)slabs * p * q);
-  int* EV = EU + nblk * p;
-  block_col_exp_kernel<<<dim3((unsigned)ceil_div(p, 32), (unsigned)ceil_div(nblk, 8)), 256, 0,
-                         st>>>(n, U, p, nblk, EU);
-  LOB_LAUNCHED();
-  block_col_exp_kernel<<<dim3((unsigned)ceil_div(q, 32), (unsigned)ceil_div(nblk, 8)), 256, 0,
-                         st>>>(n, V, q, nblk, EV);
+  int* EU = (int*)(partial + (int64_t)g.slabs * p * q);
+  int* EV = EU + g.nblk * p;
+  block_col_exp_kernel<<<dim3((unsigned)g.nblk, (unsigned)(ceil_div(p, 32) + ceil_div(q, 32))), 256,
+                         0, st>>>(n, U, p, V, q, g.cpb * TCK, EU, EV);
   LOB_LAUNCHED();
   int rc;
   switch (slices) {
-    case 3: rc = gram_tc_launch<3>(st, n, U, p, V, q, slabs, per, EU, EV, partial); break;
-    case 4: rc = gram_tc_launch<4>(st, n, U, p, V, q, slabs, per, EU, EV, partial); break;
-    case 5: rc = gram_tc_launch<5>(st, n, U, p, V, q, slabs, per, EU, EV, partial); break;
-    case 6: rc = gram_tc_launch<6>(st, n, U, p, V, q, slabs, per, EU, EV, partial); break;
-    default: rc = gram_tc_launch<7>(st, n, U, p, V, q, slabs, per, EU, EV, partial); break;
+    case 3: rc = gram_tc_launch<3>(st, n, U, p, V, q, g, EU, EV, partial); break;
+    case 4: rc = gram_tc_launch<4>(st, n, U, p, V, q, g, EU, EV, partial); break;
+    case 5: rc = gram_tc_launch<5>(st, n, U, p, V, q, g, EU, EV, partial); break;
+    case 6: rc = gram_tc_launch<6>(st, n, U, p, V, q, g, EU, EV, partial); break;
+    default: rc = gram_tc_launch<7>(st, n, U, p, V, q, g, EU, EV, partial); break;
   }
   if (rc) return rc;
   const int64_t total = (int64_t)p * q;
-  gram_tc_reduce_kernel<<<(unsigned)ceil_div(total, 32), 256, 0, st>>>(partial, slabs, p, q, G,
+  gram_tc_reduce_kernel<<<(unsigned)ceil_div(total, 32), 256, 0, st>>>(partial, g.slabs, p, q, G,
                                                                         ldg);
   LOB_LAUNCHED();
   return LOBPCG_OK;
