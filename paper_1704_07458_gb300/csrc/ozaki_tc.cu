@@ -384,7 +384,8 @@ constexpr int kURegs = 96, kURegsCompute = 104, kURegsHelper = 64;
 static_assert(kUThr * kURegsCompute + (kUThrAll - kUThr) * kURegsHelper == kUThrAll * kURegs,
               "register shares must add up to the launch's registers");
 constexpr int kUStagesA = 4;            // most digit stages of A in TMEM
-constexpr int kUStagesB = 4;            // stages of C's digits in shared memory
+constexpr int kUSlots = 4;              // chunks in flight; stages of C's digits in shared memory
+static_assert(kUStagesA <= kUSlots, "a slot's barrier outlives its digit stage");
 constexpr int kUPitch = NTMAX / 4 + 1;  // int64 slots per row and warp (odd: no bank conflicts)
 
 // widest output tile: the accumulators leave TMEM room for two digit stages of A
@@ -494,12 +495,13 @@ size_t gram_smem_bytes(int NT) {
 
 // E[b][c] = exponent bound of column c over the rows of block b: the biased
 // exponent maximum (at least 1) minus 1022.  One CTA per (block, 32 columns),
-// lanes over columns, the rows dealt to its eight warps (with a warp per block
-// a 32-column Gram of 262,144 rows had 1,024 warps in all: 33 us; 32 us
-// now); the columns of U, then those of V; high words only.
+// lanes over columns, the block's 8 R rows dealt to its eight warps and all in
+// flight at once (with a warp per block a 32-column Gram of 262,144 rows had
+// 1,024 warps in all: 33 us a launch, two of them); the columns of U, then those
+// of V; high words only.
+template <int R>
 __global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n, SegList U, int p, SegList V,
-                                                            int q, int rows,
-                                                            int* __restrict__ EU,
+                                                            int q, int* __restrict__ EU,
                                                             int* __restrict__ EV) {
   __shared__ int red[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -512,16 +514,19 @@ __global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n, SegList U
     const double* ptr;
     long long ld;
     seg_col_ptr(isv ? V : U, c, &ptr, &ld);
-    const int64_t r1 = min(n, (b + 1) * rows);
-#pragma unroll 1
-    for (int64_t r = b * rows + warp; r < r1; r += 128) {
-      int hw[16];
+    const int64_t r0 = b * 8 * R, r1 = min(n, r0 + 8 * R);
+    const int* src = reinterpret_cast<const int*>(ptr + (r0 + warp) * ld) + 1;
+    int hw[R];
+    if (r0 + 8 * R <= n) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
-        hw[i] = __ldg(reinterpret_cast<const int*>(ptr + min(r + 8 * i, r1 - 1) * ld) + 1);
+      for (int i = 0; i < R; ++i) hw[i] = __ldg(src + 16 * i * ld);
+    } else {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) e = max(e, (hw[i] >> 20) & 0x7FF);
+      for (int i = 0; i < R; ++i)
+        hw[i] = r0 + warp + 8 * i < r1 ? __ldg(src + 16 * i * ld) : 0;
     }
+#pragma unroll
+    for (int i = 0; i < R; ++i) e = max(e, (hw[i] >> 20) & 0x7FF);
   }
   red[warp][lane] = e;
   __syncthreads();
@@ -533,15 +538,16 @@ __global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n, SegList U
 
 // One CTA per (128 columns of U, NT columns of V, row slab), built like the
 // update kernel: 16 compute warps, an elected MMA thread, mbarriers and no
-// CTA-wide barrier in the loop.  In a chunk of 16 rows half of the compute warps
+// CTA-wide barrier in the loop.  In a chunk of 16 rows some of the compute warps
 // cut the U columns (a thread owns one column, its TMEM lane, and 8 rows) into
-// digit planes in TMEM and the other half the V columns into planes in shared
-// memory; the halves change places from chunk to chunk, and each warp's loads
-// for the chunk after next are in flight meanwhile.  The columns' reference
+// digit planes in TMEM and others the V columns into planes in shared memory;
+// a warp needs about 2,000 cycles for 32 x 8 values, so the work of a chunk is
+// dealt over all of them in turn, and each warp's loads for its next turn are in
+// flight meanwhile.  The columns' reference
 // exponents over the slab are known beforehand (block_col_exp_kernel), so a
 // block's sums only shift and add.  The form before this one (all digits in
 // shared memory, 8 warps, one CTA barrier per chunk) took 896 us at
-// n = 262,144, p = 213, q = 142; 640 us now.
+// n = 262,144, p = 213, q = 142; 540 us now.
 template <int S>
 __global__ void __launch_bounds__(kUThrAll, 1)
     ozaki_gram_tc_kernel(int64_t n, const __grid_constant__ SegList U, int p,
@@ -564,15 +570,18 @@ __global__ void __launch_bounds__(kUThrAll, 1)
   const int64_t r0 = b0 * cpb * TCK, r1 = min(n, b1 * cpb * TCK);
   const int nchunks = (int)((r1 - r0 + TCK - 1) / TCK), nb = (int)(b1 - b0);
   const int bunits = NT / 16;  // warps that cut the V columns of a chunk
+  // lane quarters with U columns: the others are neither cut nor read (their
+  // rows of the products hold whatever TMEM held)
+  const int quarters = (np_ + 31) / 32;
 
   if (warp == 0) tmem_alloc(smem_u32(&sh.tmem_base));
   if (tid == 0) {
     for (int i = 0; i < kUStagesA; ++i) {
-      mbar_init(smem_u32(&sh.full[i]), kUWarps / 2 + bunits);
+      mbar_init(smem_u32(&sh.full[i]), 2 * quarters + bunits);
       mbar_init(smem_u32(&sh.mdone[i]), 1);
     }
     mbar_init(smem_u32(&sh.accfull), 1);
-    mbar_init(smem_u32(&sh.accempty), kUWarps);
+    mbar_init(smem_u32(&sh.accempty), 4 * quarters);
     sh.fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n");
   }
@@ -597,10 +606,21 @@ __global__ void __launch_bounds__(kUThrAll, 1)
     const uint32_t lane_off = (uint32_t)(32 * qd) << 16;
     const int W = NT / 4;  // output columns of a warp
     long long* slots = all_slots + (size_t)warp * 32 * kUPitch;
-    // U column of this lane; V column and row half of its item
+    // The U columns of a quarter are cut by its four warps, each in every second
+    // chunk.  The V columns are `bunits` items of 32 (column, row half) pairs; an
+    // item belongs to vper warps in turn, those without U columns when they are
+    // enough, so that no warp has more than it can do in the time of the MMAs.
+    const bool cuts_u = qd < quarters;
+    const int idle = 4 * (4 - quarters);
+    const bool by_idle = idle >= bunits;
+    // (not more than NSA warps: one that sat out longer could be two phases ahead
+    // of the barrier it waits on, where the parity no longer tells them apart)
+    const int vper = min((by_idle ? idle : kUWarps) / bunits, NSA);
+    const int vidx = by_idle ? (qd - quarters) * 4 + grp : warp;  // place among these warps
+    const bool cuts_v = vidx >= 0 && vidx < vper * bunits;
+    const int vturn = cuts_v ? vidx / bunits : 0;  // cuts its item in chunks vturn mod vper
+    const int item = (cuts_v ? vidx % bunits : 0) * 32 + lane;
     const int ca = min(32 * qd + lane, np_ - 1);
-    const int item = (half * 4 + qd) * 32 + lane;
-    const bool cuts_v = half * 4 + qd < bunits;
     const int vj = item % NT, vh = item / NT, cb = min(vj, nq_ - 1);
     const int* ea = EU + b0 * p + tp + ca;
     const int* eb = EV + b0 * q + tq + cb;
@@ -608,10 +628,9 @@ __global__ void __launch_bounds__(kUThrAll, 1)
     long long lda, ldv;
     seg_col_ptr(U, tp + ca, &pa, &lda);
     seg_col_ptr(V, tq + cb, &pv, &ldv);
-    // this lane's addresses in its first chunks: U in chunks par, par + 2, ..,
-    // V in the others
+    // this lane's addresses in its first chunks (U: par, par + 2, ..)
     pa += (r0 + (int64_t)par * TCK + 8 * half) * lda;
-    pv += (r0 + (int64_t)(1 - par) * TCK + 8 * vh) * ldv;
+    pv += (r0 + (int64_t)vturn * TCK + 8 * vh) * ldv;
     const uint32_t vdst = (uint32_t)((vh * (NT / 8) + (vj >> 3)) * 128 + (vj & 7) * 16);
     int RA = kEZero;  // reference exponent of the U column over the slab
 #pragma unroll 8
@@ -641,29 +660,27 @@ __global__ void __launch_bounds__(kUThrAll, 1)
     // accumulators of block b -> the warp's int64 sums
     uint32_t fphase = 0;
     auto flush = [&](int b) -> bool {
+      if (!cuts_u) return true;
+      // the block's distances from the references, read before the wait: lane j
+      // holds that of the warp's column j
+      const int si = RA - __ldg(ea + (int64_t)b * p);  // >= 0
+      const int jl = W * grp + min(lane, W - 1);
+      const int sl = sh.RB[jl] - __ldg(EV + (b0 + b) * q + tq + min(jl, nq_ - 1));
       if (!__all_sync(0xffffffffu, wait_or_fail(smem_u32(&sh.accfull), fphase, &sh.fail)))
         return false;
       fphase ^= 1;
       asm volatile("tcgen05.fence::after_thread_sync;\n");
-      const int si = RA - __ldg(ea + (int64_t)b * p);  // >= 0
-      const int* ev = EV + (b0 + b) * q + tq;
 #pragma unroll 1
       for (int j = 0; j < W; j += 4) {
         float v[5][4];
 #pragma unroll
         for (int a = 0; a < NA; ++a) tmem_ld4(tmem + lane_off + a * NT + W * grp + j, v[a]);
-        int sj[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int jj = W * grp + j + e;
-          sj[e] = sh.RB[jj] - __ldg(ev + min(jj, nq_ - 1));
-        }
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float w[5] = {v[0][e], v[1][e], v[2][e], v[3][e], v[4][e]};
           long long* slot = slots + lane * kUPitch + j + e;
-          const int k = si + sj[e];
+          const int k = si + __shfl_sync(0xffffffffu, sl, j + e);
           long long T = acc_sum<S, gram_frac<S>()>(w);
           if (k > 0) T = k < 62 ? (T + (1LL << (k - 1))) >> k : 0;  // round to nearest
           *slot += T;
@@ -676,14 +693,15 @@ __global__ void __launch_bounds__(kUThrAll, 1)
     };
 
     double xa[8], xv[8];
-    if (par < nchunks) load8(pa, lda, r0 + (int64_t)par * TCK + 8 * half, xa);
-    if (cuts_v && 1 - par < nchunks) load8(pv, ldv, r0 + (int64_t)(1 - par) * TCK + 8 * vh, xv);
+    if (cuts_u && par < nchunks) load8(pa, lda, r0 + (int64_t)par * TCK + 8 * half, xa);
+    if (cuts_v && vturn < nchunks) load8(pv, ldv, r0 + (int64_t)vturn * TCK + 8 * vh, xv);
     // E of the block of the chunk at hand: read when a block is entered
     int Ea = __ldg(ea), Ev = __ldg(eb);
     int blk = 0, inblk = 0;    // block of chunk c and its chunk in it
     int fl = 0, fend = min(cpb, nchunks) - 1;  // next block to flush, its last chunk
     int st = 0;
     uint32_t phase = 1;
+    int vnext = vturn;
     bool ok = true;
     for (int c = 0;; ++c) {
       while (ok && fl < nb && (c >= nchunks || c > fend + NSA - 1)) {
@@ -692,30 +710,35 @@ __global__ void __launch_bounds__(kUThrAll, 1)
         fend = min(fend + cpb, nchunks - 1);
       }
       if (!ok || c >= nchunks) break;
-      const bool mine_a = (c & 1) == par;
-      if (mine_a || cuts_v) {
-        Split<S> sp;
-        const int64_t r = r0 + (int64_t)c * TCK;
-        if (mine_a) {
-          split(xa, Ea, sp);
-          pa += 2 * TCK * lda;
-          if (c + 2 < nchunks) load8(pa, lda, r + 2 * TCK + 8 * half, xa);
-        } else {
-          split(xv, Ev, sp);
-          pv += 2 * TCK * ldv;
-          if (c + 2 < nchunks) load8(pv, ldv, r + 2 * TCK + 8 * vh, xv);
-        }
+      const bool do_u = cuts_u && (c & 1) == par, do_v = cuts_v && c == vnext;
+      auto stage_free = [&]() {
         if (c >= NSA && !wait_or_fail(smem_u32(&sh.mdone[st]), phase, &sh.fail)) ok = false;
-        if (!(ok = __all_sync(0xffffffffu, ok))) break;
-        if (mine_a) {
-          asm volatile("tcgen05.fence::after_thread_sync;\n");
-          store_planes<S, 0>(sp, tmemA + lane_off + (uint32_t)(st * 8 * S + half * 4));
-          asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-          asm volatile("tcgen05.fence::before_thread_sync;\n");
-        } else {
-          store_planes_shared<S, 0>(sp, bS0 + (uint32_t)st * S * pb + vdst, pb);
-          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        }
+        ok = __all_sync(0xffffffffu, ok);
+        return ok;
+      };
+      const int64_t r = r0 + (int64_t)c * TCK;
+      if (do_u) {
+        Split<S> sp;
+        split(xa, Ea, sp);
+        pa += 2 * TCK * lda;
+        if (c + 2 < nchunks) load8(pa, lda, r + 2 * TCK + 8 * half, xa);
+        if (!stage_free()) break;
+        asm volatile("tcgen05.fence::after_thread_sync;\n");
+        store_planes<S, 0>(sp, tmemA + lane_off + (uint32_t)(st * 8 * S + half * 4));
+        asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sh.full[st]));
+      }
+      if (do_v) {
+        Split<S> sp;
+        split(xv, Ev, sp);
+        vnext += vper;
+        pv += (int64_t)vper * TCK * ldv;
+        if (vnext < nchunks) load8(pv, ldv, r + vper * TCK + 8 * vh, xv);
+        if (!stage_free()) break;
+        store_planes_shared<S, 0>(sp, bS0 + (uint32_t)st * S * pb + vdst, pb);
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sh.full[st]));
       }
@@ -959,9 +982,10 @@ struct UpdOut {
 
 struct UpdShared {
   UpdOut out[kUWarps];
-  unsigned long long afull[kUStagesA], mdone[kUStagesA];  // digits of S written / multiplied
-  unsigned long long bfull[kUStagesB], bempty[kUStagesB];
-  unsigned long long accfull, accempty;                   // accumulators of a K block
+  // chunk g uses slot g % kUSlots: its digits of S are written and those of C
+  // have arrived (full), its MMAs are done (mdone)
+  unsigned long long full[kUSlots], mdone[kUSlots];
+  unsigned long long accfull, accempty;  // accumulators of a K block
   uint32_t tmem_base;
   int fail;
   int cxmin, cxmax;  // range of the column exponents
@@ -998,7 +1022,7 @@ __global__ void row_exp_kernel(int64_t n, SegList Sg, int s, const int* __restri
 
 template <int S>
 size_t upd_smem_bytes(int NT, int s) {
-  return (size_t)kUStagesB * S * planeB_bytes(NT) + sizeof(UpdShared) +
+  return (size_t)kUSlots * S * planeB_bytes(NT) + sizeof(UpdShared) +
          (size_t)ceil_div(std::max(s, 1), TCK) * TCK * 4 +
          (size_t)kUThr * kUPitch * 8 + 1024 + 64;
 }
@@ -1024,7 +1048,7 @@ size_t upd_smem_bytes(int NT, int s) {
 // integer pipe, 45 per output).  The form before this one (digits in shared
 // memory, one CTA barrier per chunk, 64-bit shifts, the tensor core idle during
 // the outputs) took 1,010 us at n = 262,144, s = 213, m = 142 and 79.0 ms at
-// n = 2,097,152, s = 846, m = 564; this one 540 us and 39 ms.
+// n = 2,097,152, s = 846, m = 564; this one 455 us and 34 ms.
 // kOneBlock: s <= 256, a single block of columns; otherwise the int64 sums are
 // kept in shared memory across the blocks, one slot per thread and output.
 // kY0: Y0 is added (an instantiation of its own: without it the loads and
@@ -1042,7 +1066,7 @@ __global__ void __launch_bounds__(kUThrAll, 1)
   unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
   const uint32_t pb = (uint32_t)planeB_bytes(NT);
   const uint32_t bS0 = smem_u32(base);
-  unsigned char* after = base + (size_t)kUStagesB * S * pb;
+  unsigned char* after = base + (size_t)kUSlots * S * pb;
   UpdShared& sh = *reinterpret_cast<UpdShared*>(after);
   const int nch = (s + TCK - 1) / TCK;
   int* cx = reinterpret_cast<int*>(after + ((sizeof(UpdShared) + 15) / 16) * 16);
@@ -1053,13 +1077,9 @@ __global__ void __launch_bounds__(kUThrAll, 1)
 
   if (warp == 0) tmem_alloc(smem_u32(&sh.tmem_base));
   if (tid == 0) {
-    for (int i = 0; i < kUStagesA; ++i) {
-      mbar_init(smem_u32(&sh.afull[i]), kUWarps / 2);
+    for (int i = 0; i < kUSlots; ++i) {
+      mbar_init(smem_u32(&sh.full[i]), kUWarps / 2 + 1);
       mbar_init(smem_u32(&sh.mdone[i]), 1);
-    }
-    for (int i = 0; i < kUStagesB; ++i) {
-      mbar_init(smem_u32(&sh.bfull[i]), 1);
-      mbar_init(smem_u32(&sh.bempty[i]), 1);
     }
     mbar_init(smem_u32(&sh.accfull), 1);
     mbar_init(smem_u32(&sh.accempty), kUWarps);
@@ -1143,12 +1163,8 @@ __global__ void __launch_bounds__(kUThrAll, 1)
       } while (k0 >= nch * TCK);
       if (g < my_chunks) enter_tile();
     };
-    int st = g;  // digit stage of chunk g and parity of the wait for it to be free
-    uint32_t phase = 1;
-    while (st >= NSA) {
-      st -= NSA;
-      phase ^= 1;
-    }
+    int st = g;  // digit stage of chunk g
+    while (st >= NSA) st -= NSA;
     // next block of accumulators to move: tile pt, block pblk of it, ending at
     // chunk pend; parity of its barrier phases
     int pt = t0, pblk = 0, pend = min(kChunksPerBlock, nch) - 1;
@@ -1286,28 +1302,27 @@ __global__ void __launch_bounds__(kUThrAll, 1)
         }
       }
       const int gc = g, sc = st;
-      const uint32_t pc = phase;
       g += 2;
       k0 += 2 * TCK;
       p += 2 * TCK;
       st += 2;
-      while (st >= NSA) {
-        st -= NSA;
-        phase ^= 1;
-      }
+      while (st >= NSA) st -= NSA;
       if (k0 >= nch * TCK)
         wrap();
       else if (k0 >= segend && k0 < s)
         locate();
       if (g < my_chunks) load8(x);
-      if (gc >= NSA && !wait_or_fail(smem_u32(&sh.mdone[sc]), pc, &sh.fail)) ok = false;
+      // the stage is free when the MMAs of chunk gc - NSA are done
+      const unsigned go = (unsigned)(gc - NSA);
+      if (gc >= NSA && !wait_or_fail(smem_u32(&sh.mdone[go % kUSlots]), (go / kUSlots) & 1u, &sh.fail))
+        ok = false;
       if (!(ok = __all_sync(0xffffffffu, ok))) break;
       asm volatile("tcgen05.fence::after_thread_sync;\n");
       store_planes<S, 0>(sp, tmemA + lane_off + (uint32_t)(sc * 8 * S + half * 4));
       asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;\n");
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&sh.afull[sc]));
+      if (lane == 0) mbar_arrive(smem_u32(&sh.full[(unsigned)gc % kUSlots]));
       if (ou < W) {
         if (spread3)
           out_steps(std::integral_constant<int, 3>());
@@ -1333,24 +1348,22 @@ __global__ void __launch_bounds__(kUThrAll, 1)
         const uint64_t pb16 = pb >> 4;
         const uint32_t idesc = instr_desc(TCM, NT);
         const uint64_t db_first = smem_desc(bS0, (uint32_t)(NT / 8) * 128, 128);
-        const uint32_t afull0 = smem_u32(&sh.afull[0]), bfull0 = smem_u32(&sh.bfull[0]);
-        const uint32_t mdone0 = smem_u32(&sh.mdone[0]), bempty0 = smem_u32(&sh.bempty[0]);
+        const uint32_t full0 = smem_u32(&sh.full[0]), mdone0 = smem_u32(&sh.mdone[0]);
         int gc = 0, left = 0, c = 0;  // chunks to the end of the block; chunk of the tile
-        uint32_t blk = 0, phA = 0, phB = 0;
-        int stA = 0, stB = 0;
+        uint32_t blk = 0;
+        int st = 0;
         for (; gc < my_chunks; ++gc) {
+          const uint32_t slot = (uint32_t)gc % kUSlots;
           uint32_t seen = 0xFFu;
           if (left == 0) {  // a block starts: its accumulators must have been read
             seen = 0u;
             left = min(kChunksPerBlock, nch - c);
             if (blk > 0 && !wait_or_fail(smem_u32(&sh.accempty), (blk - 1) & 1u, &sh.fail)) break;
           }
-          if (!wait_or_fail(bfull0 + 8 * stB, phB, &sh.fail) ||
-              !wait_or_fail(afull0 + 8 * stA, phA, &sh.fail))
-            break;
+          if (!wait_or_fail(full0 + 8 * slot, ((uint32_t)gc / kUSlots) & 1u, &sh.fail)) break;
           asm volatile("tcgen05.fence::after_thread_sync;\n");
-          const uint64_t db0 = db_first + (uint64_t)stB * S * pb16;
-          const uint32_t a0 = tmemA + (uint32_t)(stA * 8 * S);
+          const uint64_t db0 = db_first + (uint64_t)slot * S * pb16;
+          const uint32_t a0 = tmemA + (uint32_t)(st * 8 * S);
 #pragma unroll
           for (int sl = 0; sl < S; ++sl)
 #pragma unroll
@@ -1360,58 +1373,48 @@ __global__ void __launch_bounds__(kUThrAll, 1)
                           (seen >> a) & 1u);
               seen |= 1u << a;
             }
-          mma_commit(mdone0 + 8 * stA);
-          mma_commit(bempty0 + 8 * stB);
+          mma_commit(mdone0 + 8 * slot);
           if (--left == 0) {
             mma_commit(smem_u32(&sh.accfull));
             ++blk;
           }
           if (++c == nch) c = 0;
-          if (++stA == NSA) {
-            stA = 0;
-            phA ^= 1;
-          }
-          if (++stB == kUStagesB) {
-            stB = 0;
-            phB ^= 1;
-          }
+          if (++st == NSA) st = 0;
         }
-        // every committed MMA (and its arrivals on these barriers) ends before the CTA
-        if (gc > 0) {
-          mbar_wait(smem_u32(&sh.mdone[(gc - 1) % NSA]), (uint32_t)((gc - 1) / NSA) & 1u);
-          mbar_wait(smem_u32(&sh.bempty[(gc - 1) % kUStagesB]), (uint32_t)((gc - 1) / kUStagesB) & 1u);
-        }
+        // every committed MMA (and its arrival) ends before the CTA
+        if (gc > 0)
+          mbar_wait(mdone0 + 8 * ((gc - 1) % kUSlots), (uint32_t)((gc - 1) / kUSlots) & 1u);
       }
     } else if (tid == kUThr + 32) {
       // ------------------------------------------------- copies of C's digits
       const uint32_t bbytes = cs_blk * 2;
       bool ok = true;
-      int64_t gc = 0;
+      unsigned gc = 0;
       for (int t = t0; t < ntile_total && ok; t += tstep) {
         const int tile = t % ntiles;
         for (int c = 0; c < nch; ++c) {
-          const int st = (int)(gc % kUStagesB);
-          const uint32_t use = (uint32_t)(gc / kUStagesB);
-          if (gc >= kUStagesB &&
-              !(ok = wait_or_fail(smem_u32(&sh.bempty[st]), (use - 1) & 1u, &sh.fail)))
+          const uint32_t slot = gc % kUSlots, use = gc / kUSlots;
+          if (use > 0 && !(ok = wait_or_fail(smem_u32(&sh.mdone[slot]), (use - 1) & 1u, &sh.fail)))
             break;
           const uint16_t* src = Cs + ((size_t)c * ntiles + (size_t)tile) * cs_blk;
           uint64_t state;
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;\n"
                        : "=l"(state)
-                       : "r"(smem_u32(&sh.bfull[st])), "r"(bbytes)
+                       : "r"(smem_u32(&sh.full[slot])), "r"(bbytes)
                        : "memory");
           asm volatile(
               "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
-              "[%3];\n" ::"r"(bS0 + (uint32_t)st * S * pb),
-              "l"(src), "r"(bbytes), "r"(smem_u32(&sh.bfull[st]))
+              "[%3];\n" ::"r"(bS0 + slot * S * pb),
+              "l"(src), "r"(bbytes), "r"(smem_u32(&sh.full[slot]))
               : "memory");
           ++gc;
         }
       }
-      // no copy outlives the CTA (on success the MMAs have consumed them all)
-      for (int64_t u = max((int64_t)0, gc - kUStagesB); u < gc; ++u)
-        mbar_wait(smem_u32(&sh.bfull[u % kUStagesB]), (uint32_t)(u / kUStagesB) & 1u);
+      // no copy outlives the CTA: on success the MMAs have consumed them all;
+      // after a failure a copy in flight is given time to land
+      if (!ok || *reinterpret_cast<volatile int*>(&sh.fail))
+        for (unsigned u = gc > kUSlots ? gc - kUSlots : 0u; u < gc; ++u)
+          mbar_wait(smem_u32(&sh.full[u % kUSlots]), (u / kUSlots) & 1u, 4096);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
@@ -1535,8 +1538,11 @@ int gram_tc(cudaStream_t st, int64_t n, const SegList& U, const SegList& V, doub
   int4* partial = (int4*)work;
   int* EU = (int*)(partial + (int64_t)g.slabs * p * q);
   int* EV = EU + g.nblk * p;
-  block_col_exp_kernel<<<dim3((unsigned)g.nblk, (unsigned)(ceil_div(p, 32) + ceil_div(q, 32))), 256,
-                         0, st>>>(n, U, p, V, q, g.cpb * TCK, EU, EV);
+  const dim3 egrid((unsigned)g.nblk, (unsigned)(ceil_div(p, 32) + ceil_div(q, 32)));
+  if (g.cpb == kChunksPerBlock)
+    block_col_exp_kernel<kBlock / 8><<<egrid, 256, 0, st>>>(n, U, p, V, q, EU, EV);
+  else
+    block_col_exp_kernel<kBlock / 32><<<egrid, 256, 0, st>>>(n, U, p, V, q, EU, EV);
   LOB_LAUNCHED();
   int rc;
   switch (slices) {
