@@ -28,9 +28,6 @@ struct DevDense {
   double* vec = nullptr;                 // 8 nmax
   double* scal = nullptr;                // 16 device scalars
   int* ints = nullptr;                   // flags, permutation, cluster runs
-  double* part = nullptr;                // GEMM split-K partial tiles
-  unsigned* cnt = nullptr;               // GEMM split-K tile counters (zero between launches)
-  int cnt_tiles = 0;
   int init(int64_t n_max);
   void release();
   // Layout of the buffers in one block for orders up to n_max: bytes needed;
@@ -125,10 +122,11 @@ int small_stats(DenseLayer& L, const double* G, int rows, int cols, int ldg, boo
 
 // ---- device-resident path (dense_dev.cu)
 // C = alpha op(A) op(B) + beta Cin, column-major, m, n <= 2 * the layer's
-// order; skip: device flag, the launch is a no-op when it is non-zero.
+// order; skip: device flag, the launch is a no-op when it is non-zero; sym: see
+// gemm64_kernel.
 int dev_gemm(DenseLayer& L, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
              int lda, const double* B, int ldb, double beta, const double* Cin, int ldcin,
-             double* C, int ldc, const int* skip);
+             double* C, int ldc, const int* skip, int sym = 0);
 int dev_chol(DenseLayer& L, int n, double* A, int lda, int* info);
 int dev_trinv(DenseLayer& L, int n, const double* R, int ldr, double* X, int ldx, const int* skip);
 int dev_syev(DenseLayer& L, int n, const double* A, int lda, double* Z, int ldz, double* w,

@@ -9,7 +9,7 @@
 //   * O(n^3) work that must be exact to FP64 (the Ogita-Aishima refinement of
 //     the eigenvectors, the products forming the projected matrix and the
 //     back-transformation) runs as small FP64 GEMMs spread over the whole GPU
-//     (16 x 16 output tiles, a deterministic split of the contraction);
+//     (8 x 8 output tiles);
 //   * the O(n^3) work that only has to be close (the first eigendecomposition
 //     and the Householder QR of C_p) runs in FP32 on one CTA, then FP64
 //     refinement steps (eigenvectors) or Newton-Schulz steps (QR factor)
@@ -29,9 +29,8 @@ namespace lob {
 namespace {
 
 constexpr double kEps64 = 2.220446049250313e-16;  // 2^-52
-constexpr int kGT = 16;                            // GEMM output tile
-constexpr int kGK = 32;                            // GEMM contraction chunk
-constexpr int kMaxKs = 8;                          // GEMM contraction splits
+constexpr int kGT = 8;                             // GEMM output tile
+constexpr int kGK = 64;                            // GEMM contraction chunk
 constexpr int kRefSteps = 4;                       // Ogita-Aishima steps
 constexpr int kMaxRunDev = 32;                     // cluster width of the final Jacobi
 
@@ -44,72 +43,85 @@ constexpr int kMaxRunDev = 32;                     // cluster width of the final
 
 // ------------------------------------------------------------------ GEMM
 // C = alpha op(A) op(B) + beta Cin (column-major; Cin may equal C but neither
-// may alias A or B).  One 16 x 16 output tile per CTA (one output per thread)
-// and a split of the contraction into ks slices; with ks > 1 every slice
-// stores its partial tile, and the CTA that arrives last at the tile's counter
-// adds the partials in slice order (deterministic) and resets the counter.
+// may alias A or B).  One 8 x 8 output tile per CTA, its 256 threads being four
+// interleaved slices of the contraction x 64 outputs, summed in slice order
+// (deterministic); the next chunk's operands are loaded while a chunk is
+// multiplied.  The tiles are small because the products are: at order 81 a
+// 16 x 16 tile leaves 36 CTAs, and splitting the contraction over CTAs costs a
+// fence, a counter and a second pass through L2 (5.6 us at order 81, 31 us at
+// 213; 3.1 and 19 us on average now, the symmetric products among them; FP64 pipe at 213: 18.6 us).
 // skip != nullptr: the whole launch is a no-op when *skip is non-zero.
+// sym = s > 0: s products of m x m whose results are symmetric, B and C of the
+// later ones m columns on; only the upper triangles are computed (half of the
+// FP64 work that bounds a product of order 213) and mirrored.
 __global__ void __launch_bounds__(256) gemm64_kernel(int m, int n, int k, int ta, int tb,
                                                      double alpha, const double* __restrict__ A,
                                                      int lda, const double* __restrict__ B, int ldb,
                                                      double beta, const double* Cin, int ldcin,
-                                                     double* C, int ldc, int ks, int kper,
-                                                     double* part, unsigned* cnt, const int* skip) {
+                                                     double* C, int ldc, const int* skip, int sym) {
   if (skip && *skip) return;
   __shared__ double As[kGK][kGT + 1], Bs[kGK][kGT + 1];
-  __shared__ int s_last;
-  const int tiles_m = (m + kGT - 1) / kGT;
-  const int tile = blockIdx.x, slice = blockIdx.y;
-  const int row0 = (tile % tiles_m) * kGT, col0 = (tile / tiles_m) * kGT;
-  const int k0 = slice * kper, k1 = min(k, k0 + kper);
-  const int t = threadIdx.x, i = t % kGT, j = t / kGT;
-  double acc = 0.0;
-  for (int kc = k0; kc < k1; kc += kGK) {
+  __shared__ double red[3][kGT * kGT];
+  const int tiles_m = (m + kGT - 1) / kGT, tile = blockIdx.x;
+  int row0 = (tile % tiles_m) * kGT, col0 = (tile / tiles_m) * kGT;
+  if (sym) {  // tile number of the upper triangle of product number `which`
+    const int per = tiles_m * (tiles_m + 1) / 2, which = tile / per;
+    int u = tile - which * per, tj = 0;
+    while (u > tj) u -= ++tj;  // column tj holds tj + 1 tiles
+    row0 = u * kGT;
+    col0 = tj * kGT;
+    B += (int64_t)which * m * ldb;
+    C += (int64_t)which * m * ldc;
+    n = m;
+  }
+  const int t = threadIdx.x, sl = t >> 6, i = t & 7, j = (t >> 3) & 7;
+  // this thread's two elements of an operand chunk
+  double ra[2], rb[2];
+  auto fetch = [&](int kc) {
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int e = t + 256 * r;
-      int ii, kk;
-      if (!ta) { ii = e % kGT; kk = e / kGT; } else { kk = e % kGK; ii = e / kGK; }
-      const int row = row0 + ii, kq = kc + kk;
-      double a = 0.0;
-      if (row < m && kq < k1) a = ta ? A[kq + (int64_t)row * lda] : A[row + (int64_t)kq * lda];
-      As[kk][ii] = a;
-      int jj;
-      if (!tb) { kk = e % kGK; jj = e / kGK; } else { jj = e % kGT; kk = e / kGT; }
-      const int col = col0 + jj, kb = kc + kk;
-      double b = 0.0;
-      if (col < n && kb < k1) b = tb ? B[col + (int64_t)kb * ldb] : B[kb + (int64_t)col * ldb];
-      Bs[kk][jj] = b;
+      const int ai = ta ? e >> 6 : e & 7, ak = kc + (ta ? e & 63 : e >> 3), row = row0 + ai;
+      ra[r] = (row < m && ak < k) ? (ta ? A[ak + (int64_t)row * lda] : A[row + (int64_t)ak * lda])
+                                  : 0.0;
+      const int bj = tb ? e & 7 : e >> 6, bk = kc + (tb ? e >> 3 : e & 63), col = col0 + bj;
+      rb[r] = (col < n && bk < k) ? (tb ? B[col + (int64_t)bk * ldb] : B[bk + (int64_t)col * ldb])
+                                  : 0.0;
+    }
+  };
+  double acc0 = 0.0, acc1 = 0.0;
+  fetch(0);
+  for (int kc = 0; kc < k; kc += kGK) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int e = t + 256 * r;
+      if (ta)
+        As[e & 63][e >> 6] = ra[r];
+      else
+        As[e >> 3][e & 7] = ra[r];
+      if (tb)
+        Bs[e >> 3][e & 7] = rb[r];
+      else
+        Bs[e & 63][e >> 6] = rb[r];
     }
     __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < kGK; ++kk) acc = fma(As[kk][i], Bs[kk][j], acc);
+    if (kc + kGK < k) fetch(kc + kGK);
+    const int left = min(kGK, k - kc);
+    for (int kk = sl; kk < left; kk += 8) {
+      acc0 = fma(As[kk][i], Bs[kk][j], acc0);
+      acc1 = fma(As[kk + 4][i], Bs[kk + 4][j], acc1);  // zero past k
+    }
     __syncthreads();
   }
+  const double acc = acc0 + acc1;
+  if (sl > 0) red[sl - 1][t & 63] = acc;
+  __syncthreads();
   const int row = row0 + i, col = col0 + j;
-  if (ks == 1) {
-    if (row < m && col < n) {
-      double v = alpha * acc;
-      if (beta != 0.0) v = fma(beta, Cin[row + (int64_t)col * ldcin], v);
-      C[row + (int64_t)col * ldc] = v;
-    }
-    return;
-  }
-  part[((int64_t)tile * ks + slice) * 256 + t] = acc;
-  __threadfence();
-  __syncthreads();
-  if (t == 0) s_last = (atomicAdd(&cnt[tile], 1u) == (unsigned)(ks - 1));
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  double sum = 0.0;
-  for (int s = 0; s < ks; ++s) sum += __ldcg(&part[((int64_t)tile * ks + s) * 256 + t]);
-  if (row < m && col < n) {
-    double v = alpha * sum;
-    if (beta != 0.0) v = fma(beta, Cin[row + (int64_t)col * ldcin], v);
-    C[row + (int64_t)col * ldc] = v;
-  }
-  if (t == 0) cnt[tile] = 0u;
+  if (sl > 0 || row >= m || col >= n || (sym && row > col)) return;
+  double v = alpha * (acc + red[0][t] + red[1][t] + red[2][t]);
+  if (beta != 0.0) v = fma(beta, Cin[row + (int64_t)col * ldcin], v);
+  C[row + (int64_t)col * ldc] = v;
+  if (sym) C[col + (int64_t)row * ldc] = v;
 }
 
 // ------------------------------------------------------- FP64 Cholesky
@@ -302,12 +314,14 @@ __global__ void __launch_bounds__(1024, 1) tridiag32_kernel(int n, const double*
 // that does.  Tiles left of or above the trailing block are skipped.  Bound by
 // the chain of a step (two reductions of five shuffles, a square root, two
 // divisions, two barriers); with the matrix in shared memory each element cost
-// two loads and a store per step (811 us at n = 213; 394 us now).
+// two loads and a store per step (811 us at n = 213; 361 us now).
 constexpr int kTridRegMax = 224;
 
 template <int NB>
 struct TridiagShared {
-  float xs[2][32 * NB], ps[32 * NB];
+  // xp[k & 1][i]: x_i of step k (the column being reduced) and p_i, side by
+  // side so that a row's pair is one load
+  float2 xp[2][32 * NB];
 };
 
 // The steps k whose next column k + 1 lies in column tile C0: tiles left of it
@@ -320,24 +334,26 @@ __device__ __forceinline__ void tridiag_phase(int n, float (&a)[2 * NB][NB], Tri
   const int kend = min(n - 2, 32 * C0 + 31);
 #pragma unroll 1
   for (int k = C0 > 0 ? 32 * C0 - 1 : 0; k < kend; ++k) {
-    const float* x = sh.xs[k & 1];
+    float2* xp = sh.xp[k & 1];
     __syncthreads();  // column k is complete; p of the step before has been read
     // reflector of x(k + 1 : n): v_{k+1} = 1, v_j = x_j scale
     float vj[NB], ss = 0.f;
 #pragma unroll
     for (int c = C0; c < NB; ++c) {
       const int j = tx + 32 * c;
-      vj[c] = j > k ? x[j] : 0.f;  // rows past n are zero
+      vj[c] = j > k ? xp[j].x : 0.f;  // rows past n are zero
       ss = fmaf(j == k + 1 ? 0.f : vj[c], vj[c], ss);
     }
 #pragma unroll
     for (int q = 16; q > 0; q >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, q);
-    const float alpha = x[k + 1];
+    // (approximate quotients: tau and v are formed from the same rounded values,
+    // and FP64 refines the vectors)
+    const float alpha = xp[k + 1].x;
     float tk = 0.f, beta = alpha, scale = 0.f;
     if (ss > 0.f) {
-      beta = -copysignf(sqrtf(alpha * alpha + ss), alpha);
-      tk = (beta - alpha) / beta;
-      scale = 1.f / (alpha - beta);
+      beta = -copysignf(__fsqrt_rn(fmaf(alpha, alpha, ss)), alpha);
+      tk = __fdividef(beta - alpha, beta);
+      scale = __fdividef(1.f, alpha - beta);
     }
 #pragma unroll
     for (int c = C0; c < NB; ++c) vj[c] = tx + 32 * c == k + 1 ? 1.f : vj[c] * scale;
@@ -348,7 +364,7 @@ __device__ __forceinline__ void tridiag_phase(int n, float (&a)[2 * NB][NB], Tri
         if (j > k && j < n) V[j + (int64_t)k * ldv] = vj[c];
       }
       if (tx == 0) {
-        d[k] = x[k];
+        d[k] = xp[k].x;
         e[k] = beta;
         tau[k] = tk;
       }
@@ -372,13 +388,13 @@ __device__ __forceinline__ void tridiag_phase(int n, float (&a)[2 * NB][NB], Tri
       }
     }
     s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
-    if ((tx & 1) == 0 && (tx >> 1) < NR) sh.ps[ty + 16 * (tx >> 1)] = tk * s[0];
+    if ((tx & 1) == 0 && (tx >> 1) < NR) xp[ty + 16 * (tx >> 1)].y = tk * s[0];
     __syncthreads();
     // K = tau p^T v / 2, w = p - K v, A -= v w^T + w v^T
     float wj[NB], pv = 0.f;
 #pragma unroll
     for (int c = C0; c < NB; ++c) {
-      wj[c] = sh.ps[tx + 32 * c];
+      wj[c] = xp[tx + 32 * c].y;
       pv = fmaf(wj[c], vj[c], pv);
     }
 #pragma unroll
@@ -387,15 +403,16 @@ __device__ __forceinline__ void tridiag_phase(int n, float (&a)[2 * NB][NB], Tri
 #pragma unroll
     for (int c = C0; c < NB; ++c) wj[c] = fmaf(-K, vj[c], wj[c]);
     const bool own = tx == ((k + 1) & 31);  // column k + 1, published for the next step
-    float* xn = sh.xs[(k + 1) & 1];
+    float2* xn = sh.xp[(k + 1) & 1];
 #pragma unroll
     for (int r = R0; r < NR; ++r) {
       const int i = ty + 16 * r;
-      const float vi = i == k + 1 ? 1.f : (i > k ? x[i] * scale : 0.f);
-      const float wi = fmaf(-K, vi, sh.ps[i]);
+      const float2 xi = xp[i];
+      const float vi = i == k + 1 ? 1.f : (i > k ? xi.x * scale : 0.f);
+      const float wi = fmaf(-K, vi, xi.y);
 #pragma unroll
       for (int c = C0; c < NB; ++c) a[r][c] -= fmaf(vi, wj[c], wi * vj[c]);
-      if (own) xn[i] = a[r][C0];
+      if (own) xn[i].x = a[r][C0];
     }
   }
   if constexpr (C0 + 1 < NB) {
@@ -422,7 +439,7 @@ __global__ void __launch_bounds__(512, 1) tridiag32_reg_kernel(int n, const doub
     }
   if (tx == 0)
 #pragma unroll
-    for (int r = 0; r < NR; ++r) sh.xs[0][ty + 16 * r] = a[r][0];
+    for (int r = 0; r < NR; ++r) sh.xp[0][ty + 16 * r].x = a[r][0];
   tridiag_phase<NB, 0>(n, a, sh, d, e, V, ldv, tau);
 #pragma unroll
   for (int r = 0; r < NR; ++r)
@@ -1350,51 +1367,60 @@ __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, con
     }
     __syncthreads();
   };
-  // out = MB in:  top = in_top + F in_w;  w = F^T in_top + Bw in_w
-  auto mb_apply = [&](const float* in, float* res) {
-    for (int i = t; i < ns; i += blockDim.x) {
-      float s = 0.f;
-      if (i < o) {
-        s = in[i];
-        for (int j = 0; j < nw; ++j) s = fmaf(F[i + j * o], in[o + j], s);
-      } else {
-        const int iw = i - o;
-        for (int j = 0; j < o; ++j) s = fmaf(F[j + iw * o], in[j], s);
-        for (int j = 0; j < nw; ++j) s = fmaf(Bw[iw + j * nw], in[o + j], s);
-      }
-      res[i] = s;
+  // res(i) = sum over eight lanes of part(i, lane): with a thread per row only
+  // ns of the 1024 threads worked, each on a chain of ns products (43 us at
+  // ns = 81; 38 us now)
+  auto apply = [&](auto part, float* res) {
+    const int sub = t & 7;
+    for (int i0 = 0; i0 < ns; i0 += (int)blockDim.x >> 3) {
+      const int i = i0 + (t >> 3);
+      float s = i < ns ? part(i, sub) : 0.f;
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 4);
+      if (i < ns && sub == 0) res[i] = s;
     }
     __syncthreads();
+  };
+  // out = MB in:  top = in_top + F in_w;  w = F^T in_top + Bw in_w
+  auto mb_apply = [&](const float* in, float* res) {
+    apply([&](int i, int sub) {
+      float s = 0.f;
+      if (i < o) {
+        s = sub == 0 ? in[i] : 0.f;
+        for (int j = sub; j < nw; j += 8) s = fmaf(F[i + j * o], in[o + j], s);
+      } else {
+        const int iw = i - o;
+        for (int j = sub; j < o; j += 8) s = fmaf(F[j + iw * o], in[j], s);
+        for (int j = sub; j < nw; j += 8) s = fmaf(Bw[iw + j * nw], in[o + j], s);
+      }
+      return s;
+    }, res);
   };
   // res = R^-T in: top = in_top; w = Yt^T in_top + Yw^T in_w
   auto rit_apply = [&](const float* in, float* res) {
-    for (int i = t; i < ns; i += blockDim.x) {
-      float s;
-      if (i < o) {
-        s = in[i];
-      } else {
-        const int iw = i - o;
-        s = 0.f;
-        for (int j = 0; j < o; ++j) s = fmaf(Yt[j + iw * o], in[j], s);
-        for (int j = 0; j < nw; ++j) s = fmaf(Yw[j + iw * nw], in[o + j], s);
-      }
-      res[i] = s;
-    }
-    __syncthreads();
+    apply([&](int i, int sub) {
+      if (i < o) return sub == 0 ? in[i] : 0.f;
+      const int iw = i - o;
+      float s = 0.f;
+      for (int j = sub; j < o; j += 8) s = fmaf(Yt[j + iw * o], in[j], s);
+      for (int j = sub; j < nw; j += 8) s = fmaf(Yw[j + iw * nw], in[o + j], s);
+      return s;
+    }, res);
   };
   // res = R^-1 in: top = in_top + Yt in_w; w = Yw in_w
   auto ri_apply = [&](const float* in, float* res) {
-    for (int i = t; i < ns; i += blockDim.x) {
-      float s = i < o ? in[i] : 0.f;
+    apply([&](int i, int sub) {
+      float s = 0.f;
       if (i < o) {
-        for (int j = 0; j < nw; ++j) s = fmaf(Yt[i + j * o], in[o + j], s);
+        s = sub == 0 ? in[i] : 0.f;
+        for (int j = sub; j < nw; j += 8) s = fmaf(Yt[i + j * o], in[o + j], s);
       } else {
         const int iw = i - o;
-        for (int j = 0; j < nw; ++j) s = fmaf(Yw[iw + j * nw], in[o + j], s);
+        for (int j = sub; j < nw; j += 8) s = fmaf(Yw[iw + j * nw], in[o + j], s);
       }
-      res[i] = s;
-    }
-    __syncthreads();
+      return s;
+    }, res);
   };
   auto power = [&](int which) -> float {
     for (int i = t; i < ns; i += blockDim.x) x[i] = 1.0f + 0.001f * (float)(i % 7);
@@ -1495,14 +1521,12 @@ unsigned nblk(int64_t total) { return (unsigned)std::max<int64_t>(1, ceil_div(to
 size_t DevDense::carve(int64_t nmax_, char* base, size_t* clear_bytes) {
   const int nm = (int)std::min<int64_t>(nmax_, kDevDenseMax);
   const size_t nn = (size_t)nm * nm;
-  const int tiles = (int)(ceil_div(nm, kGT) * ceil_div(2 * nm, kGT));
   size_t at = 0;
   auto take = [&](size_t bytes) {
     char* p = base ? base + at : nullptr;
     at += (bytes + 255) / 256 * 256;
     return (void*)p;
   };
-  unsigned* c = (unsigned*)take((size_t)tiles * sizeof(unsigned));
   int* in = (int*)take((5 * (size_t)nm + 64) * sizeof(int));
   if (clear_bytes) *clear_bytes = at;
   double* m[8];
@@ -1514,15 +1538,12 @@ size_t DevDense::carve(int64_t nmax_, char* base, size_t* clear_bytes) {
   float* fv = (float*)take(4 * (size_t)nm * sizeof(float));
   double* ve = (double*)take((8 * (size_t)nm + 256) * sizeof(double));
   double* sc = (double*)take(16 * sizeof(double));
-  double* pt = (double*)take((size_t)tiles * kMaxKs * 256 * sizeof(double));
   if (base) {
     nmax = nm;
-    cnt_tiles = tiles;
-    cnt = c;
     ints = in;
     X = m[0]; X1 = m[1]; E = m[2]; Zt = m[3];
     T1 = m[4]; T2 = m[5]; T3 = m[6]; T4 = m[7];
-    XA = xa; GS = gs; V32 = v32; Y32 = y32; f32v = fv; vec = ve; scal = sc; part = pt;
+    XA = xa; GS = gs; V32 = v32; Y32 = y32; f32v = fv; vec = ve; scal = sc;
   }
   return at;
 }
@@ -1550,23 +1571,16 @@ void DevDense::release() {
 
 int dev_gemm(DenseLayer& L, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
              int lda, const double* B, int ldb, double beta, const double* Cin, int ldcin,
-             double* C, int ldc, const int* skip) {
+             double* C, int ldc, const int* skip, int sym) {
   if (m <= 0 || n <= 0) return LOBPCG_OK;
-  DevDense& D = L.dev;
-  const int tiles = (int)(ceil_div(m, kGT) * ceil_div(n, kGT));
-  if (tiles > D.cnt_tiles) return LOBPCG_ERR_ARG;
-  const int kchunks = (int)std::max<int64_t>(1, ceil_div(k, kGK));
-  int ks = (int)std::min<int64_t>(std::min<int64_t>(kMaxKs, kchunks),
-                                  std::max<int64_t>(1, ceil_div(2 * 152, tiles)));
-  const int kper = (int)(ceil_div(kchunks, ks) * kGK);
-  ks = (int)ceil_div(std::max(k, 1), kper);
+  const int tm = (int)ceil_div(m, kGT);
+  const int tiles = sym ? sym * tm * (tm + 1) / 2 : tm * (int)ceil_div(n, kGT);
   if (!Cin) {
     Cin = C;
     ldcin = ldc;
   }
-  gemm64_kernel<<<dim3((unsigned)tiles, (unsigned)ks), 256, 0, L.st>>>(
-      m, n, k, ta ? 1 : 0, tb ? 1 : 0, alpha, A, lda, B, ldb, beta, Cin, ldcin, C, ldc, ks, kper,
-      D.part, D.cnt, skip);
+  gemm64_kernel<<<(unsigned)tiles, 256, 0, L.st>>>(m, n, k, ta ? 1 : 0, tb ? 1 : 0, alpha, A, lda,
+                                                   B, ldb, beta, Cin, ldcin, C, ldc, skip, sym);
   DLAUNCH(L);
   return LOBPCG_OK;
 }
@@ -1716,7 +1730,7 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
     if ((rc = dev_gemm(L, false, false, n, n, n, 1.0, A, lda, X, n, 0.0, nullptr, 0, AX, n, done)))
       return rc;
     if ((rc = dev_gemm(L, true, false, n, 2 * n, n, 1.0, X, n, D.XA, n, 0.0, nullptr, 0, G, n,
-                       done)))
+                       done, 2)))
       return rc;
     oa_norms_kernel<<<kOaBlocks, 256, 0, L.st>>>(n, D.GS, D.vec, D.vec + 2 * kOaBlocks, done);
     DLAUNCH(L);
@@ -1736,7 +1750,8 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
   // step leaves ||I - X^T X|| up to ~1e-4 on pairs it has just separated;
   // each step squares it
   for (int s = 0; s < 2; ++s) {
-    if ((rc = dev_gemm(L, true, false, n, n, n, 1.0, X, n, X, n, 0.0, nullptr, 0, G, n, nullptr)))
+    if ((rc = dev_gemm(L, true, false, n, n, n, 1.0, X, n, X, n, 0.0, nullptr, 0, G, n, nullptr,
+                       1)))
       return rc;
     if ((rc = dev_gemm(L, false, false, n, n, n, -0.5, X, n, G, n, 1.5, X, n, D.X1, n, nullptr)))
       return rc;
@@ -1747,7 +1762,7 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
   if ((rc = dev_gemm(L, false, false, n, n, n, 1.0, A, lda, X, n, 0.0, nullptr, 0, AX, n, nullptr)))
     return rc;
   if ((rc = dev_gemm(L, true, false, n, 2 * n, n, 1.0, X, n, D.XA, n, 0.0, nullptr, 0, G, n,
-                     nullptr)))
+                     nullptr, 2)))
     return rc;
   int* nonfin = D.ints + 4 * D.nmax + 60;
   int* reach = D.ints + 4 * D.nmax + 64;
