@@ -977,7 +977,7 @@ __global__ void split_c_tc_kernel(const double* __restrict__ C, int64_t ldc, int
 struct UpdOut {
   const double* y0base;
   int64_t y0ld;
-  int row0;
+  int64_t row0;
 };
 
 struct UpdShared {
@@ -1212,12 +1212,12 @@ __global__ void __launch_bounds__(kUThrAll, 1)
         if (kY0) {
           const double* y0 = fin.y0base;
           out += y0 ? y0[r[u] * fin.y0ld + j[u]]
-                    : seg_load(Y0, ocol + j[u], (int64_t)fin.row0 + r[u]);
+                    : seg_load(Y0, ocol + j[u], fin.row0 + r[u]);
         }
         if (ybase)
           ybase[(int64_t)r[u] * oyld + j[u]] = out;
         else
-          *out_addr(Y, ocol + j[u], (int64_t)fin.row0 + r[u]) = out;
+          *out_addr(Y, ocol + j[u], fin.row0 + r[u]) = out;
       }
       ou += kU;
     };
@@ -1267,7 +1267,7 @@ __global__ void __launch_bounds__(kUThrAll, 1)
             fin.y0base = Y0.nseg == 1 ? Y0.ptr[0] + row0 * Y0.ld[0] + ocol : nullptr;
             fin.y0ld = Y0.ld[0];
           }
-          fin.row0 = (int)row0;
+          fin.row0 = row0;
         }
         __syncwarp();
         pblk = 0;

@@ -48,7 +48,11 @@ cudaMemPool_t pool_of_device() {
 
 int scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
   *p = nullptr;
-  cudaMemPool_t pool = pool_of_device();
+  // a captured allocation belongs to the graph, whatever the pool, and making a
+  // pool is no part of a capture
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+  cudaMemPool_t pool = cap == cudaStreamCaptureStatusNone ? pool_of_device() : nullptr;
   const size_t b = bytes < 16 ? 16 : bytes;
   if ((pool ? cudaMallocFromPoolAsync(p, b, pool, st) : cudaMallocAsync(p, b, st)) != cudaSuccess) {
     cudaGetLastError();
