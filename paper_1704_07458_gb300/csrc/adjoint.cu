@@ -239,8 +239,8 @@ __global__ void grad_coeff_kernel(int k, const double* __restrict__ lam,
 }
 
 int col_finish(cudaStream_t st, int k, void* partial, double* out) {
-  colsum_finish_kernel<<<(unsigned)ceil_div(k, kSumCols), kSumCols * kSumLanes, 0, st>>>(
-      (const double*)partial, kRB, k, out);
+  launch_chained(colsum_finish_kernel, (unsigned)ceil_div(k, kSumCols), kSumCols * kSumLanes, 0, st,
+                 (const double*)partial, kRB, k, out);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }

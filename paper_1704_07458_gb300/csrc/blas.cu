@@ -268,9 +268,9 @@ __global__ void __launch_bounds__(kColThreads) residual_kernel(
 }
 
 __global__ void __launch_bounds__(kSumCols* kSumLanes)
-    residual_finish_kernel(const double* __restrict__ partial, int blocks, int mm, int c0,
-                           const double* __restrict__ theta, double normA, double normB,
-                           double* __restrict__ be) {
+    residual_finish_kernel(const double* partial, int blocks, int mm, int c0, const double* theta,
+                           double normA, double normB, double* be) {
+  chain_wait();
   const int j = blockIdx.x * kSumCols + threadIdx.x % kSumCols;
   double s[2];
   sum_partials<2>(partial, blocks, mm, j, s);
@@ -292,8 +292,8 @@ int residual(cudaStream_t st, int64_t n, const double* X, const double* AX, cons
     residual_kernel<false><<<blocks, kColThreads, 0, st>>>(n, X, AX, BX, ld, m, c0, TX, theta,
                                                            kinv, W, ldw, xb, (double*)partial);
   LOB_LAUNCHED();
-  residual_finish_kernel<<<(unsigned)ceil_div(mm, kSumCols), kSumCols * kSumLanes, 0, st>>>(
-      (const double*)partial, blocks, mm, c0, theta, normA, normB, be);
+  launch_chained(residual_finish_kernel, (unsigned)ceil_div(mm, kSumCols), kSumCols * kSumLanes, 0,
+                 st, (const double*)partial, blocks, mm, c0, theta, normA, normB, be);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
@@ -335,8 +335,8 @@ int colsumsq(cudaStream_t st, int64_t n, const double* Y, int64_t ld, int m, dou
   const int blocks = row_blocks(n);
   colsumsq_kernel<<<blocks, kColThreads, 0, st>>>(n, Y, ld, m, col_tile(m), (double*)partial);
   LOB_LAUNCHED();
-  colsum_finish_kernel<<<(unsigned)ceil_div(m, kSumCols), kSumCols * kSumLanes, 0, st>>>(
-      (const double*)partial, blocks, m, out);
+  launch_chained(colsum_finish_kernel, (unsigned)ceil_div(m, kSumCols), kSumCols * kSumLanes, 0, st,
+                 (const double*)partial, blocks, m, out);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
@@ -428,8 +428,8 @@ int sign_normalise(cudaStream_t st, int64_t n, int m, double* X, int64_t ldx, vo
 // ------------------------------------------------------ balance exponents
 // out[k] = floor(log2(G_kk) / 2), i.e. 2^out[k] is within a factor 2 of the
 // column norm sqrt(G_kk) (0 for a non-positive diagonal).  Integer ops only.
-__global__ void diag_exponents_kernel(int n, const double* __restrict__ G, int64_t ldg,
-                                      int* __restrict__ out) {
+__global__ void diag_exponents_kernel(int n, const double* G, int64_t ldg, int* out) {
+  chain_wait();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const long long b = __double_as_longlong(G[k + (int64_t)k * ldg]);
@@ -444,7 +444,7 @@ __global__ void diag_exponents_kernel(int n, const double* __restrict__ G, int64
 
 int diag_exponents(cudaStream_t st, int n, const double* G, int64_t ldg, int* out) {
   if (n <= 0) return LOBPCG_OK;
-  diag_exponents_kernel<<<(unsigned)ceil_div(n, 128), 128, 0, st>>>(n, G, ldg, out);
+  launch_chained(diag_exponents_kernel, (unsigned)ceil_div(n, 128), 128, 0, st, n, G, ldg, out);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }

@@ -41,7 +41,7 @@ __device__ __forceinline__ double col_reduce(double v, double* red, int tx, int 
 // Fixed-order sum over blocks of partial[(z * NV + v) * m + j]: kSumCols
 // columns x kSumLanes lanes per CTA; the result is valid in lane 0.
 template <int NV>
-__device__ __forceinline__ void sum_partials(const double* __restrict__ partial, int blocks, int m,
+__device__ __forceinline__ void sum_partials(const double* partial, int blocks, int m,
                                              int j, double (&out)[NV]) {
   __shared__ double red[NV][kSumLanes][kSumCols];
   const int tx = threadIdx.x % kSumCols, ty = threadIdx.x / kSumCols;
@@ -68,8 +68,8 @@ __device__ __forceinline__ void sum_partials(const double* __restrict__ partial,
 
 // out[j] = sum over blocks of partial[z * m + j]
 static __global__ void __launch_bounds__(kSumCols* kSumLanes)
-    colsum_finish_kernel(const double* __restrict__ partial, int blocks, int m,
-                         double* __restrict__ out) {
+    colsum_finish_kernel(const double* partial, int blocks, int m, double* out) {
+  chain_wait();
   const int j = blockIdx.x * kSumCols + threadIdx.x % kSumCols;
   double s[1];
   sum_partials<1>(partial, blocks, m, j, s);

@@ -89,6 +89,7 @@ __global__ void svqb_t_kernel(int nu, int first, int nkeep, const double* d, con
 __global__ void assemble_kernel(int nx, int np, int nw, int c0, const double* theta,
                                 const double* PAP, int ldpap, const double* GAw,
                                 const double* GBw, int ldgw, double* SAS, double* SBS) {
+  chain_wait();
   const int ns = nx + np + nw;
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ns * ns) return;
@@ -1021,9 +1022,8 @@ int assemble(DenseLayer& L, int nx, int np, int nw, const double* theta, const d
              double* SBS, int c0) {
   const int ns = nx + np + nw;
   if (c0 < 0) c0 = nx + np;
-  assemble_kernel<<<blocks_for((int64_t)ns * ns), 256, 0, L.st>>>(nx, np, nw, c0, theta, PAP,
-                                                                  std::max(ldpap, 1), GAw, GBw,
-                                                                  ldgw, SAS, SBS);
+  launch_chained(assemble_kernel, blocks_for((int64_t)ns * ns), 256, 0, L.st, nx, np, nw, c0,
+                 theta, PAP, std::max(ldpap, 1), GAw, GBw, ldgw, SAS, SBS);
   LAUNCH_OK(L);
   return LOBPCG_OK;
 }

@@ -55,10 +55,11 @@ constexpr int kMaxRunDev = 32;                     // cluster width of the final
 // later ones m columns on; only the upper triangles are computed (half of the
 // FP64 work that bounds a product of order 213) and mirrored.
 __global__ void __launch_bounds__(256) gemm64_kernel(int m, int n, int k, int ta, int tb,
-                                                     double alpha, const double* __restrict__ A,
-                                                     int lda, const double* __restrict__ B, int ldb,
+                                                     double alpha, const double* A,
+                                                     int lda, const double* B, int ldb,
                                                      double beta, const double* Cin, int ldcin,
                                                      double* C, int ldc, const int* skip, int sym) {
+  chain_wait();
   if (skip && *skip) return;
   __shared__ double As[kGK][kGT + 1], Bs[kGK][kGT + 1];
   __shared__ double red[3][kGT * kGT];
@@ -131,6 +132,7 @@ __global__ void __launch_bounds__(256) gemm64_kernel(int m, int n, int k, int ta
 constexpr int kCholMax = 160;
 
 __global__ void __launch_bounds__(256) chol64_kernel(int n, double* A, int lda, int* info) {
+  chain_wait();
   extern __shared__ double sa[];  // n x n, column-major, leading dimension n
   __shared__ int s_fail;
   __shared__ double s_r, s_inv;
@@ -175,6 +177,7 @@ __global__ void __launch_bounds__(256) chol64_kernel(int n, double* A, int lda, 
 // skip: no-op when *skip != 0 (the factorisation failed).
 __global__ void __launch_bounds__(256) trinv64_kernel(int n, const double* R, int ldr, double* X,
                                                       int ldx, const int* skip) {
+  chain_wait();
   if (skip && *skip) return;
   extern __shared__ double sm[];  // n x n: R, rows turning into X from the bottom
   __shared__ double dinv[kCholMax];
@@ -222,6 +225,7 @@ __device__ __forceinline__ int pk(int n, int i, int j) {  // (i >= j) packed low
 __global__ void __launch_bounds__(1024, 1) tridiag32_kernel(int n, const double* A, int lda,
                                                             float* d, float* e, float* V, int ldv,
                                                             float* tau) {
+  chain_wait();
   extern __shared__ float P[];  // n (n + 1) / 2
   __shared__ float v[256], p[256];
   __shared__ float wpart[32];
@@ -423,9 +427,10 @@ __device__ __forceinline__ void tridiag_phase(int n, float (&a)[2 * NB][NB], Tri
 }
 
 template <int NB>
-__global__ void __launch_bounds__(512, 1) tridiag32_reg_kernel(int n, const double* __restrict__ A,
+__global__ void __launch_bounds__(512, 1) tridiag32_reg_kernel(int n, const double* A,
                                                                int lda, float* d, float* e,
                                                                float* V, int ldv, float* tau) {
+  chain_wait();
   constexpr int NR = 2 * NB;
   __shared__ TridiagShared<NB> sh;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -479,10 +484,11 @@ __device__ __forceinline__ float hash_unit(uint32_t a, uint32_t b) {
 // refines).  A round is a chain of n quotients, so its count is what to save:
 // four points per eigenvalue and IEEE division took 204 us at n = 213; 51 us
 // now.  bounds[0], bounds[1]: ||T|| bound and pivot guard for the eigenvectors.
-__global__ void __launch_bounds__(256) bisect_kernel(int n, const float* __restrict__ dg,
-                                                     const float* __restrict__ eg,
-                                                     float* __restrict__ lam,
-                                                     float* __restrict__ bounds) {
+__global__ void __launch_bounds__(256) bisect_kernel(int n, const float* dg,
+                                                     const float* eg,
+                                                     float* lam,
+                                                     float* bounds) {
+  chain_wait();
   __shared__ float d[256], e2[257];
   __shared__ float s_gl[8], s_gu[8], s_em[8];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -553,11 +559,12 @@ __global__ void __launch_bounds__(256) bisect_kernel(int n, const float* __restr
 // Per-thread work arrays live in shared memory interleaved by lane.  Y(:, j)
 // (FP32, n x n column-major) receives the unit eigenvector of T.
 // The pivots are stored as reciprocals, so the substitutions hold no division.
-__global__ void __launch_bounds__(32) tridiag_eig_kernel(int n, const float* __restrict__ dg,
-                                                         const float* __restrict__ eg,
-                                                         const float* __restrict__ lam,
-                                                         const float* __restrict__ bounds,
-                                                         float* __restrict__ Y, int ldy) {
+__global__ void __launch_bounds__(32) tridiag_eig_kernel(int n, const float* dg,
+                                                         const float* eg,
+                                                         const float* lam,
+                                                         const float* bounds,
+                                                         float* Y, int ldy) {
+  chain_wait();
   extern __shared__ float ws[];  // d, e (2 n) then 6 arrays of n x 32
   float* d = ws;
   float* e = ws + n;
@@ -641,8 +648,9 @@ __global__ void __launch_bounds__(32) tridiag_eig_kernel(int n, const float* __r
 // vectors): each cluster's vectors are orthonormalised in eigenvalue order
 // by modified Gram-Schmidt (one warp per cluster, clusters found by thread
 // 0).  Vectors of well separated eigenvalues are left as they are.
-__global__ void __launch_bounds__(1024, 1) cluster_orth_kernel(int n, const float* __restrict__ lam,
-                                                               float* __restrict__ Y, int ldy) {
+__global__ void __launch_bounds__(1024, 1) cluster_orth_kernel(int n, const float* lam,
+                                                               float* Y, int ldy) {
+  chain_wait();
   __shared__ int runs[2 * 128];
   __shared__ int nruns, near;
   __shared__ float ls[256];
@@ -707,10 +715,11 @@ __device__ __forceinline__ int vpk(int n, int k) {  // start of reflector k (row
 }
 
 template <int NB>
-__global__ void __launch_bounds__(256) backtransform_kernel(int n, const float* __restrict__ V,
-                                                            int ldv, const float* __restrict__ tau,
-                                                            const float* __restrict__ Y, int ldy,
-                                                            double* __restrict__ Z, int ldz) {
+__global__ void __launch_bounds__(256) backtransform_kernel(int n, const float* V,
+                                                            int ldv, const float* tau,
+                                                            const float* Y, int ldy,
+                                                            double* Z, int ldz) {
+  chain_wait();
   extern __shared__ float vp[];  // n (n - 1) / 2
   __shared__ float ts[256];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -762,9 +771,10 @@ __global__ void __launch_bounds__(256) backtransform_kernel(int n, const float* 
 // Two kernels over the whole GPU: partial norms and d, then delta and E.
 constexpr int kOaBlocks = 64;
 
-__global__ void __launch_bounds__(256) oa_norms_kernel(int n, const double* __restrict__ GS,
-                                                       double* __restrict__ part,
-                                                       double* __restrict__ dvec, const int* done) {
+__global__ void __launch_bounds__(256) oa_norms_kernel(int n, const double* GS,
+                                                       double* part,
+                                                       double* dvec, const int* done) {
+  chain_wait();
   if (*done) return;
   __shared__ double red[2][8];
   const double* G = GS;
@@ -805,13 +815,14 @@ __global__ void __launch_bounds__(256) oa_norms_kernel(int n, const double* __re
   }
 }
 
-__global__ void __launch_bounds__(256) oa_e_kernel(int n, const double* __restrict__ GS,
-                                                   const double* __restrict__ part,
-                                                   const double* __restrict__ dvec,
-                                                   const double* __restrict__ scal,
-                                                   double* __restrict__ E, int* done,
+__global__ void __launch_bounds__(256) oa_e_kernel(int n, const double* GS,
+                                                   const double* part,
+                                                   const double* dvec,
+                                                   const double* scal,
+                                                   double* E, int* done,
                                                    double* delta_out,
                                                    unsigned long long* emax) {
+  chain_wait();
   if (*done) return;
   __shared__ double s_delta;
   __shared__ unsigned long long s_max[8];
@@ -868,6 +879,7 @@ __global__ void __launch_bounds__(256) oa_e_kernel(int n, const double* __restri
 // orthogonality defect of order |s_ij - s_ji| / |d_j - d_i| (the rounding
 // asymmetry of X^T A X over the gap) even when its corrections are tiny.
 __global__ void oa_next_kernel(const int* cur, const unsigned long long* emax, int* next) {
+  chain_wait();
   if (threadIdx.x == 0)
     next[0] = (cur[0] || __longlong_as_double((long long)emax[0]) <= 1e-10) ? 1 : 0;
 }
@@ -893,12 +905,13 @@ __device__ __forceinline__ long long order_key(double x) {  // sorts as x does (
 
 // reach[pos(i)]: furthest sorted position coupled to column i; part[i]: column
 // i's share of ||I - G||_F^2; perm and w; nonfin[0] = 1 for a non-finite d_i.
-__global__ void __launch_bounds__(256) eig_scan_kernel(int n, const double* __restrict__ GS,
-                                                       const double* __restrict__ scal,
-                                                       int* __restrict__ perm,
-                                                       int* __restrict__ reach,
-                                                       double* __restrict__ part,
-                                                       double* __restrict__ w, int* nonfin) {
+__global__ void __launch_bounds__(256) eig_scan_kernel(int n, const double* GS,
+                                                       const double* scal,
+                                                       int* perm,
+                                                       int* reach,
+                                                       double* part,
+                                                       double* w, int* nonfin) {
+  chain_wait();
   __shared__ long long key[256];
   __shared__ int pos[256];
   const double* G = GS;
@@ -943,11 +956,12 @@ __global__ void __launch_bounds__(256) eig_scan_kernel(int n, const double* __re
   }
 }
 
-__global__ void __launch_bounds__(256) eig_finalize_kernel(int n, const int* __restrict__ reach_g,
-                                                           const double* __restrict__ part,
-                                                           int* __restrict__ runs,
-                                                           int* __restrict__ nruns_out,
+__global__ void __launch_bounds__(256) eig_finalize_kernel(int n, const int* reach_g,
+                                                           const double* part,
+                                                           int* runs,
+                                                           int* nruns_out,
                                                            int* nonfin, int* status) {
+  chain_wait();
   __shared__ int reach[256];
   __shared__ double red[8];
   __shared__ int coupled;
@@ -986,9 +1000,10 @@ __global__ void __launch_bounds__(256) eig_finalize_kernel(int n, const int* __r
 }
 
 // Zo(:, k) = X(:, perm[k]) (column permutation into the output).
-__global__ void permute_cols_dev_kernel(int n, const double* __restrict__ X, int ldxx,
-                                        const int* __restrict__ perm, double* __restrict__ Zo,
+__global__ void permute_cols_dev_kernel(int n, const double* X, int ldxx,
+                                        const int* perm, double* Zo,
                                         int ldo) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)n * n) return;
   const int r = (int)(e % n), k = (int)(e / n);
@@ -999,12 +1014,13 @@ __global__ void permute_cols_dev_kernel(int n, const double* __restrict__ X, int
 // perm[a + j]) of each run [a, a + m), one CTA per run (CTAs beyond the run
 // count exit), then Zo(:, a : a + m) <- Zo(:, a : a + m) Q and w(a : a + m)
 // the block's eigenvalues ascending.
-__global__ void __launch_bounds__(256) run_jacobi_kernel(int n, const double* __restrict__ GS,
-                                                         const int* __restrict__ perm,
-                                                         const int* __restrict__ runs,
-                                                         const int* __restrict__ nruns,
-                                                         double* __restrict__ Zo, int ldo,
-                                                         double* __restrict__ w) {
+__global__ void __launch_bounds__(256) run_jacobi_kernel(int n, const double* GS,
+                                                         const int* perm,
+                                                         const int* runs,
+                                                         const int* nruns,
+                                                         double* Zo, int ldo,
+                                                         double* w) {
+  chain_wait();
   if ((int)blockIdx.x >= nruns[0]) return;
   if (runs[2 * blockIdx.x + 1] > kMaxRunDev) return;  // flagged by the finalize pass
   const double* S = GS + (int64_t)n * n;
@@ -1094,8 +1110,9 @@ __global__ void __launch_bounds__(256) run_jacobi_kernel(int n, const double* __
 // Each reflector is column-wise backward stable, so the span of a column of
 // M is kept to FP32 accuracy relative to that column's own norm whatever
 // the other columns' norms; the caller restores FP64 orthonormality.
-__global__ void __launch_bounds__(1024, 1) qr32_kernel(int m, int c, const double* __restrict__ M,
-                                                       int ldm, double* __restrict__ Q, int ldq) {
+__global__ void __launch_bounds__(1024, 1) qr32_kernel(int m, int c, const double* M,
+                                                       int ldm, double* Q, int ldq) {
+  chain_wait();
   extern __shared__ float qs[];
   float* a = qs;          // m x c
   float* q = qs + m * c;  // m x c
@@ -1167,8 +1184,9 @@ __global__ void __launch_bounds__(1024, 1) qr32_kernel(int m, int c, const doubl
 
 // ------------------------------------------------- small helpers
 // D = S (rows x cols), skipped when *skip != 0
-__global__ void copy_skip_kernel(int rows, int cols, const double* __restrict__ S, int lds,
-                                 double* __restrict__ D, int ldd, const int* skip) {
+__global__ void copy_skip_kernel(int rows, int cols, const double* S, int lds,
+                                 double* D, int ldd, const int* skip) {
+  chain_wait();
   if (skip && *skip) return;
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)rows * cols) return;
@@ -1178,15 +1196,17 @@ __global__ void copy_skip_kernel(int rows, int cols, const double* __restrict__ 
 
 // order 1: Z = [1], w = a, status 0
 __global__ void eig1_kernel(const double* A, double* Z, double* w, int* status) {
+  chain_wait();
   w[0] = A[0];
   Z[0] = 1.0;
   status[0] = 0;
 }
 
 // S = (A + A^T) / 2 (n x n), with each CTA's share of ||S||_F^2
-__global__ void __launch_bounds__(256) symmetrize_copy_kernel(int n, const double* __restrict__ A,
-                                                              int lda, double* __restrict__ S,
-                                                              int lds, double* __restrict__ part) {
+__global__ void __launch_bounds__(256) symmetrize_copy_kernel(int n, const double* A,
+                                                              int lda, double* S,
+                                                              int lds, double* part) {
+  chain_wait();
   __shared__ double red[8];
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double v = 0.0;
@@ -1207,8 +1227,9 @@ __global__ void __launch_bounds__(256) symmetrize_copy_kernel(int n, const doubl
 }
 
 // out[0] = sqrt of the sum of m partials (m <= 256, fixed order)
-__global__ void __launch_bounds__(256) norm_finish_kernel(int m, const double* __restrict__ part,
+__global__ void __launch_bounds__(256) norm_finish_kernel(int m, const double* part,
                                                           double* out) {
+  chain_wait();
   __shared__ double red[8];
   double v = threadIdx.x < m ? part[threadIdx.x] : 0.0;
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1221,8 +1242,9 @@ __global__ void __launch_bounds__(256) norm_finish_kernel(int m, const double* _
   }
 }
 
-__global__ void copy_block_cm_kernel(int rows, int cols, const double* __restrict__ S, int lds,
-                                     double* __restrict__ D, int ldd, double scale) {
+__global__ void copy_block_cm_kernel(int rows, int cols, const double* S, int lds,
+                                     double* D, int ldd, double scale) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)rows * cols) return;
   const int i = (int)(e % rows), j = (int)(e / rows);
@@ -1230,9 +1252,10 @@ __global__ void copy_block_cm_kernel(int rows, int cols, const double* __restric
 }
 
 // X(i, j) *= r[i] (row scaling), optionally adding Add(i, j) for i < add_rows first
-__global__ void scale_rows_add_kernel(int rows, int cols, const double* __restrict__ r,
-                                      double* __restrict__ X, int ldx, const double* __restrict__ Add,
+__global__ void scale_rows_add_kernel(int rows, int cols, const double* r,
+                                      double* X, int ldx, const double* Add,
                                       int ldadd, int add_rows) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)rows * cols) return;
   const int i = (int)(e % rows), j = (int)(e / rows);
@@ -1243,9 +1266,10 @@ __global__ void scale_rows_add_kernel(int rows, int cols, const double* __restri
 
 // d_i = G_ii^-1/2 (0 for a zero column); MB = D GB D, MA = D GA D (both
 // symmetrised).  GA may be null (only MB).
-__global__ void dscale2_kernel(int n, const double* __restrict__ GB, int ldb,
-                               const double* __restrict__ GA, int lda, double* __restrict__ d,
-                               double* __restrict__ MB, double* __restrict__ MA, int ldm) {
+__global__ void dscale2_kernel(int n, const double* GB, int ldb,
+                               const double* GA, int lda, double* d,
+                               double* MB, double* MA, int ldm) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)n * n) return;
   const int i = (int)(e % n), j = (int)(e / n);
@@ -1264,10 +1288,11 @@ __global__ void dscale2_kernel(int n, const double* __restrict__ GB, int ldb,
 // transpose below the diagonal, MB on the trailing block; SA' has the GEMM's
 // leading block, Ka[:, o:] = Y11^T MA[0:o, o:] off the diagonal and MA on the
 // trailing block.  Both come out with both triangles.
-__global__ void pre_fill_kernel(int ns, int o, const double* __restrict__ MB,
-                                const double* __restrict__ MA, int ldm,
-                                const double* __restrict__ Ka, int ldk, double* __restrict__ SB,
-                                double* __restrict__ SA, int lds) {
+__global__ void pre_fill_kernel(int ns, int o, const double* MB,
+                                const double* MA, int ldm,
+                                const double* Ka, int ldk, double* SB,
+                                double* SA, int lds) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ns * ns) return;
   const int i = (int)(e % ns), j = (int)(e / ns);
@@ -1286,9 +1311,10 @@ __global__ void pre_fill_kernel(int ns, int o, const double* __restrict__ MB,
 
 // C(i, j) = d_i (i < o ? Ct(i, j) : C(i, j)): the coefficients in the basis
 // S back from the congruence, C = D blkdiag(Y11, I) C'.
-__global__ void pre_back_kernel(int ns, int m, int o, const double* __restrict__ d,
-                                const double* __restrict__ Ct, int ldt, double* __restrict__ C,
+__global__ void pre_back_kernel(int ns, int m, int o, const double* d,
+                                const double* Ct, int ldt, double* C,
                                 int ldc) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ns * m) return;
   const int i = (int)(e % ns), j = (int)(e / ns);
@@ -1298,9 +1324,10 @@ __global__ void pre_back_kernel(int ns, int m, int o, const double* __restrict__
 
 // H (ns x ns): H[0:o, 0:o] = MA[0:o, 0:o]; H[0:o, o:] = Qm[0:o, :] and its
 // transpose below; H[o:, o:] is written by a GEMM.
-__global__ void assemble_h_kernel(int ns, int o, const double* __restrict__ MA, int ldm,
-                                  const double* __restrict__ Qm, int ldq, double* __restrict__ H,
+__global__ void assemble_h_kernel(int ns, int o, const double* MA, int ldm,
+                                  const double* Qm, int ldq, double* H,
                                   int ldh) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)ns * ns) return;
   const int i = (int)(e % ns), j = (int)(e / ns);
@@ -1318,9 +1345,10 @@ __global__ void assemble_h_kernel(int ns, int o, const double* __restrict__ MA, 
 // memory (the value feeds an order-of-magnitude test).  out[0] = cond(R),
 // inf when a factor is non-finite; skip: no-op when *skip != 0 (then out[0]
 // is set to inf).
-__global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, const double* __restrict__ MB,
-                                                              int ldm, const double* __restrict__ Y,
+__global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, const double* MB,
+                                                              int ldm, const double* Y,
                                                               int ldy, double* out, const int* skip) {
+  chain_wait();
   if (skip && *skip) {
     if (threadIdx.x == 0) out[0] = INFINITY;
     return;
@@ -1460,9 +1488,10 @@ __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, con
 }
 
 // Q2(i, j) = th[i] * Q(i, j)
-__global__ void scale_rows_by_kernel(int rows, int cols, const double* __restrict__ th,
-                                     const double* __restrict__ Q, int ldq, double* __restrict__ Q2,
+__global__ void scale_rows_by_kernel(int rows, int cols, const double* th,
+                                     const double* Q, int ldq, double* Q2,
                                      int ldq2) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)rows * cols) return;
   const int i = (int)(e % rows), j = (int)(e / rows);
@@ -1473,9 +1502,10 @@ __global__ void scale_rows_by_kernel(int rows, int cols, const double* __restric
 // Z) of D G D: keep J = {j : w_j > tau max|w|} (drop) or all with w clamped
 // at tau max|w| (replace); T(:, t) = d .* Z(:, first + t) / sqrt(w); nkeep[0]
 // is the kept count.  One CTA computes the split, all threads fill T.
-__global__ void svqb_dev_kernel(int nu, const double* __restrict__ w, const double* __restrict__ d,
-                                const double* __restrict__ Z, int ldz, int drop, double tau,
-                                double* __restrict__ T, int ldt, int* nkeep) {
+__global__ void svqb_dev_kernel(int nu, const double* w, const double* d,
+                                const double* Z, int ldz, int drop, double tau,
+                                double* T, int ldt, int* nkeep) {
+  chain_wait();
   __shared__ int s_first;
   __shared__ double s_floor;
   if (threadIdx.x == 0) {
@@ -1504,8 +1534,9 @@ __global__ void svqb_dev_kernel(int nu, const double* __restrict__ w, const doub
 }
 
 // D = diag(w[0:n]) (n x n, leading dimension ldd)
-__global__ void diag_matrix_kernel(int n, const double* __restrict__ w, double* __restrict__ D,
+__global__ void diag_matrix_kernel(int n, const double* w, double* D,
                                    int ldd) {
+  chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)n * n) return;
   const int i = (int)(e % n), j = (int)(e / n);
@@ -1579,8 +1610,8 @@ int dev_gemm(DenseLayer& L, bool ta, bool tb, int m, int n, int k, double alpha,
     Cin = C;
     ldcin = ldc;
   }
-  gemm64_kernel<<<(unsigned)tiles, 256, 0, L.st>>>(m, n, k, ta ? 1 : 0, tb ? 1 : 0, alpha, A, lda,
-                                                   B, ldb, beta, Cin, ldcin, C, ldc, skip, sym);
+  launch_chained(gemm64_kernel, (unsigned)tiles, 256, 0, L.st, m, n, k, ta ? 1 : 0, tb ? 1 : 0,
+                 alpha, A, lda, B, ldb, beta, Cin, ldcin, C, ldc, skip, sym);
   DLAUNCH(L);
   return LOBPCG_OK;
 }
@@ -1598,14 +1629,15 @@ int dev_chol(DenseLayer& L, int n, double* A, int lda, int* info) {
                                      kCholMax * kCholMax * 8));
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
-  chol64_kernel<<<1, 256, sh, L.st>>>(n, A, lda, info);
+  launch_chained(chol64_kernel, 1, 256, sh, L.st, n, A, lda, info);
   DLAUNCH(L);
   return LOBPCG_OK;
 }
 
 int dev_trinv(DenseLayer& L, int n, const double* R, int ldr, double* X, int ldx, const int* skip) {
   if (n > kCholMax) return LOBPCG_ERR_ARG;
-  trinv64_kernel<<<1, 256, (size_t)n * n * sizeof(double), L.st>>>(n, R, ldr, X, ldx, skip);
+  launch_chained(trinv64_kernel, 1, 256, (size_t)n * n * sizeof(double), L.st, n, R, ldr, X, ldx,
+                 skip);
   DLAUNCH(L);
   return LOBPCG_OK;
 }
@@ -1637,7 +1669,7 @@ int dev_syev(DenseLayer& L, int n, const double* A, int lda, double* Z, int ldz,
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   if (n == 1) {
-    eig1_kernel<<<1, 1, 0, L.st>>>(A, Z, w, status);
+    launch_chained(eig1_kernel, 1, 1, 0, L.st, A, Z, w, status);
     DLAUNCH(L);
     return LOBPCG_OK;
   }
@@ -1649,20 +1681,21 @@ int dev_syev(DenseLayer& L, int n, const double* A, int lda, double* Z, int ldz,
   // the refinement multiplies by the symmetric part of A (a projected
   // matrix formed by products is symmetric only to rounding)
   // (its norm partials lie where the refinement's vectors will)
-  symmetrize_copy_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, A, lda, D.Zt, n, D.vec);
+  launch_chained(symmetrize_copy_kernel, nblk((int64_t)n * n), 256, 0, L.st, n, A, lda, D.Zt, n,
+                 D.vec);
   DLAUNCH(L);
-  norm_finish_kernel<<<1, 256, 0, L.st>>>((int)nblk((int64_t)n * n), D.vec, normA);
+  launch_chained(norm_finish_kernel, 1, 256, 0, L.st, (int)nblk((int64_t)n * n), D.vec, normA);
   DLAUNCH(L);
   A = D.Zt;
   lda = n;
   const int nb = (int)ceil_div(n, 32);
   float* bounds = reinterpret_cast<float*>(D.scal + 8);
   auto tridiag = [&](auto* kernel) {
-    kernel<<<1, 512, 0, L.st>>>(n, A, lda, d32, e32, D.V32, n, tau32);
+    launch_chained(kernel, 1, 512, 0, L.st, n, A, lda, d32, e32, D.V32, n, tau32);
   };
   if (n > kTridRegMax)
-    tridiag32_kernel<<<1, 1024, (size_t)n * (n + 1) / 2 * 4, L.st>>>(n, A, lda, d32, e32, D.V32,
-                                                                     n, tau32);
+    launch_chained(tridiag32_kernel, 1, 1024, (size_t)n * (n + 1) / 2 * 4, L.st, n, A, lda, d32,
+                   e32, D.V32, n, tau32);
   else if (nb == 1) tridiag(tridiag32_reg_kernel<1>);
   else if (nb == 2) tridiag(tridiag32_reg_kernel<2>);
   else if (nb == 3) tridiag(tridiag32_reg_kernel<3>);
@@ -1671,18 +1704,18 @@ int dev_syev(DenseLayer& L, int n, const double* A, int lda, double* Z, int ldz,
   else if (nb == 6) tridiag(tridiag32_reg_kernel<6>);
   else tridiag(tridiag32_reg_kernel<7>);
   DLAUNCH(L);
-  bisect_kernel<<<(unsigned)ceil_div(n, 8), 256, 0, L.st>>>(n, d32, e32, lam32, bounds);
+  launch_chained(bisect_kernel, (unsigned)ceil_div(n, 8), 256, 0, L.st, n, d32, e32, lam32, bounds);
   DLAUNCH(L);
-  tridiag_eig_kernel<<<(unsigned)ceil_div(n, 32), 32, (size_t)(2 * n + 6 * 32 * n) * 4, L.st>>>(
-      n, d32, e32, lam32, bounds, D.Y32, n);
+  launch_chained(tridiag_eig_kernel, (unsigned)ceil_div(n, 32), 32,
+                 (size_t)(2 * n + 6 * 32 * n) * 4, L.st, n, d32, e32, lam32, bounds, D.Y32, n);
   DLAUNCH(L);
-  cluster_orth_kernel<<<1, 1024, 0, L.st>>>(n, lam32, D.Y32, n);
+  launch_chained(cluster_orth_kernel, 1, 1024, 0, L.st, n, lam32, D.Y32, n);
   DLAUNCH(L);
   // X (first n columns of XA) = Q Y
   double* X = D.XA;
   auto back = [&](auto* kernel) {
-    kernel<<<(unsigned)ceil_div(n, 8), 256, (size_t)(n * (n - 1)) / 2 * 4, L.st>>>(
-        n, D.V32, n, tau32, D.Y32, n, X, n);
+    launch_chained(kernel, (unsigned)ceil_div(n, 8), 256, (size_t)(n * (n - 1)) / 2 * 4, L.st, n,
+                   D.V32, n, tau32, D.Y32, n, X, n);
   };
   switch (nb) {
     case 1: back(backtransform_kernel<1>); break;
@@ -1732,18 +1765,19 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
     if ((rc = dev_gemm(L, true, false, n, 2 * n, n, 1.0, X, n, D.XA, n, 0.0, nullptr, 0, G, n,
                        done, 2)))
       return rc;
-    oa_norms_kernel<<<kOaBlocks, 256, 0, L.st>>>(n, D.GS, D.vec, D.vec + 2 * kOaBlocks, done);
+    launch_chained(oa_norms_kernel, kOaBlocks, 256, 0, L.st, n, D.GS, D.vec, D.vec + 2 * kOaBlocks,
+                   done);
     DLAUNCH(L);
-    oa_e_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, D.GS, D.vec, D.vec + 2 * kOaBlocks,
-                                                        normA, D.E, done, delta, emax + s);
+    launch_chained(oa_e_kernel, nblk((int64_t)n * n), 256, 0, L.st, n, D.GS, D.vec,
+                   D.vec + 2 * kOaBlocks, normA, D.E, done, delta, emax + s);
     DLAUNCH(L);
-    oa_next_kernel<<<1, 32, 0, L.st>>>(done, emax + s, flag + s + 1);
+    launch_chained(oa_next_kernel, 1, 32, 0, L.st, done, emax + s, flag + s + 1);
     DLAUNCH(L);
     // X1 = X + X E
     if ((rc = dev_gemm(L, false, false, n, n, n, 1.0, X, n, D.E, n, 1.0, X, n, D.X1, n, done)))
       return rc;
     // X = X1 (skipped with the step)
-    copy_skip_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, n, D.X1, n, X, n, done);
+    launch_chained(copy_skip_kernel, nblk((int64_t)n * n), 256, 0, L.st, n, n, D.X1, n, X, n, done);
     DLAUNCH(L);
   }
   // two Newton-Schulz steps X = X (3/2 I - 1/2 X^T X): the last first-order
@@ -1755,7 +1789,8 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
       return rc;
     if ((rc = dev_gemm(L, false, false, n, n, n, -0.5, X, n, G, n, 1.5, X, n, D.X1, n, nullptr)))
       return rc;
-    copy_block_cm_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, n, D.X1, n, X, n, 1.0);
+    launch_chained(copy_block_cm_kernel, nblk((int64_t)n * n), 256, 0, L.st, n, n, D.X1, n, X, n,
+                   1.0);
     DLAUNCH(L);
   }
   // final [G, S] = X^T [X, A X]
@@ -1766,15 +1801,17 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
     return rc;
   int* nonfin = D.ints + 4 * D.nmax + 60;
   int* reach = D.ints + 4 * D.nmax + 64;
-  eig_scan_kernel<<<(unsigned)ceil_div(n, 8), 256, 0, L.st>>>(n, D.GS, normA, perm, reach, D.vec, w,
-                                                              nonfin);
+  launch_chained(eig_scan_kernel, (unsigned)ceil_div(n, 8), 256, 0, L.st, n, D.GS, normA, perm,
+                 reach, D.vec, w, nonfin);
   DLAUNCH(L);
-  eig_finalize_kernel<<<1, 256, 0, L.st>>>(n, reach, D.vec, runs, nruns, nonfin, status);
+  launch_chained(eig_finalize_kernel, 1, 256, 0, L.st, n, reach, D.vec, runs, nruns, nonfin,
+                 status);
   DLAUNCH(L);
-  permute_cols_dev_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, X, n, perm, Z, ldz);
+  launch_chained(permute_cols_dev_kernel, nblk((int64_t)n * n), 256, 0, L.st, n, X, n, perm, Z,
+                 ldz);
   DLAUNCH(L);
-  run_jacobi_kernel<<<(unsigned)std::max(1, n / 2), 256, 0, L.st>>>(n, D.GS, perm, runs, nruns, Z,
-                                                                     ldz, w);
+  launch_chained(run_jacobi_kernel, (unsigned)std::max(1, n / 2), 256, 0, L.st, n, D.GS, perm, runs,
+                 nruns, Z, ldz, w);
   DLAUNCH(L);
   return LOBPCG_OK;
 }
@@ -1793,7 +1830,7 @@ int dev_orth_basis(DenseLayer& L, int m, int c, const double* M, int ldm, double
   }
   const size_t sh = 2 * (size_t)m * c * sizeof(float);
   if (sh > 200 * 1024 || c > 256) return LOBPCG_ERR_ARG;
-  qr32_kernel<<<1, 1024, sh, L.st>>>(m, c, M, ldm, Q, ldq);
+  launch_chained(qr32_kernel, 1, 1024, sh, L.st, m, c, M, ldm, Q, ldq);
   DLAUNCH(L);
   int rc;
   for (int s = 0; s < 2; ++s) {
@@ -1803,7 +1840,8 @@ int dev_orth_basis(DenseLayer& L, int m, int c, const double* M, int ldm, double
     if ((rc = dev_gemm(L, false, false, m, c, c, -0.5, Q, ldq, D.T4, c, 1.5, Q, ldq, D.T3, m,
                        nullptr)))
       return rc;
-    copy_block_cm_kernel<<<nblk((int64_t)m * c), 256, 0, L.st>>>(m, c, D.T3, m, Q, ldq, 1.0);
+    launch_chained(copy_block_cm_kernel, nblk((int64_t)m * c), 256, 0, L.st, m, c, D.T3, m, Q, ldq,
+                   1.0);
     DLAUNCH(L);
   }
   return LOBPCG_OK;
@@ -1890,7 +1928,7 @@ int eig_recover(DenseLayer& L, int n, const double* H, double* Z, int mask) {
     if (fl == 0) return LOBPCG_OK;
     note_check(L, fl);
   }
-  copy_block_cm_kernel<<<nblk((int64_t)n * n), 256, 0, L.st>>>(n, n, H, n, Z, n, 1.0);
+  launch_chained(copy_block_cm_kernel, nblk((int64_t)n * n), 256, 0, L.st, n, n, H, n, Z, n, 1.0);
   DLAUNCH(L);
   return syevd_fallback(L, n, Z, n);
 }
@@ -1906,14 +1944,16 @@ int rr_tail(DenseLayer& L, const double* TZ, const double* Z, int ns, int nx, in
   const int mrow = ns - nx, mcol = nx - nc;
   const int npn = std::min(mrow, mcol);
   int rc;
-  copy_block_cm_kernel<<<nblk((int64_t)ns * nx), 256, 0, L.st>>>(ns, nx, TZ, ns, C, ns, 1.0);
+  launch_chained(copy_block_cm_kernel, nblk((int64_t)ns * nx), 256, 0, L.st, ns, nx, TZ, ns, C, ns,
+                 1.0);
   DLAUNCH(L);
   if (npn > 0) {
     if (mcol >= mrow) {  // M spans the whole (ns - nx)-dimensional space: Q = I
-      copy_block_cm_kernel<<<nblk((int64_t)ns * mrow), 256, 0, L.st>>>(
-          ns, mrow, TZ + (int64_t)nx * ns, ns, C + (int64_t)nx * ns, ns, 1.0);
+      launch_chained(copy_block_cm_kernel, nblk((int64_t)ns * mrow), 256, 0, L.st, ns, mrow,
+                     TZ + (int64_t)nx * ns, ns, C + (int64_t)nx * ns, ns, 1.0);
       DLAUNCH(L);
-      diag_matrix_kernel<<<nblk((int64_t)npn * npn), 256, 0, L.st>>>(npn, L.ev + nx, PAP, npn);
+      launch_chained(diag_matrix_kernel, nblk((int64_t)npn * npn), 256, 0, L.st, npn, L.ev + nx,
+                     PAP, npn);
       DLAUNCH(L);
     } else {
       double* M = D.Zt;
@@ -1926,8 +1966,8 @@ int rr_tail(DenseLayer& L, const double* TZ, const double* Z, int ns, int nx, in
       if ((rc = dev_gemm(L, false, false, ns, mcol, mrow, 1.0, TZ + (int64_t)nx * ns, ns, Q, mrow,
                          0.0, nullptr, 0, C + (int64_t)nx * ns, ns, nullptr)))
         return rc;
-      scale_rows_by_kernel<<<nblk((int64_t)mrow * mcol), 256, 0, L.st>>>(mrow, mcol, L.ev + nx, Q,
-                                                                          mrow, Q2, mrow);
+      launch_chained(scale_rows_by_kernel, nblk((int64_t)mrow * mcol), 256, 0, L.st, mrow, mcol,
+                     L.ev + nx, Q, mrow, Q2, mrow);
       DLAUNCH(L);
       if ((rc = dev_gemm(L, true, false, mcol, mcol, mrow, 1.0, Q, mrow, Q2, mrow, 0.0, nullptr, 0,
                          PAP, npn, nullptr)))
@@ -1959,14 +1999,16 @@ int rr_initial_dev(DenseLayer& L, const double* GA, const double* GB, int nx, do
   int rc;
   if ((rc = configure_cond(L))) return rc;
   LOB_CUDA_OK(cudaMemsetAsync(info, 0, 2 * sizeof(int), L.st));
-  dscale2_kernel<<<nblk((int64_t)nx * nx), 256, 0, L.st>>>(nx, GB, nx, GA, nx, L.d, MB, MA, nx);
+  launch_chained(dscale2_kernel, nblk((int64_t)nx * nx), 256, 0, L.st, nx, GB, nx, GA, nx, L.d, MB,
+                 MA, nx);
   DLAUNCH(L);
-  copy_block_cm_kernel<<<nblk((int64_t)nx * nx), 256, 0, L.st>>>(nx, nx, MB, nx, Rf, nx, 1.0);
+  launch_chained(copy_block_cm_kernel, nblk((int64_t)nx * nx), 256, 0, L.st, nx, nx, MB, nx, Rf, nx,
+                 1.0);
   DLAUNCH(L);
   if ((rc = dev_chol(L, nx, Rf, nx, info))) return rc;
   if ((rc = dev_trinv(L, nx, Rf, nx, Ri, nx, info))) return rc;
-  cond_struct_kernel<<<1, 1024, (size_t)(2 * nx * nx + 3 * nx) * 4, L.st>>>(nx, 0, MB, nx, Ri, nx,
-                                                                            cr, info);
+  launch_chained(cond_struct_kernel, 1, 1024, (size_t)(2 * nx * nx + 3 * nx) * 4, L.st, nx, 0, MB,
+                 nx, Ri, nx, cr, info);
   DLAUNCH(L);
   // H = Ri^T MA Ri
   if ((rc = dev_gemm(L, false, false, nx, nx, nx, 1.0, MA, nx, Ri, nx, 0.0, nullptr, 0, T, nx, info)))
@@ -1989,7 +2031,8 @@ int rr_initial_dev(DenseLayer& L, const double* GA, const double* GB, int nx, do
   if ((rc = dev_gemm(L, false, false, nx, nx, nx, 1.0, Ri, nx, Z, nx, 0.0, nullptr, 0, C, nx,
                      nullptr)))
     return rc;
-  scale_rows_add_kernel<<<nblk((int64_t)nx * nx), 256, 0, L.st>>>(nx, nx, L.d, C, nx, nullptr, 0, 0);
+  launch_chained(scale_rows_add_kernel, nblk((int64_t)nx * nx), 256, 0, L.st, nx, nx, L.d, C, nx,
+                 nullptr, 0, 0);
   DLAUNCH(L);
   LOB_CUDA_OK(cudaMemcpyAsync(theta, L.ev, nx * sizeof(double), cudaMemcpyDeviceToDevice, L.st));
   return LOBPCG_OK;
@@ -2032,7 +2075,8 @@ int rr_modified_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
     if (fl[0] != 0 && (rc = eig_recover(L, ns, SAS, Z, fl[0]))) return rc;
     return rr_tail(L, Z, Z, ns, nx, nc, C, npn_out, theta, PAP);
   }
-  dscale2_kernel<<<nblk((int64_t)ns * ns), 256, 0, L.st>>>(ns, SBS, ns, SAS, ns, L.d, MB, MA, ns);
+  launch_chained(dscale2_kernel, nblk((int64_t)ns * ns), 256, 0, L.st, ns, SBS, ns, SAS, ns, L.d,
+                 MB, MA, ns);
   DLAUNCH(L);
   const double* Hsrc = MA;
   if (nw > 0) {
@@ -2046,13 +2090,14 @@ int rr_modified_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
     if ((rc = dev_gemm(L, false, false, o, nw, nw, -1.0, F, ns, Y + o, ns, 0.0, nullptr, 0, Y, ns,
                        info)))
       return rc;
-    cond_struct_kernel<<<1, 1024, (size_t)(2 * o * nw + 2 * nw * nw + 3 * ns) * 4, L.st>>>(
-        ns, o, MB, ns, Y, ns, cr, info);
+    launch_chained(cond_struct_kernel, 1, 1024, (size_t)(2 * o * nw + 2 * nw * nw + 3 * ns) * 4,
+                   L.st, ns, o, MB, ns, Y, ns, cr, info);
     DLAUNCH(L);
     if ((rc = dev_gemm(L, false, false, ns, nw, ns, 1.0, MA, ns, Y, ns, 0.0, nullptr, 0, Qm, ns,
                        info)))
       return rc;
-    assemble_h_kernel<<<nblk((int64_t)ns * ns), 256, 0, L.st>>>(ns, o, MA, ns, Qm, ns, H, ns);
+    launch_chained(assemble_h_kernel, nblk((int64_t)ns * ns), 256, 0, L.st, ns, o, MA, ns, Qm, ns,
+                   H, ns);
     DLAUNCH(L);
     if ((rc = dev_gemm(L, true, false, nw, nw, ns, 1.0, Y, ns, Qm, ns, 0.0, nullptr, 0,
                        H + o + (int64_t)o * ns, ns, info)))
@@ -2083,11 +2128,14 @@ int rr_modified_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
     if ((rc = dev_gemm(L, false, false, ns, ns, nw, 1.0, Y, ns, Z + o, ns, 0.0, nullptr, 0, TZ, ns,
                        nullptr)))
       return rc;
-    scale_rows_add_kernel<<<nblk((int64_t)ns * ns), 256, 0, L.st>>>(ns, ns, L.d, TZ, ns, Z, ns, o);
+    launch_chained(scale_rows_add_kernel, nblk((int64_t)ns * ns), 256, 0, L.st, ns, ns, L.d, TZ, ns,
+                   Z, ns, o);
   } else {
-    copy_block_cm_kernel<<<nblk((int64_t)ns * ns), 256, 0, L.st>>>(ns, ns, Z, ns, TZ, ns, 1.0);
+    launch_chained(copy_block_cm_kernel, nblk((int64_t)ns * ns), 256, 0, L.st, ns, ns, Z, ns, TZ,
+                   ns, 1.0);
     DLAUNCH(L);
-    scale_rows_add_kernel<<<nblk((int64_t)ns * ns), 256, 0, L.st>>>(ns, ns, L.d, TZ, ns, nullptr, 0, 0);
+    launch_chained(scale_rows_add_kernel, nblk((int64_t)ns * ns), 256, 0, L.st, ns, ns, L.d, TZ, ns,
+                   nullptr, 0, 0);
   }
   DLAUNCH(L);
   return rr_tail(L, TZ, Z, ns, nx, nc, C, npn_out, theta, PAP);
@@ -2130,9 +2178,11 @@ int rr_explicit_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
   double* MA = L.A[1];
   int* info = D.ints + 4 * D.nmax + 16;
   int rc;
-  dscale2_kernel<<<nblk((int64_t)ns * ns), 256, 0, L.st>>>(ns, SBS, ns, SAS, ns, d0, MB, MA, ns);
+  launch_chained(dscale2_kernel, nblk((int64_t)ns * ns), 256, 0, L.st, ns, SBS, ns, SAS, ns, d0, MB,
+                 MA, ns);
   DLAUNCH(L);
-  copy_block_cm_kernel<<<nblk((int64_t)o * o), 256, 0, L.st>>>(o, o, MB, ns, R11, o, 1.0);
+  launch_chained(copy_block_cm_kernel, nblk((int64_t)o * o), 256, 0, L.st, o, o, MB, ns, R11, o,
+                 1.0);
   DLAUNCH(L);
   LOB_CUDA_OK(cudaMemsetAsync(info, 0, sizeof(int), L.st));
   if ((rc = dev_chol(L, o, R11, o, info))) return rc;
@@ -2157,7 +2207,8 @@ int rr_explicit_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
   if (nw > 0 && (rc = dev_gemm(L, true, false, o, nw, o, 1.0, Y, o, MB + (int64_t)o * ns, ns, 0.0,
                                nullptr, 0, SB + (int64_t)o * ns, ns, nullptr)))
     return rc;
-  pre_fill_kernel<<<nblk((int64_t)ns * ns), 256, 0, L.st>>>(ns, o, MB, MA, ns, Ka, o, SB, SA, ns);
+  launch_chained(pre_fill_kernel, nblk((int64_t)ns * ns), 256, 0, L.st, ns, o, MB, MA, ns, Ka, o,
+                 SB, SA, ns);
   DLAUNCH(L);
   int npn = 0;
   if ((rc = rr_modified_dev(L, SA, SB, ns, nx, np, nc, false, tau_skip, flip, condR, C, &npn,
@@ -2167,7 +2218,7 @@ int rr_explicit_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
   const int m = nx + npn;
   if ((rc = dev_gemm(L, false, false, o, m, o, 1.0, Y, o, C, ns, 0.0, nullptr, 0, Ka, o, nullptr)))
     return rc;
-  pre_back_kernel<<<nblk((int64_t)ns * m), 256, 0, L.st>>>(ns, m, o, d0, Ka, o, C, ns);
+  launch_chained(pre_back_kernel, nblk((int64_t)ns * m), 256, 0, L.st, ns, m, o, d0, Ka, o, C, ns);
   DLAUNCH(L);
   *npn_out = npn;
   return LOBPCG_OK;
@@ -2182,18 +2233,20 @@ int svqb_transform_dev(DenseLayer& L, const double* G, int nu, bool drop, double
   int* est = D.ints + 2;
   int* keep = D.ints + 3;
   int rc;
-  dscale2_kernel<<<nblk((int64_t)nu * nu), 256, 0, L.st>>>(nu, G, nu, nullptr, 0, L.d, MB, nullptr,
-                                                           nu);
+  launch_chained(dscale2_kernel, nblk((int64_t)nu * nu), 256, 0, L.st, nu, G, nu, nullptr, 0, L.d,
+                 MB, nullptr, nu);
   DLAUNCH(L);
   if ((rc = eig_into(L, nu, MB, Z, est))) return rc;
-  svqb_dev_kernel<<<1, 256, 0, L.st>>>(nu, L.ev, L.d, Z, nu, drop ? 1 : 0, tau, T, nu, keep);
+  launch_chained(svqb_dev_kernel, 1, 256, 0, L.st, nu, L.ev, L.d, Z, nu, drop ? 1 : 0, tau, T, nu,
+                 keep);
   DLAUNCH(L);
   int fl[2];
   if ((rc = read_flags(L, est, 2, nullptr, 0, fl, nullptr))) return rc;
   note_check(L, fl[0]);
   if (fl[0] != 0) {
     if ((rc = eig_recover(L, nu, MB, Z, fl[0]))) return rc;
-    svqb_dev_kernel<<<1, 256, 0, L.st>>>(nu, L.ev, L.d, Z, nu, drop ? 1 : 0, tau, T, nu, keep);
+    launch_chained(svqb_dev_kernel, 1, 256, 0, L.st, nu, L.ev, L.d, Z, nu, drop ? 1 : 0, tau, T, nu,
+                   keep);
     DLAUNCH(L);
     if ((rc = read_flags(L, keep, 1, nullptr, 0, fl + 1, nullptr))) return rc;
   }

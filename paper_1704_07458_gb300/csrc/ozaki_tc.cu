@@ -832,9 +832,9 @@ __global__ void __launch_bounds__(kUThrAll, 1)
 // A warp's 32 lanes are 8 slab lanes x 4 outputs: with one thread per output
 // the two passes over up to 152 slabs are chains of dependent L2 loads on a few
 // warps (p = q = 32: 52 us; 9 us now).
-__global__ void __launch_bounds__(256) gram_tc_reduce_kernel(const int4* __restrict__ partial,
-                                                             int slabs, int p, int q,
-                                                             double* __restrict__ G, int64_t ldg) {
+__global__ void __launch_bounds__(256) gram_tc_reduce_kernel(const int4* partial, int slabs, int p,
+                                                             int q, double* G, int64_t ldg) {
+  chain_wait();
   const int sl = (threadIdx.x & 31) >> 2;
   const int64_t idx =
       ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 4 + (threadIdx.x & 3);
@@ -1554,8 +1554,8 @@ int gram_tc(cudaStream_t st, int64_t n, const SegList& U, const SegList& V, doub
   }
   if (rc) return rc;
   const int64_t total = (int64_t)p * q;
-  gram_tc_reduce_kernel<<<(unsigned)ceil_div(total, 32), 256, 0, st>>>(partial, g.slabs, p, q, G,
-                                                                        ldg);
+  launch_chained(gram_tc_reduce_kernel, (unsigned)ceil_div(total, 32), 256, 0, st, partial,
+                 g.slabs, p, q, G, ldg);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
