@@ -11,175 +11,287 @@
 //               norms of Eq. (9), one pass over X, AX, BX.
 // These run on the FP64 units; the tensor-core versions are in ozaki.cu.
 #include <algorithm>
+#include <type_traits>
 
 #include "colpass.cuh"
 
 namespace lob {
 
 // ---------------------------------------------------------------- Gram (FP64)
+//
+// The FP64 contractions are bound by the FP64 pipe (two FMAs per clock and SM),
+// so what counts is that no FMA is spent on padding and that every SM has a
+// share: 16 x 16 threads hold NI x NJ outputs each, tiles are NI, NJ <= 4 units
+// of 16 rows or columns dealt out evenly (213 columns: 4, 4, 3, 3 units and not
+// 64, 64, 64, 21 columns of a 64-wide tile), and a small contraction is split
+// down to 16 rows a CTA.  With 64 x 64 tiles and 256 rows a CTA the Gram of
+// 1,024 x 30 x 10 took 328 us, 14 times the useful FMAs on 4 SMs.
 
-constexpr int kGT = 64;  // output tile
-constexpr int kGK = 16;  // rows per shared-memory stage
+constexpr int kU16 = 16;       // rows or columns of a tile unit
+constexpr int kTileUnits = 4;  // most units of a tile
+constexpr int kGK = 16;        // contraction length of a shared-memory stage
 
-static void gram_f64_plan(int64_t n, int p, int q, int* slabs, int64_t* rows_per_slab) {
-  const int64_t tiles = ceil_div(p, kGT) * ceil_div(q, kGT);
+// tile t of `tiles` covers units [first, first + count) of `units`
+__host__ __device__ __forceinline__ int unit_at(int t, int units, int tiles) {
+  return (int)((int64_t)t * units / tiles);
+}
+
+// calls f(NI, NJ) with the counts 1 .. 4 as compile-time constants
+template <int NI, typename F>
+__device__ __forceinline__ void with_nj(int nj, F&& f) {
+  using I = std::integral_constant<int, NI>;
+  if (nj == 1) f(I(), std::integral_constant<int, 1>());
+  else if (nj == 2) f(I(), std::integral_constant<int, 2>());
+  else if (nj == 3) f(I(), std::integral_constant<int, 3>());
+  else f(I(), std::integral_constant<int, 4>());
+}
+template <typename F>
+__device__ __forceinline__ void with_units(int ni, int nj, F&& f) {
+  if (ni == 1) with_nj<1>(nj, f);
+  else if (ni == 2) with_nj<2>(nj, f);
+  else if (ni == 3) with_nj<3>(nj, f);
+  else with_nj<4>(nj, f);
+}
+
+struct GramF64Plan {
+  int up, uq, tp, tq;  // units and tiles of p and q
+  int slabs;
+  int64_t rows;  // per slab
+};
+
+// One wave of four CTAs per SM, at least 16 rows each.
+static GramF64Plan gram_f64_plan(int64_t n, int p, int q) {
+  GramF64Plan g;
+  g.up = (int)ceil_div(p, kU16);
+  g.uq = (int)ceil_div(q, kU16);
+  g.tp = (int)ceil_div(g.up, kTileUnits);
+  g.tq = (int)ceil_div(g.uq, kTileUnits);
+  const int64_t tiles = (int64_t)g.tp * g.tq;
   int64_t s = std::max<int64_t>(1, ceil_div(4 * 152, tiles));
-  s = std::min<int64_t>(s, std::max<int64_t>(1, ceil_div(n, 256)));
-  int64_t r = round_up(ceil_div(n, s), kGK);
-  s = std::max<int64_t>(1, ceil_div(n, r));
-  *slabs = (int)s;
-  *rows_per_slab = r;
+  s = std::min<int64_t>(s, std::max<int64_t>(1, ceil_div(n, kGK)));
+  g.rows = round_up(ceil_div(n, s), kGK);
+  g.slabs = (int)std::max<int64_t>(1, ceil_div(n, g.rows));
+  return g;
 }
 
 int64_t gram_f64_workspace(int64_t n, int p, int q) {
-  int slabs;
-  int64_t r;
-  gram_f64_plan(n, p, q, &slabs, &r);
-  return (int64_t)slabs * p * q * (int64_t)sizeof(double);
+  if (p <= 0 || q <= 0) return 0;
+  return (int64_t)gram_f64_plan(n, p, q).slabs * p * q * (int64_t)sizeof(double);
 }
 
-__global__ void __launch_bounds__(256) gram_f64_kernel(int64_t n, SegList U, int p, SegList V,
-                                                       int q, int64_t rows_per_slab,
+__global__ void __launch_bounds__(256) gram_f64_kernel(int64_t n, const __grid_constant__ SegList U,
+                                                       int p, const __grid_constant__ SegList V,
+                                                       int q, GramF64Plan g,
                                                        double* __restrict__ partial) {
-  __shared__ double Us[kGK][kGT + 1];
-  __shared__ double Vs[kGK][kGT + 1];
-  const int tp = blockIdx.x * kGT, tq = blockIdx.y * kGT;
-  const int64_t r0 = (int64_t)blockIdx.z * rows_per_slab;
-  const int64_t r1 = min(n, r0 + rows_per_slab);
+  __shared__ double Us[kGK][kTileUnits * kU16 + 1], Vs[kGK][kTileUnits * kU16 + 1];
+  const int up0 = unit_at(blockIdx.x, g.up, g.tp), uq0 = unit_at(blockIdx.y, g.uq, g.tq);
+  const int tp = up0 * kU16, tq = uq0 * kU16;
+  const int64_t r0 = (int64_t)blockIdx.z * g.rows, r1 = min(n, r0 + g.rows);
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double acc[4][4];
+  auto tile = [&](auto NIc, auto NJc) {
+    constexpr int NI = decltype(NIc)::value, NJ = decltype(NJc)::value;
+    // this thread loads row ty of a stage, columns tx + 16 i
+    const double *pu[NI], *pv[NJ];
+    int64_t ldu[NI], ldv[NJ];
+    auto column = [&](const SegList& S, int c, int cols, const double** ptr, int64_t* ld) {
+      if (c >= cols) {
+        *ptr = nullptr;
+        *ld = 0;
+        return;
+      }
+      int k = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+      for (int t = 1; t < kMaxSeg; ++t) k += (t < S.nseg && c >= S.off[t]) ? 1 : 0;
+      *ld = S.ld[k];
+      *ptr = S.ptr[k] + (c - S.off[k]) + (r0 + ty) * S.ld[k];
+    };
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  for (int64_t r = r0; r < r1; r += kGK) {
-    for (int e = threadIdx.x; e < kGK * kGT; e += blockDim.x) {
-      const int rr = e / kGT, cc = e % kGT;
-      const int64_t row = r + rr;
-      const bool ok = row < r1;
-      Us[rr][cc] = (ok && tp + cc < p) ? seg_load(U, tp + cc, row) : 0.0;
-      Vs[rr][cc] = (ok && tq + cc < q) ? seg_load(V, tq + cc, row) : 0.0;
-    }
-    __syncthreads();
+    for (int i = 0; i < NI; ++i) column(U, tp + tx + 16 * i, p, &pu[i], &ldu[i]);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) column(V, tq + tx + 16 * j, q, &pv[j], &ldv[j]);
+    double ru[NI], rv[NJ];
+    auto fetch = [&](int64_t r) {  // rows r .. r + 15 of the slab
+      const bool in = r + ty < r1;
+#pragma unroll
+      for (int i = 0; i < NI; ++i) ru[i] = in && pu[i] ? __ldg(pu[i] + (r - r0) * ldu[i]) : 0.0;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) rv[j] = in && pv[j] ? __ldg(pv[j] + (r - r0) * ldv[j]) : 0.0;
+    };
+    double acc[NI][NJ];
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) acc[i][j] = 0.0;
+    fetch(r0);
+    for (int64_t r = r0; r < r1; r += kGK) {
+#pragma unroll
+      for (int i = 0; i < NI; ++i) Us[ty][tx + 16 * i] = ru[i];
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) Vs[ty][tx + 16 * j] = rv[j];
+      __syncthreads();
+      if (r + kGK < r1) fetch(r + kGK);
 #pragma unroll 4
-    for (int k = 0; k < kGK; ++k) {
-      double a[4], b[4];
+      for (int k = 0; k < kGK; ++k) {
+        double a[NI], b[NJ];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = Us[k][ty + 16 * i];
+        for (int i = 0; i < NI; ++i) a[i] = Us[k][ty + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Vs[k][tx + 16 * j];
+        for (int j = 0; j < NJ; ++j) b[j] = Vs[k][tx + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < NI; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+          for (int j = 0; j < NJ; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      }
+      __syncthreads();
     }
-    __syncthreads();
-  }
-  double* out = partial + (int64_t)blockIdx.z * p * q;
+    double* out = partial + (int64_t)blockIdx.z * p * q;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < NI; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gi = tp + ty + 16 * i, gj = tq + tx + 16 * j;
-      if (gi < p && gj < q) out[(int64_t)gi * q + gj] = acc[i][j];
-    }
+      for (int j = 0; j < NJ; ++j) {
+        const int gi = tp + ty + 16 * i, gj = tq + tx + 16 * j;
+        if (gi < p && gj < q) out[(int64_t)gi * q + gj] = acc[i][j];
+      }
+  };
+  with_units(unit_at(blockIdx.x + 1, g.up, g.tp) - up0, unit_at(blockIdx.y + 1, g.uq, g.tq) - uq0,
+             tile);
 }
 
-__global__ void slab_reduce_kernel(const double* __restrict__ partial, int slabs, int p, int q,
-                                   double* __restrict__ G, int64_t ldg) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)p * q) return;
+// G(i, j) = fixed-order sum over the slabs, 8 lanes per output (a chain of up to
+// 608 dependent loads otherwise)
+__global__ void __launch_bounds__(256) slab_reduce_kernel(const double* partial, int slabs, int p,
+                                                          int q, double* G, int64_t ldg) {
+  chain_wait();
+  __shared__ double red[8][32];
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const int64_t e = (int64_t)blockIdx.x * 32 + tx, pq = (int64_t)p * q;
   double s = 0.0;
-  for (int z = 0; z < slabs; ++z) s += partial[(int64_t)z * p * q + e];
-  const int i = (int)(e / q), j = (int)(e % q);
-  G[i + (int64_t)j * ldg] = s;
+  if (e < pq)
+#pragma unroll 4
+    for (int z = ty; z < slabs; z += 8) s += partial[z * pq + e];
+  red[ty][tx] = s;
+  __syncthreads();
+  if (ty != 0 || e >= pq) return;
+  for (int t = 1; t < 8; ++t) s += red[t][tx];
+  G[(int)(e / q) + (int64_t)(e % q) * ldg] = s;
 }
 
 int gram_f64(cudaStream_t st, int64_t n, const SegList& U, const SegList& V, double* G,
              int64_t ldg, void* work, int64_t work_bytes) {
   const int p = U.off[U.nseg], q = V.off[V.nseg];
   if (p <= 0 || q <= 0) return LOBPCG_OK;
-  int slabs;
-  int64_t rps;
-  gram_f64_plan(std::max<int64_t>(n, 1), p, q, &slabs, &rps);
+  const GramF64Plan g = gram_f64_plan(std::max<int64_t>(n, 1), p, q);
+  int slabs = g.slabs;
   if (work_bytes < (int64_t)slabs * p * q * (int64_t)sizeof(double)) return LOBPCG_ERR_ARG;
   double* partial = (double*)work;
   if (n > 0) {
-    dim3 grid((unsigned)ceil_div(p, kGT), (unsigned)ceil_div(q, kGT), (unsigned)slabs);
-    gram_f64_kernel<<<grid, 256, 0, st>>>(n, U, p, V, q, rps, partial);
+    dim3 grid((unsigned)g.tp, (unsigned)g.tq, (unsigned)slabs);
+    gram_f64_kernel<<<grid, 256, 0, st>>>(n, U, p, V, q, g, partial);
     LOB_LAUNCHED();
   } else {
     slabs = 1;
     LOB_CUDA_OK(cudaMemsetAsync(partial, 0, (size_t)p * q * sizeof(double), st));
   }
   const int64_t tot = (int64_t)p * q;
-  slab_reduce_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, st>>>(partial, slabs, p, q, G, ldg);
+  launch_chained(slab_reduce_kernel, (unsigned)ceil_div(tot, 32), 256, 0, st, partial, slabs, p, q,
+                 G, ldg);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }
 
 // -------------------------------------------------------------- update (FP64)
 
-constexpr int kUT = 64;  // rows and output columns per tile
-constexpr int kUK = 16;  // contraction stage
-
-__global__ void __launch_bounds__(256) update_f64_kernel(int64_t n, SegList S, int s,
+// Tiles of NI x 16 rows (NI a launch constant) by up to four units of 16 output
+// columns; stages of 16 of the s contraction columns, the next one's loads in
+// flight.
+template <int NI>
+__global__ void __launch_bounds__(256) update_f64_kernel(int64_t n, const __grid_constant__ SegList S, int s,
                                                          const double* __restrict__ C,
                                                          int64_t ldc, int m, double alpha,
-                                                         double beta, SegList Y0, OutList Y) {
-  __shared__ double Ss[kUT][kUK + 1];
-  __shared__ double Cs[kUK][kUT + 1];
-  const int64_t r0 = (int64_t)blockIdx.x * kUT;
-  const int c0 = blockIdx.y * kUT;
+                                                         double beta, const __grid_constant__ SegList Y0,
+                                                         const __grid_constant__ OutList Y,
+                                                         int units, int tiles) {
+  __shared__ double Ss[NI * kU16][kGK + 1], Cs[kGK][kTileUnits * kU16 + 1];
+  const int64_t r0 = (int64_t)blockIdx.x * (NI * kU16);
+  const int u0 = unit_at(blockIdx.y, units, tiles), c0 = u0 * kU16;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double acc[4][4];
+  auto tile = [&](auto, auto NJc) {
+    constexpr int NJ = decltype(NJc)::value;
+    double rs[NI], rc[NJ];
+    auto fetch = [&](int k0) {  // column k0 + tx of S and row k0 + tx of C
+      const bool in = k0 + tx < s;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  for (int k0 = 0; k0 < s; k0 += kUK) {
-    for (int e = threadIdx.x; e < kUT * kUK; e += blockDim.x) {
-      const int rr = e / kUK, kk = e % kUK;
-      const int64_t row = r0 + rr;
-      Ss[rr][kk] = (row < n && k0 + kk < s) ? seg_load(S, k0 + kk, row) : 0.0;
-      const int kc = e / kUT, cc = e % kUT;
-      Cs[kc][cc] = (k0 + kc < s && c0 + cc < m) ? C[(k0 + kc) + (int64_t)(c0 + cc) * ldc] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < kUK; ++k) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = Ss[ty + 16 * i][k];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Cs[k][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t row = r0 + ty + 16 * i;
-      const int c = c0 + tx + 16 * j;
-      if (row < n && c < m) {
-        double v = alpha * acc[i][j];
-        if (beta != 0.0) v = fma(beta, seg_load(Y0, c, row), v);
-        *out_addr(Y, c, row) = v;
+      for (int i = 0; i < NI; ++i) {
+        const int64_t row = r0 + ty + 16 * i;
+        rs[i] = in && row < n ? seg_load(S, k0 + tx, row) : 0.0;
       }
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const int c = c0 + ty + 16 * j;
+        rc[j] = in && c < m ? C[(k0 + tx) + (int64_t)c * ldc] : 0.0;
+      }
+    };
+    double acc[NI][NJ];
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) acc[i][j] = 0.0;
+    fetch(0);
+    for (int k0 = 0; k0 < s; k0 += kGK) {
+#pragma unroll
+      for (int i = 0; i < NI; ++i) Ss[ty + 16 * i][tx] = rs[i];
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) Cs[tx][ty + 16 * j] = rc[j];
+      __syncthreads();
+      if (k0 + kGK < s) fetch(k0 + kGK);
+      const int left = min(kGK, s - k0);
+#pragma unroll 4
+      for (int k = 0; k < left; ++k) {
+        double a[NI], b[NJ];
+#pragma unroll
+        for (int i = 0; i < NI; ++i) a[i] = Ss[ty + 16 * i][k];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) b[j] = Cs[k][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      }
+      __syncthreads();
     }
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const int64_t row = r0 + ty + 16 * i;
+        const int c = c0 + tx + 16 * j;
+        if (row < n && c < m) {
+          double v = alpha * acc[i][j];
+          if (beta != 0.0) v = fma(beta, seg_load(Y0, c, row), v);
+          *out_addr(Y, c, row) = v;
+        }
+      }
+  };
+  with_nj<NI>(unit_at(blockIdx.y + 1, units, tiles) - u0, tile);
 }
 
 int update_f64(cudaStream_t st, int64_t n, const SegList& S, const double* C, int64_t ldc,
                int m, double alpha, double beta, const SegList& Y0, const OutList& Y) {
   const int s = S.off[S.nseg];
   if (n <= 0 || m <= 0) return LOBPCG_OK;
-  dim3 grid((unsigned)ceil_div(n, kUT), (unsigned)ceil_div(m, kUT));
-  update_f64_kernel<<<grid, 256, 0, st>>>(n, S, s, C, ldc, m, alpha, beta, Y0, Y);
+  const int units = (int)ceil_div(m, kU16);
+  // 64-row tiles of up to four units when they give every SM four CTAs, 16-row
+  // tiles of one unit when not
+  int tiles = (int)ceil_div(units, kTileUnits);
+  const bool small = ceil_div(n, 4 * kU16) * tiles < 4 * 152;
+  if (small) tiles = units;
+  const dim3 grid((unsigned)ceil_div(n, (small ? 1 : 4) * kU16), (unsigned)tiles);
+  if (small)
+    update_f64_kernel<1><<<grid, 256, 0, st>>>(n, S, s, C, ldc, m, alpha, beta, Y0, Y, units,
+                                               tiles);
+  else
+    update_f64_kernel<4><<<grid, 256, 0, st>>>(n, S, s, C, ldc, m, alpha, beta, Y0, Y, units,
+                                               tiles);
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }

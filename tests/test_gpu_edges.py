@@ -127,6 +127,26 @@ def test_update_tc_edges(n, s, m, slices, scale, beta):
     np.testing.assert_array_equal(host(Y, m)[0], beta * Y0[0])
 
 
+# the FP64 forms: unequal tiles of 16-wide units, one unit, 16-row slabs and
+# stages with a remainder; the update's 64-row (many rows) and 16-row tiles
+@pytest.mark.parametrize("n,s,m", [(1, 1, 1), (17, 15, 16), (1024, 30, 10), (1000, 81, 65),
+                                   (609, 213, 142), (20001, 33, 130), (39000, 17, 16)])
+def test_fp64_contraction_tiles(n, s, m):
+    torch = torch_cuda()
+    S, C = synth.normal_block(5, 1, n, s), synth.normal_block(6, 1, s, m)
+    V = synth.normal_block(7, 1, n, m)
+    Sd, Vd = dev(S, s + 1), dev(V, m + 3)
+    Y, G = dev(np.full((n, m), np.nan), m + 1), dev(np.full(s * m, np.nan))
+    assert gb.lobpcg_update(n, Sd, s + 1, s, dev(C.T.copy().reshape(-1)), s, m, -1.5, 0.5, Vd,
+                            m + 3, Y, m + 1, gb.LOBPCG_GEMM_F64, 0) == 0
+    assert gb.lobpcg_gram(n, Sd, s + 1, s, Vd, m + 3, m, G, s, gb.LOBPCG_GEMM_F64, 0) == 0
+    torch.cuda.synchronize()
+    bound = 2 * gamma(s + 2) * (1.5 * np.abs(S) @ np.abs(C) + 0.5 * np.abs(V))
+    assert np.all(np.abs(host(Y, m) - (0.5 * V - 1.5 * (S @ C))) <= bound)
+    got = host(G).reshape(m, s).T
+    assert np.all(np.abs(got - S.T @ V) <= 2 * gamma(n) * (np.abs(S).T @ np.abs(V)))
+
+
 # fewer rows than a CTA's row lanes, one column, several column tiles (128)
 @pytest.mark.parametrize("n,m,c0", [(2, 128, 0), (7, 129, 0), (700, 282, 25), (700, 1, 0),
                                     (4097, 257, 256)])
