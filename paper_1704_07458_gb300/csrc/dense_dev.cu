@@ -142,14 +142,14 @@ __global__ void __launch_bounds__(256) chol64_kernel(int n, double* A, int lda, 
   if (t == 0) s_fail = 0;
   __syncthreads();
   for (int j = 0; j < n; ++j) {
-    if (t == 0) {  // one square root and one division per step
+    if (t == 0) {
       const double piv = sa[j + j * n];
-      if (!(piv > 0.0) || !isfinite(piv)) {
+      if (!(piv > 0.0) || !isfinite(piv))
         s_fail = j + 1;
-      } else {
+      else
         s_r = sqrt(piv);
-        s_inv = 1.0 / s_r;
-      }
+    } else if (t == 32) {  // beside the root, not after it
+      s_inv = rsqrt(sa[j + j * n]);
     }
     __syncthreads();
     if (s_fail) break;
@@ -188,20 +188,26 @@ __global__ void __launch_bounds__(256) trinv64_kernel(int n, const double* R, in
   __syncthreads();
   // eight lanes per column c share its dot product (a shuffle reduction), so
   // a row costs (n - i) / 8 dependent steps instead of n - i
+  // (a warp without a column left takes no part: its shuffled sums of zeros would
+  // occupy the FP64 pipe all the same; order 27: 60 -> 24 us)
   const int sub = t & 7, grp = t >> 3, ngrp = (int)blockDim.x >> 3;
   for (int i = n - 1; i >= 0; --i) {
     const double inv = dinv[i];
     double val[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
     for (int h = 0; h < 5; ++h) {
+      if (i + 4 * warp + h * ngrp >= n) break;
       const int c = i + grp + h * ngrp;  // uniform within each group of 8 lanes
       double sacc = 0.0;
       if (c < n && c > i)
-        for (int kk = i + 1 + sub; kk <= c; kk += 8) sacc = fma(sm[i + kk * n], sm[kk + c * n], sacc);
+        for (int kk = i + 1 + sub; kk <= c; kk += 8)
+          sacc = fma(sm[i + kk * n], sm[kk + c * n], sacc);
       for (int o = 4; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
       val[h] = c == i ? inv : -sacc * inv;
     }
     __syncthreads();
     if (sub == 0)
+#pragma unroll
       for (int h = 0; h < 5; ++h) {
         const int c = i + grp + h * ngrp;
         if (c < n) sm[i + c * n] = val[h];
