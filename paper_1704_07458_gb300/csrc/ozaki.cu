@@ -383,7 +383,7 @@ __global__ void split_c_kernel(const double* __restrict__ C, int64_t ldc, int s,
 // for 8 bytes and fills 213 CTAs (349 us at n = 262,144, s = 213; 78 us now).
 constexpr int kCxZero = -2139062144;  // 0x80808080, the memset pattern
 
-__global__ void __launch_bounds__(256) colexp_rows_kernel(int64_t n, SegList Sg, int s,
+__global__ void __launch_bounds__(256) colexp_rows_kernel(int64_t n, const __grid_constant__ SegList Sg, int s,
                                                           int* __restrict__ colexp) {
   __shared__ int red[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

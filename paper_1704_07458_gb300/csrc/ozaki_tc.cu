@@ -500,8 +500,10 @@ size_t gram_smem_bytes(int NT) {
 // 1,024 warps in all: 33 us a launch, two of them); the columns of U, then those
 // of V; high words only.
 template <int R>
-__global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n, SegList U, int p, SegList V,
-                                                            int q, int* __restrict__ EU,
+__global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n,
+                                                            const __grid_constant__ SegList U, int p,
+                                                            const __grid_constant__ SegList V, int q,
+                                                            int* __restrict__ EU,
                                                             int* __restrict__ EV) {
   __shared__ int red[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -992,32 +994,50 @@ struct UpdShared {
 };
 
 // ER[i] = exponent bound of row i of the balanced S(i, k) 2^-colexp[k] over all
-// k (kEZero for a zero row).  One warp per row, lanes over the columns of each
-// segment in turn (plain pointer arithmetic within a segment).
-__global__ void row_exp_kernel(int64_t n, SegList Sg, int s, const int* __restrict__ colexp,
-                               int* __restrict__ ER) {
+// k (kEZero for a zero row).  A warp takes kErRows rows at a time, lanes over the
+// columns of each segment in turn (plain pointer arithmetic within a segment),
+// the rows' loads all in flight: with one row per warp a pass over 262,144 x 32
+// took 31 us against 10 us of bytes.
+constexpr int kErRows = 4;
+__global__ void __launch_bounds__(256) row_exp_kernel(int64_t n,
+                                                      const __grid_constant__ SegList Sg, int s,
+                                                      const int* __restrict__ colexp,
+                                                      int* __restrict__ ER) {
   const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int64_t row = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kErRows;
   if (row >= n) return;
-  int e = -1000000;
+  int e[kErRows];
+#pragma unroll
+  for (int i = 0; i < kErRows; ++i) e[i] = -1000000;
 #pragma unroll
   for (int g = 0; g < kMaxSeg; ++g) {
     if (g >= Sg.nseg) break;
     const int c0 = Sg.off[g], w = Sg.off[g + 1] - c0;
-    const double* base = Sg.ptr[g] + row * Sg.ld[g];
-    for (int c = lane; c < w; c += 64) {  // two loads in flight per lane
+    const int64_t ld = Sg.ld[g];
+    const double* base = Sg.ptr[g] + row * ld;
+    for (int c = lane; c < w; c += 64) {  // two columns of every row in flight
       const bool two = c + 32 < w;
-      const long long b0 = __double_as_longlong(__ldg(base + c));
-      const long long b1 = two ? __double_as_longlong(__ldg(base + c + 32)) : 0LL;
+      long long b0[kErRows], b1[kErRows];
+#pragma unroll
+      for (int i = 0; i < kErRows; ++i) {
+        const bool in = row + i < n;
+        b0[i] = in ? __double_as_longlong(__ldg(base + i * ld + c)) : 0LL;
+        b1[i] = in && two ? __double_as_longlong(__ldg(base + i * ld + c + 32)) : 0LL;
+      }
       const int x0 = colexp ? __ldg(colexp + c0 + c) : 0;
       const int x1 = (colexp && two) ? __ldg(colexp + c0 + c + 32) : 0;
-      if ((b0 << 1) != 0) e = max(e, max((int)((b0 >> 52) & 0x7FF), 1) - x0);
-      if ((b1 << 1) != 0) e = max(e, max((int)((b1 >> 52) & 0x7FF), 1) - x1);
+#pragma unroll
+      for (int i = 0; i < kErRows; ++i) {
+        if ((b0[i] << 1) != 0) e[i] = max(e[i], max((int)((b0[i] >> 52) & 0x7FF), 1) - x0);
+        if ((b1[i] << 1) != 0) e[i] = max(e[i], max((int)((b1[i] >> 52) & 0x7FF), 1) - x1);
+      }
     }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-  if (lane == 0) ER[row] = e > -1000000 ? e - 1022 : kEZero;
+  for (int i = 0; i < kErRows; ++i) {
+    const int m = __reduce_max_sync(0xffffffffu, e[i]);
+    if (lane == 0 && row + i < n) ER[row + i] = m > -1000000 ? m - 1022 : kEZero;
+  }
 }
 
 template <int S>
@@ -1224,11 +1244,35 @@ __global__ void __launch_bounds__(kUThrAll, 1)
     auto drain_outputs = [&]() {
       while (ou < W) out_steps(std::integral_constant<int, 2>());
     };
+    // outputs are formed a few steps after each chunk, spread over the chunks of
+    // the next tile, so that the tensor core never waits for them
+    const int own = max(1, min(nch, kChunksPerBlock) / 2);
+    const bool spread3 = W <= 3 * own;  // three steps a chunk are enough
+    // With Y0 (s <= 256) a tile's outputs are formed at once, eight a thread with
+    // their Y0 in flight together, the first eight since before the wait for the
+    // MMAs: steps of two or three waited for Y0 each time (n = 262,144: 204 ->
+    // 153 us at 32 x 32, 268 -> 235 at 96 x 32, 933 -> 744 at 213 x 142).
+    constexpr int kNow = 8;
+    constexpr bool kNowY0 = kOneBlock && kY0;
+    double y0[kNow];
+    auto load_y0 = [&](int b) {
+      const int64_t row0 = (int64_t)(pt / ntiles) * TCM + 32 * q;
+      const int col = (pt % ntiles) * NT + W * grp;
+      const double* yb = Y0.ptr[0] + row0 * Y0.ld[0] + col;
+#pragma unroll
+      for (int u = 0; u < kNow; ++u) {
+        const unsigned idx = 32u * (b + u) + lane;
+        const int r = (int)((idx * inv) >> 16), j = (int)idx - r * W;
+        y0[u] = r < 32 && row0 + r < n && col + j < m ? yb[r * Y0.ld[0] + j] : 0.0;
+      }
+    };
     // accumulators -> int64 sums in this warp's slots; the tensor core has TMEM
     // back before the outputs are formed
     auto flush = [&]() -> bool {
       drain_outputs();  // the previous tile's outputs leave the slots
       __syncwarp();
+      const bool now = kNowY0 && Y0.nseg == 1;
+      if (now) load_y0(0);
       if (!__all_sync(0xffffffffu, wait_or_fail(smem_u32(&sh.accfull), pphase, &sh.fail)))
         return false;
       asm volatile("tcgen05.fence::after_thread_sync;\n");
@@ -1270,16 +1314,32 @@ __global__ void __launch_bounds__(kUThrAll, 1)
           fin.row0 = row0;
         }
         __syncwarp();
+        if (now) {
+          for (int b = 0; b < W; b += kNow) {
+            if (b > 0) load_y0(b);
+#pragma unroll
+            for (int u = 0; u < kNow; ++u) {
+              const unsigned idx = 32u * (b + u) + lane;
+              const int r = (int)((idx * inv) >> 16), j = (int)idx - r * W;
+              const int er = __shfl_sync(0xffffffffu, oerow, r & 31);
+              if (r < onrow && ocol + j < m) {
+                const double v =
+                    i64_scaled(slots[r * kUPitch + j], er + __ldg(Ce + ocol + j)) + y0[u];
+                if (ybase)
+                  ybase[(int64_t)r * oyld + j] = v;
+                else
+                  *out_addr(Y, ocol + j, fin.row0 + r) = v;
+              }
+            }
+          }
+          ou = W;
+        }
         pblk = 0;
         pt += tstep;
       }
       pend += min(kChunksPerBlock, nch - pblk * kChunksPerBlock);
       return true;
     };
-    // outputs are formed a few steps after each chunk, spread over the chunks of
-    // the next tile, so that the tensor core never waits for them
-    const int own = max(1, min(nch, kChunksPerBlock) / 2);
-    const bool spread3 = W <= 3 * own;  // three steps a chunk are enough
 
     for (;;) {
       const bool more = g < my_chunks;
@@ -1449,7 +1509,7 @@ int update_tc_launch(cudaStream_t st, int64_t n, const SegList& Sg, int s, const
     if (rc) return rc;
     colexp = cxw;
   }
-  row_exp_kernel<<<(unsigned)ceil_div(n, 8), 256, 0, st>>>(n, Sg, s, colexp, ER);
+  row_exp_kernel<<<(unsigned)ceil_div(n, 8 * kErRows), 256, 0, st>>>(n, Sg, s, colexp, ER);
   LOB_LAUNCHED();
   {
     const int64_t warps = (int64_t)ntiles * NT;
