@@ -497,8 +497,10 @@ size_t gram_smem_bytes(int NT) {
 // exponent maximum (at least 1) minus 1022.  One CTA per (block, 32 columns),
 // lanes over columns, the block's 8 R rows dealt to its eight warps and all in
 // flight at once (with a warp per block a 32-column Gram of 262,144 rows had
-// 1,024 warps in all: 33 us a launch, two of them); the columns of U, then those
-// of V; high words only.
+// 1,024 warps in all: 33 us a launch, two of them; 21 us for both now); the columns
+// of U, then those of V; high words only.  __grid_constant__: indexed by segment, a
+// plain parameter is copied to the stack by every thread (Gram 262,144 x 213 x 142
+// 709 -> 666 us).
 template <int R>
 __global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n,
                                                             const __grid_constant__ SegList U, int p,
@@ -997,7 +999,7 @@ struct UpdShared {
 // k (kEZero for a zero row).  A warp takes kErRows rows at a time, lanes over the
 // columns of each segment in turn (plain pointer arithmetic within a segment),
 // the rows' loads all in flight: with one row per warp a pass over 262,144 x 32
-// took 31 us against 10 us of bytes.
+// took 31 us against 10 us of bytes (18 us now, cold).
 constexpr int kErRows = 4;
 __global__ void __launch_bounds__(256) row_exp_kernel(int64_t n,
                                                       const __grid_constant__ SegList Sg, int s,
