@@ -20,9 +20,9 @@ constexpr int kDevDenseMax = 256;
 struct DevDense {
   int nmax = 0;
   std::vector<void*> bufs;
-  double *X = nullptr, *X1 = nullptr, *E = nullptr, *Zt = nullptr;  // nmax x nmax
+  double *X = nullptr, *E = nullptr, *Zt = nullptr;  // nmax x nmax
   double *T1 = nullptr, *T2 = nullptr, *T3 = nullptr, *T4 = nullptr;
-  double *XA = nullptr, *GS = nullptr;  // nmax x 2 nmax: [X | A X], [G | S]
+  double *XA = nullptr, *XB = nullptr, *GS = nullptr;  // nmax x 2 nmax: [X | A X] twice, [G | S]
   float *V32 = nullptr, *Y32 = nullptr;  // nmax x nmax FP32
   float* f32v = nullptr;                 // 4 nmax FP32 vectors
   double* vec = nullptr;                 // 8 nmax
@@ -122,11 +122,12 @@ int small_stats(DenseLayer& L, const double* G, int rows, int cols, int ldg, boo
 
 // ---- device-resident path (dense_dev.cu)
 // C = alpha op(A) op(B) + beta Cin, column-major, m, n <= 2 * the layer's
-// order; skip: device flag, the launch is a no-op when it is non-zero; sym: see
-// gemm64_kernel.
+// order; skip: device flag, the launch is a no-op when it is non-zero; sym, next
+// and emax: see gemm64_kernel.
 int dev_gemm(DenseLayer& L, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
              int lda, const double* B, int ldb, double beta, const double* Cin, int ldcin,
-             double* C, int ldc, const int* skip, int sym = 0);
+             double* C, int ldc, const int* skip, int sym = 0, int* next = nullptr,
+             const unsigned long long* emax = nullptr);
 int dev_chol(DenseLayer& L, int n, double* A, int lda, int* info);
 int dev_trinv(DenseLayer& L, int n, const double* R, int ldr, double* X, int ldx, const int* skip);
 int dev_syev(DenseLayer& L, int n, const double* A, int lda, double* Z, int ldz, double* w,
