@@ -1340,37 +1340,37 @@ __global__ void assemble_h_kernel(int ns, int o, const double* MA, int ldm,
 // cond(R) of R = [[I, F], [0, Rw]] (o + nw = ns; o = 0: R = Rw) from 8 power
 // iterations on M = R^T R = MB and 8 on R^-1 R^-T = MB^-1, with R^-1 =
 // [[I, Yt], [0, Yw]] given by its last nw columns Y (ns x nw); FP32 in shared
-// memory (the value feeds an order-of-magnitude test).  out[0] = cond(R),
-// inf when a factor is non-finite; skip: no-op when *skip != 0 (then out[0]
-// is set to inf).
+// memory (the value feeds an order-of-magnitude test).  One CTA for each of the
+// two, side by side: out[0] and out[1] are the largest eigenvalues of M and
+// M^-1, cond(R) = sqrt(out[0] out[1]) (cond_of); inf when non-finite, or when
+// *skip != 0.  A chain of barriers: 49 us at ns = 81 with one CTA for
+// both (32 x 32 solve 26.9 -> 24.8 ms, 48 x 40 x 36 solve 124.6 -> 119.8 ms).
 __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, const double* MB,
                                                               int ldm, const double* Y,
                                                               int ldy, double* out, const int* skip) {
   chain_wait();
+  const int which = blockIdx.x;
   if (skip && *skip) {
-    if (threadIdx.x == 0) out[0] = INFINITY;
+    if (threadIdx.x == 0) out[which] = INFINITY;
     return;
   }
   extern __shared__ float cs[];
   const int nw = ns - o;
-  float* F = cs;               // o x nw   (MB[0:o, o:])
-  float* Bw = F + o * nw;      // nw x nw  (MB[o:, o:])
-  float* Yt = Bw + nw * nw;    // o x nw
-  float* Yw = Yt + o * nw;     // nw x nw
-  float* x = Yw + nw * nw;     // ns
+  float* F = cs;               // o x nw: MB[0:o, o:], or Yt
+  float* Bw = F + o * nw;      // nw x nw: MB[o:, o:], or Yw
+  const float *Yt = F, *Yw = Bw;
+  float* x = Bw + nw * nw;     // ns
   float* y = x + ns;           // ns
   float* z = y + ns;           // ns
   __shared__ float red[3][32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   for (int e = t; e < o * nw; e += blockDim.x) {
     const int i = e % o, j = e / o;
-    F[e] = (float)MB[i + (int64_t)(o + j) * ldm];
-    Yt[e] = (float)Y[i + (int64_t)j * ldy];
+    F[e] = (float)(which ? Y[i + (int64_t)j * ldy] : MB[i + (int64_t)(o + j) * ldm]);
   }
   for (int e = t; e < nw * nw; e += blockDim.x) {
     const int i = e % nw, j = e / nw;
-    Bw[e] = (float)MB[(o + i) + (int64_t)(o + j) * ldm];
-    Yw[e] = (float)Y[(o + i) + (int64_t)j * ldy];
+    Bw[e] = (float)(which ? Y[(o + i) + (int64_t)j * ldy] : MB[(o + i) + (int64_t)(o + j) * ldm]);
   }
   __syncthreads();
   auto sum3 = [&](float a, float b, float c, float& ra, float& rb, float& rc) {
@@ -1386,7 +1386,8 @@ __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, con
     }
     __syncthreads();
     ra = rb = rc = 0.f;
-    for (int w = 0; w < 32; ++w) {
+    const int nwarps = (ns + 31) / 32;  // the others hold zeros
+    for (int w = 0; w < nwarps; ++w) {
       ra += red[0][w];
       rb += red[1][w];
       rc += red[2][w];
@@ -1448,7 +1449,7 @@ __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, con
       return s;
     }, res);
   };
-  auto power = [&](int which) -> float {
+  auto power = [&]() -> float {
     for (int i = t; i < ns; i += blockDim.x) x[i] = 1.0f + 0.001f * (float)(i % 7);
     __syncthreads();
     float lam = 0.f;
@@ -1477,12 +1478,8 @@ __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, con
     }
     return lam;
   };
-  const float lmax = power(0);
-  const float imax = power(1);
-  if (t == 0)
-    out[0] = (isfinite(lmax) && isfinite(imax) && lmax > 0.f && imax > 0.f)
-                 ? sqrt((double)lmax * (double)imax)
-                 : INFINITY;
+  const float lmax = power();
+  if (t == 0) out[which] = isfinite(lmax) && lmax > 0.f ? (double)lmax : INFINITY;
 }
 
 // Q2(i, j) = th[i] * Q(i, j)
@@ -1899,6 +1896,11 @@ int read_flags(DenseLayer& L, const int* ints, int n_ints, const double* dbl, in
   return LOBPCG_OK;
 }
 
+// cond(R) from the two results of cond_struct_kernel
+double cond_of(const double* cr) {
+  return std::isfinite(cr[0]) && std::isfinite(cr[1]) ? std::sqrt(cr[0] * cr[1]) : INFINITY;
+}
+
 // count the reasons of a failed check of the device eigensolver
 void note_check(DenseLayer& L, int mask) {
   if (mask & 1) ++L.check_fail[0];
@@ -2008,7 +2010,7 @@ int rr_initial_dev(DenseLayer& L, const double* GA, const double* GB, int nx, do
   DLAUNCH(L);
   if ((rc = dev_chol(L, nx, Rf, nx, info))) return rc;
   if ((rc = dev_trinv(L, nx, Rf, nx, Ri, nx, info))) return rc;
-  launch_chained(cond_struct_kernel, 1, 1024, (size_t)(2 * nx * nx + 3 * nx) * 4, L.st, nx, 0, MB,
+  launch_chained(cond_struct_kernel, 2, 1024, (size_t)(nx * nx + 3 * nx) * 4, L.st, nx, 0, MB,
                  nx, Ri, nx, cr, info);
   DLAUNCH(L);
   // H = Ri^T MA Ri
@@ -2018,8 +2020,9 @@ int rr_initial_dev(DenseLayer& L, const double* GA, const double* GB, int nx, do
     return rc;
   if ((rc = eig_into(L, nx, H, Z, est))) return rc;
   int fl[2];
-  double condR;
-  if ((rc = read_flags(L, info, 2, cr, 1, fl, &condR))) return rc;
+  double crh[2];
+  if ((rc = read_flags(L, info, 2, cr, 2, fl, crh))) return rc;
+  const double condR = cond_of(crh);
   // breakdown: Cholesky failed or D X0^T B X0 D = R^T R is numerically
   // singular, cond(R)^2 >= 1 / (n_x eps)
   if (fl[0] != 0 || !(condR * condR < 1.0 / (nx * kEps64))) {
@@ -2091,7 +2094,7 @@ int rr_modified_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
     if ((rc = dev_gemm(L, false, false, o, nw, nw, -1.0, F, ns, Y + o, ns, 0.0, nullptr, 0, Y, ns,
                        info)))
       return rc;
-    launch_chained(cond_struct_kernel, 1, 1024, (size_t)(2 * o * nw + 2 * nw * nw + 3 * ns) * 4,
+    launch_chained(cond_struct_kernel, 2, 1024, (size_t)(o * nw + nw * nw + 3 * ns) * 4,
                    L.st, ns, o, MB, ns, Y, ns, cr, info);
     DLAUNCH(L);
     if ((rc = dev_gemm(L, false, false, ns, nw, ns, 1.0, MA, ns, Y, ns, 0.0, nullptr, 0, Qm, ns,
@@ -2105,13 +2108,13 @@ int rr_modified_dev(DenseLayer& L, const double* SAS, const double* SBS, int ns,
       return rc;
     Hsrc = H;
   } else {
-    LOB_CUDA_OK(cudaMemsetAsync(cr, 0, sizeof(double), L.st));  // cond(I) = 1, set below
+    LOB_CUDA_OK(cudaMemsetAsync(cr, 0, 2 * sizeof(double), L.st));  // cond(I) = 1, set below
   }
   if ((rc = eig_into(L, ns, Hsrc, Z, est))) return rc;
   int fl[2];
-  double c = 1.0;
-  if ((rc = read_flags(L, info, 2, cr, 1, fl, &c))) return rc;
-  if (nw == 0) c = 1.0;
+  double crh[2];
+  if ((rc = read_flags(L, info, 2, cr, 2, fl, crh))) return rc;
+  const double c = nw == 0 ? 1.0 : cond_of(crh);
   if (fl[0] != 0) {
     *flip = true;
     *condR = INFINITY;
