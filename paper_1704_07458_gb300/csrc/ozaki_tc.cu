@@ -110,13 +110,23 @@ __device__ __forceinline__ void digits(double x, int E, float (&d)[S]) {
 // S <= 6, on the FP32 pipe.  The integer pipe takes an instruction every two
 // cycles, so a split by shifts and byte permutes (25 integer instructions per
 // value) bounded the kernels at 1,400 to 2,200 cycles a chunk against 1,300 of
-// MMAs.  Here x 2^(7-E) is a sum a + b of two floats: a takes the top 24 bits of
-// the mantissa with the exponent field moved by one multiply-add (values below
+// MMAs.  Here x 2^(7-E) is a sum of two floats: a takes the top 24 bits of the
+// mantissa with the exponent field moved by one multiply-add (values below
 // 2^-87 of the bound are raised to it: all their digits are zero), b the other
-// 29 bits through one conversion.  Digit s is what the sum rounds to at a
-// multiple of 2^-8s: adding and subtracting 1.5 * 2^(23-8s) leaves it, exact,
-// pre-weighted and balanced (|d_s| <= 128); b joins at the third digit.  Nine
-// integer instructions per value remain.
+// 29 bits.  Digit s is what the sum rounds to at a multiple of 2^-8s: adding and
+// subtracting 1.5 * 2^(23-8s) leaves it, exact, pre-weighted and balanced
+// (|d_s| <= 129, the 129 in the last digit only).
+//
+// The digits sum to F of `digits`, every bit of it: F is one rounding of x, and
+// 29 bits do not fit a float, so b and all that follows it round down and b
+// carries the half unit of the last digit, 2^(7-8S), with it.  Then the last
+// digit is a floor, and a floor is not changed by floors at finer multiples
+// before it.  (Rounded to the nearest at each step, x was rounded twice for
+// S = 6: largest error 0.73 units of the last digit and not 0.5, 17 % of the
+// values in the top binade with another F.)  A negative x takes the one's
+// complement of its low bits, which breaks its ties away from zero as F does.  b
+// joins a after the fourth digit (a + b is exact enough before that only to
+// choose a digit).  Ten integer instructions per value remain.
 constexpr int kFastEMin = -900, kFastEMax = 1100;
 
 __host__ __device__ constexpr uint32_t split_thr(int E) { return (uint32_t)(E + 889) << 20; }
@@ -145,10 +155,12 @@ struct Split {
     const uint32_t m = (uint32_t)max((int)(xh & 0x7FFFFFFFu), (int)(thr + (40u << 20)));
     // exponent field be - E - 889 = (be - 1023) + (7 - E) + 127
     const uint32_t w = __funnelshift_l(xl, m, 3) - thr * 8u;
-    const uint32_t sw = (xh & 0x80000000u) | w;
-    a[i] = __uint_as_float(sw);
-    b[i] = (float)(int)(xl & 0x1FFFFFFFu) * pow2f(-52) * __uint_as_float(sw & 0xFF800000u);
+    a[i] = __uint_as_float((xh & 0x80000000u) | w);
+    const int low = (int)((xl & 0x1FFFFFFFu) ^ (uint32_t)((int)xh >> 31));
+    b[i] = __fmaf_rd(__int2float_rd(low) * pow2f(-52), __uint_as_float(w & 0x7F800000u),
+                     pow2f(7 - 8 * S));
   }
+  // a + b is F itself: no bits below the last digit, so no half unit
   __device__ __forceinline__ void load_any(int i, double x, int E) {
     constexpr int sh = 8 * S - 24;
     const long long F = fixed_any<S>(x, E);
@@ -158,13 +170,18 @@ struct Split {
   template <int s>
   __device__ __forceinline__ void plane(uint32_t (&w)[4]) {
     constexpr float M = 1.5f * pow2f(23 - 8 * s);
+    constexpr int kJoin = S > 4 ? 3 : S - 1;  // where b joins a
     float d[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      // b is below the third digit's unit, but may decide its rounding
-      d[i] = ((s == 2 ? a[i] + b[i] : a[i]) + M) - M;
-      if (s + 1 < S) a[i] -= d[i];
-      if (s == 2) a[i] += b[i];
+      if (s == S - 1) {
+        if (s == kJoin) a[i] = __fadd_rd(a[i], b[i]);
+        d[i] = __fadd_rd(a[i], M) - M;
+      } else {
+        d[i] = ((s >= 2 && s <= kJoin ? a[i] + b[i] : a[i]) + M) - M;
+        a[i] -= d[i];
+        if (s == kJoin) a[i] = __fadd_rd(a[i], b[i]);
+      }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
