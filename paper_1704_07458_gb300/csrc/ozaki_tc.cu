@@ -341,6 +341,27 @@ __device__ __forceinline__ double i64_scaled(long long v, int e) {
   return int_to_double(v, e);
 }
 
+// v * 2^e + y0, aligned in 62 bits and rounded once; integer operations only.
+__device__ __noinline__ double i64_scaled_sum(long long v, int e, double y0) {
+  long long my;
+  int ey;
+  double_parts(y0, my, ey);
+  if (my == 0) return int_to_double(v, e);
+  const int base = max(e + bitlen(v), ey + bitlen(my)) - 61;
+  auto shifted = [&](long long m, int k) {
+    return k >= 0 ? m << k : (k < -62 ? 0LL : m >> -k);
+  };
+  return int_to_double(shifted(v, e - base) + shifted(my, ey - base), base);
+}
+
+// v * 2^e + y0 with one rounding: below 2^53 the integer is a double as it stands
+// (always so over one block of 256 columns: levels below 2^52 + 2^45), above it
+// would be rounded before Y0 joins.
+__device__ __forceinline__ double i64_scaled_plus(long long v, int e, double y0) {
+  if ((unsigned long long)(v + (1LL << 53)) <= (1ULL << 54)) return i64_scaled(v, e) + y0;
+  return i64_scaled_sum(v, e, y0);
+}
+
 // float -> int without the conversion unit (which takes 16 values per clock
 // and SM): f + kMagic for |f| <= 2^22 holds the integer nearest f in its low
 // mantissa bits, as_int(f + kMagic) - kMagicInt.
@@ -1247,11 +1268,14 @@ __global__ void __launch_bounds__(kUThrAll, 1)
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         if (r[u] < 0) continue;
-        double out = i64_scaled(T[u], e[u]);
+        double out;
         if (kY0) {
-          const double* y0 = fin.y0base;
-          out += y0 ? y0[r[u] * fin.y0ld + j[u]]
-                    : seg_load(Y0, ocol + j[u], fin.row0 + r[u]);
+          const double* yb = fin.y0base;
+          const double y0 = yb ? yb[r[u] * fin.y0ld + j[u]]
+                               : seg_load(Y0, ocol + j[u], fin.row0 + r[u]);
+          out = kOneBlock ? i64_scaled(T[u], e[u]) + y0 : i64_scaled_plus(T[u], e[u], y0);
+        } else {
+          out = i64_scaled(T[u], e[u]);
         }
         if (ybase)
           ybase[(int64_t)r[u] * oyld + j[u]] = out;

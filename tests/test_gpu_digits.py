@@ -145,3 +145,26 @@ def test_update_digits_are_one_rounding(slices, scale):
     got = host(Y, 16)
     for j in (0, 7, 15):
         _check(got[:, j], x, E, slices, terms, 30)
+
+
+def test_update_adds_y0_before_it_rounds():
+    """Over several blocks of 256 columns a sum may need more than the 53 bits
+    of a double; Y0 joins it before the one rounding.  2,049 products of 64 x 64
+    digits (2^53 + 2^42 in units of 2^-30) and one unit: less the first, the unit
+    is left, exactly."""
+    torch = torch_cuda()
+    n, m, s = 130, 16, 2050
+    S = np.full((n, s), 0.5)
+    C = np.full((s, m), 0.5)
+    C[-1] = 2.0 ** -43
+    big, unit = 2049 * 0.25, 2.0 ** -44
+    Y0 = np.tile([-big, big, 1.0, 0.0], (n, m // 4))
+    Y = dev(np.full((n, m), np.nan), m)
+    rc = gb.lobpcg_update(n, dev(S, s), s, s, dev(C.T.copy().reshape(-1)), s, m, 1.0, 1.0,
+                          dev(Y0, m), m, Y, m, TC, 6)
+    torch.cuda.synchronize()
+    assert rc == 0
+    got = host(Y, m)
+    np.testing.assert_array_equal(got[:, ::4], unit)
+    for c in (1, 2, 3):  # big + unit, one part in 2^53, is lost in a double
+        np.testing.assert_array_equal(got[:, c::4], big + Y0[0, c])
