@@ -51,6 +51,10 @@ struct Cols<true> {
     v.x += x.v.x;
     v.y += x.v.y;
   }
+  __device__ __forceinline__ void sub(const Cols& x) {
+    v.x -= x.v.x;
+    v.y -= x.v.y;
+  }
   // both columns when the second exists
   __device__ __forceinline__ void store(double* p, bool two) const {
     if (two && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
@@ -69,10 +73,11 @@ struct Cols<false> {
   __device__ __forceinline__ void fma_(double a, const Cols& x) { v = fma(a, x.v, v); }
   __device__ __forceinline__ void scale(double a) { v *= a; }
   __device__ __forceinline__ void add(const Cols& x) { v += x.v; }
+  __device__ __forceinline__ void sub(const Cols& x) { v -= x.v; }
   __device__ __forceinline__ void store(double* p, bool) const { *p = v; }
 };
 
-// acc += sgn A(row, :) X(:, c) for this thread's columns; kBatch nonzeros of
+// acc += A(row, :) X(:, c) for this thread's columns; kBatch nonzeros of
 // the row are in flight (their column indices and values, then their X pieces).
 // The loop ends at the longest row of the warp by a branch: an FMA predicated
 // off for all lanes occupies the FP64 pipe like any other (three of eight of
@@ -83,7 +88,7 @@ __device__ __forceinline__ void row_product(const int32_t* __restrict__ rowptr,
                                             const int32_t* __restrict__ col,
                                             const double* __restrict__ val,
                                             const double* __restrict__ X, int64_t ldx, int64_t row,
-                                            int c, bool live, bool neg, Cols<kPair>& acc) {
+                                            int c, bool live, Cols<kPair>& acc) {
   const int lo = live ? __ldg(rowptr + row) : 0, hi = live ? __ldg(rowptr + row + 1) : 0;
   const int longest = __reduce_max_sync(0xffffffffu, hi - lo);
   for (int p = 0; p < longest; p += kBatch) {
@@ -104,7 +109,7 @@ __device__ __forceinline__ void row_product(const int32_t* __restrict__ rowptr,
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
       if (p + j >= longest) break;
-      acc.fma_(neg ? -a[j] : a[j], x[j]);
+      acc.fma_(a[j], x[j]);
     }
   }
 }
@@ -132,7 +137,7 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) spmm_csr_kernel(
   const bool live = it.row < n && c < m, two = c + 1 < m;
   Cols<kPair> acc;
   acc.zero();
-  row_product<kPair>(rowptr, col, val, X, ldx, it.row, c, live, false, acc);
+  row_product<kPair>(rowptr, col, val, X, ldx, it.row, c, live, acc);
   if (!live) return;
   acc.store(Y + it.row * ldy + c, two);
   if (b) {
@@ -144,7 +149,10 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) spmm_csr_kernel(
 }
 
 // One Chebyshev step on the fly (see precond.cu): with z = D^-1 (r - A w),
-// d <- a d + bz z and w' = w + d.  The last step writes w' only.
+// d <- a d + bz z and w' = w + d.  The last step writes w' only.  A w is summed
+// by itself and z rounded before bz multiplies it, as in separate passes: terms
+// of A w taken from r one by one would cost r the bits that they cancel among
+// themselves.
 template <bool kPair>
 __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) cheb_step_kernel(
     int64_t n, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
@@ -154,17 +162,20 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) cheb_step_kernel(
   const Item it = item_of(width);
   const int c = kPair ? 2 * it.q : it.q;
   const bool live = it.row < n && c < m, two = c + 1 < m;
-  Cols<kPair> acc, dn, wn;
+  Cols<kPair> acc, z, dn, wn;
   acc.zero();
   if (live) {
-    acc.load(R + it.row * ldr + c);
+    z.load(R + it.row * ldr + c);
     dn.load(d + it.row * ld + c);
     wn.load(w + it.row * ld + c);
   }
-  row_product<kPair>(rowptr, col, val, w, ld, it.row, c, live, true, acc);
+  row_product<kPair>(rowptr, col, val, w, ld, it.row, c, live, acc);
   if (!live) return;
-  dn.scale(a);
-  dn.fma_(bz * __ldg(dinv + it.row), acc);
+  z.sub(acc);
+  z.scale(__ldg(dinv + it.row));
+  z.scale(bz);
+  z.fma_(a, dn);  // a d + bz z
+  dn = z;
   wn.add(dn);
   if (!last) dn.store(d + it.row * ld + c, two);
   wn.store(wnew + it.row * ldw + c, two);
