@@ -35,8 +35,12 @@ struct Cols;
 template <>
 struct Cols<true> {
   double2 v;
-  __device__ __forceinline__ void load(const double* p) {
+  // ro: memory that nothing writes while the kernel runs
+  __device__ __forceinline__ void load_ro(const double* p) {
     v = __ldg(reinterpret_cast<const double2*>(p));
+  }
+  __device__ __forceinline__ void load(const double* p) {
+    v = *reinterpret_cast<const double2*>(p);
   }
   __device__ __forceinline__ void zero() { v = make_double2(0.0, 0.0); }
   __device__ __forceinline__ void fma_(double a, const Cols& x) {
@@ -68,7 +72,8 @@ struct Cols<true> {
 template <>
 struct Cols<false> {
   double v;
-  __device__ __forceinline__ void load(const double* p) { v = __ldg(p); }
+  __device__ __forceinline__ void load_ro(const double* p) { v = __ldg(p); }
+  __device__ __forceinline__ void load(const double* p) { v = *p; }
   __device__ __forceinline__ void zero() { v = 0.0; }
   __device__ __forceinline__ void fma_(double a, const Cols& x) { v = fma(a, x.v, v); }
   __device__ __forceinline__ void scale(double a) { v *= a; }
@@ -104,7 +109,7 @@ __device__ __forceinline__ void row_product(const int32_t* __restrict__ rowptr,
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
       x[j].zero();
-      if (ci[j] >= 0) x[j].load(X + (int64_t)ci[j] * ldx + c);
+      if (ci[j] >= 0) x[j].load_ro(X + (int64_t)ci[j] * ldx + c);
     }
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
@@ -142,7 +147,7 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) spmm_csr_kernel(
   acc.store(Y + it.row * ldy + c, two);
   if (b) {
     Cols<kPair> x;
-    x.load(X + it.row * ldx + c);
+    x.load_ro(X + it.row * ldx + c);
     x.scale(__ldg(b + it.row));
     x.store(BY + it.row * ldby + c, two);
   }
@@ -152,13 +157,15 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) spmm_csr_kernel(
 // d <- a d + bz z and w' = w + d.  The last step writes w' only.  A w is summed
 // by itself and z rounded before bz multiplies it, as in separate passes: terms
 // of A w taken from r one by one would cost r the bits that they cancel among
-// themselves.
+// themselves.  d and, where W is R, r are written by the thread that has read
+// them: ordinary loads, not the read-only path, which is for memory that stays as
+// it is while the kernel runs.
 template <bool kPair>
 __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) cheb_step_kernel(
     int64_t n, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     const double* __restrict__ val, const double* __restrict__ w, int64_t ld, int m, int width,
-    const double* __restrict__ R, int64_t ldr, const double* __restrict__ dinv, double a, double bz,
-    double* __restrict__ d, double* __restrict__ wnew, int64_t ldw, bool last) {
+    const double* R, int64_t ldr, const double* __restrict__ dinv, double a, double bz, double* d,
+    double* wnew, int64_t ldw, bool last) {
   const Item it = item_of(width);
   const int c = kPair ? 2 * it.q : it.q;
   const bool live = it.row < n && c < m, two = c + 1 < m;
@@ -167,7 +174,7 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) cheb_step_kernel(
   if (live) {
     z.load(R + it.row * ldr + c);
     dn.load(d + it.row * ld + c);
-    wn.load(w + it.row * ld + c);
+    wn.load_ro(w + it.row * ld + c);
   }
   row_product<kPair>(rowptr, col, val, w, ld, it.row, c, live, acc);
   if (!live) return;

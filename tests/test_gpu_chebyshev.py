@@ -10,13 +10,14 @@ pytestmark = pytest.mark.gpu
 N = 70
 
 
-def _apply(rows, R, m, ldr, degree):
+def _apply(rows, R, m, ldr, degree, in_place=False):
     """rows: per row a list of (column, value)."""
     torch = torch_cuda()
     rp = dev_i32(np.cumsum([0] + [len(r) for r in rows]))
     ci = dev_i32(np.array([c for r in rows for c, _ in r]))
     va = dev(np.array([v for r in rows for _, v in r]))
     Rd, W = dev(R, ldr), dev(np.full((len(rows), m), np.nan), ldr)
+    W = Rd if in_place else W
     c = gb.lobpcg_chebyshev_create(len(rows), rp, ci, va, None, degree, 0.05, 2.0, m)
     rc = gb.lobpcg_chebyshev_apply(c, len(rows), m, Rd, ldr, W, ldr, None)
     torch.cuda.synchronize()
@@ -40,3 +41,14 @@ def test_terms_that_cancel_in_a_w_cost_r_no_bits(m, ldr, degree):
     coupled = plain[:2] + [[(0, big), (1, -big), (i, d[i])] for i in range(2, N)]
     np.testing.assert_array_equal(_apply(coupled, R, m, ldr, degree),
                                   _apply(plain, R, m, ldr, degree))
+
+
+@pytest.mark.parametrize("m,ldr", [(1, 1), (4, 4), (5, 5), (5, 8), (71, 72)])
+@pytest.mark.parametrize("degree", [1, 2, 5])
+def test_result_may_replace_r(m, ldr, degree):
+    """Every element of R is read before W's takes its place."""
+    R = np.random.default_rng(m).standard_normal((N, m))
+    rows = [[(j, 4.0 if i == j else -1.0) for j in (i - 7, i - 1, i, i + 1, i + 7) if 0 <= j < N]
+            for i in range(N)]
+    np.testing.assert_array_equal(_apply(rows, R, m, ldr, degree, in_place=True),
+                                  _apply(rows, R, m, ldr, degree))
