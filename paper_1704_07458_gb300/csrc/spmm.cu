@@ -35,12 +35,13 @@ struct Cols;
 template <>
 struct Cols<true> {
   double2 v;
-  // ro: memory that nothing writes while the kernel runs
-  __device__ __forceinline__ void load_ro(const double* p) {
-    v = __ldg(reinterpret_cast<const double2*>(p));
+  // ro: memory that nothing writes while the kernel runs.  two: the second
+  // column exists; if not, it is not read (the caller's block may end there).
+  __device__ __forceinline__ void load_ro(const double* p, bool two) {
+    v = two ? __ldg(reinterpret_cast<const double2*>(p)) : make_double2(__ldg(p), 0.0);
   }
-  __device__ __forceinline__ void load(const double* p) {
-    v = *reinterpret_cast<const double2*>(p);
+  __device__ __forceinline__ void load(const double* p, bool two) {
+    v = two ? *reinterpret_cast<const double2*>(p) : make_double2(*p, 0.0);
   }
   __device__ __forceinline__ void zero() { v = make_double2(0.0, 0.0); }
   __device__ __forceinline__ void fma_(double a, const Cols& x) {
@@ -72,8 +73,8 @@ struct Cols<true> {
 template <>
 struct Cols<false> {
   double v;
-  __device__ __forceinline__ void load_ro(const double* p) { v = __ldg(p); }
-  __device__ __forceinline__ void load(const double* p) { v = *p; }
+  __device__ __forceinline__ void load_ro(const double* p, bool) { v = __ldg(p); }
+  __device__ __forceinline__ void load(const double* p, bool) { v = *p; }
   __device__ __forceinline__ void zero() { v = 0.0; }
   __device__ __forceinline__ void fma_(double a, const Cols& x) { v = fma(a, x.v, v); }
   __device__ __forceinline__ void scale(double a) { v *= a; }
@@ -93,7 +94,7 @@ __device__ __forceinline__ void row_product(const int32_t* __restrict__ rowptr,
                                             const int32_t* __restrict__ col,
                                             const double* __restrict__ val,
                                             const double* __restrict__ X, int64_t ldx, int64_t row,
-                                            int c, bool live, Cols<kPair>& acc) {
+                                            int c, bool live, bool two, Cols<kPair>& acc) {
   const int lo = live ? __ldg(rowptr + row) : 0, hi = live ? __ldg(rowptr + row + 1) : 0;
   const int longest = __reduce_max_sync(0xffffffffu, hi - lo);
   for (int p = 0; p < longest; p += kBatch) {
@@ -109,7 +110,7 @@ __device__ __forceinline__ void row_product(const int32_t* __restrict__ rowptr,
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
       x[j].zero();
-      if (ci[j] >= 0) x[j].load_ro(X + (int64_t)ci[j] * ldx + c);
+      if (ci[j] >= 0) x[j].load_ro(X + (int64_t)ci[j] * ldx + c, two);
     }
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
@@ -142,12 +143,12 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) spmm_csr_kernel(
   const bool live = it.row < n && c < m, two = c + 1 < m;
   Cols<kPair> acc;
   acc.zero();
-  row_product<kPair>(rowptr, col, val, X, ldx, it.row, c, live, acc);
+  row_product<kPair>(rowptr, col, val, X, ldx, it.row, c, live, two, acc);
   if (!live) return;
   acc.store(Y + it.row * ldy + c, two);
   if (b) {
     Cols<kPair> x;
-    x.load_ro(X + it.row * ldx + c);
+    x.load_ro(X + it.row * ldx + c, two);
     x.scale(__ldg(b + it.row));
     x.store(BY + it.row * ldby + c, two);
   }
@@ -172,11 +173,11 @@ __global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) cheb_step_kernel(
   Cols<kPair> acc, z, dn, wn;
   acc.zero();
   if (live) {
-    z.load(R + it.row * ldr + c);
-    dn.load(d + it.row * ld + c);
-    wn.load_ro(w + it.row * ld + c);
+    z.load(R + it.row * ldr + c, two);
+    dn.load(d + it.row * ld + c, two);
+    wn.load_ro(w + it.row * ld + c, two);
   }
-  row_product<kPair>(rowptr, col, val, w, ld, it.row, c, live, acc);
+  row_product<kPair>(rowptr, col, val, w, ld, it.row, c, live, two, acc);
   if (!live) return;
   z.sub(acc);
   z.scale(__ldg(dinv + it.row));
@@ -202,10 +203,9 @@ dim3 grid_of(int64_t n, Tiles t) {
   return dim3((unsigned)ceil_div(n * t.width, kSpmmThreads), (unsigned)t.count);
 }
 
-// pairs: rows 16-byte aligned (base and leading dimension even), and an odd m
-// only with a padded row (the pair's second half stays inside it)
-bool pairs_ok(const double* X, int64_t ldx, int m) {
-  return ((uintptr_t)X % 16 == 0) && (ldx % 2 == 0) && (m % 2 == 0 || ldx > m);
+// pairs: rows 16-byte aligned (base and leading dimension even)
+bool pairs_ok(const double* X, int64_t ldx) {
+  return ((uintptr_t)X % 16 == 0) && (ldx % 2 == 0);
 }
 
 }  // namespace
@@ -215,7 +215,7 @@ int spmm(cudaStream_t st, int64_t n, const int32_t* rowptr, const int32_t* col,
          const double* b, double* BY, int64_t ldby) {
   if (n <= 0 || m <= 0) return LOBPCG_OK;
   const double* bb = BY ? b : nullptr;
-  if (pairs_ok(X, ldx, m)) {
+  if (pairs_ok(X, ldx)) {
     const Tiles t = tiles_of((m + 1) / 2);
     spmm_csr_kernel<true><<<grid_of(n, t), kSpmmThreads, 0, st>>>(
         n, rowptr, col, val, X, ldx, m, t.width, Y, ldy, bb, BY, ldby);
@@ -233,7 +233,7 @@ int cheb_step(cudaStream_t st, int64_t n, const int32_t* rowptr, const int32_t* 
               const double* dinv, double a, double bz, double* d, double* wnew, int64_t ldw,
               bool last) {
   if (n <= 0 || m <= 0) return LOBPCG_OK;
-  if (pairs_ok(w, ld, m) && pairs_ok(d, ld, m) && pairs_ok(R, ldr, m)) {
+  if (pairs_ok(w, ld) && pairs_ok(d, ld) && pairs_ok(R, ldr)) {
     const Tiles t = tiles_of((m + 1) / 2);
     cheb_step_kernel<true><<<grid_of(n, t), kSpmmThreads, 0, st>>>(
         n, rowptr, col, val, w, ld, m, t.width, R, ldr, dinv, a, bz, d, wnew, ldw, last);
