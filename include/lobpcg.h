@@ -275,8 +275,14 @@ void lobpcg_destroy(lobpcg_t h);
 
 /* ---------------------------------------------------------------------------
  * Kernel-level entry points: single steps of one iteration on device buffers,
- * ordered on `stream`.  They allocate nothing unless noted.
+ * ordered on `stream`.  They allocate nothing unless noted.  Scratch that a call
+ * allocates comes from a pool of the library, which keeps up to 64 MB a device
+ * for the next call; lobpcg_destroy and lobpcg_chebyshev_destroy (on the device of
+ * their object) and lobpcg_release_scratch (on the current device, which it
+ * synchronises) give it back.
  * ------------------------------------------------------------------------- */
+
+int lobpcg_release_scratch(void);
 
 /* Block sparse product Y = A X for an n x m row-major block X (the A W and
  * B W products of Algorithm 8, Sec. 5.2), optionally also BY = diag(b) X

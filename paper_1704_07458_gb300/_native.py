@@ -38,7 +38,7 @@ EXPORTED = [
     "lobpcg_update", "lobpcg_residual", "lobpcg_philox_normal", "lobpcg_gram_noalloc",
     "lobpcg_eig_adjoint", "lobpcg_syev",
     "lobpcg_chebyshev_create", "lobpcg_chebyshev_apply", "lobpcg_chebyshev_destroy",
-    "lobpcg_wait_selftest", "lobpcg_set_operator_ex",
+    "lobpcg_wait_selftest", "lobpcg_set_operator_ex", "lobpcg_release_scratch",
 ]
 
 
@@ -163,6 +163,7 @@ def load(build_if_missing=False):
         "lobpcg_chebyshev_apply": (I32, [P, I64, I64, P, I64, P, I64, P]),
         "lobpcg_chebyshev_destroy": (None, [P]),
         "lobpcg_wait_selftest": (I32, [I32, P]),
+        "lobpcg_release_scratch": (I32, []),
         "lobpcg_set_operator_ex": (I32, [P, I64, P, P, P, I64, I32, P, P, P, I64, P, I32, I32,
                                          I32]),
     }
@@ -282,6 +283,10 @@ def lobpcg_last_error(h):
 
 def lobpcg_destroy(h):
     load().lobpcg_destroy(h)
+
+
+def lobpcg_release_scratch():
+    return load().lobpcg_release_scratch()
 
 
 def lobpcg_spmm(n, rowptr, col, val, X, ldx, m, Y, ldy, b=None, BY=None, ldby=0, stream=None):

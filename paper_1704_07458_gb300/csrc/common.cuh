@@ -67,7 +67,7 @@ __device__ __forceinline__ double* out_addr(const OutList& o, int c, int64_t row
 // Device scratch in stream order from this library's pool (scratch.cu).
 int scratch_alloc(void** p, size_t bytes, cudaStream_t st);
 void scratch_free(void* p, cudaStream_t st);
-void scratch_trim();  // the current device's kept memory goes back
+void scratch_trim(int device);  // the memory kept on a device goes back
 
 // Launches that follow one another on a stream without the gap of a full
 // completion (programmatic dependent launch): the next kernel's CTAs take their

@@ -21,6 +21,7 @@
 #include "colpass.cuh"
 
 struct lobpcg_chebyshev {
+  int device = 0;
   int64_t n = 0, max_cols = 0, ld = 0;
   const int32_t* rowptr = nullptr;
   const int32_t* col = nullptr;
@@ -90,6 +91,7 @@ LOBPCG_EXPORT int lobpcg_chebyshev_create(lobpcg_chebyshev_t* out, int64_t n,
     return LOBPCG_ERR_ARG;
   auto* c = new (std::nothrow) lobpcg_chebyshev();
   if (!c) return LOBPCG_ERR_OOM;
+  cudaGetDevice(&c->device);
   c->n = n;
   c->max_cols = max_cols;
   c->ld = lob::round_up(max_cols, 8);
@@ -161,5 +163,6 @@ LOBPCG_EXPORT void lobpcg_chebyshev_destroy(lobpcg_chebyshev_t c) {
   if (c->w) cudaFree(c->w);
   if (c->d) cudaFree(c->d);
   if (c->aw) cudaFree(c->aw);
+  lob::scratch_trim(c->device);
   delete c;
 }

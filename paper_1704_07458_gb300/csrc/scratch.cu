@@ -6,9 +6,9 @@
 // stream, so a caller that waits for its result pays for a fresh mapping on the
 // next call (about 200 us at any size: 651 us alone against 431 us in a row for
 // the residual of 262,144 x 71).  This pool keeps at most kKeep bytes a device;
-// what lies above goes back at the next synchronisation, and destroying any
-// handle returns the rest.  The driver orders reuse by stream, so threads and
-// streams may share the pool.
+// what lies above goes back at the next synchronisation, and lobpcg_destroy,
+// lobpcg_chebyshev_destroy and lobpcg_release_scratch return the rest.  The driver
+// orders reuse by stream, so threads and streams may share the pool.
 #include <mutex>
 
 #include "kernels.cuh"
@@ -66,9 +66,20 @@ void scratch_free(void* p, cudaStream_t st) {
   if (p) cudaFreeAsync(p, st);
 }
 
-void scratch_trim() {
-  cudaMemPool_t pool = pool_of_device();
-  if (pool) cudaMemPoolTrimTo(pool, 0);
+// Memory whose free is still pending on a stream is not returned: callers have
+// synchronised (cudaFree does, over the whole device).
+void scratch_trim(int device) {
+  if (device < 0 || device >= kDevices) return;
+  std::lock_guard<std::mutex> lock(g_mutex);
+  if (g_pool[device]) cudaMemPoolTrimTo(g_pool[device], 0);
 }
 
 }  // namespace lob
+
+LOBPCG_EXPORT int lobpcg_release_scratch(void) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
+    return LOBPCG_ERR_CUDA;
+  lob::scratch_trim(dev);
+  return LOBPCG_OK;
+}

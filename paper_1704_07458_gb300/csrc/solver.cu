@@ -1132,9 +1132,10 @@ LOBPCG_EXPORT int lobpcg_create(lobpcg_t* out, const lobpcg_options_t* opts, voi
 
 LOBPCG_EXPORT void lobpcg_destroy(lobpcg_t h) {
   if (!h) return;
+  const int device = h->device;
   cudaStreamSynchronize(h->st);
   delete h;
-  scratch_trim();
+  scratch_trim(device);
 }
 
 LOBPCG_EXPORT const char* lobpcg_last_error(lobpcg_t h) { return h ? h->err.c_str() : "null handle"; }
