@@ -7,6 +7,7 @@ _build/libgb300lobpcg.so against cuBLAS and cuSOLVER.  Run as
 import concurrent.futures as cf
 import glob
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -36,6 +37,28 @@ def _cuda_lib_dir(nvcc):
     return os.path.join(root, "lib64")
 
 
+# Kernels whose warps share out the registers of the launch among themselves
+# (setmaxnreg): built with another count than the constant in their source says,
+# their launches would wait for shares that never come free, so the library
+# refuses them at run time.  (source, constant, kernels)
+REGISTER_SHARES = [("ozaki_tc.cu", "kURegs", r"ozaki_(gram|update)_tc_kernel")]
+
+
+def check_registers(src, log):
+    """Raise when ptxas -v's output shows such a kernel with another count."""
+    for name, const, kernels in REGISTER_SHARES:
+        if os.path.basename(src) != name:
+            continue
+        want = int(re.search(rf"\b{const} = (\d+)", open(src).read()).group(1))
+        found = [(f, int(r)) for f, r in
+                 re.findall(r"Compiling entry function '(\w+)'.*?Used (\d+) registers", log, re.S)
+                 if re.search(kernels, f)]
+        bad = [f"{f}: {r}" for f, r in found if r != want]
+        if bad or not found:
+            raise RuntimeError(f"{name}: {const} = {want} registers a thread, but ptxas gave "
+                               f"{', '.join(bad) or 'no kernel'}")
+
+
 def build(verbose=False, extra=()):
     nvcc = _nvcc()
     os.makedirs(OUT, exist_ok=True)
@@ -49,10 +72,16 @@ def build(verbose=False, extra=()):
         if (os.path.exists(obj) and os.path.getmtime(obj) > os.path.getmtime(src)
                 and os.path.getmtime(obj) > newest_hdr):
             return obj
-        cmd = [nvcc, *ARCH, *FLAGS, *extra, "-c", src, "-o", obj]
+        usage = ["-Xptxas", "-v"] * any(os.path.basename(src) == s for s, _, _ in REGISTER_SHARES)
+        cmd = [nvcc, *ARCH, *FLAGS, *usage, *extra, "-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
+        try:
+            check_registers(src, r.stdout + r.stderr)
+        except RuntimeError:
+            os.remove(obj)
+            raise
         if verbose and (r.stdout or r.stderr):
             print(r.stdout, r.stderr, file=sys.stderr)
         return obj
