@@ -336,10 +336,17 @@ __global__ void __launch_bounds__(1024, 1) tridiag32_kernel(int n, const double*
 // touching memory, and a step costs two barriers: one for the column that the
 // owners of its elements publish, one for p = tau A v.  Every warp forms the
 // reflector and p^T v for itself (a few shuffles) instead of waiting for one
-// that does.  Tiles left of or above the trailing block are skipped.  Bound by
-// the chain of a step (two reductions of five shuffles, a square root, two
-// divisions, two barriers); with the matrix in shared memory each element cost
-// two loads and a store per step (811 us at n = 213; 361 us now).
+// that does.  Tiles left of or above the trailing block are skipped.  Each
+// element is updated by the operations of its mirror image, in their order, so
+// that the matrix stays symmetric to the last bit: the reduction does not carry an
+// antisymmetric part along, and with one growing from rounding 18 % of the final
+// checks in 64^3 solves failed on groups too wide (12 % so: 603 and 375 of some
+// 3,260 eigenproblems).  The correction is rounded by itself: two FMAs into the
+// element round twice at its size, and twice as many matrices with eigenvalues
+// 1e-5 apart fail the check.  Bound by the chain of a step (two reductions of five
+// shuffles, a square root, two divisions, two barriers); with the matrix in shared
+// memory each element cost two loads and a store per step (811 us at n = 213; 361
+// us now).
 constexpr int kTridRegMax = 224;
 
 template <int NB>
@@ -436,7 +443,14 @@ __device__ __forceinline__ void tridiag_phase(int n, float (&a)[2 * NB][NB], Tri
       const float vi = i == k + 1 ? 1.f : (i > k ? xi.x * scale : 0.f);
       const float wi = fmaf(-K, vi, xi.y);
 #pragma unroll
-      for (int c = C0; c < NB; ++c) a[r][c] -= fmaf(vi, wj[c], wi * vj[c]);
+      for (int c = C0; c < NB; ++c) {  // below, above and on the diagonal tile
+        if (r / 2 > c)
+          a[r][c] -= fmaf(vi, wj[c], wi * vj[c]);
+        else if (r / 2 < c)
+          a[r][c] -= fmaf(vj[c], wi, wj[c] * vi);
+        else
+          a[r][c] -= __fadd_rn(__fmul_rn(vi, wj[c]), __fmul_rn(wi, vj[c]));
+      }
       if (own) xn[i].x = a[r][C0];
     }
   }
