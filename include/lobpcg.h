@@ -387,8 +387,8 @@ int lobpcg_eig_adjoint(lobpcg_t h, int64_t k, const double* lambda, const double
  * to FP64 (Ogita-Aishima steps, a Newton-Schulz orthonormalisation, Jacobi on
  * eigenvalue clusters; FP64 syevd when its residual check fails); mode 2:
  * this library's device-resident eigensolver (FP32 Householder
- * tridiagonalisation, bisection and inverse iteration, then FP64
- * Ogita-Aishima refinement, a Newton-Schulz step and Jacobi on clusters,
+ * tridiagonalisation, multisection and inverse iteration, then FP64
+ * Ogita-Aishima refinement, two Newton-Schulz steps and Jacobi on clusters,
  * n <= 256), cuSOLVER FP64 syevd when its check fails; mode 3: mode 2
  * without the fallback, returning LOBPCG_ERR_NOT_CONVERGED (outputs written)
  * when the check fails.  n <= 8192.  Allocates its workspace per call and

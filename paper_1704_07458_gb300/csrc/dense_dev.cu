@@ -49,7 +49,8 @@ constexpr int kMaxRunDev = 32;                     // cluster width of the final
 // multiplied.  The tiles are small because the products are: at order 81 a
 // 16 x 16 tile leaves 36 CTAs, and splitting the contraction over CTAs costs a
 // fence, a counter and a second pass through L2 (5.6 us at order 81, 31 us at
-// 213; 3.1 and 19 us on average now, the symmetric products among them; FP64 pipe at 213: 18.6 us).
+// 213; 4.8 and 21 us on average now, the symmetric products among them, in a cold
+// launch list; FP64 pipe at 213: 18.6 us).
 // skip != nullptr: the whole launch is a no-op when *skip is non-zero.
 // sym = s > 0: s products of m x m whose results are symmetric, B and C of the
 // later ones m columns on; only the upper triangles are computed (half of the
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(1024, 1) tridiag32_kernel(int n, const double*
 // element round twice at its size, and twice as many matrices with eigenvalues
 // 1e-5 apart fail the check.  Bound by the chain of a step (two reductions of five
 // shuffles, a square root, two divisions, two barriers); with the matrix in shared
-// memory each element cost two loads and a store per step (811 us at n = 213; 361
+// memory each element cost two loads and a store per step (811 us at n = 213; 374
 // us now).
 constexpr int kTridRegMax = 224;
 
@@ -1357,8 +1358,8 @@ __global__ void assemble_h_kernel(int ns, int o, const double* MA, int ldm,
 // memory (the value feeds an order-of-magnitude test).  One CTA for each of the
 // two, side by side: out[0] and out[1] are the largest eigenvalues of M and
 // M^-1, cond(R) = sqrt(out[0] out[1]) (cond_of); inf when non-finite, or when
-// *skip != 0.  A chain of barriers: 49 us at ns = 81 with one CTA for
-// both (32 x 32 solve 26.9 -> 24.8 ms, 48 x 40 x 36 solve 124.6 -> 119.8 ms).
+// *skip != 0.  A chain of barriers: 20 us at ns = 81, 38 us with one CTA for both
+// (32 x 32 solve 26.9 -> 24.8 ms, 48 x 40 x 36 solve 124.6 -> 119.8 ms).
 __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, const double* MB,
                                                               int ldm, const double* Y,
                                                               int ldy, double* out, const int* skip) {
@@ -1409,8 +1410,8 @@ __global__ void __launch_bounds__(1024, 1) cond_struct_kernel(int ns, int o, con
     __syncthreads();
   };
   // res(i) = sum over eight lanes of part(i, lane): with a thread per row only
-  // ns of the 1024 threads worked, each on a chain of ns products (43 us at
-  // ns = 81; 38 us now)
+  // ns of the 1024 threads worked, each on a chain of ns products (an eighth more
+  // time at ns = 81)
   auto apply = [&](auto part, float* res) {
     const int sub = t & 7;
     for (int i0 = 0; i0 < ns; i0 += (int)blockDim.x >> 3) {
@@ -1792,10 +1793,10 @@ int dev_syev_refine(DenseLayer& L, int n, double* Z, int ldz, double* w, int* st
       return rc;
     std::swap(X, Y);
   }
-  // two Newton-Schulz steps X = X (3/2 I - 1/2 X^T X), always: a first-order step
-  // leaves an orthogonality defect of order |s_ij - s_ji| / |d_j - d_i| (the
-  // rounding asymmetry of X^T A X over the gap) even when its corrections are
-  // tiny, up to ~1e-4 on pairs it has just separated; each step squares it
+  // two Newton-Schulz steps X = X (3/2 I - 1/2 X^T X), always: I + E is orthogonal
+  // to first order only (S and G are mirrored, so E_ij + E_ji = r_ij), and the last
+  // step that ran leaves a defect of order E^T E, up to ~1e-4 on pairs it has just
+  // separated (|E_ij| <= 1e-2); each Newton-Schulz step squares it
   for (int s = 0; s < 2; ++s) {
     if ((rc = dev_gemm(L, true, false, n, n, n, 1.0, X, n, X, n, 0.0, nullptr, 0, G, n, nullptr,
                        1)))
@@ -1864,6 +1865,8 @@ int dev_orth_basis(DenseLayer& L, int m, int c, const double* M, int ldm, double
 // The device path takes a projected pencil when every piece fits its
 // one-CTA kernels: order <= 256 (eigensolver), Cholesky factors of order
 // <= 160, the cond(R) estimate's FP32 copies and the C_p QR in shared memory.
+// (The cond(R) bound counts the matrices of both estimates, which one CTA once
+// held: pencils of n_s = 2 n_x, n_x > 112, stay on cuSOLVER, not measured here.)
 bool dev_rr_fits(const DenseLayer& L, int ns, int nx, int nw) {
   if (L.eig_mode != 0 || ns > L.dev.nmax || ns > kDevDenseMax) return false;
   if (nw > kCholMax || nx > kCholMax) return false;

@@ -16,7 +16,7 @@
 //  * the contraction runs in chunks of 16 (rows of U and V for the Gram,
 //    columns of S for the update), grouped in blocks of at most 256 (the Gram's
 //    share one exponent per operand column; the update has one per row).  With
-//    |digit| <= 128 the sums of levels 0, 1, 2 (and 3 for S = 7) stay below 2^24
+//    |digit| <= 128 (129 in the last of up to six) the sums of levels 0, 1, 2 (and 3 for S = 7) stay below 2^24
 //    in their units over a block, so they are exact in FP32; the deeper levels
 //    (below 2^-24 resp. 2^-32 of level 0) share one inexact accumulator.  4 or 5
 //    accumulators x NT columns and two to four digit stages of A fit the 512
@@ -55,8 +55,6 @@ __host__ __device__ constexpr int nacc() { return S >= 7 ? 5 : (S < 4 ? S : 4); 
 // accumulator of digit level l = s + t (0-based digit indices)
 template <int S>
 __host__ __device__ constexpr int acc_of(int l) { return l < nacc<S>() - 1 ? l : nacc<S>() - 1; }
-template <int S>
-__host__ __device__ constexpr size_t planeA_bytes() { return (size_t)KG * (TCM / 8) * 128; }
 __host__ __device__ inline size_t planeB_bytes(int NT) { return (size_t)KG * (NT / 8) * 128; }
 
 // 0x80 in each of the S-1 low bytes: adding it turns the fixed-point value
@@ -589,7 +587,7 @@ __global__ void __launch_bounds__(256) block_col_exp_kernel(int64_t n,
 // exponents over the slab are known beforehand (block_col_exp_kernel), so a
 // block's sums only shift and add.  The form before this one (all digits in
 // shared memory, 8 warps, one CTA barrier per chunk) took 896 us at
-// n = 262,144, p = 213, q = 142; 540 us now.
+// n = 262,144, p = 213, q = 142; 552 us now.
 template <int S>
 __global__ void __launch_bounds__(kUThrAll, 1)
     ozaki_gram_tc_kernel(int64_t n, const __grid_constant__ SegList U, int p,
@@ -974,8 +972,8 @@ int gram_tc_launch(cudaStream_t st, int64_t n, const SegList& U, int p, const Se
 // with rows scaled by 2^colexp[k] (one exponent per column over all k), cut
 // once per call by split_c_tc_kernel into the shared-memory plane layout
 // [chunk][tile][S][KG][NT/8][8][8].  Persistent CTAs walk the (row block,
-// column tile) pairs; the row exponents of a CTA's next tile are computed
-// during its current tile.
+// column tile) pairs; the row exponents come from a pass of their own
+// (row_exp_kernel).
 
 template <int S>
 __global__ void split_c_tc_kernel(const double* __restrict__ C, int64_t ldc, int s, int m,
@@ -1101,7 +1099,7 @@ size_t upd_smem_bytes(int NT, int s) {
 //  * warp 16: an elected thread issues the S (S + 1) / 2 MMAs of a chunk (a
 //    thread found by its index instead makes every operand pass through a
 //    lane-by-lane move to uniform registers: 1,430 cycles a chunk, 870 so);
-//  * warp 17: one thread fetches C's digits, kUStagesB chunks ahead.
+//  * warp 17: one thread fetches C's digits, kUSlots chunks ahead.
 // The floor is the tensor pipe's 61 cycles for an M = 128, K = 16 MMA up to
 // N = 80 (64 at 96), 21 of them per chunk; what bounds it is the instruction
 // issue of the compute warps (about 30 per value cut, at the half rate of the

@@ -14,7 +14,7 @@
 // K^-1 = D^-1/2 p(D^-1/2 A D^-1/2) D^-1/2 is symmetric positive definite: a
 // valid LOBPCG preconditioner.  Every step is one kernel: the product A w with
 // the recurrence in its epilogue, so that A w is never stored (a product and an
-// elementwise pass took 570 us a step at 64^3, 71 columns; 400 us now); no
+// elementwise pass took 570 us a step at 64^3, 71 columns; 410 us now); no
 // host work per call.
 #include <algorithm>
 
