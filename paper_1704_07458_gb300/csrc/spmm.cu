@@ -164,8 +164,8 @@ __device__ __forceinline__ Item item_of(const Tiles& tl, int G) {
           (int)(t - dr * (uint32_t)tl.width) + (int)blockIdx.y * tl.width * G};
 }
 
-template <bool kPair, int G>
-__global__ void __launch_bounds__(kSpmmThreads, kSpmmCtas) spmm_csr_kernel(
+template <bool kPair, int G, int kCtas>
+__global__ void __launch_bounds__(kSpmmThreads, kCtas) spmm_csr_kernel(
     int64_t n, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     const double* __restrict__ val, const double* __restrict__ X, int64_t ldx, int m,
     const Tiles tl, double* __restrict__ Y, int64_t ldy, const double* __restrict__ b,
@@ -260,20 +260,27 @@ int spmm(cudaStream_t st, int64_t n, const int32_t* rowptr, const int32_t* col,
     kernel<<<grid_of(n, t), kSpmmThreads, 0, st>>>(n, rowptr, col, val, X, ldx, m, t, Y, ldy, bb,
                                                    BY, ldby);
   };
-  // Aligned rows in pairs, if these make two CTAs an SM (30 x 26 x 28, 4 columns:
-  // 6.0 us in pairs, 5.0 singly).  Others in two single columns a thread, twice the
-  // work behind each row's chain of loads (64^3, 64 columns: 248 us with one, 203
-  // with two), where at most one lane in fourteen is then idle (512^2, 7 columns:
-  // 20.7 and 22.8 us) and four waves of CTAs remain (200 x 90, 31 columns, 1.2
-  // waves: 8.6 and 10.1 us).
+  // Two columns a thread where few lanes are then idle: aligned rows in pairs up to
+  // one in ten (512^2, 7 columns: 22.8 us, 20.7 singly; diagonal B, 9 columns: 35.2
+  // and 37.3), if these make four CTAs an SM (30 x 26 x 28: 6.0 us in pairs at 4
+  // columns, 5.3 singly, with diagonal B at 8 columns 8.4 and 7.1); others in two
+  // single columns up to one in fourteen, twice the work behind each row's chain of
+  // loads (64^3, 64 columns: 248 us with one, 203 with two), if four waves of CTAs
+  // remain (200 x 90, 31 columns, 1.2 waves: 8.6 and 10.1 us).  One column a thread
+  // takes 64 warps an SM, with a few values spilled, for blocks that do not stay in
+  // L2 (100^3, 7 columns: 95 us, 105 with 48 warps; 64^3, 6 columns: 25.0 and 23.4);
+  // a row of A is taken as seven nonzeros.
+  const bool even = m % 2 == 0;
   const Tiles pairs = tiles_of((m + 1) / 2, 1, kMaxWidth), two = tiles_of(m, 2, 32);
   auto ctas = [&](const Tiles& t) { return ceil_div(n * t.width, kSpmmThreads) * t.count; };
-  if (pairs_ok(X, ldx) && ctas(pairs) >= 2 * 152)
-    run(spmm_csr_kernel<true, 1>, pairs);
-  else if (m > 4 && (m % 2 == 0 || m > 12) && ctas(two) >= 4 * kSpmmCtas * 152)
-    run(spmm_csr_kernel<false, 2>, two);
+  if ((even || m > 8) && pairs_ok(X, ldx) && ctas(pairs) >= 4 * 152)
+    run(spmm_csr_kernel<true, 1, kSpmmCtas>, pairs);
+  else if ((even || m > 12) && m > 4 && ctas(two) >= 4 * kSpmmCtas * 152)
+    run(spmm_csr_kernel<false, 2, kSpmmCtas>, two);
+  else if (n * (8 * (ldx + ldy) + 84) <= (96 << 20))
+    run(spmm_csr_kernel<false, 1, kSpmmCtas>, tiles_of(m, 1, 32));
   else
-    run(spmm_csr_kernel<false, 1>, tiles_of(m, 1, 32));
+    run(spmm_csr_kernel<false, 1, 8>, tiles_of(m, 1, 32));
   LOB_LAUNCHED();
   return LOBPCG_OK;
 }

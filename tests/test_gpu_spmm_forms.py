@@ -22,8 +22,9 @@ def _matrix(n, seed):
 
 
 @pytest.mark.parametrize("n", [97, 140001])
-@pytest.mark.parametrize("m,ld", [(1, 1), (2, 2), (3, 3), (3, 4), (4, 4), (5, 7), (6, 9), (8, 9),
-                                  (13, 13), (13, 14), (14, 17), (33, 33), (66, 67), (81, 82)])
+@pytest.mark.parametrize("m,ld", [(1, 1), (2, 2), (3, 3), (3, 4), (4, 4), (5, 7), (5, 61), (6, 9),
+                                  (8, 9), (9, 10), (13, 13), (13, 14), (14, 17), (33, 33), (66, 67),
+                                  (81, 82)])
 def test_spmm_forms_on_integers(n, m, ld):
     torch = torch_cuda()
     rowptr, col, val = _matrix(n, m)
