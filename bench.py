@@ -60,7 +60,7 @@ ORACLE_ITERS_FALLBACK = {"lap3d_64_diagB": 715, "lap2d_32": 101}
 # (source file, sha16, bytes per launch)
 NCU_TRAFFIC = {
     ("lap3d_64_diagB", "update", "ozaki_tc", 6):
-        ("paper_1704_07458_gb300/csrc/ozaki_tc.cu", "8abb673856b2052c", 450.009856e6 + 266.715392e6),
+        ("paper_1704_07458_gb300/csrc/ozaki_tc.cu", "b4051dea4187b867", 455.567360e6 + 262.135552e6),
 }
 # algorithmic bytes of one full-shape launch of each family at the workload
 # (the unit the traffic above is compared against)
