@@ -189,6 +189,7 @@ typedef int (*lobpcg_precond_fn)(void* ctx, int64_t n, int64_t ncols, const doub
  * (the solver's block width).  Allocates 3 n x max_cols work blocks.
  * lobpcg_chebyshev_apply has the lobpcg_precond_fn signature:
  *   lobpcg_set_precond_callback(h, lobpcg_chebyshev_apply, cheb);
+ * W may be R (the same pointer and leading dimension).
  * Errors: LOBPCG_ERR_ARG (degree outside 1..64, 0 < lmin < lmax violated,
  * ncols > max_cols or n different from the object's), LOBPCG_ERR_OOM. */
 typedef struct lobpcg_chebyshev* lobpcg_chebyshev_t;
@@ -286,7 +287,8 @@ int lobpcg_release_scratch(void);
 
 /* Block sparse product Y = A X for an n x m row-major block X (the A W and
  * B W products of Algorithm 8, Sec. 5.2), optionally also BY = diag(b) X
- * (b != NULL).  All pointers are device pointers. */
+ * (b != NULL).  All pointers are device pointers; nothing past the m columns of a
+ * row is read or written. */
 int lobpcg_spmm(int64_t n, const int32_t* rowptr, const int32_t* col, const double* val,
                 const double* X, int64_t ldx, int64_t m, double* Y, int64_t ldy,
                 const double* b, double* BY, int64_t ldby, void* stream);
